@@ -333,8 +333,8 @@ int lrvol_mlp_infer_timeout_test(const float *feat_dev, int64_t n, const uint16_
  * (LRVOL_MLP_PARAMS floats) and the loss (1 float); lrvol_mlp_train_step then
  * applies Adam (beta1 0.9, beta2 0.999, eps 1e-8, step count t >= 1) to params
  * with moment buffers m, v (LRVOL_MLP_PARAMS floats each, zero at t = 1).
- * scratch_dev must hold lrvol_mlp_scratch_floats(n) floats (activations, their
- * gradients and one gradient vector).  Batch n in 1 .. 2^20. */
+ * scratch_dev must hold lrvol_mlp_scratch_floats(n) floats (partial gradients
+ * and one gradient vector).  Batch n in 1 .. 2^20. */
 int64_t lrvol_mlp_scratch_floats(int64_t n);
 int lrvol_mlp_grad(const float *x_dev, const float *target_dev, int64_t n, const float *params_dev, float *grad_dev,
                    float *loss_dev, float *scratch_dev, void *stream);

@@ -751,26 +751,31 @@ int lrvol_mlp_check(void) {
   return fail(LRVOL_ERR_TIMEOUT, "a tensor-core wait of lrvol_mlp_infer ran out; its rows got multiplier 1");
 }
 
-// activations and their gradients (n x (6*64 + 2)), then one gradient vector
+// room for the partial gradients (n x (6*64 + 2)), then one gradient vector
 int64_t lrvol_mlp_scratch_floats(int64_t n) { return n < 0 ? 0 : n * (6 * (int64_t)kHid + 2) + kParams; }
+
+static int mlp_gradient(const float *x, const float *target, int64_t n, float *params, float *grad, float *loss,
+                        float *scratch, const AdamStep *adam, void *stream) {
+  if (!x || !target || !params || !grad || !scratch) return fail(LRVOL_ERR_ARG, "null pointer");
+  if (n < 1 || n > ((int64_t)1 << 20)) return fail(LRVOL_ERR_ARG, "batch must be 1 .. 2^20 rows");
+  CU(launch_mlp_grad(x, target, n, params, grad, loss, scratch, adam, (cudaStream_t)stream), "mlp training kernels");
+  return LRVOL_OK;
+}
 
 int lrvol_mlp_grad(const float *x, const float *target, int64_t n, const float *params, float *grad, float *loss,
                    float *scratch, void *stream) {
-  if (!x || !target || !params || !grad || !scratch) return fail(LRVOL_ERR_ARG, "null pointer");
-  if (n < 1 || n > ((int64_t)1 << 20)) return fail(LRVOL_ERR_ARG, "batch must be 1 .. 2^20 rows");
-  CU(launch_mlp_grad(x, target, n, params, grad, loss, scratch, (cudaStream_t)stream), "mlp grad kernels");
-  return LRVOL_OK;
+  // without an Adam step the parameters are only read
+  return mlp_gradient(x, target, n, const_cast<float *>(params), grad, loss, scratch, nullptr, stream);
 }
 
 int lrvol_mlp_train_step(const float *x, const float *target, int64_t n, float *params, float *m, float *vv,
                          int64_t t, float lr, float *loss, float *scratch, void *stream) {
   if (!m || !vv || t < 1 || !(lr > 0.f)) return fail(LRVOL_ERR_ARG, "bad optimiser arguments");
+  if (!scratch) return fail(LRVOL_ERR_ARG, "null pointer");
   // the gradient lands in the last kParams floats of the scratch
   float *grad = scratch + lrvol_mlp_scratch_floats(n) - kParams;
-  int rc = lrvol_mlp_grad(x, target, n, params, grad, loss, scratch, stream);
-  if (rc) return rc;
-  CU(launch_adam(params, grad, m, vv, t, lr, (cudaStream_t)stream), "adam kernel");
-  return LRVOL_OK;
+  const AdamStep adam = {m, vv, t, lr};
+  return mlp_gradient(x, target, n, params, grad, loss, scratch, &adam, stream);
 }
 
 int lrvol_labels(lrvol_t v, const lrvol_camera *cam, const lrvol_tf *tf, const lrvol_step *step, double h_fine,

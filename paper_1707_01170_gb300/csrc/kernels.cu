@@ -8,10 +8,11 @@
 //   k_eval         look-up + Bezier block evaluation at points.
 //   (k_render, the per-pixel ray casting of Sec. 4, is in render.cu; the
 //   device helpers both files use are in device_common.cuh.)
-//   k_features, k_mlp_infer, k_labels, k_dense_*, k_adam
+//   k_features, k_mlp_infer, k_labels
 //                  learned step multipliers (not in the paper; Eq. 4 stays the
 //                  base): per-element features, the network on the tcgen05
-//                  tensor cores, training labels and FP32 training.
+//                  tensor cores and training labels (its FP32 training is in
+//                  train.cu).
 //   k_streamlines, k_streamline_error, k_tube_*
 //                  Sec. 5 streamlines (Eq. 4 steps), the Eq. 7 error, tubes.
 //   k_trim_raster  Sec. 4.1 trimming: per-pixel interval of a boundary mesh.
@@ -425,8 +426,7 @@ cudaError_t launch_eval_grad(const lrvol_s *v, const float *pts, int64_t n, floa
 
 
 // ----------------------------------------------------------------------------
-// Learned step sizes: features, BF16 tensor-core inference, FP32 training,
-// fine-step labels.  The network is 16 -> 64 -> 64 -> 64 -> 1 (ReLU).
+// Learned step sizes: features, BF16 tensor-core inference, fine-step labels.  The network is 16 -> 64 -> 64 -> 64 -> 1 (ReLU).
 // ----------------------------------------------------------------------------
 namespace {
 
@@ -814,77 +814,6 @@ __global__ void __launch_bounds__(128 * kTcGroups, 4) k_mlp_infer(const float *_
   }
 }
 
-// ---- FP32 training (plain CUDA-core kernels; batch up to 2^20 rows) ----
-// out[b][j] = act(sum_k in[b][k] W[k][j] + bias[j])
-__global__ void k_dense_fwd(const float *__restrict__ in, int K, const float *__restrict__ W,
-                            const float *__restrict__ bias, int N, int64_t n, bool relu, float *__restrict__ out) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n * N) return;
-  const int64_t b = q / N;
-  const int j = (int)(q % N);
-  float acc = bias[j];
-  for (int k = 0; k < K; ++k) acc = fmaf(in[b * K + k], W[k * N + j], acc);
-  out[q] = relu ? fmaxf(acc, 0.f) : acc;
-}
-
-// dy[b] = (y[b] - t[b]) / n and the loss (one CTA, fixed order)
-__global__ void k_loss(const float *__restrict__ y, const float *__restrict__ tgt, int64_t n, float *__restrict__ dy,
-                       float *__restrict__ loss) {
-  __shared__ double red[256];
-  double acc = 0.0;
-  for (int64_t b = threadIdx.x; b < n; b += blockDim.x) {
-    const float r = y[b] - tgt[b];
-    dy[b] = r / (float)n;
-    acc += 0.5 * (double)r * (double)r;
-  }
-  red[threadIdx.x] = acc;
-  __syncthreads();
-  for (int s2 = blockDim.x / 2; s2 > 0; s2 >>= 1) {
-    if (threadIdx.x < s2) red[threadIdx.x] += red[threadIdx.x + s2];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && loss) *loss = (float)(red[0] / (double)n);
-}
-
-// gW[k][j] = sum_b in[b][k] d[b][j];  gb[j] = sum_b d[b][j]   (thread per (k, j), fixed order)
-__global__ void k_dense_wgrad(const float *__restrict__ in, int K, const float *__restrict__ d, int N, int64_t n,
-                              float *__restrict__ gW, float *__restrict__ gb) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= (K + 1) * N) return;
-  const int k = q / N, j = q % N;
-  float acc = 0.f;
-  if (k < K) {
-    for (int64_t b = 0; b < n; ++b) acc = fmaf(in[b * K + k], d[b * N + j], acc);
-    gW[k * N + j] = acc;
-  } else {
-    for (int64_t b = 0; b < n; ++b) acc += d[b * N + j];
-    gb[j] = acc;
-  }
-}
-
-// din[b][k] = (sum_j d[b][j] W[k][j]) * (in[b][k] > 0)   (in = post-ReLU activations)
-__global__ void k_dense_dgrad(const float *__restrict__ d, int N, const float *__restrict__ W,
-                              const float *__restrict__ in, int K, int64_t n, float *__restrict__ din) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n * K) return;
-  const int64_t b = q / K;
-  const int k = (int)(q % K);
-  float acc = 0.f;
-  for (int j = 0; j < N; ++j) acc = fmaf(d[b * N + j], W[k * N + j], acc);
-  din[q] = in[q] > 0.f ? acc : 0.f;
-}
-
-__global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, int count, float lr, float c1, float c2) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= count) return;
-  const float mq = 0.9f * m[q] + 0.1f * g[q];
-  const float vq = 0.999f * v[q] + 0.001f * g[q] * g[q];
-  m[q] = mq;
-  v[q] = vq;
-  p[q] -= lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
-}
-
 // ---- fine-step labels (scalar volumes, FP32 storage) ----
 struct SegState {
   uint32_t e;
@@ -1045,34 +974,6 @@ cudaError_t launch_mlp_infer(const float *x, int64_t n, const uint16_t *packed, 
   const int64_t blocks = std::min<int64_t>((tiles + kTcGroups - 1) / kTcGroups, 4 * (int64_t)sms);
   k_mlp_infer<<<(unsigned)std::max<int64_t>(blocks, 1), 128 * kTcGroups, kTcSmemBytes, s>>>(x, n, packed, ymin, ymax,
                                                                                            out, status, no_mma);
-  return cudaGetLastError();
-}
-
-// Scratch layout (floats): h1, h2, h3 (n x 64 each), y (n), dy (n), d3, d2, d1 (n x 64 each)
-cudaError_t launch_mlp_grad(const float *x, const float *target, int64_t n, const float *p, float *grad,
-                            float *loss, float *scratch, cudaStream_t s) {
-  float *h1 = scratch, *h2 = h1 + n * kHid, *h3 = h2 + n * kHid, *y = h3 + n * kHid, *dy = y + n;
-  float *d3 = dy + n, *d2 = d3 + n * kHid, *d1 = d2 + n * kHid;
-  const unsigned thr = 256;
-  auto blocks = [&](int64_t c) { return (unsigned)((c + thr - 1) / thr); };
-  k_dense_fwd<<<blocks(n * kHid), thr, 0, s>>>(x, kIn, p + kOffW1, p + kOffB1, kHid, n, true, h1);
-  k_dense_fwd<<<blocks(n * kHid), thr, 0, s>>>(h1, kHid, p + kOffW2, p + kOffB2, kHid, n, true, h2);
-  k_dense_fwd<<<blocks(n * kHid), thr, 0, s>>>(h2, kHid, p + kOffW3, p + kOffB3, kHid, n, true, h3);
-  k_dense_fwd<<<blocks(n), thr, 0, s>>>(h3, kHid, p + kOffW4, p + kOffB4, 1, n, false, y);
-  k_loss<<<1, 256, 0, s>>>(y, target, n, dy, loss);
-  k_dense_wgrad<<<blocks((kHid + 1) * 1), thr, 0, s>>>(h3, kHid, dy, 1, n, grad + kOffW4, grad + kOffB4);
-  k_dense_dgrad<<<blocks(n * kHid), thr, 0, s>>>(dy, 1, p + kOffW4, h3, kHid, n, d3);
-  k_dense_wgrad<<<blocks((kHid + 1) * kHid), thr, 0, s>>>(h2, kHid, d3, kHid, n, grad + kOffW3, grad + kOffB3);
-  k_dense_dgrad<<<blocks(n * kHid), thr, 0, s>>>(d3, kHid, p + kOffW3, h2, kHid, n, d2);
-  k_dense_wgrad<<<blocks((kHid + 1) * kHid), thr, 0, s>>>(h1, kHid, d2, kHid, n, grad + kOffW2, grad + kOffB2);
-  k_dense_dgrad<<<blocks(n * kHid), thr, 0, s>>>(d2, kHid, p + kOffW2, h1, kHid, n, d1);
-  k_dense_wgrad<<<blocks((kIn + 1) * kHid), thr, 0, s>>>(x, kIn, d1, kHid, n, grad + kOffW1, grad + kOffB1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_adam(float *params, const float *grad, float *m, float *v, int64_t t, float lr, cudaStream_t s) {
-  const float c1 = 1.f - powf(0.9f, (float)t), c2 = 1.f - powf(0.999f, (float)t);
-  k_adam<<<(kParams + 255) / 256, 256, 0, s>>>(params, grad, m, v, kParams, lr, c1, c2);
   return cudaGetLastError();
 }
 

@@ -300,9 +300,14 @@ cudaError_t launch_mlp_infer(const float *x, int64_t n, const uint16_t *packed, 
                              uint32_t *status, cudaStream_t s, bool no_mma = false);
 // the library's status word for lrvol_mlp_infer calls (device address)
 uint32_t *mlp_status_word();
-cudaError_t launch_mlp_grad(const float *x, const float *target, int64_t n, const float *params, float *grad,
-                            float *loss, float *scratch, cudaStream_t s);
-cudaError_t launch_adam(float *params, const float *grad, float *m, float *v, int64_t t, float lr, cudaStream_t s);
+// train.cu: the gradient and loss of a batch, and with `adam` one step of p
+struct AdamStep {
+  float *m, *v;
+  int64_t t;
+  float lr;
+};
+cudaError_t launch_mlp_grad(const float *x, const float *target, int64_t n, float *p, float *grad, float *loss,
+                            float *scratch, const AdamStep *adam, cudaStream_t s);
 cudaError_t launch_labels(const RenderParams &prm, int degree, float h_fine, float tau, const float *cand, int n_cand,
                           int32_t *label, cudaStream_t s);
 
