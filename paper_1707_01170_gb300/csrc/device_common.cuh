@@ -300,8 +300,10 @@ __device__ __forceinline__ unsigned short f16_bits(float x) { return __half_as_u
 //   FP16 blocks (MIXED) stay as 16-bit pairs in registers (half the registers
 //   of FP32 values), and the first contraction stage multiplies them with the
 //   x monomials rounded to FP16 in mixed-precision FMAs (exact products, FP32
-//   sums); the later stages run in FP32 as for the other storages.
-template <int P, int FIELD, int STORE>
+//   sums); the later stages run in FP32 as for the other storages.  Point
+//   evaluation, which reads a block once, converts FP16 values instead (MIX
+//   false): nothing but their storage is rounded.
+template <int P, int FIELD, int STORE, bool MIX = STORE == LRVOL_STORE_F16>
 struct Block {
   static constexpr int N = P + 1;
   static constexpr int NB = N * N * N;
@@ -314,7 +316,7 @@ struct Block {
   static constexpr int PAIRF = (2 * NB + 7) & ~7;          // slots of the component pair block
   static constexpr int C2F = (NB + 7) & ~7;                // slots of one plain component
 
-  static constexpr bool MIXED = STORE == LRVOL_STORE_F16;
+  static constexpr bool MIXED = MIX;
   f2 rp[ROWPAIR && !MIXED ? 8 : 1][4];       // row pairs (2m, 2m+1), value i
   unsigned rh[ROWPAIR && MIXED ? 8 : 1][4];  // MIXED: FP16 words (row 2m, row 2m+1), value i
   float sg[SCALAR_GENERIC && !MIXED ? ((SGF + 7) & ~7) : 1];

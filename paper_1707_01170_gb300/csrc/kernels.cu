@@ -4,10 +4,9 @@
 //                  coefficients of every incident B-spline's univariate factors
 //                  over the element, by blossoming, accumulated with gamma*c.
 //   k_elem_records element boxes -> FP32 records (rounded-up corners, Eq. 4 step).
-//   k_lookup       Alg. 1 element look-up through the k-d forest.
-//   k_eval         look-up + Bezier block evaluation at points.
-//   (k_render, the per-pixel ray casting of Sec. 4, is in render.cu; the
-//   device helpers both files use are in device_common.cuh.)
+//   (k_render, the per-pixel ray casting of Sec. 4, is in render.cu, look-up
+//   and evaluation at points in points.cu; the device helpers these files
+//   share are in device_common.cuh.)
 //   k_features, k_mlp_infer, k_labels
 //                  learned step multipliers (not in the paper; Eq. 4 stays the
 //                  base): per-element features, the network on the tcgen05
@@ -210,175 +209,6 @@ __global__ void k_elem_records(const double *__restrict__ box, int64_t n_elem, i
   out[e] = r;
 }
 
-
-__global__ void k_lookup(ForestView f, int64_t n_elem, const float *__restrict__ pts, int64_t n,
-                         uint32_t *__restrict__ out, uint32_t *status) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  const float x = pts[3 * q], y = pts[3 * q + 1], z = pts[3 * q + 2];
-  uint32_t e = kNone;
-  if (x >= 0.f && x <= 1.f && y >= 0.f && y <= 1.f && z >= 0.f && z <= 1.f) {
-    e = forest_lookup(f, x, y, z, status);
-    if (e != kNone && (int64_t)e >= n_elem) {
-      set_status(status, kStatusBounds);
-      e = kNone;
-    }
-  }
-  out[q] = e;
-}
-
-
-// Generic-degree evaluation for the point kernel (any p0,p1,p2 <= 4).
-__device__ float eval_generic(const float *c, const int *deg, float ux, float uy, float uz) {
-  float b[3][kMaxDeg + 1];
-  const float u[3] = {ux, uy, uz};
-  for (int a = 0; a < 3; ++a) {
-    const int p = deg[a];
-    const float v = 1.f - u[a];
-    for (int i = 0; i <= p; ++i) {
-      float m = 1.f;
-      for (int q = 0; q < i; ++q) m *= u[a];
-      for (int q = i; q < p; ++q) m *= v;
-      b[a][i] = m;
-    }
-  }
-  const int n0 = deg[0] + 1, n1 = deg[1] + 1, n2 = deg[2] + 1;
-  float f = 0.f;
-  for (int k = 0; k < n2; ++k) {
-    float t = 0.f;
-    for (int j = 0; j < n1; ++j) {
-      float s = 0.f;
-      for (int i = 0; i < n0; ++i) s = fmaf(c[(k * n1 + j) * n0 + i], b[0][i], s);
-      t = fmaf(s, b[1][j], t);
-    }
-    f = fmaf(t, b[2][k], f);
-  }
-  return f;
-}
-
-// Value and derivatives in local coordinates (d/du, d/dv, d/dw) of the same block.
-__device__ float eval_generic_grad(const float *c, const int *deg, float ux, float uy, float uz, float *g) {
-  float b[3][kMaxDeg + 1], db[3][kMaxDeg + 1];
-  const float u[3] = {ux, uy, uz};
-  for (int a = 0; a < 3; ++a) {
-    const int p = deg[a];
-    const float v = 1.f - u[a];
-    for (int i = 0; i <= p; ++i) {
-      float m = 1.f, d1 = 0.f, d2 = 0.f;
-      for (int q = 0; q < i; ++q) m *= u[a];
-      for (int q = i; q < p; ++q) m *= v;
-      if (i > 0) {  // i u^(i-1) v^(p-i)
-        d1 = (float)i;
-        for (int q = 0; q < i - 1; ++q) d1 *= u[a];
-        for (int q = i; q < p; ++q) d1 *= v;
-      }
-      if (i < p) {  // (p-i) u^i v^(p-i-1)
-        d2 = (float)(p - i);
-        for (int q = 0; q < i; ++q) d2 *= u[a];
-        for (int q = i + 1; q < p; ++q) d2 *= v;
-      }
-      b[a][i] = m;
-      db[a][i] = d1 - d2;
-    }
-  }
-  const int n0 = deg[0] + 1, n1 = deg[1] + 1, n2 = deg[2] + 1;
-  float f = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-  for (int k = 0; k < n2; ++k) {
-    float t = 0.f, tx = 0.f, ty = 0.f;
-    for (int j = 0; j < n1; ++j) {
-      float s = 0.f, sx = 0.f;
-      for (int i = 0; i < n0; ++i) {
-        const float cc = c[(k * n1 + j) * n0 + i];
-        s = fmaf(cc, b[0][i], s);
-        sx = fmaf(cc, db[0][i], sx);
-      }
-      t = fmaf(s, b[1][j], t);
-      tx = fmaf(sx, b[1][j], tx);
-      ty = fmaf(s, db[1][j], ty);
-    }
-    f = fmaf(t, b[2][k], f);
-    gx = fmaf(tx, b[2][k], gx);
-    gy = fmaf(ty, b[2][k], gy);
-    gz = fmaf(t, db[2][k], gz);
-  }
-  g[0] = gx;
-  g[1] = gy;
-  g[2] = gz;
-  return f;
-}
-
-__device__ __forceinline__ float load_slot(const unsigned char *eb, int storage, int slot) {
-  if (storage == LRVOL_STORE_F32) return __ldg(reinterpret_cast<const float *>(eb) + slot);
-  const unsigned short h = __ldg(reinterpret_cast<const unsigned short *>(eb + kHeaderBytes) + slot);
-  if (storage == LRVOL_STORE_F16) return __half2float(__ushort_as_half(h));
-  return __uint_as_float((unsigned)h << 16);
-}
-
-__global__ void k_eval(ForestView f, const ElemRec *__restrict__ elem, int64_t n_elem,
-                       const unsigned char *__restrict__ bez, int ebytes, int storage, int p0, int p1, int p2, int nc,
-                       const float *__restrict__ pts, int64_t n, float *__restrict__ out, uint32_t *status) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  const float x = pts[3 * q], y = pts[3 * q + 1], z = pts[3 * q + 2];
-  uint32_t e = kNone;
-  if (x >= 0.f && x <= 1.f && y >= 0.f && y <= 1.f && z >= 0.f && z <= 1.f) e = forest_lookup(f, x, y, z, status);
-  if (e == kNone || (int64_t)e >= n_elem) {
-    for (int c = 0; c < nc; ++c) out[q * nc + c] = 0.f;
-    return;
-  }
-  const ElemRec r = elem[e];
-  const float ux = local_u(x, r.a.x, r.c.x, r.d.x);
-  const float uy = local_u(y, r.a.y, r.c.y, r.d.y);
-  const float uz = local_u(z, r.a.z, r.c.z, r.d.z);
-  const int deg[3] = {p0, p1, p2};
-  const int n0 = p0 + 1, n1 = p1 + 1, nb = n0 * n1 * (p2 + 1);
-  const unsigned char *eb = bez + (int64_t)e * ebytes;
-  for (int c = 0; c < nc; ++c) {
-    float cl[(kMaxDeg + 1) * (kMaxDeg + 1) * (kMaxDeg + 1)];
-    for (int t = 0; t < nb; ++t) cl[t] = load_slot(eb, storage, render_slot(nc, n0, nb, t / n0, t % n0, c));
-    const float v = eval_generic(cl, deg, ux, uy, uz);
-    if (storage == LRVOL_STORE_F32) {
-      out[q * nc + c] = v;
-    } else {
-      const float *hdr = reinterpret_cast<const float *>(eb);
-      out[q * nc + c] = fmaf(__ldg(hdr + 3 + c), v, __ldg(hdr + c));
-    }
-  }
-}
-
-// Value and world-space gradient of a scalar volume at points (n x 4 out).
-__global__ void k_eval_grad(ForestView f, const ElemRec *__restrict__ elem, int64_t n_elem,
-                            const unsigned char *__restrict__ bez, int ebytes, int storage, int p0, int p1, int p2,
-                            const float *__restrict__ pts, int64_t n, float *__restrict__ out, uint32_t *status) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= n) return;
-  const float x = pts[3 * q], y = pts[3 * q + 1], z = pts[3 * q + 2];
-  uint32_t e = kNone;
-  if (x >= 0.f && x <= 1.f && y >= 0.f && y <= 1.f && z >= 0.f && z <= 1.f) e = forest_lookup(f, x, y, z, status);
-  float4 *o = reinterpret_cast<float4 *>(out) + q;
-  if (e == kNone || (int64_t)e >= n_elem) {
-    *o = make_float4(0.f, 0.f, 0.f, 0.f);
-    return;
-  }
-  const ElemRec r = elem[e];
-  const int deg[3] = {p0, p1, p2};
-  const int n0 = p0 + 1, nb = n0 * (p1 + 1) * (p2 + 1);
-  const unsigned char *eb = bez + (int64_t)e * ebytes;
-  float cl[(kMaxDeg + 1) * (kMaxDeg + 1) * (kMaxDeg + 1)];
-  for (int t = 0; t < nb; ++t) cl[t] = load_slot(eb, storage, render_slot(1, n0, nb, t / n0, t % n0, 0));
-  float g[3];
-  float v = eval_generic_grad(cl, deg, local_u(x, r.a.x, r.c.x, r.d.x), local_u(y, r.a.y, r.c.y, r.d.y),
-                              local_u(z, r.a.z, r.c.z, r.d.z), g);
-  float sc = 1.f;
-  if (storage != LRVOL_STORE_F32) {
-    const float *hdr = reinterpret_cast<const float *>(eb);
-    sc = __ldg(hdr + 3);
-    v = fmaf(sc, v, __ldg(hdr));
-  }
-  *o = make_float4(v, sc * g[0] * r.d.x, sc * g[1] * r.d.y, sc * g[2] * r.d.z);
-}
-
-
 }  // namespace
 
 cudaError_t launch_to_bezier(const lrvol_s *v, cudaStream_t s) {
@@ -404,26 +234,6 @@ cudaError_t launch_elem_records(const lrvol_s *v, cudaStream_t s) {
   k_elem_records<<<(unsigned)((v->n_elem + 255) / 256), 256, 0, s>>>(v->d_box, v->n_elem, d, v->d_elem);
   return cudaGetLastError();
 }
-
-cudaError_t launch_lookup(const lrvol_s *v, const float *pts, int64_t n, uint32_t *out, cudaStream_t s) {
-  k_lookup<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(forest_view(v), v->n_elem, pts, n, out, v->d_status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_eval(const lrvol_s *v, const float *pts, int64_t n, float *out, cudaStream_t s) {
-  k_eval<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(forest_view(v), v->d_elem, v->n_elem, v->d_bez,
-                                                    v->elem_bytes, v->storage, v->p[0], v->p[1], v->p[2],
-                                                    v->nc, pts, n, out, v->d_status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_eval_grad(const lrvol_s *v, const float *pts, int64_t n, float *out, cudaStream_t s) {
-  k_eval_grad<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(forest_view(v), v->d_elem, v->n_elem, v->d_bez,
-                                                         v->elem_bytes, v->storage, v->p[0], v->p[1], v->p[2], pts,
-                                                         n, out, v->d_status);
-  return cudaGetLastError();
-}
-
 
 // ----------------------------------------------------------------------------
 // Learned step sizes: features, BF16 tensor-core inference, fine-step labels.  The network is 16 -> 64 -> 64 -> 64 -> 1 (ReLU).
