@@ -26,20 +26,23 @@ __device__ __forceinline__ void set_status(uint32_t *status, uint32_t code) { at
 // Element holding the FP32 point (x, y, z), each coordinate in [0, 1] (every
 // caller clamps or checks first): head word of its block, then the tree walk.
 __device__ __forceinline__ uint32_t forest_lookup(const ForestView &f, float x, float y, float z, uint32_t *status) {
-  // block index floor(p * blocks) (0 <= p <= 1, blocks <= 1024) as 2^23 + floor
-  // by a round-down add, without a float-int conversion
-  const int bx = min(__float_as_int(__fadd_rd(x * f.fbx, 8388608.f)) - 0x4b000000, f.bx - 1);
-  const int by = min(__float_as_int(__fadd_rd(y * f.fby, 8388608.f)) - 0x4b000000, f.by - 1);
-  const int bz = min(__float_as_int(__fadd_rd(z * f.fbz, 8388608.f)) - 0x4b000000, f.bz - 1);
-  uint32_t w = __ldg(f.head + ((int64_t)bz * f.by + by) * f.bx + bx);
-  for (int depth = 0; !(w & kLeaf); ++depth) {
-    if ((int64_t)w >= f.n_nodes || depth >= kMaxDepth) {
-      set_status(status, kStatusBounds);
-      return kNone;
-    }
+  // block index floor(p * blocks) (blocks a power of two <= 1024, so the
+  // product is exact) as the low bits of 2^23 + floor by a round-down FMA; the
+  // index of p = 1 falls on the table's last, repeated layer.  The three
+  // offsets of 2^23's bits are taken off by f.head_bias, modulo 2^32.
+  const uint32_t hx = __float_as_uint(__fmaf_rd(x, f.fbx, 8388608.f));
+  const uint32_t hy = __float_as_uint(__fmaf_rd(y, f.fby, 8388608.f));
+  const uint32_t hz = __float_as_uint(__fmaf_rd(z, f.fbz, 8388608.f));
+  uint32_t w = __ldg(f.head + (hz * f.head_sz + (hy * f.head_sy + (hx - f.head_bias))));
+  // one exit: a leaf and a word outside the tree both compare >= n_nodes < 2^31
+  for (int depth = 0; w < f.n_nodes && depth < kMaxDepth; ++depth) {
     const uint4 n = __ldg(f.nodes + w);
     const float pa = n.y == 0 ? x : (n.y == 1 ? y : z);
     w = pa < __uint_as_float(n.x) ? n.z : n.w;
+  }
+  if (!(w & kLeaf)) {
+    set_status(status, kStatusBounds);
+    return kNone;
   }
   return w & ~kLeaf;
 }
@@ -131,6 +134,13 @@ __device__ __forceinline__ float lg2_approx(float x) {
   return y;
 }
 
+// a * b + c rounded once, then clamped to [0, 1] by the same instruction (NaN gives 0)
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+  float d;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 struct Ray {
   float o[3], d[3], tin, tout;
 };
@@ -175,40 +185,41 @@ __device__ __forceinline__ bool make_ray(const RayConsts &K, int i, int j, Ray &
   return hit && tin < tout;
 }
 
-// Transfer function lookup and one Alg. 2 update in transmittance form
-// (Tr = 1 - alpha_dst): w = (1 - T) Tr, C += w C_src, Tr *= T.
-__device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, float v, float seg,
-                                          const RenderParams &prm, float &C0, float &C1, float &C2, float &Tr) {
-  const float x = fminf(fmaxf(fmaf(v, prm.tf_scale, prm.tf_bias), 0.f), 255.f);
-  // floor(x) without a float-int conversion (those issue on the narrow XU
-  // pipe): adding 2^23 rounding down leaves 2^23 + floor(x) exactly
-  const float r = __fadd_rd(x, 8388608.f);
-  const int q = min(__float_as_int(r) - 0x4b000000, 254);
-  const float fr = x - fminf(__fsub_rn(r, 8388608.f), 254.f);
-  const float4 e0 = tfb[q], de = tfd[q];
-  const float sa = fmaf(fr, de.w, e0.w);
-  const float T = ex2_approx(lg2_approx(fmaxf(1.f - sa, 0.f)) * (seg * prm.inv_xi));
-  const float w = fmaf(-Tr, T, Tr);
-  C0 = fmaf(w, fmaf(fr, de.x, e0.x), C0);
-  C1 = fmaf(w, fmaf(fr, de.y, e0.y), C1);
-  C2 = fmaf(w, fmaf(fr, de.z, e0.z), C2);
-  Tr *= T;
+// The TF in shared memory: entry i and the difference to entry i + 1 (0 at the
+// last), and entry 256 of zeros (kTfNothing).
+constexpr int kTfEntries = 257;
+__device__ __forceinline__ void load_tf(const RenderParams &prm, float4 *tfb, float4 *tfd) {
+  for (int q = threadIdx.x; q < 256; q += blockDim.x) {
+    const float4 e0 = prm.tf[q], e1 = prm.tf[q < 255 ? q + 1 : 255];
+    tfb[q] = e0;
+    tfd[q] = make_float4(e1.x - e0.x, e1.y - e0.y, e1.z - e0.z, e1.w - e0.w);
+  }
+  if (threadIdx.x == 0) tfb[256] = tfd[256] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Alg. 2 with C_src multiplied by the shading intensity sh (Sec. 4.1).
-__device__ __forceinline__ void composite_shaded(const float4 *tfb, const float4 *tfd, float v, float seg, float sh,
-                                                 const RenderParams &prm, float &C0, float &C1, float &C2,
-                                                 float &Tr) {
-  const float x = fminf(fmaxf(fmaf(v, prm.tf_scale, prm.tf_bias), 0.f), 255.f);
-  // floor(x) without a float-int conversion (those issue on the narrow XU
-  // pipe): adding 2^23 rounding down leaves 2^23 + floor(x) exactly
-  const float r = __fadd_rd(x, 8388608.f);
-  const int q = min(__float_as_int(r) - 0x4b000000, 254);
-  const float fr = x - fminf(__fsub_rn(r, 8388608.f), 254.f);
+// TF coordinate of a field value, in [0, 1].
+__device__ __forceinline__ float tf_coord(const RenderParams &prm, float v) {
+  return fma_sat(v, prm.tf_scale, prm.tf_bias);
+}
+// The coordinate that reads the table's extra entry: no opacity, no colour.
+constexpr float kTfNothing = 256.5f / 255.f;
+
+// One Alg. 2 update in transmittance form (Tr = 1 - alpha_dst) for a sample of
+// TF coordinate x: w = (1 - T) Tr, C += w C_src, Tr *= T; with SHADE, C_src is
+// multiplied by the intensity sh (Sec. 4.1).
+template <bool SHADE>
+__device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, float x, float seg, float sh,
+                                          const RenderParams &prm, float &C0, float &C1, float &C2, float &Tr) {
+  // entry floor(255 x) without a float-int conversion (those issue on the
+  // narrow XU pipe): 255 x + 2^23 rounded down is 2^23 + floor(255 x) exactly;
+  // x = 1 reads entry 255, whose difference is 0
+  const float r = __fmaf_rd(x, 255.f, 8388608.f);
+  const int q = __float_as_int(r) - 0x4b000000;
+  const float fr = __fmaf_rn(x, 255.f, __fsub_rn(8388608.f, r));
   const float4 e0 = tfb[q], de = tfd[q];
   const float sa = fmaf(fr, de.w, e0.w);
   const float T = ex2_approx(lg2_approx(fmaxf(1.f - sa, 0.f)) * (seg * prm.inv_xi));
-  const float w = fmaf(-Tr, T, Tr) * sh;
+  const float w = SHADE ? fmaf(-Tr, T, Tr) * sh : fmaf(-Tr, T, Tr);
   C0 = fmaf(w, fmaf(fr, de.x, e0.x), C0);
   C1 = fmaf(w, fmaf(fr, de.y, e0.y), C1);
   C2 = fmaf(w, fmaf(fr, de.z, e0.z), C2);
@@ -317,6 +328,8 @@ struct Block {
   static constexpr int C2F = (NB + 7) & ~7;                // slots of one plain component
 
   static constexpr bool MIXED = MIX;
+  // bytes of an element's block, as launch_pack lays it out (FIELD 2: of the per-component copy)
+  static constexpr int BYTES = elem_bytes(STORE, FIELD == 2 ? 3 * C2F : render_slots(FIELD == 1 ? 3 : 1, N, N, N));
   f2 rp[ROWPAIR && !MIXED ? 8 : 1][4];       // row pairs (2m, 2m+1), value i
   unsigned rh[ROWPAIR && MIXED ? 8 : 1][4];  // MIXED: FP16 words (row 2m, row 2m+1), value i
   float sg[SCALAR_GENERIC && !MIXED ? ((SGF + 7) & ~7) : 1];

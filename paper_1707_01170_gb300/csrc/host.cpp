@@ -138,13 +138,23 @@ float round_up_f32(double x) {
 struct ForestBuilder {
   const lrvol_s *v;
   std::vector<Node> nodes;
-  std::vector<uint32_t> head;
+  std::vector<uint32_t> head;  // as ForestView::head
   std::vector<int32_t> depth;  // per block
   int B[3];
   bool midpoint = false;       // octree-style splits (LRVOL_SPLIT_MIDPOINT)
   bool unresolved = false;     // a midpoint tree reached kMaxDepth
 
   const double *box(int32_t e) const { return &v->box[6 * (size_t)e]; }
+  size_t head_at(int x, int y, int z) const { return ((size_t)z * (B[1] + 1) + y) * (B[0] + 1) + x; }
+
+  // The repeated last layer of each axis.
+  void pad_head() {
+    for (int z = 0; z < B[2]; ++z)
+      for (int y = 0; y < B[1]; ++y) head[head_at(B[0], y, z)] = head[head_at(B[0] - 1, y, z)];
+    for (int z = 0; z < B[2]; ++z)
+      std::copy_n(head.begin() + head_at(0, B[1] - 1, z), B[0] + 1, head.begin() + head_at(0, B[1], z));
+    std::copy_n(head.begin() + head_at(0, 0, B[2] - 1), head_at(0, 0, 1), head.begin() + head_at(0, 0, B[2]));
+  }
 
   // Build a tree over `els` inside region [rlo, rhi); returns a reference.
   uint32_t build(std::vector<int32_t> &els, const double *rlo, const double *rhi, int d, int *maxd) {
@@ -264,9 +274,8 @@ struct ForestBuilder {
       for (int z = b0[2]; z < b1[2]; ++z)
         for (int y = b0[1]; y < b1[1]; ++y)
           for (int x = b0[0]; x < b1[0]; ++x) {
-            size_t q = ((size_t)z * B[1] + y) * B[0] + x;
-            head[q] = kLeaf | (uint32_t)els[0];
-            depth[q] = 0;
+            head[head_at(x, y, z)] = kLeaf | (uint32_t)els[0];
+            depth[((size_t)z * B[1] + y) * B[0] + x] = 0;
           }
       return true;
     }
@@ -280,9 +289,8 @@ struct ForestBuilder {
       int maxd = 0;
       uint32_t r = build(els, lo, hi, 0, &maxd);
       if (r == kNone) return false;
-      size_t q = ((size_t)b0[2] * B[1] + b0[1]) * B[0] + b0[0];
-      head[q] = r;
-      depth[q] = maxd;
+      head[head_at(b0[0], b0[1], b0[2])] = r;
+      depth[((size_t)b0[2] * B[1] + b0[1]) * B[0] + b0[0]] = maxd;
       return true;
     }
     int a = 0;
@@ -343,10 +351,10 @@ ForestView forest_view(const lrvol_s *v) {
   ForestView f;
   f.head = v->d_head;
   f.nodes = v->d_nodes;
-  f.n_nodes = v->n_nodes;
-  f.bx = v->blocks[0];
-  f.by = v->blocks[1];
-  f.bz = v->blocks[2];
+  f.n_nodes = (uint32_t)v->n_nodes;
+  f.head_sy = (uint32_t)v->blocks[0] + 1;
+  f.head_sz = f.head_sy * ((uint32_t)v->blocks[1] + 1);
+  f.head_bias = 0x4b000000u * (1u + f.head_sy + f.head_sz);
   f.fbx = (float)v->blocks[0];
   f.fby = (float)v->blocks[1];
   f.fbz = (float)v->blocks[2];
@@ -399,9 +407,7 @@ int prepare_render(const lrvol_s *v, const lrvol_camera *cam, const lrvol_tf *tf
   prm->elem = v->d_elem;
   prm->n_elem = v->n_elem;
   prm->bez = v->d_bez;
-  prm->elem_bytes = v->elem_bytes;
   prm->bezc = v->d_bezc;
-  prm->elemc_bytes = v->elemc_bytes;
   prm->comp = field == LRVOL_FIELD_COMPONENT ? step->component : 0;
   prm->forest = forest_view(v);
   prm->out = rgba_dev;
@@ -417,8 +423,8 @@ int prepare_render(const lrvol_s *v, const lrvol_camera *cam, const lrvol_tf *tf
   prm->h = (float)step->h;
   prm->inv_xi = (float)(1.0 / step->xi);
   prm->alpha_stop = (float)step->alpha_stop;
-  prm->tf_scale = (float)(255.0 / (tf->vmax - tf->vmin));
-  prm->tf_bias = (float)(-tf->vmin * 255.0 / (tf->vmax - tf->vmin));
+  prm->tf_scale = (float)(1.0 / (tf->vmax - tf->vmin));
+  prm->tf_bias = (float)(-tf->vmin / (tf->vmax - tf->vmin));
   for (int q = 0; q < 256; ++q) prm->tf[q] = make_float4(tf->rgba[q][0], tf->rgba[q][1], tf->rgba[q][2], tf->rgba[q][3]);
   prm->trim = reinterpret_cast<const float2 *>(step->trim);
   if (step->shading == LRVOL_SHADE_GRADIENT) {
@@ -554,7 +560,7 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   fb.midpoint = split == LRVOL_SPLIT_MIDPOINT;
   for (int a = 0; a < 3; ++a) fb.B[a] = blocks[a];
   size_t nblk = (size_t)blocks[0] * blocks[1] * blocks[2];
-  fb.head.assign(nblk, kNone);
+  fb.head.assign(fb.head_at(0, 0, blocks[2] + 1), kNone);
   fb.depth.assign(nblk, 0);
   std::vector<int32_t> all(v->n_elem);
   std::iota(all.begin(), all.end(), 0);
@@ -564,6 +570,7 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
       return fail(LRVOL_ERR_UNSUPPORTED, "midpoint splits do not resolve this mesh (faces at non-dyadic coordinates)");
     return fail(LRVOL_ERR_ARG, "elements do not form a box partition of [0,1]^3");
   }
+  fb.pad_head();
   for (uint32_t h : fb.head)
     if (h == kNone) return fail(LRVOL_ERR_ARG, "a forest block holds no element");
   if (fb.nodes.size() >= kLeaf) return fail(LRVOL_ERR_ARG, "forest too large");
@@ -581,10 +588,10 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   // from here the previous forest is replaced: until the new one is complete
   // the handle has none (a failed host build above left the previous one)
   v->have_accel = false;
-  if ((rc = dev_alloc(v, &v->d_head, nblk, "alloc forest head")) ||
+  if ((rc = dev_alloc(v, &v->d_head, fb.head.size(), "alloc forest head")) ||
       (rc = dev_alloc(v, &v->d_nodes, fb.nodes.size(), "alloc forest nodes")))
     return rc;
-  CU(cudaMemcpyAsync(v->d_head, fb.head.data(), sizeof(uint32_t) * nblk, cudaMemcpyHostToDevice, st), "upload head");
+  CU(cudaMemcpyAsync(v->d_head, fb.head.data(), sizeof(uint32_t) * fb.head.size(), cudaMemcpyHostToDevice, st), "upload head");
   if (!fb.nodes.empty())
     CU(cudaMemcpyAsync(v->d_nodes, fb.nodes.data(), sizeof(Node) * fb.nodes.size(), cudaMemcpyHostToDevice, st),
        "upload nodes");
@@ -800,7 +807,6 @@ int lrvol_labels(lrvol_t v, const lrvol_camera *cam, const lrvol_tf *tf, const l
   prm.elem = v->d_elem;
   prm.n_elem = v->n_elem;
   prm.bez = v->d_bez;
-  prm.elem_bytes = v->elem_bytes;
   prm.forest = forest_view(v);
   prm.width = cam->width;
   prm.height = cam->height;
@@ -812,8 +818,8 @@ int lrvol_labels(lrvol_t v, const lrvol_camera *cam, const lrvol_tf *tf, const l
   prm.mode = LRVOL_STEP_HEURISTIC;
   prm.inv_xi = (float)(1.0 / step->xi);
   prm.alpha_stop = (float)step->alpha_stop;
-  prm.tf_scale = (float)(255.0 / (tf->vmax - tf->vmin));
-  prm.tf_bias = (float)(-tf->vmin * 255.0 / (tf->vmax - tf->vmin));
+  prm.tf_scale = (float)(1.0 / (tf->vmax - tf->vmin));
+  prm.tf_bias = (float)(-tf->vmin / (tf->vmax - tf->vmin));
   prm.counters = v->d_counters;
   prm.status = v->d_status;
   for (int q = 0; q < 256; ++q) prm.tf[q] = make_float4(tf->rgba[q][0], tf->rgba[q][1], tf->rgba[q][2], tf->rgba[q][3]);
@@ -879,7 +885,6 @@ int lrvol_streamlines(lrvol_t v, const lrvol_streamline_params *P, const double 
   sp.elem = v->d_elem;
   sp.n_elem = v->n_elem;
   sp.bez = v->d_bez;
-  sp.elem_bytes = v->elem_bytes;
   sp.forest = forest_view(v);
   sp.status = v->d_status;
   sp.queue = v->d_counters + kCntQueue;
@@ -913,7 +918,6 @@ int lrvol_tubes(lrvol_t v, const lrvol_camera *cam, const double *samples, const
   tp.field.elem = v->d_elem;
   tp.field.n_elem = v->n_elem;
   tp.field.bez = v->d_bez;
-  tp.field.elem_bytes = v->elem_bytes;
   tp.field.forest = forest_view(v);
   tp.field.status = v->d_status;
   camera_consts(cam, &tp.ray);

@@ -637,13 +637,13 @@ __device__ __forceinline__ bool seg_locate(const RenderParams &prm, SegState &st
                       py < st.rb.y && pz < st.rb.z;
   if (inside) return true;
   const uint32_t e = forest_lookup(prm.forest, px, py, pz, prm.status);
-  if (e == kNone || (int64_t)e >= prm.n_elem) {
+  if (e >= (uint32_t)prm.n_elem) {   // kNone included
     set_status(prm.status, kStatusBounds);
     return false;
   }
   st.e = e;
   load_record(prm.elem + e, st.ra, st.rb, st.rc, st.rd);
-  blk.load(prm.bez + (int64_t)e * prm.elem_bytes, 0);
+  blk.load(prm.bez + (int64_t)e * blk.BYTES, 0);
   return true;
 }
 
@@ -658,9 +658,9 @@ __device__ void seg_composite(const RenderParams &prm, const Ray &ray, const flo
   for (int k = 0; k < kMaxSamplesPerRay; ++k) {
     const float t = __fmaf_rn((float)k, h, ta);
     if (!(t < tb)) break;
-    const float px = fminf(fmaxf(__fmaf_rn(t, ray.d[0], ray.o[0]), 0.f), 1.f);
-    const float py = fminf(fmaxf(__fmaf_rn(t, ray.d[1], ray.o[1]), 0.f), 1.f);
-    const float pz = fminf(fmaxf(__fmaf_rn(t, ray.d[2], ray.o[2]), 0.f), 1.f);
+    const float px = fma_sat(t, ray.d[0], ray.o[0]);
+    const float py = fma_sat(t, ray.d[1], ray.o[1]);
+    const float pz = fma_sat(t, ray.d[2], ray.o[2]);
     if (!seg_locate<P>(prm, st, blk, px, py, pz)) return;
     float bx[N], by[N], bz[N];
     monomials<P>(local_u(px, st.ra.x, st.rc.x, st.rd.x), bx);
@@ -668,7 +668,7 @@ __device__ void seg_composite(const RenderParams &prm, const Ray &ray, const flo
     monomials<P>(local_u(pz, st.ra.z, st.rc.z, st.rd.z), bz);
     const float v = blk.eval(bx, by, bz);
     const float tn = __fmaf_rn((float)(k + 1), h, ta);
-    composite(tfb, tfd, v, __fsub_rn(fminf(tn, tb), t), prm, C0, C1, C2, Tr);
+    composite<false>(tfb, tfd, tf_coord(prm, v), __fsub_rn(fminf(tn, tb), t), 1.f, prm, C0, C1, C2, Tr);
   }
 }
 
@@ -676,12 +676,8 @@ template <int P>
 __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
                                                 const float *__restrict__ cand, int n_cand,
                                                 int32_t *__restrict__ label) {
-  __shared__ float4 tfb[256], tfd[256];
-  for (int q = threadIdx.x; q < 256; q += blockDim.x) {
-    const float4 e0 = prm.tf[q], e1 = prm.tf[q < 255 ? q + 1 : 255];
-    tfb[q] = e0;
-    tfd[q] = make_float4(e1.x - e0.x, e1.y - e0.y, e1.z - e0.z, e1.w - e0.w);
-  }
+  __shared__ float4 tfb[kTfEntries], tfd[kTfEntries];
+  load_tf(prm, tfb, tfd);
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int i = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
@@ -697,9 +693,9 @@ __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderPa
   float t = ray.tin;
   for (int visit = 0; visit < kMaxSamplesPerRay && t < ray.tout && Tfront > tr_stop; ++visit) {
     // the visit: element of the heuristic sample at t, up to the first heuristic sample past it
-    float px = fminf(fmaxf(__fmaf_rn(t, ray.d[0], ray.o[0]), 0.f), 1.f);
-    float py = fminf(fmaxf(__fmaf_rn(t, ray.d[1], ray.o[1]), 0.f), 1.f);
-    float pz = fminf(fmaxf(__fmaf_rn(t, ray.d[2], ray.o[2]), 0.f), 1.f);
+    float px = fma_sat(t, ray.d[0], ray.o[0]);
+    float py = fma_sat(t, ray.d[1], ray.o[1]);
+    float pz = fma_sat(t, ray.d[2], ray.o[2]);
     if (!seg_locate<P>(prm, st, blk, px, py, pz)) return;
     const uint32_t e = st.e;
     const float4 ra = st.ra, rb = st.rb;
@@ -708,9 +704,9 @@ __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderPa
     for (int q = 0; q < kMaxSamplesPerRay; ++q) {
       tb = __fadd_rn(tb, ds);
       if (!(tb < ray.tout)) break;
-      px = fminf(fmaxf(__fmaf_rn(tb, ray.d[0], ray.o[0]), 0.f), 1.f);
-      py = fminf(fmaxf(__fmaf_rn(tb, ray.d[1], ray.o[1]), 0.f), 1.f);
-      pz = fminf(fmaxf(__fmaf_rn(tb, ray.d[2], ray.o[2]), 0.f), 1.f);
+      px = fma_sat(tb, ray.d[0], ray.o[0]);
+      py = fma_sat(tb, ray.d[1], ray.o[1]);
+      pz = fma_sat(tb, ray.d[2], ray.o[2]);
       if (!(px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z)) break;
     }
     tb = fminf(tb, ray.tout);
@@ -724,9 +720,9 @@ __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderPa
       for (int k = 1; k < kMaxSamplesPerRay; ++k) {
         tc = __fmaf_rn((float)k, sc, t);
         if (!(tc < ray.tout)) break;
-        px = fminf(fmaxf(__fmaf_rn(tc, ray.d[0], ray.o[0]), 0.f), 1.f);
-        py = fminf(fmaxf(__fmaf_rn(tc, ray.d[1], ray.o[1]), 0.f), 1.f);
-        pz = fminf(fmaxf(__fmaf_rn(tc, ray.d[2], ray.o[2]), 0.f), 1.f);
+        px = fma_sat(tc, ray.d[0], ray.o[0]);
+        py = fma_sat(tc, ray.d[1], ray.o[1]);
+        pz = fma_sat(tc, ray.d[2], ray.o[2]);
         if (!(px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z)) break;
       }
       tc = fminf(tc, ray.tout);
@@ -1113,13 +1109,13 @@ struct SLField {
   __device__ __forceinline__ bool locate(const SLParams &sp, float px, float py, float pz) {
     if (cur != kNone && px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z) return true;
     const uint32_t e = forest_lookup(sp.forest, px, py, pz, sp.status);
-    if (e == kNone || (int64_t)e >= sp.n_elem) {
+    if (e >= (uint32_t)sp.n_elem) {   // kNone included
       set_status(sp.status, kStatusBounds);
       return false;
     }
     cur = e;
     load_record(sp.elem + e, ra, rb, rc, rd);
-    blk.load(sp.bez + (int64_t)e * sp.elem_bytes, 0);
+    blk.load(sp.bez + (int64_t)e * blk.BYTES, 0);
     return true;
   }
 };

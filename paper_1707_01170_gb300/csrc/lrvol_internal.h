@@ -53,11 +53,14 @@ struct Node {
 };
 
 struct ForestView {
-  const uint32_t *head;  // blocks[2] x blocks[1] x blocks[0], x fastest
+  // One word per block, x fastest, and each axis' last layer once more (what
+  // p = 1 finds without a clamp): (blocks[0]+1) x (blocks[1]+1) x (blocks[2]+1).
+  const uint32_t *head;
   const uint4 *nodes;
-  int64_t n_nodes;
-  int bx, by, bz;        // block counts (powers of two)
-  float fbx, fby, fbz;
+  uint32_t n_nodes;              // < 2^31
+  uint32_t head_sy, head_sz;     // strides of y and z
+  uint32_t head_bias;            // 0x4b000000 (1 + head_sy + head_sz) mod 2^32, see forest_lookup
+  float fbx, fby, fbz;           // block counts (powers of two)
 };
 
 struct RayConsts {
@@ -80,10 +83,10 @@ struct RayConsts {
 // a 32-byte header of FP32 offsets o[3] and scales s[3], holding
 // q' = (c' - binomial*o)/s, so a component's value is o + s * contraction(q').
 // Element strides are multiples of 32 bytes.
-__host__ __device__ inline int roundup8(int x) { return (x + 7) & ~7; }
-__host__ __device__ inline int roundup32(int x) { return (x + 31) & ~31; }
-__host__ __device__ inline int render_pair_slots(int nb) { return roundup8(2 * nb); }
-__host__ __device__ inline int render_slots(int nc, int n0, int n1, int n2) {
+__host__ __device__ constexpr int roundup8(int x) { return (x + 7) & ~7; }
+__host__ __device__ constexpr int roundup32(int x) { return (x + 31) & ~31; }
+__host__ __device__ constexpr int render_pair_slots(int nb) { return roundup8(2 * nb); }
+__host__ __device__ constexpr int render_slots(int nc, int n0, int n1, int n2) {
   const int nb = n0 * n1 * n2;
   if (nc == 1) return roundup8(((n1 * n2 + 1) / 2) * 2 * n0);
   return render_pair_slots(nb) + roundup8(nb);
@@ -94,9 +97,9 @@ __host__ __device__ inline int render_slot(int nc, int n0, int nb, int r, int i,
   return c < 2 ? 2 * q + c : render_pair_slots(nb) + q;
 }
 constexpr int kHeaderBytes = 32;  // FP32 o[3], s[3], 2 unused (16-bit storage only)
-__host__ __device__ inline int slot_bytes(int storage) { return storage == LRVOL_STORE_F32 ? 4 : 2; }
-__host__ __device__ inline int header_bytes(int storage) { return storage == LRVOL_STORE_F32 ? 0 : kHeaderBytes; }
-__host__ __device__ inline int elem_bytes(int storage, int slots) {
+__host__ __device__ constexpr int slot_bytes(int storage) { return storage == LRVOL_STORE_F32 ? 4 : 2; }
+__host__ __device__ constexpr int header_bytes(int storage) { return storage == LRVOL_STORE_F32 ? 0 : kHeaderBytes; }
+__host__ __device__ constexpr int elem_bytes(int storage, int slots) {
   return roundup32(header_bytes(storage) + slot_bytes(storage) * slots);
 }
 
@@ -108,9 +111,7 @@ struct RenderParams {
   const ElemRec *elem;
   int64_t n_elem;
   const unsigned char *bez;   // render blocks (layout above)
-  int elem_bytes;             // bytes per element
   const unsigned char *bezc;  // vector volumes: plain per-component copy
-  int elemc_bytes;            // bytes per element of bezc
   int comp;               // component evaluated (FIELD_COMPONENT)
   ForestView forest;
   float *out;
@@ -120,7 +121,7 @@ struct RenderParams {
   int mode;               // LRVOL_STEP_*
   const float *mult;      // LEARNED: per-element step multipliers
   float h, inv_xi, alpha_stop;
-  float tf_scale, tf_bias; // x = v * tf_scale + tf_bias, clamped to [0, 255]
+  float tf_scale, tf_bias; // x = v * tf_scale + tf_bias, clamped to [0, 1]
   const float2 *trim;     // NULL or per pixel (t_front, t_back), row major over the full image
   int light_set;          // shading: 1 = light[] (unit), 0 = towards the eye along the ray
   float light[3];
@@ -249,7 +250,6 @@ struct SLParams {
   const ElemRec *elem;
   int64_t n_elem;
   const unsigned char *bez;
-  int elem_bytes;
   ForestView forest;
   uint32_t *status;   // device status word (bounds)
   unsigned long long *queue;  // streamlines: next seed to trace (zeroed per call)

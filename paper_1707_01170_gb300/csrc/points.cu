@@ -44,8 +44,7 @@ __device__ __forceinline__ uint32_t find_element(const ForestView &f, int64_t n_
 // block took 52 to 56 us, and more registers a thread 52 us.
 template <int P, int NC, int STORE, bool GRAD>
 __global__ void __launch_bounds__(128) k_eval_points(const ForestView f, const ElemRec *__restrict__ elem, int64_t n_elem,
-                                                     const unsigned char *__restrict__ bez, int ebytes,
-                                                     const float *__restrict__ pts, int64_t n, float *__restrict__ out,
+                                                     const unsigned char *__restrict__ bez, const float *__restrict__ pts, int64_t n, float *__restrict__ out,
                                                      uint32_t *status) {
   constexpr int N = P + 1;
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -59,7 +58,7 @@ __global__ void __launch_bounds__(128) k_eval_points(const ForestView f, const E
     float4 ra, rb, rc, rd;
     Block<P, NC == 3 ? 1 : 0, STORE, false> blk;
     load_record(elem + e, ra, rb, rc, rd);
-    blk.load(bez + (int64_t)e * ebytes, 0);
+    blk.load(bez + (int64_t)e * blk.BYTES, 0);
     const float ux = local_u(x, ra.x, rc.x, rd.x), uy = local_u(y, ra.y, rc.y, rd.y), uz = local_u(z, ra.z, rc.z, rd.z);
     float bx[N], by[N], bz[N];
     monomials<P>(ux, bx);
@@ -244,7 +243,7 @@ cudaError_t launch_points_p(const lrvol_s *v, const float *pts, int64_t n, float
   const ForestView f = forest_view(v);
   switch (v->storage) {
 #define LRVOL_PTS(S_)                                                                                             \
-  k_eval_points<P, NC, S_, GRAD><<<blocks, 128, 0, s>>>(f, v->d_elem, v->n_elem, v->d_bez, v->elem_bytes, pts, n, out, \
+  k_eval_points<P, NC, S_, GRAD><<<blocks, 128, 0, s>>>(f, v->d_elem, v->n_elem, v->d_bez, pts, n, out, \
                                                         v->d_status);                                             \
   break
     case LRVOL_STORE_F32: LRVOL_PTS(LRVOL_STORE_F32);
