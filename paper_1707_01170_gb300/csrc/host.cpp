@@ -1,6 +1,5 @@
-// liblrvol host side: the C ABI of lrvol.h, input validation, the
-// element-to-B-spline incidence used by the change of basis, and the k-d
-// forest build (Sec. 3.2.1).  Every per-sample computation runs in kernels.cu.
+// liblrvol host side: the C ABI of lrvol.h, input validation and the k-d forest
+// build (Sec. 3.2.1).  Everything else runs in the kernels.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -54,73 +53,22 @@ int dev_alloc(lrvol_s *v, T **p, size_t count, const char *what) {
   return LRVOL_OK;
 }
 
-bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
+// Scratch of one call.  cudaFree waits for the device, so kernels in flight
+// (after an error between launches) are done with it.
+struct DeviceBuffer {
+  unsigned char *p = nullptr;
+  int alloc(int64_t bytes, const char *what) {
+    const cudaError_t e = cudaMalloc((void **)&p, (size_t)std::max<int64_t>(bytes, 1));
+    if (e == cudaSuccess) return LRVOL_OK;
+    p = nullptr;
+    return cuda_fail(e, what);
+  }
+  ~DeviceBuffer() {
+    if (p) cudaFree(p);
+  }
+};
 
-// ----------------------------------------------------------------------------
-// element -> B-spline incidence: B-splines whose support contains the element
-// ----------------------------------------------------------------------------
-int build_incidence(lrvol_s *v, std::vector<int64_t> &ptr, std::vector<int32_t> &idx) {
-  const int64_t N = v->n_elem, M = v->n_basis;
-  // bucket elements by centre on an R^3 grid
-  int R = (int)std::cbrt((double)N / 4.0);
-  R = std::max(1, std::min(R, 96));
-  std::vector<int64_t> cell_ptr((size_t)R * R * R + 1, 0);
-  std::vector<int32_t> cell_of(N);
-  auto cell_coord = [&](double x) { return std::min(R - 1, std::max(0, (int)(x * R))); };
-  for (int64_t e = 0; e < N; ++e) {
-    const double *b = &v->box[6 * e];
-    int c[3];
-    for (int a = 0; a < 3; ++a) c[a] = cell_coord(0.5 * (b[a] + b[3 + a]));
-    cell_of[e] = (c[2] * R + c[1]) * R + c[0];
-    cell_ptr[cell_of[e] + 1]++;
-  }
-  for (size_t i = 1; i < cell_ptr.size(); ++i) cell_ptr[i] += cell_ptr[i - 1];
-  std::vector<int32_t> cell_el(N);
-  {
-    std::vector<int64_t> fill(cell_ptr.begin(), cell_ptr.end() - 1);
-    for (int64_t e = 0; e < N; ++e) cell_el[fill[cell_of[e]]++] = (int32_t)e;
-  }
-  // pairs (element, bspline), bspline-major
-  std::vector<int64_t> count(N + 1, 0);
-  std::vector<std::pair<int32_t, int32_t>> pairs;
-  pairs.reserve((size_t)N * 64);
-  const int off[3] = {0, v->p[0] + 2, v->p[0] + v->p[1] + 4};
-  for (int64_t i = 0; i < M; ++i) {
-    const double *k = &v->knots[(size_t)i * v->kw];
-    double lo[3], hi[3];
-    int c0[3], c1[3];
-    for (int a = 0; a < 3; ++a) {
-      lo[a] = k[off[a]];
-      hi[a] = k[off[a] + v->p[a] + 1];
-      c0[a] = cell_coord(lo[a]);
-      c1[a] = cell_coord(hi[a]);
-    }
-    for (int cz = c0[2]; cz <= c1[2]; ++cz)
-      for (int cy = c0[1]; cy <= c1[1]; ++cy)
-        for (int cx = c0[0]; cx <= c1[0]; ++cx) {
-          int cell = (cz * R + cy) * R + cx;
-          for (int64_t q = cell_ptr[cell]; q < cell_ptr[cell + 1]; ++q) {
-            int32_t e = cell_el[q];
-            const double *b = &v->box[6 * (size_t)e];
-            bool in = true;
-            for (int a = 0; a < 3 && in; ++a) in = lo[a] <= b[a] && b[3 + a] <= hi[a];
-            if (in) {
-              pairs.push_back({e, (int32_t)i});
-              count[e + 1]++;
-            }
-          }
-        }
-  }
-  for (int64_t e = 0; e < N; ++e) {
-    if (count[e + 1] == 0) return fail(LRVOL_ERR_ARG, "an element lies in no B-spline support");
-    count[e + 1] += count[e];
-  }
-  ptr.assign(count.begin(), count.end());
-  idx.resize(pairs.size());
-  std::vector<int64_t> fill(count.begin(), count.end() - 1);
-  for (auto &pr : pairs) idx[fill[pr.first]++] = pr.second;  // B-spline order kept per element
-  return LRVOL_OK;
-}
+bool is_pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
 // ----------------------------------------------------------------------------
 // k-d forest (Sec. 3.2.1).  Split rule (the paper balances depth by counting,
@@ -517,9 +465,6 @@ int lrvol_create(const int32_t deg[3], int32_t ncomp, int64_t n_elem, const doub
   v->n_basis = n_basis;
   v->kw = kw;
   v->box.assign(elem_box, elem_box + 6 * n_elem);
-  v->knots.assign(knots, knots + kw * n_basis);
-  v->coef.assign(coef, coef + ncomp * n_basis);
-  v->weight.assign(weight, weight + n_basis);
   int rc;
   if ((rc = dev_alloc(v, &v->d_box, 6 * n_elem, "alloc boxes")) ||
       (rc = dev_alloc(v, &v->d_knots, (size_t)kw * n_basis, "alloc knots")) ||
@@ -610,35 +555,42 @@ int lrvol_to_bezier(lrvol_t v, int32_t storage, void *stream) {
   if (!v) return fail(LRVOL_ERR_ARG, "null handle");
   if (storage != LRVOL_STORE_F32 && storage != LRVOL_STORE_F16 && storage != LRVOL_STORE_BF16)
     return fail(LRVOL_ERR_ARG, "bad storage");
-  std::vector<int64_t> ptr;
-  std::vector<int32_t> idx;
-  int rc = build_incidence(v, ptr, idx);
-  if (rc) return rc;
   cudaStream_t st = (cudaStream_t)stream;
+  int rc;
+  Incidence inc;
+  DeviceBuffer scratch, unsorted;
+  if ((rc = scratch.alloc(inc.plan(v->n_elem), "alloc incidence scratch"))) return rc;
+  CU(inc.count(v, scratch.p, st), "incidence count kernels");
+  int64_t entries = 0;
+  uint32_t empty = 0;
+  CU(cudaMemcpyAsync(&entries, inc.ptr() + v->n_elem, sizeof entries, cudaMemcpyDeviceToHost, st), "read incidence size");
+  CU(cudaMemcpyAsync(&empty, inc.empty(), sizeof empty, cudaMemcpyDeviceToHost, st), "read incidence check");
+  CU(cudaStreamSynchronize(st), "incidence sync");
+  if (empty) return fail(LRVOL_ERR_ARG, "an element lies in no B-spline support");
+  if ((rc = unsorted.alloc(4 * entries, "alloc incidence lists"))) return rc;
   const int n0 = v->p[0] + 1, n1 = v->p[1] + 1, n2 = v->p[2] + 1, nb = n0 * n1 * n2;
   v->have_bezier = false;   // the blocks are replaced: none until the new ones are complete
   v->storage = storage;
   v->elem_bytes = elem_bytes(storage, render_slots(v->nc, n0, n1, n2));
   v->elemc_bytes = v->nc == 3 ? elem_bytes(storage, 3 * roundup8(nb)) : 0;
-  if ((rc = dev_alloc(v, &v->d_inc_ptr, ptr.size(), "alloc incidence ptr")) ||
-      (rc = dev_alloc(v, &v->d_inc_idx, idx.size(), "alloc incidence")) ||
+  if ((rc = dev_alloc(v, &v->d_inc_ptr, (size_t)v->n_elem + 1, "alloc incidence ptr")) ||
+      (rc = dev_alloc(v, &v->d_inc_idx, (size_t)entries, "alloc incidence")) ||
       (rc = dev_alloc(v, &v->d_bez64, (size_t)v->n_elem * v->nc * nb, "alloc bezier64")) ||
       (rc = dev_alloc(v, &v->d_bez, (size_t)v->n_elem * v->elem_bytes, "alloc render blocks")) ||
       (v->nc == 3 && (rc = dev_alloc(v, &v->d_bezc, (size_t)v->n_elem * v->elemc_bytes, "alloc render copy"))) ||
       (rc = dev_alloc(v, &v->d_elem, (size_t)v->n_elem, "alloc element records")) ||
       (rc = dev_alloc(v, &v->d_range, (size_t)v->n_elem * v->nc, "alloc coefficient ranges")))
     return rc;
-  CU(cudaMemcpyAsync(v->d_inc_ptr, ptr.data(), sizeof(int64_t) * ptr.size(), cudaMemcpyHostToDevice, st),
-     "upload incidence ptr");
-  CU(cudaMemcpyAsync(v->d_inc_idx, idx.data(), sizeof(int32_t) * idx.size(), cudaMemcpyHostToDevice, st),
-     "upload incidence");
+  CU(cudaMemcpyAsync(v->d_inc_ptr, inc.ptr(), sizeof(int64_t) * (v->n_elem + 1), cudaMemcpyDeviceToDevice, st),
+     "keep incidence ptr");
+  CU(inc.fill(v, reinterpret_cast<int32_t *>(unsorted.p), v->d_inc_idx, st), "incidence list kernels");
   CU(cudaMemsetAsync(v->d_bez, 0, (size_t)v->n_elem * v->elem_bytes, st), "clear render blocks");
   if (v->d_bezc) CU(cudaMemsetAsync(v->d_bezc, 0, (size_t)v->n_elem * v->elemc_bytes, st), "clear render copy");
   CU(launch_to_bezier(v, st), "to_bezier kernel");
   CU(launch_pack(v, st), "pack kernel");
   CU(launch_elem_records(v, st), "element record kernel");
-  CU(cudaStreamSynchronize(st), "to_bezier sync");  // host incidence goes out of scope
-  v->inc_entries = (int64_t)idx.size();
+  CU(cudaStreamSynchronize(st), "to_bezier sync");  // the scratch goes out of scope
+  v->inc_entries = entries;
   v->have_bezier = true;
   return LRVOL_OK;
 }

@@ -1,12 +1,5 @@
 // liblrvol kernels for sm_103a.
 //
-//   k_to_bezier    Sec. 3.2.3 change of basis, FP64: per element, the Bernstein
-//                  coefficients of every incident B-spline's univariate factors
-//                  over the element, by blossoming, accumulated with gamma*c.
-//   k_elem_records element boxes -> FP32 records (rounded-up corners, Eq. 4 step).
-//   (k_render, the per-pixel ray casting of Sec. 4, is in render.cu, look-up
-//   and evaluation at points in points.cu; the device helpers these files
-//   share are in device_common.cuh.)
 //   k_features, k_mlp_infer, k_labels
 //                  learned step multipliers (not in the paper; Eq. 4 stays the
 //                  base): per-element features, the network on the tcgen05
@@ -15,228 +8,18 @@
 //   k_streamlines, k_streamline_error, k_tube_*
 //                  Sec. 5 streamlines (Eq. 4 steps), the Eq. 7 error, tubes.
 //   k_trim_raster  Sec. 4.1 trimming: per-pixel interval of a boundary mesh.
+//   (k_render, the per-pixel ray casting of Sec. 4, is in render.cu, a volume's
+//   change of basis in setup.cu, look-up and evaluation at points in points.cu;
+//   the device helpers these files share are in device_common.cuh.)
 #include <algorithm>
 
 #include "device_common.cuh"
 
 namespace lrvol {
-namespace {
 
 // ----------------------------------------------------------------------------
-// change of basis (FP64)
-// ----------------------------------------------------------------------------
-
-// Bernstein coefficients over [a, b] of the univariate B-spline on knots
-// xi[0..p+1], where [a, b] lies in one knot span.  beta_j is the blossom
-// B(a,..,a, b,..,b) with j arguments b, evaluated by the de Boor triangle of
-// the span restricted to its non-zero entries (only the B-spline itself has
-// coefficient 1), so every denominator is a positive knot difference.
-__device__ void bernstein_of_bspline(const double *xi, int p, double a, double b, double *beta) {
-  int m = 0;
-  for (int q = 1; q <= p; ++q)
-    if (xi[q] <= a) m = q;
-  // the triangle's denominators depend on (r, k) only: one FP64 division
-  // each (FP64 division is a long instruction sequence on GB300), reused for
-  // all p + 1 blossoms
-  double inv[kMaxDeg + 1][kMaxDeg + 1];
-  for (int r = 1; r <= p; ++r) {
-    const int khi = m < r ? m : r;
-    const int klo = (m - p + r) > 0 ? (m - p + r) : 0;
-    for (int k = khi; k >= klo; --k) inv[r][k] = 1.0 / (xi[k + p + 1 - r] - xi[k]);
-  }
-  for (int j = 0; j <= p; ++j) {
-    double D[kMaxDeg + 1];
-    D[0] = 1.0;
-    for (int q = 1; q <= p; ++q) D[q] = 0.0;
-    for (int r = 1; r <= p; ++r) {
-      const double t = (r <= p - j) ? a : b;
-      const int khi = m < r ? m : r;
-      const int klo = (m - p + r) > 0 ? (m - p + r) : 0;
-      for (int k = khi; k >= klo; --k) {
-        const double alpha = (t - xi[k]) * inv[r][k];
-        const double prev = k > 0 ? D[k - 1] : 0.0;
-        D[k] = (1.0 - alpha) * prev + alpha * D[k];
-      }
-    }
-    beta[j] = D[m];
-  }
-}
-
-// C(n, k) in integer arithmetic (each partial product is itself a binomial,
-// so every division is exact)
-__device__ __forceinline__ int binomial(int n, int k) {
-  int b = 1;
-  for (int i = 1; i <= k; ++i) b = b * (n - k + i) / i;
-  return b;
-}
-
-constexpr int kBezWarps = 4;
-constexpr int kChunk = 32;
-
-// One warp per element; lane l owns coefficients q = l, l+32, ... of the
-// (p0+1)(p1+1)(p2+1) block, for every component.
-__global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier(
-    const double *__restrict__ box, const double *__restrict__ knots, const double *__restrict__ coef,
-    const double *__restrict__ weight, const int64_t *__restrict__ inc_ptr, const int32_t *__restrict__ inc_idx,
-    int p0, int p1, int p2, int nc, int kw, int64_t n_elem, double *__restrict__ out64) {
-  __shared__ double sb[kBezWarps][kChunk][3 * (kMaxDeg + 1)];
-  __shared__ double sg[kBezWarps][kChunk][3];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
-  if (e >= n_elem) return;
-  const int n0 = p0 + 1, n1 = p1 + 1, n2 = p2 + 1;
-  const int nb = n0 * n1 * n2;
-  const int deg[3] = {p0, p1, p2};
-  const int off[3] = {0, p0 + 2, p0 + p1 + 4};
-  double acc[4][3];
-  for (int r = 0; r < 4; ++r)
-    for (int c = 0; c < 3; ++c) acc[r][c] = 0.0;
-  const double *eb = box + 6 * e;
-  const int64_t beg = inc_ptr[e], end = inc_ptr[e + 1];
-  for (int64_t base = beg; base < end; base += kChunk) {
-    const int cnt = (int)min((int64_t)kChunk, end - base);
-    if (lane < cnt) {
-      const int32_t i = inc_idx[base + lane];
-      for (int a = 0; a < 3; ++a) {
-        double xi[kMaxDeg + 2];
-        for (int q = 0; q <= deg[a] + 1; ++q) xi[q] = knots[(int64_t)i * kw + off[a] + q];
-        bernstein_of_bspline(xi, deg[a], eb[a], eb[3 + a], &sb[w][lane][a * (kMaxDeg + 1)]);
-      }
-      for (int c = 0; c < nc; ++c) sg[w][lane][c] = weight[i] * coef[(int64_t)i * nc + c];
-    }
-    __syncwarp();
-    for (int s = 0; s < cnt; ++s) {
-      const double *bs = sb[w][s];
-      for (int r = 0; r < 4; ++r) {
-        const int q = lane + 32 * r;
-        if (q < nb) {
-          const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
-          const double prod = bs[ix] * bs[(kMaxDeg + 1) + iy] * bs[2 * (kMaxDeg + 1) + iz];
-          for (int c = 0; c < nc; ++c) acc[r][c] += sg[w][s][c] * prod;
-        }
-      }
-    }
-    __syncwarp();
-  }
-  for (int r = 0; r < 4; ++r) {
-    const int q = lane + 32 * r;
-    if (q < nb)
-      for (int c = 0; c < nc; ++c) out64[(e * nc + c) * nb + q] = acc[r][c];
-  }
-}
-
-// Render copy of the FP64 blocks (layout and storage in lrvol_internal.h):
-// binomials folded in; for 16-bit storage a per-element, per-component offset
-// o = (max+min)/2 and scale s = (max-min)/2 of the FP64 coefficients, and
-// q' = binomial*(c - o)/s rounded once from FP64.  One warp per element.
-__device__ __forceinline__ void store_slot(unsigned char *base, int storage, int slot, double x) {
-  if (storage == LRVOL_STORE_F32) {
-    reinterpret_cast<float *>(base)[slot] = (float)x;
-  } else if (storage == LRVOL_STORE_F16) {
-    reinterpret_cast<__half *>(base + kHeaderBytes)[slot] = __double2half(x);
-  } else {
-    reinterpret_cast<__nv_bfloat16 *>(base + kHeaderBytes)[slot] = __double2bfloat16(x);
-  }
-}
-
-__global__ void __launch_bounds__(32 * kBezWarps) k_pack(const double *__restrict__ b64, int p0, int p1, int p2, int nc,
-                                                        int64_t n_elem, int storage, unsigned char *__restrict__ out,
-                                                        int ebytes, unsigned char *__restrict__ outc, int ecbytes,
-                                                        float2 *__restrict__ range) {
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
-  if (e >= n_elem) return;
-  const int n0 = p0 + 1, n1 = p1 + 1, nb = n0 * n1 * (p2 + 1);
-  const double *be = b64 + e * nc * nb;
-  double o[3] = {0.0, 0.0, 0.0}, sc[3] = {1.0, 1.0, 1.0};
-  for (int c = 0; c < nc; ++c) {
-    // coefficient range (the block's convex hull bounds the field on the element)
-    double mn = __longlong_as_double(0x7ff0000000000000ll), mx = -mn;
-    for (int q = lane; q < nb; q += 32) {
-      mn = fmin(mn, be[c * nb + q]);
-      mx = fmax(mx, be[c * nb + q]);
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-      mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    }
-    if (lane == 0) range[e * nc + c] = make_float2(__double2float_rd(mn), __double2float_ru(mx));
-    if (storage != LRVOL_STORE_F32) {
-      o[c] = 0.5 * (mx + mn);
-      sc[c] = 0.5 * (mx - mn);
-      if (!(sc[c] > 0.0)) sc[c] = 1.0;
-    }
-  }
-  if (storage != LRVOL_STORE_F32) {
-    if (lane < 8) {
-      const float hv = lane < 3 ? (float)o[lane] : (lane < 6 ? (float)sc[lane - 3] : 0.f);
-      reinterpret_cast<float *>(out + e * ebytes)[lane] = hv;
-      if (outc) reinterpret_cast<float *>(outc + e * ecbytes)[lane] = hv;
-    }
-  }
-  for (int q = lane; q < nb; q += 32) {
-    const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
-    const double binom = (double)(binomial(p0, ix) * binomial(p1, iy) * binomial(p2, iz));
-    for (int c = 0; c < nc; ++c) {
-      const double d = be[c * nb + q] - o[c];   // o = 0 and s = 1 for FP32 storage
-      const double x = storage == LRVOL_STORE_F32 ? binom * d : binom * d / sc[c];
-      store_slot(out + e * ebytes, storage, render_slot(nc, n0, nb, iz * n1 + iy, ix, c), x);
-      if (outc) store_slot(outc + e * ecbytes, storage, c * roundup8(nb) + q, x);
-    }
-  }
-}
-
-__global__ void k_elem_records(const double *__restrict__ box, int64_t n_elem, int d, ElemRec *__restrict__ out) {
-  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= n_elem) return;
-  const double *b = box + 6 * e;
-  float lo[3], hi[3], off[3], iw[3];
-  double m = b[3] - b[0];
-  if (b[4] - b[1] < m) m = b[4] - b[1];
-  if (b[5] - b[2] < m) m = b[5] - b[2];
-  for (int a = 0; a < 3; ++a) {
-    lo[a] = __double2float_ru(b[a]);
-    hi[a] = b[3 + a] == 1.0 ? __int_as_float(0x7f800000) : __double2float_ru(b[3 + a]);
-    const double inv = 1.0 / (b[3 + a] - b[a]);
-    off[a] = (float)(((double)lo[a] - b[a]) * inv);   // (lo_RU - lo) / (hi - lo), in FP64
-    iw[a] = (float)inv;
-  }
-  ElemRec r;
-  r.a = make_float4(lo[0], lo[1], lo[2], __double2float_rn(ldexp(m, -d)));
-  r.b = make_float4(hi[0], hi[1], hi[2], 0.f);
-  r.c = make_float4(off[0], off[1], off[2], 0.f);
-  r.d = make_float4(iw[0], iw[1], iw[2], 0.f);
-  out[e] = r;
-}
-
-}  // namespace
-
-cudaError_t launch_to_bezier(const lrvol_s *v, cudaStream_t s) {
-  const int64_t blocks = (v->n_elem + kBezWarps - 1) / kBezWarps;
-  k_to_bezier<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_box, v->d_knots, v->d_coef, v->d_weight, v->d_inc_ptr,
-                                                         v->d_inc_idx, v->p[0], v->p[1], v->p[2], v->nc, v->kw,
-                                                         v->n_elem, v->d_bez64);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_pack(const lrvol_s *v, cudaStream_t s) {
-  const int64_t blocks = (v->n_elem + kBezWarps - 1) / kBezWarps;
-  k_pack<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_bez64, v->p[0], v->p[1], v->p[2], v->nc, v->n_elem,
-                                                    v->storage, v->d_bez, v->elem_bytes, v->d_bezc, v->elemc_bytes,
-                                                    v->d_range);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_elem_records(const lrvol_s *v, cudaStream_t s) {
-  int d = v->p[0];
-  if (v->p[1] > d) d = v->p[1];
-  if (v->p[2] > d) d = v->p[2];
-  k_elem_records<<<(unsigned)((v->n_elem + 255) / 256), 256, 0, s>>>(v->d_box, v->n_elem, d, v->d_elem);
-  return cudaGetLastError();
-}
-
-// ----------------------------------------------------------------------------
-// Learned step sizes: features, BF16 tensor-core inference, fine-step labels.  The network is 16 -> 64 -> 64 -> 64 -> 1 (ReLU).
+// Learned step sizes: features, BF16 tensor-core inference, fine-step labels.
+// The network is 16 -> 64 -> 64 -> 64 -> 1 (ReLU).
 // ----------------------------------------------------------------------------
 namespace {
 

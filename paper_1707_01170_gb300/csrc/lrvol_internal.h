@@ -148,7 +148,7 @@ struct lrvol_s {
   int nc = 1;
   int64_t n_elem = 0, n_basis = 0;
   int kw = 0;  // knots per B-spline
-  std::vector<double> box, knots, coef, weight;
+  std::vector<double> box;  // element boxes (the forest is built on the host)
 
   // device copies of the spline
   double *d_box = nullptr, *d_knots = nullptr, *d_coef = nullptr, *d_weight = nullptr;
@@ -181,7 +181,29 @@ struct lrvol_s {
 
 namespace lrvol {
 
-// kernels.cu
+// setup.cu
+// Element -> B-spline incidence on the device: plan() gives the bytes of one
+// scratch allocation, count() the lists' offsets (ptr, n_elem + 1 entries, the
+// last the total) and whether a list is empty, fill() the lists themselves.
+struct Incidence {
+  int64_t n_elem = 0;
+  int R = 1;
+  unsigned char *base = nullptr;
+  int64_t o_ptr = 0, o_cell_ptr = 0, o_sums = 0, o_cell_count = 0, o_cell_of = 0, o_cell_el = 0, o_count = 0, o_empty = 0;
+  int64_t plan(int64_t n_elem);
+  cudaError_t count(const lrvol_s *v, unsigned char *scratch, cudaStream_t s);
+  cudaError_t fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, cudaStream_t s);
+  template <class T>
+  T *at(int64_t off) const { return reinterpret_cast<T *>(base + off); }
+  int64_t *ptr() const { return at<int64_t>(o_ptr); }
+  int64_t *cell_ptr() const { return at<int64_t>(o_cell_ptr); }
+  int64_t *sums() const { return at<int64_t>(o_sums); }
+  uint32_t *cell_count() const { return at<uint32_t>(o_cell_count); }
+  int32_t *cell_of() const { return at<int32_t>(o_cell_of); }
+  int32_t *cell_el() const { return at<int32_t>(o_cell_el); }
+  uint32_t *counts() const { return at<uint32_t>(o_count); }
+  uint32_t *empty() const { return at<uint32_t>(o_empty); }
+};
 cudaError_t launch_to_bezier(const lrvol_s *v, cudaStream_t s);
 cudaError_t launch_pack(const lrvol_s *v, cudaStream_t s);
 cudaError_t launch_elem_records(const lrvol_s *v, cudaStream_t s);

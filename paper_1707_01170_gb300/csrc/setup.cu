@@ -1,0 +1,450 @@
+// liblrvol set-up kernels for sm_103a: what lrvol_to_bezier does once per volume.
+//
+//   k_cell_*, k_incident, k_sort_lists, k_scan_*
+//                  element -> B-spline incidence: the B-splines whose support
+//                  contains the element, in ascending order.
+//   k_to_bezier    Sec. 3.2.3 change of basis, FP64: per element, the Bernstein
+//                  coefficients of every incident B-spline's univariate factors
+//                  over the element, by blossoming, accumulated with gamma*c.
+//   k_pack         the render copy of the blocks in its storage, and their ranges.
+//   k_elem_records element boxes -> FP32 records (rounded-up corners, Eq. 4 step).
+#include <algorithm>
+#include <cmath>
+
+#include "device_common.cuh"
+
+namespace lrvol {
+namespace {
+
+// ----------------------------------------------------------------------------
+// incidence.  Elements are bucketed by their centres on a grid of R^3 cells, so
+// a B-spline's candidates are the buckets its support meets: for each (y, z)
+// one contiguous run of elements.  A warp takes a B-spline and its lanes the
+// run's elements; a pass counts the elements' B-splines, the other fills their
+// lists.  The lists are filled in no fixed order and sorted afterwards, since
+// k_to_bezier adds in the list's order.  Bound by the candidates' box reads
+// from the L2: about 1 ms for 174,000 elements and 11.45 M entries, where one
+// host thread took 145 ms (388,016 elements, 10.56 M entries: 365 ms).
+// ----------------------------------------------------------------------------
+struct CellGrid {
+  int R;
+  __host__ __device__ int64_t cells() const { return (int64_t)R * R * R; }
+  __device__ __forceinline__ int coord(double x) const { return min(R - 1, max(0, (int)(x * R))); }
+};
+
+__global__ void __launch_bounds__(256) k_cell_count(const double *__restrict__ box, int64_t n_elem, CellGrid g,
+                                                    int32_t *__restrict__ cell_of, uint32_t *__restrict__ count) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n_elem) return;
+  const double *b = box + 6 * e;
+  const int cx = g.coord(0.5 * (b[0] + b[3])), cy = g.coord(0.5 * (b[1] + b[4])), cz = g.coord(0.5 * (b[2] + b[5]));
+  const int32_t c = (cz * g.R + cy) * g.R + cx;
+  cell_of[e] = c;
+  atomicAdd(count + c, 1u);
+}
+
+__global__ void __launch_bounds__(256) k_cell_fill(const int32_t *__restrict__ cell_of, int64_t n_elem,
+                                                   const int64_t *__restrict__ cell_ptr, uint32_t *__restrict__ cursor,
+                                                   int32_t *__restrict__ cell_el) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n_elem) return;
+  const int32_t c = cell_of[e];
+  cell_el[cell_ptr[c] + atomicAdd(cursor + c, 1u)] = (int32_t)e;
+}
+
+constexpr int kSetupWarps = 8;
+
+// FILL false: count[e] = B-splines whose support contains element e.  FILL
+// true: their indices from list[ptr[e]] on, count as the cursors (zeroed).
+template <bool FILL>
+__global__ void __launch_bounds__(32 * kSetupWarps) k_incident(
+    const double *__restrict__ box, const double *__restrict__ knots, int64_t n_basis, int p0, int p1, int p2, int kw,
+    CellGrid g, const int64_t *__restrict__ cell_ptr, const int32_t *__restrict__ cell_el,
+    uint32_t *__restrict__ count, const int64_t *__restrict__ ptr, int32_t *__restrict__ list) {
+  const int64_t i = (int64_t)blockIdx.x * kSetupWarps + (threadIdx.x >> 5);
+  if (i >= n_basis) return;
+  const int lane = threadIdx.x & 31;
+  const double *k = knots + i * kw;
+  const double lx = k[0], hx = k[p0 + 1], ly = k[p0 + 2], hy = k[p0 + 3 + p1], lz = k[p0 + p1 + 4],
+               hz = k[p0 + p1 + p2 + 5];
+  const int cx0 = g.coord(lx), cx1 = g.coord(hx);
+  const int cy0 = g.coord(ly), ny = g.coord(hy) - cy0 + 1;
+  const int cz0 = g.coord(lz), rows = ny * (g.coord(hz) - cz0 + 1);
+  for (int r = 0; r < rows; ++r) {
+    const int64_t row = ((int64_t)(cz0 + r / ny) * g.R + cy0 + r % ny) * g.R;
+    const int64_t end = cell_ptr[row + cx1 + 1];
+    for (int64_t q = cell_ptr[row + cx0] + lane; q < end; q += 32) {
+      const int32_t e = cell_el[q];
+      const double2 *b2 = reinterpret_cast<const double2 *>(box + 6 * (int64_t)e);   // 48 bytes an element
+      const double2 a = __ldg(b2), b = __ldg(b2 + 1), c = __ldg(b2 + 2);             // lo x y | lo z, hi x | hi y z
+      if (lx <= a.x && ly <= a.y && lz <= b.x && b.y <= hx && c.x <= hy && c.y <= hz) {
+        const uint32_t n = atomicAdd(count + e, 1u);
+        if constexpr (FILL) list[ptr[e] + n] = (int32_t)i;
+      }
+    }
+  }
+}
+
+// out = the lists of `in` in ascending order: a warp per element, every entry
+// placed at the number of smaller ones (the entries are distinct).
+__global__ void __launch_bounds__(32 * kSetupWarps) k_sort_lists(const int64_t *__restrict__ ptr, int64_t n_elem,
+                                                                const int32_t *__restrict__ in,
+                                                                int32_t *__restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * kSetupWarps + (threadIdx.x >> 5);
+  if (e >= n_elem) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t beg = ptr[e], end = ptr[e + 1];
+  for (int64_t q0 = beg; q0 < end; q0 += 32) {
+    const int32_t v = q0 + lane < end ? in[q0 + lane] : INT32_MAX;
+    int rank = 0;
+    for (int64_t t0 = beg; t0 < end; t0 += 32) {
+      const int32_t w = t0 + lane < end ? in[t0 + lane] : INT32_MAX;
+      const int n = (int)min((int64_t)32, end - t0);
+      for (int s = 0; s < n; ++s) rank += __shfl_sync(0xffffffffu, w, s) < v;
+    }
+    if (q0 + lane < end) out[beg + rank] = v;
+  }
+}
+
+// Exclusive prefix sums of n counts into out[0 .. n], three launches: tiles of
+// 2,048 counts, the tiles' totals by one CTA, and the tiles' offsets added.
+// `empty` is set when a count is 0.
+constexpr int kScanThreads = 256, kScanItems = 8, kScanTile = kScanThreads * kScanItems;
+
+// Exclusive prefix of v over the CTA's 256 threads, and the total.
+__device__ __forceinline__ int64_t cta_exclusive(int64_t v, int64_t &total) {
+  __shared__ int64_t warp_sum[kScanThreads / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t inc = v;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) warp_sum[warp] = inc;
+  __syncthreads();
+  int64_t before = 0;
+  total = 0;
+  for (int w = 0; w < kScanThreads / 32; ++w) {
+    if (w == warp) before = total;
+    total += warp_sum[w];
+  }
+  __syncthreads();
+  return before + inc - v;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_tiles(const uint32_t *__restrict__ count, int64_t n,
+                                                             int64_t *__restrict__ out, int64_t *__restrict__ sums,
+                                                             uint32_t *__restrict__ empty) {
+  const int64_t q0 = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
+  uint32_t c[kScanItems];
+  int64_t sum = 0, total;
+  bool zero = false;
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    c[i] = q0 + i < n ? count[q0 + i] : 0u;
+    zero |= q0 + i < n && c[i] == 0u;
+    sum += c[i];
+  }
+  int64_t at = cta_exclusive(sum, total);
+#pragma unroll
+  for (int i = 0; i < kScanItems; ++i) {
+    if (q0 + i < n) out[q0 + i] = at;
+    at += c[i];
+  }
+  if (threadIdx.x == 0) sums[blockIdx.x] = total;
+  if (empty && zero) *empty = 1u;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_sums(int64_t *__restrict__ sums, int64_t tiles,
+                                                            int64_t *__restrict__ grand) {
+  int64_t carry = 0;
+  for (int64_t base = 0; base < tiles; base += kScanThreads) {
+    const int64_t q = base + threadIdx.x;
+    int64_t total;
+    const int64_t v = q < tiles ? sums[q] : 0;
+    const int64_t at = cta_exclusive(v, total);
+    if (q < tiles) sums[q] = carry + at;
+    carry += total;
+  }
+  if (threadIdx.x == 0) *grand = carry;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_add(int64_t *__restrict__ out, int64_t n,
+                                                           const int64_t *__restrict__ sums) {
+  const int64_t q0 = (int64_t)blockIdx.x * kScanTile, add = sums[blockIdx.x];
+  for (int64_t q = q0 + threadIdx.x; q < min(n, q0 + kScanTile); q += kScanThreads) out[q] += add;
+}
+
+cudaError_t exclusive_scan(const uint32_t *count, int64_t n, int64_t *out, int64_t *sums, uint32_t *empty,
+                           cudaStream_t s) {
+  const int64_t tiles = (n + kScanTile - 1) / kScanTile;
+  k_scan_tiles<<<(unsigned)tiles, kScanThreads, 0, s>>>(count, n, out, sums, empty);
+  k_scan_sums<<<1, kScanThreads, 0, s>>>(sums, tiles, out + n);
+  k_scan_add<<<(unsigned)tiles, kScanThreads, 0, s>>>(out, n, sums);
+  return cudaGetLastError();
+}
+
+// ----------------------------------------------------------------------------
+// change of basis (FP64)
+// ----------------------------------------------------------------------------
+
+// Bernstein coefficients over [a, b] of the univariate B-spline on knots
+// xi[0..p+1], where [a, b] lies in one knot span.  beta_j is the blossom
+// B(a,..,a, b,..,b) with j arguments b, evaluated by the de Boor triangle of
+// the span restricted to its non-zero entries (only the B-spline itself has
+// coefficient 1), so every denominator is a positive knot difference.
+__device__ void bernstein_of_bspline(const double *xi, int p, double a, double b, double *beta) {
+  int m = 0;
+  for (int q = 1; q <= p; ++q)
+    if (xi[q] <= a) m = q;
+  // the triangle's denominators depend on (r, k) only: one FP64 division
+  // each (FP64 division is a long instruction sequence on GB300), reused for
+  // all p + 1 blossoms
+  double inv[kMaxDeg + 1][kMaxDeg + 1];
+  for (int r = 1; r <= p; ++r) {
+    const int khi = m < r ? m : r;
+    const int klo = (m - p + r) > 0 ? (m - p + r) : 0;
+    for (int k = khi; k >= klo; --k) inv[r][k] = 1.0 / (xi[k + p + 1 - r] - xi[k]);
+  }
+  for (int j = 0; j <= p; ++j) {
+    double D[kMaxDeg + 1];
+    D[0] = 1.0;
+    for (int q = 1; q <= p; ++q) D[q] = 0.0;
+    for (int r = 1; r <= p; ++r) {
+      const double t = (r <= p - j) ? a : b;
+      const int khi = m < r ? m : r;
+      const int klo = (m - p + r) > 0 ? (m - p + r) : 0;
+      for (int k = khi; k >= klo; --k) {
+        const double alpha = (t - xi[k]) * inv[r][k];
+        const double prev = k > 0 ? D[k - 1] : 0.0;
+        D[k] = (1.0 - alpha) * prev + alpha * D[k];
+      }
+    }
+    beta[j] = D[m];
+  }
+}
+
+// C(n, k) in integer arithmetic (each partial product is itself a binomial,
+// so every division is exact)
+__device__ __forceinline__ int binomial(int n, int k) {
+  int b = 1;
+  for (int i = 1; i <= k; ++i) b = b * (n - k + i) / i;
+  return b;
+}
+
+constexpr int kBezWarps = 4;
+constexpr int kChunk = 32;
+
+// One warp per element; lane l owns coefficients q = l, l+32, ... of the
+// (p0+1)(p1+1)(p2+1) block, for every component.
+__global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier(
+    const double *__restrict__ box, const double *__restrict__ knots, const double *__restrict__ coef,
+    const double *__restrict__ weight, const int64_t *__restrict__ inc_ptr, const int32_t *__restrict__ inc_idx,
+    int p0, int p1, int p2, int nc, int kw, int64_t n_elem, double *__restrict__ out64) {
+  __shared__ double sb[kBezWarps][kChunk][3 * (kMaxDeg + 1)];
+  __shared__ double sg[kBezWarps][kChunk][3];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
+  if (e >= n_elem) return;
+  const int n0 = p0 + 1, n1 = p1 + 1, n2 = p2 + 1;
+  const int nb = n0 * n1 * n2;
+  const int deg[3] = {p0, p1, p2};
+  const int off[3] = {0, p0 + 2, p0 + p1 + 4};
+  double acc[4][3];
+  for (int r = 0; r < 4; ++r)
+    for (int c = 0; c < 3; ++c) acc[r][c] = 0.0;
+  const double *eb = box + 6 * e;
+  const int64_t beg = inc_ptr[e], end = inc_ptr[e + 1];
+  for (int64_t base = beg; base < end; base += kChunk) {
+    const int cnt = (int)min((int64_t)kChunk, end - base);
+    if (lane < cnt) {
+      const int32_t i = inc_idx[base + lane];
+      for (int a = 0; a < 3; ++a) {
+        double xi[kMaxDeg + 2];
+        for (int q = 0; q <= deg[a] + 1; ++q) xi[q] = knots[(int64_t)i * kw + off[a] + q];
+        bernstein_of_bspline(xi, deg[a], eb[a], eb[3 + a], &sb[w][lane][a * (kMaxDeg + 1)]);
+      }
+      for (int c = 0; c < nc; ++c) sg[w][lane][c] = weight[i] * coef[(int64_t)i * nc + c];
+    }
+    __syncwarp();
+    for (int s = 0; s < cnt; ++s) {
+      const double *bs = sb[w][s];
+      for (int r = 0; r < 4; ++r) {
+        const int q = lane + 32 * r;
+        if (q < nb) {
+          const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
+          const double prod = bs[ix] * bs[(kMaxDeg + 1) + iy] * bs[2 * (kMaxDeg + 1) + iz];
+          for (int c = 0; c < nc; ++c) acc[r][c] += sg[w][s][c] * prod;
+        }
+      }
+    }
+    __syncwarp();
+  }
+  for (int r = 0; r < 4; ++r) {
+    const int q = lane + 32 * r;
+    if (q < nb)
+      for (int c = 0; c < nc; ++c) out64[(e * nc + c) * nb + q] = acc[r][c];
+  }
+}
+
+// Render copy of the FP64 blocks (layout and storage in lrvol_internal.h):
+// binomials folded in; for 16-bit storage a per-element, per-component offset
+// o = (max+min)/2 and scale s = (max-min)/2 of the FP64 coefficients, and
+// q' = binomial*(c - o)/s rounded once from FP64.  One warp per element.
+__device__ __forceinline__ void store_slot(unsigned char *base, int storage, int slot, double x) {
+  if (storage == LRVOL_STORE_F32) {
+    reinterpret_cast<float *>(base)[slot] = (float)x;
+  } else if (storage == LRVOL_STORE_F16) {
+    reinterpret_cast<__half *>(base + kHeaderBytes)[slot] = __double2half(x);
+  } else {
+    reinterpret_cast<__nv_bfloat16 *>(base + kHeaderBytes)[slot] = __double2bfloat16(x);
+  }
+}
+
+__global__ void __launch_bounds__(32 * kBezWarps) k_pack(const double *__restrict__ b64, int p0, int p1, int p2, int nc,
+                                                        int64_t n_elem, int storage, unsigned char *__restrict__ out,
+                                                        int ebytes, unsigned char *__restrict__ outc, int ecbytes,
+                                                        float2 *__restrict__ range) {
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
+  if (e >= n_elem) return;
+  const int n0 = p0 + 1, n1 = p1 + 1, nb = n0 * n1 * (p2 + 1);
+  const double *be = b64 + e * nc * nb;
+  double o[3] = {0.0, 0.0, 0.0}, sc[3] = {1.0, 1.0, 1.0};
+  for (int c = 0; c < nc; ++c) {
+    // coefficient range (the block's convex hull bounds the field on the element)
+    double mn = __longlong_as_double(0x7ff0000000000000ll), mx = -mn;
+    for (int q = lane; q < nb; q += 32) {
+      mn = fmin(mn, be[c * nb + q]);
+      mx = fmax(mx, be[c * nb + q]);
+    }
+    for (int off = 16; off > 0; off >>= 1) {
+      mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    }
+    if (lane == 0) range[e * nc + c] = make_float2(__double2float_rd(mn), __double2float_ru(mx));
+    if (storage != LRVOL_STORE_F32) {
+      o[c] = 0.5 * (mx + mn);
+      sc[c] = 0.5 * (mx - mn);
+      if (!(sc[c] > 0.0)) sc[c] = 1.0;
+    }
+  }
+  if (storage != LRVOL_STORE_F32) {
+    if (lane < 8) {
+      const float hv = lane < 3 ? (float)o[lane] : (lane < 6 ? (float)sc[lane - 3] : 0.f);
+      reinterpret_cast<float *>(out + e * ebytes)[lane] = hv;
+      if (outc) reinterpret_cast<float *>(outc + e * ecbytes)[lane] = hv;
+    }
+  }
+  for (int q = lane; q < nb; q += 32) {
+    const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
+    const double binom = (double)(binomial(p0, ix) * binomial(p1, iy) * binomial(p2, iz));
+    for (int c = 0; c < nc; ++c) {
+      const double d = be[c * nb + q] - o[c];   // o = 0 and s = 1 for FP32 storage
+      const double x = storage == LRVOL_STORE_F32 ? binom * d : binom * d / sc[c];
+      store_slot(out + e * ebytes, storage, render_slot(nc, n0, nb, iz * n1 + iy, ix, c), x);
+      if (outc) store_slot(outc + e * ecbytes, storage, c * roundup8(nb) + q, x);
+    }
+  }
+}
+
+__global__ void k_elem_records(const double *__restrict__ box, int64_t n_elem, int d, ElemRec *__restrict__ out) {
+  const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n_elem) return;
+  const double *b = box + 6 * e;
+  float lo[3], hi[3], off[3], iw[3];
+  double m = b[3] - b[0];
+  if (b[4] - b[1] < m) m = b[4] - b[1];
+  if (b[5] - b[2] < m) m = b[5] - b[2];
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = __double2float_ru(b[a]);
+    hi[a] = b[3 + a] == 1.0 ? __int_as_float(0x7f800000) : __double2float_ru(b[3 + a]);
+    const double inv = 1.0 / (b[3 + a] - b[a]);
+    off[a] = (float)(((double)lo[a] - b[a]) * inv);   // (lo_RU - lo) / (hi - lo), in FP64
+    iw[a] = (float)inv;
+  }
+  ElemRec r;
+  r.a = make_float4(lo[0], lo[1], lo[2], __double2float_rn(ldexp(m, -d)));
+  r.b = make_float4(hi[0], hi[1], hi[2], 0.f);
+  r.c = make_float4(off[0], off[1], off[2], 0.f);
+  r.d = make_float4(iw[0], iw[1], iw[2], 0.f);
+  out[e] = r;
+}
+
+}  // namespace
+
+// Scratch of the incidence: one allocation, carved up here.
+int64_t Incidence::plan(int64_t n_elem_) {
+  n_elem = n_elem_;
+  R = std::max(1, std::min((int)std::cbrt((double)n_elem / 4.0), 96));
+  const int64_t cells = (int64_t)R * R * R, most = std::max(cells, n_elem);
+  int64_t at = 0;
+  auto take = [&](int64_t bytes) {
+    const int64_t off = at;
+    at += (bytes + 255) & ~int64_t(255);
+    return off;
+  };
+  o_ptr = take(8 * (n_elem + 1));
+  o_cell_ptr = take(8 * (cells + 1));
+  o_sums = take(8 * ((most + kScanTile - 1) / kScanTile));
+  o_cell_count = take(4 * cells);
+  o_cell_of = take(4 * n_elem);
+  o_cell_el = take(4 * n_elem);
+  o_count = take(4 * n_elem);
+  o_empty = take(4);
+  return at;
+}
+
+cudaError_t Incidence::count(const lrvol_s *v, unsigned char *scratch, cudaStream_t s) {
+  base = scratch;
+  const CellGrid g = {R};
+  const int64_t cells = g.cells();
+  cudaError_t e;
+  if ((e = cudaMemsetAsync(cell_count(), 0, 4 * cells, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(counts(), 0, 4 * n_elem, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(empty(), 0, 4, s)) != cudaSuccess) return e;
+  const unsigned eb = (unsigned)((n_elem + 255) / 256), wb = (unsigned)((v->n_basis + kSetupWarps - 1) / kSetupWarps);
+  k_cell_count<<<eb, 256, 0, s>>>(v->d_box, n_elem, g, cell_of(), cell_count());
+  if ((e = exclusive_scan(cell_count(), cells, cell_ptr(), sums(), nullptr, s)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(cell_count(), 0, 4 * cells, s)) != cudaSuccess) return e;
+  k_cell_fill<<<eb, 256, 0, s>>>(cell_of(), n_elem, cell_ptr(), cell_count(), cell_el());
+  k_incident<false><<<wb, 32 * kSetupWarps, 0, s>>>(v->d_box, v->d_knots, v->n_basis, v->p[0], v->p[1], v->p[2], v->kw,
+                                                   g, cell_ptr(), cell_el(), counts(), nullptr, nullptr);
+  if ((e = exclusive_scan(counts(), n_elem, ptr(), sums(), empty(), s)) != cudaSuccess) return e;
+  return cudaMemsetAsync(counts(), 0, 4 * n_elem, s);   // from here the fill's cursors
+}
+
+cudaError_t Incidence::fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, cudaStream_t s) {
+  const unsigned wb = (unsigned)((v->n_basis + kSetupWarps - 1) / kSetupWarps);
+  k_incident<true><<<wb, 32 * kSetupWarps, 0, s>>>(v->d_box, v->d_knots, v->n_basis, v->p[0], v->p[1], v->p[2], v->kw,
+                                                  CellGrid{R}, cell_ptr(), cell_el(), counts(), ptr(), unsorted);
+  k_sort_lists<<<(unsigned)((n_elem + kSetupWarps - 1) / kSetupWarps), 32 * kSetupWarps, 0, s>>>(ptr(), n_elem, unsorted,
+                                                                                              list);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_to_bezier(const lrvol_s *v, cudaStream_t s) {
+  const int64_t blocks = (v->n_elem + kBezWarps - 1) / kBezWarps;
+  k_to_bezier<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_box, v->d_knots, v->d_coef, v->d_weight, v->d_inc_ptr,
+                                                         v->d_inc_idx, v->p[0], v->p[1], v->p[2], v->nc, v->kw,
+                                                         v->n_elem, v->d_bez64);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pack(const lrvol_s *v, cudaStream_t s) {
+  const int64_t blocks = (v->n_elem + kBezWarps - 1) / kBezWarps;
+  k_pack<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_bez64, v->p[0], v->p[1], v->p[2], v->nc, v->n_elem,
+                                                    v->storage, v->d_bez, v->elem_bytes, v->d_bezc, v->elemc_bytes,
+                                                    v->d_range);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_elem_records(const lrvol_s *v, cudaStream_t s) {
+  int d = v->p[0];
+  if (v->p[1] > d) d = v->p[1];
+  if (v->p[2] > d) d = v->p[2];
+  k_elem_records<<<(unsigned)((v->n_elem + 255) / 256), 256, 0, s>>>(v->d_box, v->n_elem, d, v->d_elem);
+  return cudaGetLastError();
+}
+
+}  // namespace lrvol

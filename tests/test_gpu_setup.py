@@ -1,0 +1,85 @@
+"""Incidence and change of basis on the device, at sizes where the lists and
+the scans change shape: one element; fewer elements than a warp; lists longer
+than 64 entries; elements of very different size in one bucket; more elements
+than a scan tile.
+
+Blocks against the FP64 oracle's interpolated blocks.  Interpolation carries a
+value's rounding (32 u max|c| allowed for the sum over a list, u = 2^-53) into
+the coefficients by the norms of its three inverses, so the bar is 32 u max|c|
+times their product (6e-13, 6e-12 and 1e-10 for degrees 2, 3 and 4).  The number
+of incidence entries against a direct test of supports, and two conversions bit
+for bit (the lists are filled in no fixed order and sorted).
+"""
+import math
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle.oracle import Oracle
+from paper_1707_01170_gb300 import lrvol as lv
+from paper_1707_01170_gb300.synth import volumes as V
+from paper_1707_01170_gb300.synth.lrgen import LRVolume
+
+pytestmark = pytest.mark.gpu
+
+VOLS = {
+    "one element": lambda: V.tensor_product((3, 3, 3), (1, 1, 1)),
+    "8 elements": lambda: V.tensor_product((1, 2, 3), (2, 2, 2), ncomp=3),
+    "degree 4": lambda: V.refined_ball((4, 4, 4), (3, 3, 3), radii=(0.3,), seed=1),
+    "mixed sizes": lambda: V.refined_ball((2, 2, 2), (2, 2, 2), centres=((0.2, 0.3, 0.4),), radii=(0.3, 0.2, 0.12),
+                                          ncomp=3, seed=2),
+    "scan tiles": lambda: V.tensor_product((1, 1, 1), (17, 16, 15)),
+    "flat": lambda: V.tensor_product((2, 1, 1), (40, 1, 1)),
+}
+
+
+def _amplification(deg):
+    k = 1.0
+    for p in (int(d) for d in deg):
+        x = (np.arange(p + 1) + 0.5) / (p + 1)
+        B = np.stack([math.comb(p, i) * x ** i * (1 - x) ** (p - i) for i in range(p + 1)], 1)
+        k *= np.abs(np.linalg.inv(B)).sum(1).max()
+    return k
+
+
+def _incidence(vol):
+    n = 0
+    s = vol.knot_slices()
+    lo = np.stack([vol.knots[:, q][:, 0] for q in s], 1)
+    hi = np.stack([vol.knots[:, q][:, -1] for q in s], 1)
+    for b in vol.elem_box:
+        n += int(np.all((lo <= b[:3]) & (b[3:] <= hi), axis=1).sum())
+    return n
+
+
+@pytest.mark.parametrize("name", list(VOLS))
+def test_blocks_and_incidence(name):
+    vol = VOLS[name]()
+    gv = lv.Volume(vol).to_bezier()
+    got = gv.get_bezier()
+    want = Oracle(vol).bezier_blocks()
+    assert got.shape == want.shape
+    assert np.abs(got - want).max() <= 32 * 2.0 ** -53 * _amplification(vol.deg) * np.abs(vol.coef).max()
+    assert gv.stats()["incidence_entries"] == _incidence(vol)
+    again = gv.to_bezier(lv.STORE_F16).get_bezier()
+    gv.close()
+    assert np.array_equal(got, again)
+
+
+def test_element_without_a_spline_is_refused():
+    vol = V.tensor_product((2, 2, 2), (3, 3, 3))
+    lo = vol.knots[:, 0]
+    keep = lo < lo.max()                       # drop the B-splines that reach furthest right ...
+    k = vol.knots.copy()
+    k[:, :4] = np.minimum(k[:, :4], 2 / 3)     # ... and cut the others' supports before the last elements
+    bad = LRVolume(deg=vol.deg, elem_box=vol.elem_box, knots=k[keep], coef=vol.coef[keep], weight=vol.weight[keep],
+                   grid=vol.grid)
+    gv = lv.Volume(bad)
+    with pytest.raises(lv.LrvolError) as err:
+        gv.to_bezier()
+    assert err.value.status == lv.ERR_ARG
+    with pytest.raises(lv.LrvolError):
+        gv.get_bezier()
+    gv.close()
