@@ -204,12 +204,8 @@ __device__ __forceinline__ float tf_coord(const RenderParams &prm, float v) {
 // The coordinate that reads the table's extra entry: no opacity, no colour.
 constexpr float kTfNothing = 256.5f / 255.f;
 
-// One Alg. 2 update in transmittance form (Tr = 1 - alpha_dst) for a sample of
-// TF coordinate x: w = (1 - T) Tr, C += w C_src, Tr *= T; with SHADE, C_src is
-// multiplied by the intensity sh (Sec. 4.1).
-template <bool SHADE>
-__device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, float x, float seg, float sh,
-                                          const RenderParams &prm, float &C0, float &C1, float &C2, float &Tr) {
+// The transfer function at coordinate x: colour, and log2(1 - alpha) in w.
+__device__ __forceinline__ float4 tf_sample(const float4 *tfb, const float4 *tfd, float x) {
   // entry floor(255 x) without a float-int conversion (those issue on the
   // narrow XU pipe): 255 x + 2^23 rounded down is 2^23 + floor(255 x) exactly;
   // x = 1 reads entry 255, whose difference is 0
@@ -218,11 +214,21 @@ __device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, 
   const float fr = __fmaf_rn(x, 255.f, __fsub_rn(8388608.f, r));
   const float4 e0 = tfb[q], de = tfd[q];
   const float sa = fmaf(fr, de.w, e0.w);
-  const float T = ex2_approx(lg2_approx(fmaxf(1.f - sa, 0.f)) * (seg * prm.inv_xi));
+  return make_float4(fmaf(fr, de.x, e0.x), fmaf(fr, de.y, e0.y), fmaf(fr, de.z, e0.z), lg2_approx(fmaxf(1.f - sa, 0.f)));
+}
+
+// One Alg. 2 update in transmittance form (Tr = 1 - alpha_dst) for a sample of
+// TF coordinate x: w = (1 - T) Tr, C += w C_src, Tr *= T; with SHADE, C_src is
+// multiplied by the intensity sh (Sec. 4.1).
+template <bool SHADE>
+__device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, float x, float seg, float sh,
+                                          const RenderParams &prm, float &C0, float &C1, float &C2, float &Tr) {
+  const float4 src = tf_sample(tfb, tfd, x);
+  const float T = ex2_approx(src.w * (seg * prm.inv_xi));
   const float w = SHADE ? fmaf(-Tr, T, Tr) * sh : fmaf(-Tr, T, Tr);
-  C0 = fmaf(w, fmaf(fr, de.x, e0.x), C0);
-  C1 = fmaf(w, fmaf(fr, de.y, e0.y), C1);
-  C2 = fmaf(w, fmaf(fr, de.z, e0.z), C2);
+  C0 = fmaf(w, src.x, C0);
+  C1 = fmaf(w, src.y, C1);
+  C2 = fmaf(w, src.z, C2);
   Tr *= T;
 }
 

@@ -430,41 +430,55 @@ __device__ __forceinline__ bool seg_locate(const RenderParams &prm, SegState &st
   return true;
 }
 
-// Alg. 2 from transparent over [ta, tb) with samples ta + k*h (each in its element).
+// A lane's sample at parameter t: colour and log2(1 - alpha); false on a failed look-up.
 template <int P>
-__device__ void seg_composite(const RenderParams &prm, const Ray &ray, const float4 *tfb, const float4 *tfd,
-                              float ta, float tb, float h, SegState &st, Block<P, 0, LRVOL_STORE_F32> &blk,
-                              float &C0, float &C1, float &C2, float &Tr) {
+__device__ __forceinline__ bool seg_sample(const RenderParams &prm, const Ray &ray, const float4 *tfb, const float4 *tfd,
+                                           float t, SegState &st, Block<P, 0, LRVOL_STORE_F32> &blk, float4 &src) {
   constexpr int N = P + 1;
-  C0 = C1 = C2 = 0.f;
-  Tr = 1.f;
-  for (int k = 0; k < kMaxSamplesPerRay; ++k) {
-    const float t = __fmaf_rn((float)k, h, ta);
-    if (!(t < tb)) break;
-    const float px = fma_sat(t, ray.d[0], ray.o[0]);
-    const float py = fma_sat(t, ray.d[1], ray.o[1]);
-    const float pz = fma_sat(t, ray.d[2], ray.o[2]);
-    if (!seg_locate<P>(prm, st, blk, px, py, pz)) return;
-    float bx[N], by[N], bz[N];
-    monomials<P>(local_u(px, st.ra.x, st.rc.x, st.rd.x), bx);
-    monomials<P>(local_u(py, st.ra.y, st.rc.y, st.rd.y), by);
-    monomials<P>(local_u(pz, st.ra.z, st.rc.z, st.rd.z), bz);
-    const float v = blk.eval(bx, by, bz);
-    const float tn = __fmaf_rn((float)(k + 1), h, ta);
-    composite<false>(tfb, tfd, tf_coord(prm, v), __fsub_rn(fminf(tn, tb), t), 1.f, prm, C0, C1, C2, Tr);
-  }
+  const float px = fma_sat(t, ray.d[0], ray.o[0]);
+  const float py = fma_sat(t, ray.d[1], ray.o[1]);
+  const float pz = fma_sat(t, ray.d[2], ray.o[2]);
+  if (!seg_locate<P>(prm, st, blk, px, py, pz)) return false;
+  float bx[N], by[N], bz[N];
+  monomials<P>(local_u(px, st.ra.x, st.rc.x, st.rd.x), bx);
+  monomials<P>(local_u(py, st.ra.y, st.rc.y, st.rd.y), by);
+  monomials<P>(local_u(pz, st.ra.z, st.rc.z, st.rd.z), bz);
+  src = tf_sample(tfb, tfd, tf_coord(prm, blk.eval(bx, by, bz)));
+  return true;
 }
 
+// Whether the ray at parameter t has left the box [lo, hi) or the cube.
+__device__ __forceinline__ bool seg_left(const Ray &ray, const float4 &lo, const float4 &hi, float t) {
+  const float px = fma_sat(t, ray.d[0], ray.o[0]);
+  const float py = fma_sat(t, ray.d[1], ray.o[1]);
+  const float pz = fma_sat(t, ray.d[2], ray.o[2]);
+  return !(t < ray.tout) ||
+         !(px >= lo.x && py >= lo.y && pz >= lo.z && px < hi.x && py < hi.y && pz < hi.z);
+}
+
+// One warp per ray.  A visit's fine samples are independent until they are
+// composited, so the lanes take 32 at a time: Alg. 2 over them is a prefix
+// product of transmittances and prefix sums of colours.  Lane 0's end is the
+// visit's, lane c's that of candidate c; all their fine composites start at
+// the visit's first sample, so one march serves them all, and a lane picks its
+// composite out of the prefix at its own last sample.  The candidates' own
+// samples, a few each, are spread over the lanes as (candidate, sample) slots
+// and composited by the candidates' lanes.
+//
+// With a thread per ray and a fine march per candidate the kernel evaluated
+// the visit's fine samples up to seven times, with 12 of 32 lanes active and a
+// tail of long rays: 12.5 ms for a 320x180 camera of a 174,000-element tricubic
+// volume, 3.45 ms now.
 template <int P>
 __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
                                                 const float *__restrict__ cand, int n_cand,
                                                 int32_t *__restrict__ label) {
+  constexpr unsigned kAll = 0xffffffffu;
   __shared__ float4 tfb[kTfEntries], tfd[kTfEntries];
   load_tf(prm, tfb, tfd);
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int i = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
-  const int j = prm.row_begin + blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
+  const int i = blockIdx.x * 2 + (warp & 1), j = prm.row_begin + blockIdx.y * 2 + (warp >> 1);
   if (i >= prm.width || j >= prm.row_end) return;
   Ray ray;
   if (!make_ray(prm.ray, i, j, ray)) return;
@@ -472,52 +486,142 @@ __global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderPa
   SegState st;
   st.e = kNone;
   const float tr_stop = 1.f - prm.alpha_stop;
-  float Tfront = 1.f;
-  float t = ray.tin;
+  const bool is_cand = lane > 0 && lane < n_cand;
+  const float my_cand = is_cand ? __ldg(cand + lane) : 1.f;
+  float Tfront = 1.f, t = ray.tin;
   for (int visit = 0; visit < kMaxSamplesPerRay && t < ray.tout && Tfront > tr_stop; ++visit) {
     // the visit: element of the heuristic sample at t, up to the first heuristic sample past it
-    float px = fma_sat(t, ray.d[0], ray.o[0]);
-    float py = fma_sat(t, ray.d[1], ray.o[1]);
-    float pz = fma_sat(t, ray.d[2], ray.o[2]);
-    if (!seg_locate<P>(prm, st, blk, px, py, pz)) return;
+    if (!seg_locate<P>(prm, st, blk, fma_sat(t, ray.d[0], ray.o[0]), fma_sat(t, ray.d[1], ray.o[1]),
+                       fma_sat(t, ray.d[2], ray.o[2])))
+      return;
     const uint32_t e = st.e;
-    const float4 ra = st.ra, rb = st.rb;
-    const float ds = ra.w;
+    const float4 lo = st.ra, hi = st.rb;
+    const float ds = lo.w;
     float tb = t;
-    for (int q = 0; q < kMaxSamplesPerRay; ++q) {
-      tb = __fadd_rn(tb, ds);
-      if (!(tb < ray.tout)) break;
-      px = fma_sat(tb, ray.d[0], ray.o[0]);
-      py = fma_sat(tb, ray.d[1], ray.o[1]);
-      pz = fma_sat(tb, ray.d[2], ray.o[2]);
-      if (!(px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z)) break;
+    for (int q = 0; q < kMaxSamplesPerRay; q += 32) {   // 32 steps at a time, a lane each
+      float mine = 0.f;
+#pragma unroll
+      for (int s = 0; s < 32; ++s) {
+        tb = __fadd_rn(tb, ds);
+        if (s == lane) mine = tb;
+      }
+      const unsigned left = __ballot_sync(kAll, seg_left(ray, lo, hi, mine));
+      if (left) {
+        tb = __shfl_sync(kAll, mine, __ffs(left) - 1);
+        break;
+      }
     }
     tb = fminf(tb, ray.tout);
-    float R0, R1, R2, RT;
-    seg_composite<P>(prm, ray, tfb, tfd, t, tb, h_fine, st, blk, R0, R1, R2, RT);
-    int best = 0;
-    for (int c = 1; c < n_cand; ++c) {
-      // the candidate's first sample outside e (or the ray's exit)
-      const float sc = __fmul_rn(ds, cand[c]);
-      float tc = t;
-      for (int k = 1; k < kMaxSamplesPerRay; ++k) {
-        tc = __fmaf_rn((float)k, sc, t);
-        if (!(tc < ray.tout)) break;
-        px = fma_sat(tc, ray.d[0], ray.o[0]);
-        py = fma_sat(tc, ray.d[1], ray.o[1]);
-        pz = fma_sat(tc, ray.d[2], ray.o[2]);
-        if (!(px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z)) break;
+    // a candidate's end: its first sample outside e (or the ray's exit); nk samples before it
+    const float sc = __fmul_rn(ds, my_cand);
+    float te = tb;
+    int nk = 0;
+    bool open = is_cand;
+    for (int k = 1; k < kMaxSamplesPerRay && __any_sync(kAll, open); ++k) {
+      if (open) {
+        const float tc = __fmaf_rn((float)k, sc, t);
+        open = !seg_left(ray, lo, hi, tc);
+        te = fminf(tc, ray.tout);
+        nk = k;
       }
-      tc = fminf(tc, ray.tout);
-      float F0, F1, F2, FT, A0, A1, A2, AT;
-      seg_composite<P>(prm, ray, tfb, tfd, t, tc, h_fine, st, blk, F0, F1, F2, FT);
-      seg_composite<P>(prm, ray, tfb, tfd, t, tc, sc, st, blk, A0, A1, A2, AT);
-      const float err = Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
-      if (!(err <= tau)) break;
-      best = c;
     }
-    atomicMin(label + e, best);
-    Tfront *= RT;
+    // the candidates' composites (all their samples lie in e, which every lane
+    // holds here): slots off .. off + nk - 1 are candidate `lane`'s samples
+    int off = nk;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kAll, off, o);
+      if (lane >= o) off += y;
+    }
+    const int total = __shfl_sync(kAll, off, 31);
+    off -= nk;
+    float A0 = 0.f, A1 = 0.f, A2 = 0.f, AT = 1.f;
+    for (int b = 0; b < total; b += 32) {
+      const int slot = b + lane;
+      int c = 1;
+      for (int q = 2; q < n_cand; ++q)
+        if (slot >= __shfl_sync(kAll, off, q)) c = q;
+      const float tk = __fmaf_rn((float)(slot - __shfl_sync(kAll, off, c)), __shfl_sync(kAll, sc, c), t);
+      float4 src = make_float4(0.f, 0.f, 0.f, 0.f);
+      const bool good = slot >= total || seg_sample<P>(prm, ray, tfb, tfd, tk, st, blk, src);
+      if (!__all_sync(kAll, good)) return;
+      const int k0 = max(b - off, 0), k1 = min(b + 32 - off, nk);   // this lane's samples in these slots
+      const int most = (int)__reduce_max_sync(kAll, (unsigned)max(k1 - k0, 0));
+      for (int q = 0; q < most; ++q) {
+        const int k = k0 + q, from = (off + k - b) & 31;
+        const float s0 = __shfl_sync(kAll, src.x, from), s1 = __shfl_sync(kAll, src.y, from);
+        const float s2 = __shfl_sync(kAll, src.z, from), lg = __shfl_sync(kAll, src.w, from);
+        if (k < k1) {
+          const float tq = __fmaf_rn((float)k, sc, t), tn = __fmaf_rn((float)(k + 1), sc, t);
+          const float T = ex2_approx(lg * (__fsub_rn(fminf(tn, te), tq) * prm.inv_xi)), w = fmaf(-AT, T, AT);
+          A0 = fmaf(w, s0, A0);
+          A1 = fmaf(w, s1, A1);
+          A2 = fmaf(w, s2, A2);
+          AT *= T;
+        }
+      }
+    }
+    // fine composites over [t, te)
+    float F0 = 0.f, F1 = 0.f, F2 = 0.f, FT = 1.f;
+    bool need = lane < n_cand && t < te;
+    const float te_max = __uint_as_float(__reduce_max_sync(kAll, need ? __float_as_uint(te) : 0u));   // te >= 0
+    float cT = 1.f, cC0 = 0.f, cC1 = 0.f, cC2 = 0.f;   // composite of the earlier chunks
+    for (int kb = 0; kb < kMaxSamplesPerRay && __any_sync(kAll, need); kb += 32) {
+      const float ts = __fmaf_rn((float)(kb + lane), h_fine, t), tn = __fmaf_rn((float)(kb + lane + 1), h_fine, t);
+      const bool act = ts < te_max;
+      float4 src = make_float4(0.f, 0.f, 0.f, 0.f);
+      const bool good = !act || seg_sample<P>(prm, ray, tfb, tfd, ts, st, blk, src);
+      if (!__all_sync(kAll, good)) return;
+      const float T = act ? ex2_approx(src.w * (__fsub_rn(tn, ts) * prm.inv_xi)) : 1.f;
+      float p = T;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float y = __shfl_up_sync(kAll, p, o);
+        if (lane >= o) p *= y;
+      }
+      float before = __shfl_up_sync(kAll, p, 1);
+      if (lane == 0) before = 1.f;
+      const float Tr = cT * before, w = fmaf(-Tr, T, Tr);
+      float s0 = w * src.x, s1 = w * src.y, s2 = w * src.z;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const float y0 = __shfl_up_sync(kAll, s0, o), y1 = __shfl_up_sync(kAll, s1, o), y2 = __shfl_up_sync(kAll, s2, o);
+        if (lane >= o) {
+          s0 += y0;
+          s1 += y1;
+          s2 += y2;
+        }
+      }
+      // this chunk's samples before each end; the last of them is clipped there
+      int cnt = 0;
+      for (int c = 0; c < n_cand; ++c) {
+        const unsigned m = __ballot_sync(kAll, ts < __shfl_sync(kAll, te, c));
+        if (lane == c) cnt = __popc(m);
+      }
+      const bool fin = need && (cnt < 32 || !(__fmaf_rn((float)(kb + 32), h_fine, t) < te));
+      const int last = cnt > 0 ? cnt - 1 : 0;
+      const float gt = __shfl_sync(kAll, ts, last), gTr = __shfl_sync(kAll, Tr, last), glg = __shfl_sync(kAll, src.w, last);
+      const float g0 = __shfl_sync(kAll, src.x, last), g1 = __shfl_sync(kAll, src.y, last), g2 = __shfl_sync(kAll, src.z, last);
+      const int prev = last > 0 ? last - 1 : 0;
+      float E0 = __shfl_sync(kAll, s0, prev), E1 = __shfl_sync(kAll, s1, prev), E2 = __shfl_sync(kAll, s2, prev);
+      if (fin) {
+        if (last == 0) E0 = E1 = E2 = 0.f;
+        const float Te = ex2_approx(glg * (__fsub_rn(te, gt) * prm.inv_xi)), we = fmaf(-gTr, Te, gTr);
+        F0 = fmaf(we, g0, cC0 + E0);
+        F1 = fmaf(we, g1, cC1 + E1);
+        F2 = fmaf(we, g2, cC2 + E2);
+        FT = gTr * Te;
+        need = false;
+      }
+      cT *= __shfl_sync(kAll, p, 31);
+      cC0 += __shfl_sync(kAll, s0, 31);
+      cC1 += __shfl_sync(kAll, s1, 31);
+      cC2 += __shfl_sync(kAll, s2, 31);
+    }
+    const float err = Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
+    const unsigned bad = __ballot_sync(kAll, is_cand && !(err <= tau));
+    if (lane == 0) atomicMin(label + e, bad ? __ffs(bad) - 2 : n_cand - 1);
+    Tfront *= __shfl_sync(kAll, FT, 0);
     t = tb;
   }
 }
@@ -568,7 +672,8 @@ cudaError_t launch_mlp_infer(const float *x, int64_t n, const uint16_t *packed, 
 
 cudaError_t launch_labels(const RenderParams &prm, int degree, float h_fine, float tau, const float *cand, int n_cand,
                           int32_t *label, cudaStream_t s) {
-  const dim3 grid((unsigned)((prm.width + 15) / 16), (unsigned)((prm.row_end - prm.row_begin + 7) / 8));
+  // four rays a CTA, a 2x2 patch
+  const dim3 grid((unsigned)((prm.width + 1) / 2), (unsigned)((prm.row_end - prm.row_begin + 1) / 2));
   switch (degree) {
     case 1: k_labels<1><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
     case 2: k_labels<2><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
