@@ -467,10 +467,11 @@ __device__ __forceinline__ bool seg_left(const Ray &ray, const float4 &lo, const
 //
 // With a thread per ray and a fine march per candidate the kernel evaluated
 // the visit's fine samples up to seven times, with 12 of 32 lanes active and a
-// tail of long rays: 12.5 ms for a 320x180 camera of a 174,000-element tricubic
-// volume, 3.45 ms now.
+// tail of long rays: 13.0 ms for a 320x180 camera of a 174,000-element tricubic
+// volume, 3.0 ms now.  Held to 128 registers (four CTAs an SM; 3.6 ms with the
+// 146 it would take, 3.8 ms at five CTAs).
 template <int P>
-__global__ void __launch_bounds__(128) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
+__global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
                                                 const float *__restrict__ cand, int n_cand,
                                                 int32_t *__restrict__ label) {
   constexpr unsigned kAll = 0xffffffffu;
