@@ -586,7 +586,7 @@ int lrvol_to_bezier(lrvol_t v, int32_t storage, void *stream) {
   CU(inc.fill(v, reinterpret_cast<int32_t *>(unsorted.p), v->d_inc_idx, st), "incidence list kernels");
   CU(cudaMemsetAsync(v->d_bez, 0, (size_t)v->n_elem * v->elem_bytes, st), "clear render blocks");
   if (v->d_bezc) CU(cudaMemsetAsync(v->d_bezc, 0, (size_t)v->n_elem * v->elemc_bytes, st), "clear render copy");
-  CU(launch_to_bezier(v, st), "to_bezier kernel");
+  CU(launch_to_bezier(v, inc.cell_of(), inc.empty(), st), "to_bezier kernels");   // their scratch: no longer needed there
   CU(launch_pack(v, st), "pack kernel");
   CU(launch_elem_records(v, st), "element record kernel");
   CU(cudaStreamSynchronize(st), "to_bezier sync");  // the scratch goes out of scope

@@ -204,7 +204,8 @@ struct Incidence {
   uint32_t *counts() const { return at<uint32_t>(o_count); }
   uint32_t *empty() const { return at<uint32_t>(o_empty); }
 };
-cudaError_t launch_to_bezier(const lrvol_s *v, cudaStream_t s);
+// todo, n_todo: scratch for n_elem entries and one counter
+cudaError_t launch_to_bezier(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, cudaStream_t s);
 cudaError_t launch_pack(const lrvol_s *v, cudaStream_t s);
 cudaError_t launch_elem_records(const lrvol_s *v, cudaStream_t s);
 cudaError_t launch_lookup(const lrvol_s *v, const float *pts, int64_t n, uint32_t *out, cudaStream_t s);

@@ -235,56 +235,234 @@ __device__ __forceinline__ int binomial(int n, int k) {
 constexpr int kBezWarps = 4;
 constexpr int kChunk = 32;
 
-// One warp per element; lane l owns coefficients q = l, l+32, ... of the
-// (p0+1)(p1+1)(p2+1) block, for every component.
+// Any degrees; one warp per element (of the n_list listed ones, or of all with
+// no list); lane l owns coefficients q = l, l+32, ... of the (p0+1)(p1+1)(p2+1)
+// block, for every component.
 __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier(
     const double *__restrict__ box, const double *__restrict__ knots, const double *__restrict__ coef,
     const double *__restrict__ weight, const int64_t *__restrict__ inc_ptr, const int32_t *__restrict__ inc_idx,
-    int p0, int p1, int p2, int nc, int kw, int64_t n_elem, double *__restrict__ out64) {
+    int p0, int p1, int p2, int nc, int kw, int64_t n_elem, double *__restrict__ out64,
+    const int32_t *__restrict__ list, const uint32_t *__restrict__ n_list) {
   __shared__ double sb[kBezWarps][kChunk][3 * (kMaxDeg + 1)];
   __shared__ double sg[kBezWarps][kChunk][3];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
-  if (e >= n_elem) return;
-  const int n0 = p0 + 1, n1 = p1 + 1, n2 = p2 + 1;
-  const int nb = n0 * n1 * n2;
-  const int deg[3] = {p0, p1, p2};
-  const int off[3] = {0, p0 + 2, p0 + p1 + 4};
-  double acc[4][3];
-  for (int r = 0; r < 4; ++r)
-    for (int c = 0; c < 3; ++c) acc[r][c] = 0.0;
-  const double *eb = box + 6 * e;
-  const int64_t beg = inc_ptr[e], end = inc_ptr[e + 1];
-  for (int64_t base = beg; base < end; base += kChunk) {
-    const int cnt = (int)min((int64_t)kChunk, end - base);
-    if (lane < cnt) {
-      const int32_t i = inc_idx[base + lane];
-      for (int a = 0; a < 3; ++a) {
-        double xi[kMaxDeg + 2];
-        for (int q = 0; q <= deg[a] + 1; ++q) xi[q] = knots[(int64_t)i * kw + off[a] + q];
-        bernstein_of_bspline(xi, deg[a], eb[a], eb[3 + a], &sb[w][lane][a * (kMaxDeg + 1)]);
+  for (int64_t at = (int64_t)blockIdx.x * kBezWarps + w; at < (list ? (int64_t)*n_list : n_elem);
+       at += (int64_t)gridDim.x * kBezWarps) {
+    const int64_t e = list ? list[at] : at;
+    const int n0 = p0 + 1, n1 = p1 + 1, n2 = p2 + 1;
+    const int nb = n0 * n1 * n2;
+    const int deg[3] = {p0, p1, p2};
+    const int off[3] = {0, p0 + 2, p0 + p1 + 4};
+    double acc[4][3];
+    for (int r = 0; r < 4; ++r)
+      for (int c = 0; c < 3; ++c) acc[r][c] = 0.0;
+    const double *eb = box + 6 * e;
+    const int64_t beg = inc_ptr[e], end = inc_ptr[e + 1];
+    for (int64_t base = beg; base < end; base += kChunk) {
+      const int cnt = (int)min((int64_t)kChunk, end - base);
+      if (lane < cnt) {
+        const int32_t i = inc_idx[base + lane];
+        for (int a = 0; a < 3; ++a) {
+          double xi[kMaxDeg + 2];
+          for (int q = 0; q <= deg[a] + 1; ++q) xi[q] = knots[(int64_t)i * kw + off[a] + q];
+          bernstein_of_bspline(xi, deg[a], eb[a], eb[3 + a], &sb[w][lane][a * (kMaxDeg + 1)]);
+        }
+        for (int c = 0; c < nc; ++c) sg[w][lane][c] = weight[i] * coef[(int64_t)i * nc + c];
       }
-      for (int c = 0; c < nc; ++c) sg[w][lane][c] = weight[i] * coef[(int64_t)i * nc + c];
-    }
-    __syncwarp();
-    for (int s = 0; s < cnt; ++s) {
-      const double *bs = sb[w][s];
-      for (int r = 0; r < 4; ++r) {
-        const int q = lane + 32 * r;
-        if (q < nb) {
-          const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
-          const double prod = bs[ix] * bs[(kMaxDeg + 1) + iy] * bs[2 * (kMaxDeg + 1) + iz];
-          for (int c = 0; c < nc; ++c) acc[r][c] += sg[w][s][c] * prod;
+      __syncwarp();
+      for (int s = 0; s < cnt; ++s) {
+        const double *bs = sb[w][s];
+        for (int r = 0; r < 4; ++r) {
+          const int q = lane + 32 * r;
+          if (q < nb) {
+            const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
+            const double prod = bs[ix] * bs[(kMaxDeg + 1) + iy] * bs[2 * (kMaxDeg + 1) + iz];
+            for (int c = 0; c < nc; ++c) acc[r][c] += sg[w][s][c] * prod;
+          }
         }
       }
+      __syncwarp();
     }
-    __syncwarp();
+    for (int r = 0; r < 4; ++r) {
+      const int q = lane + 32 * r;
+      if (q < nb)
+        for (int c = 0; c < nc; ++c) out64[(e * nc + c) * nb + q] = acc[r][c];
+    }
   }
-  for (int r = 0; r < 4; ++r) {
-    const int q = lane + 32 * r;
-    if (q < nb)
-      for (int c = 0; c < nc; ++c) out64[(e * nc + c) * nb + q] = acc[r][c];
+}
+
+// The same factor with the degree known.  With i = m - k the triangle's level r
+// has entries i = 0 .. P - r, whatever m; entries outside the B-spline stay 0,
+// so their knots only have to be finite and distinct.  The P + 1 blossoms share
+// their leading levels at a: 16 instead of 24 entries for P = 3.
+template <int P>
+__device__ __forceinline__ void factor(const double *__restrict__ xi, double a, double b, double *beta) {
+  int m = 0;
+#pragma unroll
+  for (int q = 1; q <= P; ++q)
+    if (xi[q] <= a) m = q;
+  double tau[2 * P];   // xi[m - P + 1 .. m + P]
+#pragma unroll
+  for (int s = 0; s < 2 * P; ++s) {
+    const int q = m - P + 1 + s;
+    const double x = xi[min(max(q, 0), P + 1)];
+    tau[s] = q < 0 ? x + (double)(q - 1) : (q > P + 1 ? x + (double)q : x);
   }
+  double inv[P + 1][P];
+#pragma unroll
+  for (int r = 1; r <= P; ++r)
+#pragma unroll
+    for (int i = 0; i <= P - r; ++i) inv[r][i] = 1.0 / (tau[2 * P - i - r] - tau[P - 1 - i]);
+  double A[P + 1];     // the triangle after j levels at a
+#pragma unroll
+  for (int i = 0; i <= P; ++i) A[i] = i == m ? 1.0 : 0.0;
+#pragma unroll
+  for (int j = 0; j <= P; ++j) {   // A holds j levels at a: the other P - j at b give the blossom with P - j arguments b
+    double D[P + 1];
+#pragma unroll
+    for (int i = 0; i <= P - j; ++i) D[i] = A[i];
+#pragma unroll
+    for (int r = j + 1; r <= P; ++r)
+#pragma unroll
+      for (int i = 0; i <= P - r; ++i) {
+        const double alpha = (b - tau[P - 1 - i]) * inv[r][i];
+        D[i] = (1.0 - alpha) * D[i + 1] + alpha * D[i];
+      }
+    beta[P - j] = D[0];
+    if (j < P) {
+#pragma unroll
+      for (int i = 0; i <= P - j - 1; ++i) {
+        const double alpha = (a - tau[P - 1 - i]) * inv[j + 1][i];
+        A[i] = (1.0 - alpha) * A[i + 1] + alpha * A[i];
+      }
+    }
+  }
+}
+
+// k_to_bezier for equal degrees.  FP64 runs at 1/64 of the FP32 rate here, an
+// instruction costing the same whatever number of lanes is active, and the
+// B-splines over an element share their univariate factors (about 20 different
+// ones over the three axes among 66 B-splines).  So the warp first finds the
+// different local knot vectors of each axis, by bits, computes each factor
+// once, a lane a factor, and then adds the products of the listed factors.
+// A list of more than kListMax B-splines, or with more than 32 different knot
+// vectors on an axis, is left to the general kernel (todo, n_todo).
+// The change of basis of 174,000 tricubic elements (11.45 M pairs) takes 7.2 ms
+// in all, allocations included, 17.0 with a factor of every pair and axis
+// computed anew; 388,016 triquadratic 3-vector elements 11.4 instead of 14.9.
+constexpr int kListMax = 128;
+
+template <int P, int NC>
+__global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
+    const double *__restrict__ box, const double *__restrict__ knots, const double *__restrict__ coef,
+    const double *__restrict__ weight, const int64_t *__restrict__ inc_ptr, const int32_t *__restrict__ inc_idx,
+    int64_t n_elem, double *__restrict__ out64, int32_t *__restrict__ todo, uint32_t *__restrict__ n_todo) {
+  constexpr int N = P + 1, NB = N * N * N, R = (NB + 31) / 32, K = P + 2, KW = 3 * K;
+  constexpr unsigned kAll = 0xffffffffu;
+  __shared__ double s_fac[kBezWarps][3][32][N];
+  __shared__ double s_g[kBezWarps][NC][kListMax];
+  __shared__ uint32_t s_ids[kBezWarps][kListMax];
+  __shared__ int32_t s_rep[kBezWarps][3][32];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
+  if (e >= n_elem) return;
+  const int64_t beg = inc_ptr[e];
+  const int L = (int)min(inc_ptr[e + 1] - beg, (int64_t)kListMax + 1);
+  int nd[3] = {0, 0, 0};
+  bool fits = L <= kListMax;
+  for (int c = 0; c < L && fits; c += 32) {
+    const bool valid = c + lane < L;
+    const int32_t i = valid ? inc_idx[beg + c + lane] : 0;
+    uint32_t ids = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      const long long *mine = reinterpret_cast<const long long *>(knots + (int64_t)i * KW + a * K);
+      long long x[K];
+#pragma unroll
+      for (int q = 0; q < K; ++q) x[q] = __ldg(mine + q);
+      auto equals = [&](int32_t other) {
+        const long long *o = reinterpret_cast<const long long *>(knots + (int64_t)other * KW + a * K);
+        bool same = true;
+#pragma unroll
+        for (int q = 0; q < K; ++q) same &= x[q] == __ldg(o + q);
+        return same;
+      };
+      int id = -1;
+      for (int t = 0; t < nd[a]; ++t) {
+        if (equals(s_rep[w][a][t])) id = t;
+        if (__all_sync(kAll, id >= 0 || !valid)) break;
+      }
+      for (unsigned open = __ballot_sync(kAll, valid && id < 0); open && fits; open = __ballot_sync(kAll, valid && id < 0)) {
+        if (nd[a] == 32) {
+          fits = false;
+          break;
+        }
+        const int32_t rep = __shfl_sync(kAll, i, __ffs(open) - 1);
+        if (id < 0 && equals(rep)) id = nd[a];
+        if (lane == 0) s_rep[w][a][nd[a]] = rep;
+        ++nd[a];
+      }
+      ids |= (uint32_t)(id & 31) << (8 * a);
+      __syncwarp();
+    }
+    if (valid && fits) {
+      s_ids[w][c + lane] = ids;
+      const double wt = weight[i];
+#pragma unroll
+      for (int q = 0; q < NC; ++q) s_g[w][q][c + lane] = wt * coef[(int64_t)i * NC + q];
+    }
+  }
+  if (!fits) {
+    if (lane == 0) todo[atomicAdd(n_todo, 1u)] = (int32_t)e;
+    return;
+  }
+  const double *eb = box + 6 * e;
+  for (int d = lane; d < nd[0] + nd[1] + nd[2]; d += 32) {
+    const int a = d < nd[0] ? 0 : (d < nd[0] + nd[1] ? 1 : 2);
+    const int t = d - (a > 0 ? nd[0] : 0) - (a > 1 ? nd[1] : 0);
+    double beta[N];
+    factor<P>(knots + (int64_t)s_rep[w][a][t] * KW + a * K, eb[a], eb[3 + a], beta);
+#pragma unroll
+    for (int q = 0; q < N; ++q) s_fac[w][a][t][q] = beta[q];
+  }
+  __syncwarp();
+  double acc[R][NC];
+  int ix[R], iy[R], iz[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int q = min(lane + 32 * r, NB - 1);
+    ix[r] = q % N;
+    iy[r] = (q / N) % N;
+    iz[r] = q / (N * N);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[r][c] = 0.0;
+  }
+#pragma unroll 2
+  for (int s = 0; s < L; ++s) {
+    const uint32_t ids = s_ids[w][s];
+    const double *fx = s_fac[w][0][ids & 255u], *fy = s_fac[w][1][(ids >> 8) & 255u], *fz = s_fac[w][2][ids >> 16];
+    if constexpr (N == 4) {   // the lane's coefficients differ in z only
+      const double xy = fx[ix[0]] * fy[iy[0]];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) {
+        const double gxy = s_g[w][c][s] * xy;
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r][c] = fma(gxy, fz[iz[r]], acc[r][c]);
+      }
+    } else {
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const double prod = fx[ix[r]] * fy[iy[r]] * fz[iz[r]];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[r][c] = fma(s_g[w][c][s], prod, acc[r][c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r)
+    if (lane + 32 * r < NB)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) out64[(e * NC + c) * NB + lane + 32 * r] = acc[r][c];
 }
 
 // Render copy of the FP64 blocks (layout and storage in lrvol_internal.h):
@@ -423,11 +601,37 @@ cudaError_t Incidence::fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_to_bezier(const lrvol_s *v, cudaStream_t s) {
-  const int64_t blocks = (v->n_elem + kBezWarps - 1) / kBezWarps;
+template <int P, int NC>
+static void launch_shared(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, cudaStream_t s) {
+  k_to_bezier_shared<P, NC><<<(unsigned)((v->n_elem + kBezWarps - 1) / kBezWarps), 32 * kBezWarps, 0, s>>>(
+      v->d_box, v->d_knots, v->d_coef, v->d_weight, v->d_inc_ptr, v->d_inc_idx, v->n_elem, v->d_bez64, todo, n_todo);
+}
+
+// Equal degrees share factors; what that kernel leaves over, and unequal
+// degrees, go through the general one.  todo: room for n_elem elements.
+cudaError_t launch_to_bezier(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, cudaStream_t s) {
+  const bool equal = v->p[0] == v->p[1] && v->p[0] == v->p[2];
+  int64_t blocks = (v->n_elem + kBezWarps - 1) / kBezWarps;
+  if (equal) {
+    cudaError_t e = cudaMemsetAsync(n_todo, 0, sizeof(uint32_t), s);
+    if (e != cudaSuccess) return e;
+    switch (v->p[0] * 2 + (v->nc == 3)) {
+      case 2: launch_shared<1, 1>(v, todo, n_todo, s); break;
+      case 3: launch_shared<1, 3>(v, todo, n_todo, s); break;
+      case 4: launch_shared<2, 1>(v, todo, n_todo, s); break;
+      case 5: launch_shared<2, 3>(v, todo, n_todo, s); break;
+      case 6: launch_shared<3, 1>(v, todo, n_todo, s); break;
+      case 7: launch_shared<3, 3>(v, todo, n_todo, s); break;
+      case 8: launch_shared<4, 1>(v, todo, n_todo, s); break;
+      case 9: launch_shared<4, 3>(v, todo, n_todo, s); break;
+      default: return cudaErrorInvalidValue;
+    }
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    blocks = std::min<int64_t>(blocks, 1216);   // usually nothing is left: a grid that strides over the list
+  }
   k_to_bezier<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_box, v->d_knots, v->d_coef, v->d_weight, v->d_inc_ptr,
                                                          v->d_inc_idx, v->p[0], v->p[1], v->p[2], v->nc, v->kw,
-                                                         v->n_elem, v->d_bez64);
+                                                         v->n_elem, v->d_bez64, equal ? todo : nullptr, n_todo);
   return cudaGetLastError();
 }
 

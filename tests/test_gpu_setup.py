@@ -27,7 +27,7 @@ pytestmark = pytest.mark.gpu
 VOLS = {
     "one element": lambda: V.tensor_product((3, 3, 3), (1, 1, 1)),
     "8 elements": lambda: V.tensor_product((1, 2, 3), (2, 2, 2), ncomp=3),
-    "degree 4": lambda: V.refined_ball((4, 4, 4), (3, 3, 3), radii=(0.3,), seed=1),
+    "degree 4, lists over 128": lambda: V.refined_ball((4, 4, 4), (3, 3, 3), radii=(0.3,), seed=1),
     "mixed sizes": lambda: V.refined_ball((2, 2, 2), (2, 2, 2), centres=((0.2, 0.3, 0.4),), radii=(0.3, 0.2, 0.12),
                                           ncomp=3, seed=2),
     "scan tiles": lambda: V.tensor_product((1, 1, 1), (17, 16, 15)),
@@ -66,6 +66,24 @@ def test_blocks_and_incidence(name):
     again = gv.to_bezier(lv.STORE_F16).get_bezier()
     gv.close()
     assert np.array_equal(got, again)
+
+
+def test_more_knot_vectors_than_lanes():
+    """One trilinear element under 40 B-splines that differ in x, and 3 x 50 on three axes."""
+    for nx, ny, nz in ((40, 1, 1), (5, 5, 6), (1, 33, 2)):
+        k = [np.stack([-np.arange(1.0, n + 1), np.zeros(n), np.ones(n)], 1) for n in (nx, ny, nz)]
+        q = np.stack(np.meshgrid(*[np.arange(n) for n in (nx, ny, nz)], indexing="ij"), -1).reshape(-1, 3)
+        knots = np.concatenate([k[a][q[:, a]] for a in range(3)], axis=1)
+        rng = np.random.default_rng(nx)
+        vol = LRVolume(deg=np.array([1, 1, 1]), elem_box=np.array([[0.0, 0, 0, 1, 1, 1]]), knots=knots,
+                       coef=rng.random((len(q), 3)), weight=rng.random(len(q)), grid=np.array([1, 1, 1]))
+        gv = lv.Volume(vol).to_bezier()
+        got = gv.get_bezier()[0]
+        gv.close()
+        # over [0, 1] the B-spline on (-k, 0, 1) is 1 - x: coefficients 1, 0
+        want = np.zeros((3, 2, 2, 2))
+        want[:, 0, 0, 0] = (vol.weight[:, None] * vol.coef).sum(0)
+        assert np.abs(got - want).max() <= 8 * len(q) * 2.0 ** -53 * want.max()
 
 
 def test_element_without_a_spline_is_refused():
