@@ -1,10 +1,12 @@
 // liblrvol host side: the C ABI of lrvol.h, input validation and the k-d forest
 // build (Sec. 3.2.1).  Everything else runs in the kernels.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <numeric>
+#include <thread>
 #include <vector>
 
 #include "lrvol_internal.h"
@@ -83,27 +85,13 @@ float round_up_f32(double x) {
   return f;
 }
 
-struct ForestBuilder {
-  const lrvol_s *v;
+struct TreeBuilder {
+  const lrvol_s *v = nullptr;
   std::vector<Node> nodes;
-  std::vector<uint32_t> head;  // as ForestView::head
-  std::vector<int32_t> depth;  // per block
-  int B[3];
   bool midpoint = false;       // octree-style splits (LRVOL_SPLIT_MIDPOINT)
   bool unresolved = false;     // a midpoint tree reached kMaxDepth
 
   const double *box(int32_t e) const { return &v->box[6 * (size_t)e]; }
-  size_t head_at(int x, int y, int z) const { return ((size_t)z * (B[1] + 1) + y) * (B[0] + 1) + x; }
-
-  // The repeated last layer of each axis.
-  void pad_head() {
-    for (int z = 0; z < B[2]; ++z)
-      for (int y = 0; y < B[1]; ++y) head[head_at(B[0], y, z)] = head[head_at(B[0] - 1, y, z)];
-    for (int z = 0; z < B[2]; ++z)
-      std::copy_n(head.begin() + head_at(0, B[1] - 1, z), B[0] + 1, head.begin() + head_at(0, B[1], z));
-    std::copy_n(head.begin() + head_at(0, 0, B[2] - 1), head_at(0, 0, 1), head.begin() + head_at(0, 0, B[2]));
-  }
-
   // Build a tree over `els` inside region [rlo, rhi); returns a reference.
   uint32_t build(std::vector<int32_t> &els, const double *rlo, const double *rhi, int d, int *maxd) {
     *maxd = std::max(*maxd, d);
@@ -213,6 +201,151 @@ struct ForestBuilder {
     if (nd.child[1] == kNone) return kNone;
     nodes[me] = nd;
     return me;
+  }
+
+};
+
+// fn(k) for k = 0 .. n - 1 on up to 16 threads, the caller's among them; false
+// if a call returned false or threw.
+template <class Fn>
+bool parallel_for(int n, Fn fn) {
+  std::atomic<int> next{0};
+  std::atomic<bool> ok{true};
+  auto work = [&]() {
+    try {
+      for (int k; (k = next.fetch_add(1)) < n;)
+        if (!fn(k)) ok = false;
+    } catch (...) {
+      ok = false;
+    }
+  };
+  std::vector<std::thread> threads;
+  const int extra = std::min<int>({n, 16, (int)std::max(1u, std::thread::hardware_concurrency())}) - 1;
+  try {
+    for (int t = 0; t < extra; ++t) threads.emplace_back(work);
+  } catch (...) {   // fewer threads than wanted
+  }
+  work();
+  for (auto &t : threads) t.join();
+  return ok;
+}
+
+struct ForestBuilder : TreeBuilder {
+  std::vector<uint32_t> head;  // as ForestView::head
+  std::vector<int32_t> depth;  // per block
+  int B[3];
+
+  size_t head_at(int x, int y, int z) const { return ((size_t)z * (B[1] + 1) + y) * (B[0] + 1) + x; }
+
+  // The repeated last layer of each axis.
+  void pad_head() {
+    for (int z = 0; z < B[2]; ++z)
+      for (int y = 0; y < B[1]; ++y) head[head_at(B[0], y, z)] = head[head_at(B[0] - 1, y, z)];
+    for (int z = 0; z < B[2]; ++z)
+      std::copy_n(head.begin() + head_at(0, B[1] - 1, z), B[0] + 1, head.begin() + head_at(0, B[1], z));
+    std::copy_n(head.begin() + head_at(0, 0, B[2] - 1), head_at(0, 0, 1), head.begin() + head_at(0, 0, B[2]));
+  }
+
+  // The forest by layers of blocks: each element is painted over the blocks it
+  // meets, a block that one element meets names it, and the others get their
+  // trees.  Layers are independent and run on several threads; their nodes
+  // follow one another in layer order.  Gives the trees of region(), and false
+  // wherever a block meets no element or a tree fails: region() then decides
+  // (it accepts some meshes with gaps, and names the error).
+  // 174,000 elements in 64^3 blocks (no trees): 19.3 ms by region(), 2.7 ms so;
+  // 388,016 elements and 562,882 nodes: 145 and 18 ms.
+  bool layers() {
+    const int64_t N = v->n_elem;
+    struct Range {
+      uint16_t lo[3], hi[3];   // blocks the element meets, [lo, hi)
+    };
+    std::vector<Range> range((size_t)N);
+    const int64_t part = 16384;
+    if (!parallel_for((int)((N + part - 1) / part), [&](int k) {
+          for (int64_t e = k * part; e < std::min(N, (k + 1) * part); ++e) {
+            const double *b = box((int32_t)e);
+            for (int a = 0; a < 3; ++a) {   // exact: B is a power of two
+              range[e].lo[a] = (uint16_t)(int)(b[a] * B[a]);
+              range[e].hi[a] = (uint16_t)(int)std::ceil(b[3 + a] * B[a]);
+            }
+          }
+          return true;
+        }))
+      return false;
+    const int n_slabs = std::min(B[2], 64), thick = B[2] / n_slabs;   // powers of two
+    std::vector<std::vector<Node>> slab_nodes(n_slabs);
+    std::vector<std::vector<int64_t>> slab_trees(n_slabs);            // blocks with a tree, as offsets into `depth`
+    const size_t plane = (size_t)B[0] * B[1];
+    auto at = [&](int64_t q) { return head_at((int)(q % B[0]), (int)(q / B[0] % B[1]), (int)(q / plane)); };
+    if (!parallel_for(n_slabs, [&](int s) {
+          const int z0 = s * thick, z1 = z0 + thick;
+          auto paint = [&](auto block) {   // block(element, offset into depth) for every block of the slab it meets
+            for (int64_t e = 0; e < N; ++e) {
+              const Range &r = range[e];
+              for (int z = std::max<int>(z0, r.lo[2]); z < std::min<int>(z1, r.hi[2]); ++z)
+                for (int y = r.lo[1]; y < r.hi[1]; ++y)
+                  for (int x = r.lo[0]; x < r.hi[0]; ++x) block((int32_t)e, ((int64_t)z * B[1] + y) * B[0] + x);
+            }
+          };
+          paint([&](int32_t e, int64_t q) {   // depth counts the elements here
+            if (depth[q]++ == 0) head[at(q)] = kLeaf | (uint32_t)e;
+          });
+          std::vector<int64_t> &trees = slab_trees[s];
+          std::vector<size_t> off(1, 0);
+          for (int64_t q = z0 * (int64_t)plane; q < z1 * (int64_t)plane; ++q) {
+            if (depth[q] == 0) return false;
+            if (depth[q] == 1) {
+              depth[q] = 0;
+              continue;
+            }
+            head[at(q)] = (uint32_t)trees.size();
+            trees.push_back(q);
+            off.push_back(off.back() + depth[q]);
+          }
+          if (trees.empty()) return true;
+          std::vector<int32_t> els(off.back());
+          std::vector<size_t> cur(off.begin(), off.end() - 1);
+          paint([&](int32_t e, int64_t q) {
+            if (depth[q] > 0) els[cur[head[at(q)]]++] = e;
+          });
+          TreeBuilder tb;
+          tb.v = v;
+          tb.midpoint = midpoint;
+          for (size_t k = 0; k < trees.size(); ++k) {
+            const int64_t q = trees[k];
+            const int b[3] = {(int)(q % B[0]), (int)(q / B[0] % B[1]), (int)(q / plane)};
+            double lo[3], hi[3];
+            for (int a = 0; a < 3; ++a) {
+              lo[a] = (double)b[a] / B[a];
+              hi[a] = (double)(b[a] + 1) / B[a];
+            }
+            std::vector<int32_t> mine(els.begin() + off[k], els.begin() + off[k + 1]);
+            int maxd = 0;
+            const uint32_t r = tb.build(mine, lo, hi, 0, &maxd);
+            if (r == kNone) return false;
+            head[at(q)] = r;
+            depth[q] = maxd;
+          }
+          slab_nodes[s] = std::move(tb.nodes);
+          return true;
+        }))
+      return false;
+    size_t total = 0;
+    for (const auto &n : slab_nodes) total += n.size();
+    if (total >= kLeaf) return false;
+    nodes.clear();
+    nodes.reserve(total);
+    for (int s = 0; s < n_slabs; ++s) {
+      const uint32_t base = (uint32_t)nodes.size();
+      auto shift = [&](uint32_t r) { return r & kLeaf ? r : r + base; };
+      for (Node n : slab_nodes[s]) {
+        n.child[0] = shift(n.child[0]);
+        n.child[1] = shift(n.child[1]);
+        nodes.push_back(n);
+      }
+      for (int64_t q : slab_trees[s]) head[at(q)] = shift(head[at(q)]);
+    }
+    return true;
   }
 
   // Recursive region subdivision over blocks [b0, b1) with the elements meeting it.
@@ -507,13 +640,18 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   size_t nblk = (size_t)blocks[0] * blocks[1] * blocks[2];
   fb.head.assign(fb.head_at(0, 0, blocks[2] + 1), kNone);
   fb.depth.assign(nblk, 0);
-  std::vector<int32_t> all(v->n_elem);
-  std::iota(all.begin(), all.end(), 0);
-  int b0[3] = {0, 0, 0}, b1[3] = {blocks[0], blocks[1], blocks[2]};
-  if (!fb.region(all, b0, b1)) {
-    if (fb.unresolved)
-      return fail(LRVOL_ERR_UNSUPPORTED, "midpoint splits do not resolve this mesh (faces at non-dyadic coordinates)");
-    return fail(LRVOL_ERR_ARG, "elements do not form a box partition of [0,1]^3");
+  if (!fb.layers()) {
+    fb.nodes.clear();
+    fb.head.assign(fb.head.size(), kNone);
+    fb.depth.assign(nblk, 0);
+    std::vector<int32_t> all(v->n_elem);
+    std::iota(all.begin(), all.end(), 0);
+    int b0[3] = {0, 0, 0}, b1[3] = {blocks[0], blocks[1], blocks[2]};
+    if (!fb.region(all, b0, b1)) {
+      if (fb.unresolved)
+        return fail(LRVOL_ERR_UNSUPPORTED, "midpoint splits do not resolve this mesh (faces at non-dyadic coordinates)");
+      return fail(LRVOL_ERR_ARG, "elements do not form a box partition of [0,1]^3");
+    }
   }
   fb.pad_head();
   for (uint32_t h : fb.head)

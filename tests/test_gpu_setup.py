@@ -1,4 +1,4 @@
-"""Incidence and change of basis on the device, at sizes where the lists and
+"""Incidence, change of basis and the forest, at sizes where the lists and
 the scans change shape: one element; fewer elements than a warp; lists longer
 than 64 entries; elements of very different size in one bucket; more elements
 than a scan tile.
@@ -20,7 +20,7 @@ torch = pytest.importorskip("torch")
 from oracle.oracle import Oracle
 from paper_1707_01170_gb300 import lrvol as lv
 from paper_1707_01170_gb300.synth import volumes as V
-from paper_1707_01170_gb300.synth.lrgen import LRVolume
+from paper_1707_01170_gb300.synth.lrgen import LRVolume, Stream
 
 pytestmark = pytest.mark.gpu
 
@@ -52,6 +52,41 @@ def _incidence(vol):
     for b in vol.elem_box:
         n += int(np.all((lo <= b[:3]) & (b[3:] <= hi), axis=1).sum())
     return n
+
+
+def _half_box():
+    return LRVolume(deg=np.array([1, 1, 1]), elem_box=np.array([[0.0, 0, 0, 0.5, 0.5, 0.5]]), knots=np.tile([0.0, 0.0, 1.0], (1, 3)),
+                    coef=np.ones((1, 1)), weight=np.ones(1), grid=np.array([2, 2, 2]))
+
+
+@pytest.mark.parametrize("blocks", [(1, 1, 1), (4, 4, 4), (2, 1, 128), (64, 1, 1), (32, 64, 16)])
+@pytest.mark.parametrize("split", [lv.SPLIT_BALANCED, lv.SPLIT_MIDPOINT])
+def test_forest_shapes(blocks, split):
+    """Look-ups are exact for every shape of the forest and both split rules, on a mesh of three element sizes."""
+    vol = V.refined_ball((2, 2, 2), (4, 4, 4), centres=((0.3, 0.4, 0.55),), radii=(0.3, 0.15), seed=2)
+    X = Stream(3, 3 * 4000 + 8).take(3 * 4000).reshape(-1, 3)
+    X[::3] = np.round(X[::3] * 32) / 32
+    gv = lv.Volume(vol).build_accel(blocks, split=split)
+    got = gv.lookup(torch.from_numpy(X.astype(np.float32)).cuda()).cpu().numpy().astype(np.uint32)
+    st = gv.stats()
+    gv.close()
+    assert np.array_equal(got, Oracle(vol).lookup(X.astype(np.float32)))
+    assert (st["depth_max"] == 0) == (st["n_nodes"] == 0)
+
+
+def test_forest_accepts_and_refuses_as_it_did():
+    """A lone element with gaps around it names every block; overlapping elements are refused."""
+    gv = lv.Volume(_half_box()).build_accel((4, 4, 4))
+    assert (gv.lookup(torch.rand((100, 3), device="cuda")) == 0).all()
+    gv.close()
+    v = V.tensor_product((1, 1, 1), (2, 2, 2))
+    v.elem_box = np.concatenate([v.elem_box, v.elem_box[:1]])
+    gv = lv.Volume(v)
+    for blocks in ((1, 1, 1), (4, 4, 4)):
+        with pytest.raises(lv.LrvolError) as err:
+            gv.build_accel(blocks)
+        assert err.value.status == lv.ERR_ARG
+    gv.close()
 
 
 @pytest.mark.parametrize("name", list(VOLS))
