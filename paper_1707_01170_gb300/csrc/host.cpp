@@ -975,6 +975,7 @@ int lrvol_streamlines(lrvol_t v, const lrvol_streamline_params *P, const double 
   sp.elem = v->d_elem;
   sp.n_elem = v->n_elem;
   sp.bez = v->d_bez;
+  sp.bezc = v->d_bezc;
   sp.forest = forest_view(v);
   sp.status = v->d_status;
   sp.queue = v->d_counters + kCntQueue;

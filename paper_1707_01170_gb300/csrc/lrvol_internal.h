@@ -273,6 +273,7 @@ struct SLParams {
   const ElemRec *elem;
   int64_t n_elem;
   const unsigned char *bez;
+  const unsigned char *bezc;  // per-component copy (streamlines)
   ForestView forest;
   uint32_t *status;   // device status word (bounds)
   unsigned long long *queue;  // streamlines: next seed to trace (zeroed per call)
