@@ -1095,20 +1095,27 @@ __device__ __forceinline__ void trace_line(const SLParams &sp, const double *__r
         }
       }
       if (left) break;
-      float D0 = 0.f, D1 = 0.f, D2 = 0.f, E0 = 0.f, E1 = 0.f, E2 = 0.f;
+      float D0 = 0.f, D1 = 0.f, D2 = 0.f;
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
         if (i < T.s) {
-          const float b = T.b[i], e = T.b[i] - T.bh[i];
+          const float b = T.b[i];
           D0 = fmaf(b, k[i][0], D0);
           D1 = fmaf(b, k[i][1], D1);
           D2 = fmaf(b, k[i][2], D2);
-          E0 = fmaf(e, k[i][0], E0);
-          E1 = fmaf(e, k[i][1], E1);
-          E2 = fmaf(e, k[i][2], E2);
         }
       }
       if (sp.rule == 2) {
+        float E0 = 0.f, E1 = 0.f, E2 = 0.f;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          if (i < T.s) {
+            const float e = T.b[i] - T.bh[i];
+            E0 = fmaf(e, k[i][0], E0);
+            E1 = fmaf(e, k[i][1], E1);
+            E2 = fmaf(e, k[i][2], E2);
+          }
+        }
         const float err = hf * sqrtf(fmaf(E0, E0, fmaf(E1, E1, E2 * E2)));
         float fac = err > 0.f ? 0.9f * powf(sp.tol_f / err, 1.f / (float)(T.q_low + 1)) : 5.f;
         fac = fminf(fmaxf(fac, 0.2f), 5.f);
@@ -1177,6 +1184,18 @@ __global__ void __launch_bounds__(128) k_streamlines(const __grid_constant__ SLP
   }
 }
 
+// NaN if any operand is NaN (fminf and fmaxf would drop it)
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+  float d;
+  asm("{\n\t.reg .f32 t;\n\tmin.NaN.f32 t, %1, %2;\n\tmin.NaN.f32 %0, t, %3;\n\t}" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float d;
+  asm("{\n\t.reg .f32 t;\n\tmax.NaN.f32 t, %1, %2;\n\tmax.NaN.f32 %0, t, %3;\n\t}" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+  return d;
+}
+
 // ---- one line by four lanes ----
 // A small rake waits for the chain of its slowest line, so a line's stage is
 // split over a group of four lanes: lane c < 3 holds coordinate c of the point
@@ -1195,8 +1214,18 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
   const int c = l4 < 3 ? l4 : 2;
   float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra, rc = ra, rd = ra;   // an empty box
   Block<P, 2, STORE> blk;
+  auto in_cube = [](float x, float y, float z) {
+    return x >= 0.f && x <= 1.f && y >= 0.f && y <= 1.f && z >= 0.f && z <= 1.f;
+  };
+  // The element holding the point, its record and block; false outside the
+  // cube.  The signs of the six differences are exact, and the smallest and
+  // largest of three take one instruction each, where a chain of six compares
+  // waits for each predicate.  A box lies in the cube.
   auto locate = [&](float px, float py, float pz) -> bool {
-    if (px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z) return true;
+    const float below = min3_nan(px - ra.x, py - ra.y, pz - ra.z);
+    const float above = max3_nan(px - rb.x, py - rb.y, pz - rb.z);
+    if (below >= 0.f && above < 0.f) return true;
+    if (!in_cube(px, py, pz)) return false;
     const uint32_t e = forest_lookup(sp.forest, px, py, pz, sp.status);
     if (e >= (uint32_t)sp.n_elem) {   // kNone included
       set_status(sp.status, kStatusBounds);
@@ -1206,13 +1235,18 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
     blk.load(sp.bezc + (int64_t)e * blk.BYTES, c);
     return true;
   };
+  auto field = [&](float px, float py, float pz) -> float {   // component c in the current element
+    float bx[N], by[N], bz[N], unused0, unused1, v;
+    monomials<P>(local_u(px, ra.x, rc.x, rd.x), bx);
+    monomials<P>(local_u(py, ra.y, rc.y, rd.y), by);
+    monomials<P>(local_u(pz, ra.z, rc.z, rd.z), bz);
+    blk.components(bx, by, bz, unused0, unused1, v);
+    return v;
+  };
   auto gather = [&](float v, float &x, float &y, float &z) {
     x = __shfl_sync(group, v, 0, 4);
     y = __shfl_sync(group, v, 1, 4);
     z = __shfl_sync(group, v, 2, 4);
-  };
-  auto in_cube = [](float x, float y, float z) {
-    return x >= 0.f && x <= 1.f && y >= 0.f && y <= 1.f && z >= 0.f && z <= 1.f;
   };
   float2 *o = reinterpret_cast<float2 *>(out + q * (int64_t)sp.max_samples) + l4;   // this lane's quarter of sample 0
   auto store = [&](int at, float hi, float lo, double t) {   // as store_sample with pairs
@@ -1224,7 +1258,7 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
   float px, py, pz;
   gather(xh, px, py, pz);
   int nout = 0, st = 0;
-  if (!in_cube(px, py, pz) || !locate(px, py, pz)) {
+  if (!locate(px, py, pz)) {
     if (l4 == 0) {
       count[q] = 0;
       status[q] = 1;
@@ -1254,9 +1288,10 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
       ds_h = dsn;
     }
     bool taken = false, left = false;
-    float nh = 0.f, nl = 0.f;
+    float nh = 0.f, nl = 0.f, k[6];
+    double tn = t + h;          // its FP64 latency passes under the first stage
+    k[0] = field(px, py, pz);   // x_n, which the last step or the seed located: the same for every attempt
     for (int tries = 0; tries < 64 && !taken; ++tries) {
-      const double tn = t + h;
       const bool last = __double_as_longlong(tn) > t_end_bits;
       double hs = h;
       float hf = hf_h;
@@ -1264,26 +1299,20 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
         hs = sp.t_end - t;
         hf = __double2float_rn(hs);
       }
-      float k[6];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) {
+      for (int i = 1; i < 6; ++i) {
         if (i < T.s) {
           float d = 0.f;
 #pragma unroll
           for (int j = 0; j < i; ++j) d = fmaf(T.a[i][j], k[j], d);
           float yh = xh, yl = xl;
-          if (i > 0) ff_add(yh, yl, hf * d);
+          ff_add(yh, yl, hf * d);
           gather(yh, px, py, pz);
           k[i] = 0.f;
-          if (!left && in_cube(px, py, pz) && locate(px, py, pz)) {
-            float bx[N], by[N], bz[N], unused0, unused1;
-            monomials<P>(local_u(px, ra.x, rc.x, rd.x), bx);
-            monomials<P>(local_u(py, ra.y, rc.y, rd.y), by);
-            monomials<P>(local_u(pz, ra.z, rc.z, rd.z), bz);
-            blk.components(bx, by, bz, unused0, unused1, k[i]);
-          } else {
+          if (!left && locate(px, py, pz))
+            k[i] = field(px, py, pz);
+          else
             left = true;
-          }
         }
       }
       if (left) break;
@@ -1304,13 +1333,16 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
           h = hs * (double)fac;
           hf_h = __double2float_rn(h);
         }
-        if (err > sp.tol_f) continue;
+        if (err > sp.tol_f) {
+          tn = t + h;
+          continue;
+        }
       }
       nh = xh;
       nl = xl;
       ff_add(nh, nl, hf * D);
       gather(nh, px, py, pz);
-      if (!in_cube(px, py, pz) || !locate(px, py, pz)) {
+      if (!locate(px, py, pz)) {
         left = true;
         break;
       }

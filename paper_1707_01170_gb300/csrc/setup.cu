@@ -536,7 +536,7 @@ __global__ void k_elem_records(const double *__restrict__ box, int64_t n_elem, i
   if (b[5] - b[2] < m) m = b[5] - b[2];
   for (int a = 0; a < 3; ++a) {
     lo[a] = __double2float_ru(b[a]);
-    hi[a] = b[3 + a] == 1.0 ? __int_as_float(0x7f800000) : __double2float_ru(b[3 + a]);
+    hi[a] = b[3 + a] == 1.0 ? __int_as_float(0x3f800001) : __double2float_ru(b[3 + a]);   // the float after 1
     const double inv = 1.0 / (b[3 + a] - b[a]);
     off[a] = (float)(((double)lo[a] - b[a]) * inv);   // (lo_RU - lo) / (hi - lo), in FP64
     iw[a] = (float)inv;
