@@ -447,6 +447,16 @@ __device__ __forceinline__ bool seg_sample(const RenderParams &prm, const Ray &r
   return true;
 }
 
+// One step of an inclusive scan over the warp: the value o lanes below, where there is one.
+__device__ __forceinline__ void scan_mul(float &v, int o) {
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .f32 y;\n\tshfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff;\n\t@p mul.rn.f32 %0, %0, y;\n\t}"
+               : "+f"(v) : "r"(o));
+}
+__device__ __forceinline__ void scan_add(float &v, int o) {
+  asm volatile("{\n\t.reg .pred p;\n\t.reg .f32 y;\n\tshfl.sync.up.b32 y|p, %0, %1, 0, 0xffffffff;\n\t@p add.rn.f32 %0, %0, y;\n\t}"
+               : "+f"(v) : "r"(o));
+}
+
 // Whether the ray at parameter t has left the box [lo, hi) or the cube.
 __device__ __forceinline__ bool seg_left(const Ray &ray, const float4 &lo, const float4 &hi, float t) {
   const float px = fma_sat(t, ray.d[0], ray.o[0]);
@@ -468,8 +478,8 @@ __device__ __forceinline__ bool seg_left(const Ray &ray, const float4 &lo, const
 // With a thread per ray and a fine march per candidate the kernel evaluated
 // the visit's fine samples up to seven times, with 12 of 32 lanes active and a
 // tail of long rays: 13.0 ms for a 320x180 camera of a 174,000-element tricubic
-// volume, 3.0 ms now.  Held to 128 registers (four CTAs an SM; 3.6 ms with the
-// 146 it would take, 3.8 ms at five CTAs).
+// volume, 2.8 ms now.  Held to 128 registers for four CTAs an SM: with the 146 it
+// would take, three fit and it is a fifth slower, and five CTAs spill.
 template <int P>
 __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
                                                 const float *__restrict__ cand, int n_cand,
@@ -486,7 +496,7 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
   Block<P, 0, LRVOL_STORE_F32> blk;
   SegState st;
   st.e = kNone;
-  const float tr_stop = 1.f - prm.alpha_stop;
+  const float tr_stop = 1.f - prm.alpha_stop, inv_h = 1.f / h_fine;
   const bool is_cand = lane > 0 && lane < n_cand;
   const float my_cand = is_cand ? __ldg(cand + lane) : 1.f;
   float Tfront = 1.f, t = ray.tin;
@@ -499,12 +509,12 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
     const float4 lo = st.ra, hi = st.rb;
     const float ds = lo.w;
     float tb = t;
-    for (int q = 0; q < kMaxSamplesPerRay; q += 32) {   // 32 steps at a time, a lane each
+    for (int q = 0; q < kMaxSamplesPerRay; q += 16) {   // 16 steps at a time, a lane each (and its shadow)
       float mine = 0.f;
 #pragma unroll
-      for (int s = 0; s < 32; ++s) {
+      for (int s = 0; s < 16; ++s) {
         tb = __fadd_rn(tb, ds);
-        if (s == lane) mine = tb;
+        if (s == (lane & 15)) mine = tb;
       }
       const unsigned left = __ballot_sync(kAll, seg_left(ray, lo, hi, mine));
       if (left) {
@@ -566,6 +576,13 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
     float F0 = 0.f, F1 = 0.f, F2 = 0.f, FT = 1.f;
     bool need = lane < n_cand && t < te;
     const float te_max = __uint_as_float(__reduce_max_sync(kAll, need ? __float_as_uint(te) : 0u));   // te >= 0
+    // fine samples before te: a quotient, corrected with the samples' own places
+    int nf = 0;
+    if (need) {
+      nf = (int)fminf((te - t) * inv_h, (float)kMaxSamplesPerRay);
+      while (nf > 0 && !(__fmaf_rn((float)(nf - 1), h_fine, t) < te)) --nf;
+      while (nf < kMaxSamplesPerRay && __fmaf_rn((float)nf, h_fine, t) < te) ++nf;
+    }
     float cT = 1.f, cC0 = 0.f, cC1 = 0.f, cC2 = 0.f;   // composite of the earlier chunks
     for (int kb = 0; kb < kMaxSamplesPerRay && __any_sync(kAll, need); kb += 32) {
       const float ts = __fmaf_rn((float)(kb + lane), h_fine, t), tn = __fmaf_rn((float)(kb + lane + 1), h_fine, t);
@@ -576,31 +593,20 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
       const float T = act ? ex2_approx(src.w * (__fsub_rn(tn, ts) * prm.inv_xi)) : 1.f;
       float p = T;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const float y = __shfl_up_sync(kAll, p, o);
-        if (lane >= o) p *= y;
-      }
+      for (int o = 1; o < 32; o <<= 1) scan_mul(p, o);
       float before = __shfl_up_sync(kAll, p, 1);
       if (lane == 0) before = 1.f;
       const float Tr = cT * before, w = fmaf(-Tr, T, Tr);
       float s0 = w * src.x, s1 = w * src.y, s2 = w * src.z;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
-        const float y0 = __shfl_up_sync(kAll, s0, o), y1 = __shfl_up_sync(kAll, s1, o), y2 = __shfl_up_sync(kAll, s2, o);
-        if (lane >= o) {
-          s0 += y0;
-          s1 += y1;
-          s2 += y2;
-        }
+        scan_add(s0, o);
+        scan_add(s1, o);
+        scan_add(s2, o);
       }
-      // this chunk's samples before each end; the last of them is clipped there
-      int cnt = 0;
-      for (int c = 0; c < n_cand; ++c) {
-        const unsigned m = __ballot_sync(kAll, ts < __shfl_sync(kAll, te, c));
-        if (lane == c) cnt = __popc(m);
-      }
-      const bool fin = need && (cnt < 32 || !(__fmaf_rn((float)(kb + 32), h_fine, t) < te));
-      const int last = cnt > 0 ? cnt - 1 : 0;
+      // an end's last sample, clipped there, is in this chunk
+      const bool fin = need && nf <= kb + 32;
+      const int last = fin ? max(nf - 1 - kb, 0) : 0;
       const float gt = __shfl_sync(kAll, ts, last), gTr = __shfl_sync(kAll, Tr, last), glg = __shfl_sync(kAll, src.w, last);
       const float g0 = __shfl_sync(kAll, src.x, last), g1 = __shfl_sync(kAll, src.y, last), g2 = __shfl_sync(kAll, src.z, last);
       const int prev = last > 0 ? last - 1 : 0;
@@ -1448,13 +1454,10 @@ __global__ void __launch_bounds__(128) k_streamline_error(const SLSample *__rest
 }  // namespace
 
 // Lines per warp up to which a line gets four lanes: as many as a warp has
-// groups of four (10,000 lines of a triquadratic FP32 volume: 1.70 ms against
-// 1.88 with a lane each; 250 lines 0.95 against 1.19, tricubic 0.41 against
-// 0.80).  A lane's own FP16 block is small, and past two lines a warp the lanes
-// are worth more as lines (10,000 lines: 1.97 against 1.80 ms).  At degree 1 a
-// component is 8 coefficients and the exchange costs what it saves.
-template <int P, int STORE>
-constexpr int kGroupedLines = P == 1 ? 0 : (P == 2 && STORE == LRVOL_STORE_F16 ? 2 : 8);
+// groups of four.  250 lines of a triquadratic FP32 volume, RK4: 0.79 against
+// 1.13 ms with a lane each; 10,000 lines 1.45 against 1.83 (FP16 1.43 against
+// 1.76; tricubic 0.60 against 1.03; trilinear 0.112 against 0.117).
+constexpr int kGroupedLines = 8;
 
 template <int P, int STORE>
 cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSample *o, int32_t *count,
@@ -1474,7 +1477,7 @@ cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSamp
   const int64_t groups = (n + 4 * fit_group - 1) / (4 * fit_group);
   if ((e = cudaMemsetAsync(sp.queue, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
   SLParams spl = sp;
-  const bool grouped = groups <= kGroupedLines<P, STORE>;
+  const bool grouped = groups <= kGroupedLines;
   spl.pair_out = grouped || lanes < 32;
   if (grouped) {
     const int64_t need = (n + 4 * groups - 1) / (4 * groups);
