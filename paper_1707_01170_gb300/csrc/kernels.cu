@@ -705,9 +705,9 @@ __device__ __forceinline__ float pick3(int k, float x, float y, float z) { retur
 // Watertight ray/triangle test (Woop, Benthin and Wald, JCGT 2013), FP32,
 // with the oracle's order of operations; component selection by value so
 // that nothing goes to local memory.
-// v: the triangle's 9 coordinates, in global memory or in registers (plain loads).
-__device__ __forceinline__ bool tri_hit(const Ray &ray, const float *__restrict__ v, float &t, bool &front) {
-  const float d0 = ray.d[0], d1 = ray.d[1], d2 = ray.d[2];
+// v: the triangle's 9 coordinates relative to the ray's origin (in registers).
+__device__ __forceinline__ bool tri_hit(const float *d, const float *v, float &t, bool &front) {
+  const float d0 = d[0], d1 = d[1], d2 = d[2];
   int kz = 0;
   if (fabsf(d1) > fabsf(pick3(kz, d0, d1, d2))) kz = 1;
   if (fabsf(d2) > fabsf(pick3(kz, d0, d1, d2))) kz = 2;
@@ -720,12 +720,7 @@ __device__ __forceinline__ bool tri_hit(const Ray &ray, const float *__restrict_
   }
   const float Sx = __fdiv_rn(pick3(kx, d0, d1, d2), dz), Sy = __fdiv_rn(pick3(ky, d0, d1, d2), dz);
   const float Sz = __fdiv_rn(1.f, dz);
-  const float a0 = __fsub_rn(v[0], ray.o[0]), a1 = __fsub_rn(v[1], ray.o[1]);
-  const float a2 = __fsub_rn(v[2], ray.o[2]);
-  const float b0 = __fsub_rn(v[3], ray.o[0]), b1 = __fsub_rn(v[4], ray.o[1]);
-  const float b2 = __fsub_rn(v[5], ray.o[2]);
-  const float c0 = __fsub_rn(v[6], ray.o[0]), c1 = __fsub_rn(v[7], ray.o[1]);
-  const float c2 = __fsub_rn(v[8], ray.o[2]);
+  const float a0 = v[0], a1 = v[1], a2 = v[2], b0 = v[3], b1 = v[4], b2 = v[5], c0 = v[6], c1 = v[7], c2 = v[8];
   const float Akz = pick3(kz, a0, a1, a2), Bkz = pick3(kz, b0, b1, b2), Ckz = pick3(kz, c0, c1, c2);
   const float Ax = __fsub_rn(pick3(kx, a0, a1, a2), __fmul_rn(Sx, Akz));
   const float Ay = __fsub_rn(pick3(ky, a0, a1, a2), __fmul_rn(Sy, Akz));
@@ -755,16 +750,21 @@ __device__ __forceinline__ bool tri_hit(const Ray &ray, const float *__restrict_
 // The pixels whose centres (i + 1/2, j + 1/2) project into the image-plane
 // box [amin, amax] x [bmin, bmax], widened by a margin: 1/4 pixel plus 1e-5
 // of the box's coordinates in pixels.  The FP32 projection of a primitive's
-// vertices and the FP32 pixel rays of make_ray are each within a few ulps of
-// exact, a few thousandths of a pixel even for narrow fields of view, so
-// every pixel whose ray can hit the primitive is in the box.  False if the
-// box holds no pixel centre.
-__device__ __forceinline__ bool pixel_box(const RayConsts &K, int width, int height, float amin, float amax,
-                                          float bmin, float bmax, int &i0, int &i1, int &j0, int &j1) {
-  const float ia = (amin - K.sxo) / K.sxs - 0.5f, ib = (amax - K.sxo) / K.sxs - 0.5f;
-  const float ja = (bmin - K.syo) / K.sys - 0.5f, jb = (bmax - K.syo) / K.sys - 0.5f;
-  const float mi = 0.25f + 1e-5f * (fabsf(amin) + fabsf(amax) + 1.f) / fabsf(K.sxs);
-  const float mj = 0.25f + 1e-5f * (fabsf(bmin) + fabsf(bmax) + 1.f) / fabsf(K.sys);
+// vertices, with approximate reciprocals (2^-22 relative), and the FP32 pixel
+// rays of make_ray are each within a few ulps of exact, a few thousandths of a
+// pixel even for narrow fields of view, so every pixel whose ray can hit the
+// primitive is in the box.  False if the box holds no pixel centre.
+struct PixelScale {
+  float ax, ay, bx, by;   // pixel = a * image-plane coordinate + b - 1/2
+  __device__ __forceinline__ explicit PixelScale(const RayConsts &K)
+      : ax(1.f / K.sxs), ay(1.f / K.sys), bx(-K.sxo / K.sxs), by(-K.syo / K.sys) {}
+};
+__device__ __forceinline__ bool pixel_box(const PixelScale &S, int width, int height, float amin, float amax, float bmin,
+                                          float bmax, int &i0, int &i1, int &j0, int &j1) {
+  const float ia = fmaf(amin, S.ax, S.bx) - 0.5f, ib = fmaf(amax, S.ax, S.bx) - 0.5f;
+  const float ja = fmaf(bmin, S.ay, S.by) - 0.5f, jb = fmaf(bmax, S.ay, S.by) - 0.5f;
+  const float mi = 0.25f + 1e-5f * (fabsf(amin) + fabsf(amax) + 1.f) * fabsf(S.ax);
+  const float mj = 0.25f + 1e-5f * (fabsf(bmin) + fabsf(bmax) + 1.f) * fabsf(S.ay);
   // clamp before converting (NaN widens to the whole image)
   const float lo_i = fmaxf(fminf(ia, ib) - mi, -1.f), hi_i = fminf(fmaxf(ia, ib) + mi, (float)width);
   const float lo_j = fmaxf(fminf(ja, jb) - mj, -1.f), hi_j = fminf(fmaxf(ja, jb) + mj, (float)height);
@@ -774,37 +774,98 @@ __device__ __forceinline__ bool pixel_box(const RayConsts &K, int width, int hei
   j1 = min(height - 1, (int)floorf(hi_j));
   return i0 <= i1 && j0 <= j1;
 }
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 
 __global__ void k_trim_init(float2 *__restrict__ out, int64_t n) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q < n) out[q] = make_float2(__int_as_float(0x7f800000), 0.f);
 }
 
+// Walks the (primitive, pixel) pairs of a warp's 32 primitives, 32 pairs at a
+// time: lane l's primitive has the cnt pairs from exc on.  A lane finds its
+// pair's primitive by counting the primitives that start at or before it: a
+// mask of the starts within the 32 pairs and the number of earlier ones, kept
+// along.  The primitives' data lie in shared memory, those with pairs first, in
+// order ("slots").
+struct PairWalk {
+  long long w0, w1;       // this warp's pairs
+  long long rel;          // the lane's first pair, relative to the current 32
+  unsigned first;         // exc modulo 2^32: a primitive has < 2^31 pairs
+  int slot;               // the lane's slot
+  int before;             // primitives that start before the current 32 pairs
+  bool has;
+
+  // `split` warps share the pairs, this one is `part`
+  __device__ __forceinline__ PairWalk(int lane, int cnt, int split, int part) {
+    const unsigned all = 0xffffffffu;
+    long long inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const long long y = __shfl_up_sync(all, inc, o);
+      if (lane >= o) inc += y;
+    }
+    const long long total = __shfl_sync(all, inc, 31), exc = inc - cnt;
+    const long long chunk = (((total + split - 1) / split) + 31) & ~31ll;
+    w0 = (long long)part * chunk;
+    w1 = w0 + chunk < total ? w0 + chunk : total;
+    rel = exc - w0;
+    first = (unsigned)exc;
+    has = cnt > 0;
+    const unsigned nonempty = __ballot_sync(all, has);
+    slot = __popc(nonempty & ((1u << lane) - 1u));
+    before = __popc(__ballot_sync(all, has && rel < 0));
+  }
+  // slot of pair base + lane, for base = w0, w0 + 32, ...
+  __device__ __forceinline__ int next(int lane) {
+    const unsigned starts = __reduce_or_sync(0xffffffffu, has && rel >= 0 && rel < 32 ? 1u << (int)rel : 0u);
+    const int s = before + __popc(starts & (0xffffffffu >> (31 - lane))) - 1;
+    before += __popc(starts);
+    rel -= 32;
+    return s;
+  }
+};
+
+// Row of pixel `pix` of a box of width bw.  Below 2^21 pixels the FP32 product
+// with 1/bw is within 0.5/bw of (pix + 1/2)/bw, so its floor is exact.
+__device__ __forceinline__ unsigned box_row(unsigned pix, unsigned bw, float inv_bw) {
+  return pix < (1u << 21) ? (unsigned)(((float)pix + 0.5f) * inv_bw) : pix / bw;
+}
+
 // One warp takes 32 consecutive triangles: lane l projects triangle l of the
 // group and finds its pixel box, then the warp walks the group's (triangle,
-// pixel) pairs 32 at a time, each lane finding its pair's triangle by a
-// search over the lanes' prefix sums and fetching that triangle by shuffles.
-// Small triangles (most of a fine mesh covers a pixel centre or none) then
-// cost one lane's set-up instead of a warp's.  `split` warps share a group,
-// each taking a contiguous part of its pairs, so a coarse mesh of large
-// triangles still spreads over the GPU.
+// pixel) pairs.  Small triangles (most of a fine mesh covers a pixel centre or
+// none) then cost one lane's set-up instead of a warp's.  `split` warps share a
+// group, each taking a contiguous part of its pairs, so a coarse mesh of large
+// triangles still spreads over the GPU.  A fine mesh is bound by the set-up of
+// its triangles (2.4 M of them at 1280x720: 92 us; 104 with divisions in the
+// projection and the pairs searched by shuffles; 99 with the vertices staged
+// through shared memory).
 __global__ void __launch_bounds__(128) k_trim_raster(const RayConsts K, int width, int height,
                                                      const float *__restrict__ tri, int64_t n_tri, int split,
                                                      float2 *__restrict__ out) {
-  const unsigned full_mask = 0xffffffffu;
+  // A triangle that has pairs: its vertices (perspective: relative to the eye),
+  // 1/width, width, first pair and corner of its box.  80 bytes, so that eight
+  // lanes' 16-byte accesses to eight slots touch every bank once.
+  struct Slot {
+    float4 q[5];
+  };
+  __shared__ Slot slots[4][32];
   const int lane = threadIdx.x & 31;
+  Slot *sl = slots[threadIdx.x >> 5];
   const int64_t wid = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
   const int64_t group = wid / split;
   const int part = (int)(wid - group * split);
   if (group * 32 >= n_tri) return;   // whole warp
-  const int64_t tr = group * 32 + lane;
   float v[9];
+  const int64_t tr = group * 32 + lane;
 #pragma unroll
-  for (int c = 0; c < 9; ++c) v[c] = 0.f;
+  for (int c = 0; c < 9; ++c) v[c] = tr < n_tri ? __ldg(tri + 9 * tr + c) : 0.f;
   int i0 = 0, j0 = 0, bw = 1, cnt = 0;
   if (tr < n_tri) {
-#pragma unroll
-    for (int c = 0; c < 9; ++c) v[c] = __ldg(tri + 9 * tr + c);
     // conservative pixel box of the projected triangle (whole image when a
     // vertex is at or behind the eye plane; nothing when all three are)
     float amin = __int_as_float(0x7f800000), amax = -amin, bmin = amin, bmax = -amin;
@@ -823,8 +884,9 @@ __global__ void __launch_bounds__(128) k_trim_raster(const RayConsts K, int widt
           ++behind;
           continue;
         }
-        a = r / z;
-        b = u / z;
+        const float iz = rcp_approx(z);
+        a = r * iz;
+        b = u * iz;
       }
       amin = fminf(amin, a);
       amax = fmaxf(amax, a);
@@ -832,7 +894,7 @@ __global__ void __launch_bounds__(128) k_trim_raster(const RayConsts K, int widt
       bmax = fmaxf(bmax, b);
     }
     int i1 = width - 1, j1 = height - 1;
-    if (behind < 3 && (full || pixel_box(K, width, height, amin, amax, bmin, bmax, i0, i1, j0, j1))) {
+    if (behind < 3 && (full || pixel_box(PixelScale(K), width, height, amin, amax, bmin, bmax, i0, i1, j0, j1))) {
       if (full) {
         i0 = 0;
         j0 = 0;
@@ -843,38 +905,36 @@ __global__ void __launch_bounds__(128) k_trim_raster(const RayConsts K, int widt
       cnt = bw * (j1 - j0 + 1);   // <= 32768^2 < 2^31
     }
   }
-  // prefix sums of the lanes' pair counts
-  long long inc = cnt;
+  PairWalk walk(lane, cnt, split, part);
+  if (walk.has) {
+    Slot &m = sl[walk.slot];
+    if (K.persp) {
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const long long y = __shfl_up_sync(full_mask, inc, o);
-    if (lane >= o) inc += y;
-  }
-  const long long total = __shfl_sync(full_mask, inc, 31), exc = inc - cnt;
-  const long long chunk = (((total + split - 1) / split) + 31) & ~31ll;
-  const long long w0 = (long long)part * chunk, w1 = w0 + chunk < total ? w0 + chunk : total;
-  for (long long base = w0; base < w1; base += 32) {
-    const long long w = base + lane;
-    int q = 0;   // the last lane whose pairs start at or before w (its count is then > 0)
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-      const long long e = __shfl_sync(full_mask, exc, q + step);
-      if (e <= w) q += step;
+      for (int c = 0; c < 9; ++c) v[c] = __fsub_rn(v[c], K.E[c % 3]);
     }
-    const long long eq = __shfl_sync(full_mask, exc, q);
-    const int qi0 = __shfl_sync(full_mask, i0, q), qj0 = __shfl_sync(full_mask, j0, q);
-    const int qbw = __shfl_sync(full_mask, bw, q);
-    float tv[9];
-#pragma unroll
-    for (int c = 0; c < 9; ++c) tv[c] = __shfl_sync(full_mask, v[c], q);
-    if (w >= w1) continue;
-    const unsigned pix = (unsigned)(w - eq);
-    const int i = qi0 + (int)(pix % (unsigned)qbw), j = qj0 + (int)(pix / (unsigned)qbw);
+    m.q[0] = make_float4(v[0], v[1], v[2], v[3]);
+    m.q[1] = make_float4(v[4], v[5], v[6], v[7]);
+    m.q[2] = make_float4(v[8], 1.f / (float)bw, __int_as_float(bw), __uint_as_float(walk.first));
+    m.q[3] = make_float4(__int_as_float(i0), __int_as_float(j0), 0.f, 0.f);
+  }
+  __syncwarp();
+  for (long long base = walk.w0; base < walk.w1; base += 32) {
+    const Slot &m = sl[walk.next(lane)];
+    if (base + lane >= walk.w1) continue;
+    const float4 q0 = m.q[0], q1 = m.q[1], q2 = m.q[2], q3 = m.q[3];
+    const unsigned bw = __float_as_uint(q2.z), pix = (unsigned)(base + lane) - __float_as_uint(q2.w);
+    const unsigned row = box_row(pix, bw, q2.y);
+    const int i = __float_as_int(q3.x) + (int)(pix - row * bw), j = __float_as_int(q3.y) + (int)row;
     Ray ray;
     make_ray(K, i, j, ray);   // origin and direction; the unit-cube interval is not needed here
+    float tv[9] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w, q2.x};
+    if (!K.persp) {
+#pragma unroll
+      for (int c = 0; c < 9; ++c) tv[c] = __fsub_rn(tv[c], ray.o[c % 3]);
+    }
     float t;
     bool front;
-    if (!tri_hit(ray, tv, t, front)) continue;
+    if (!tri_hit(ray.d, tv, t, front)) continue;
     unsigned *slot = reinterpret_cast<unsigned *>(out + (int64_t)j * width + i);
     if (front)
       atomicMin(slot, __float_as_uint(t));
@@ -1527,56 +1587,63 @@ __device__ __forceinline__ float dot3r(float x0, float x1, float x2, float y0, f
   return __fadd_rn(__fadd_rn(__fmul_rn(x0, y0), __fmul_rn(x1, y1)), __fmul_rn(x2, y2));
 }
 
+// What the ray/capsule test needs of a segment and the ray's origin: computed
+// once per segment when all rays start at the eye.
+struct Capsule {
+  float ba[3], baba;   // b - a and its square
+  float oa[3], baoa;   // origin - a, and its product with b - a
+  float ob[3], C;      // origin - b; baba |oa|^2 - baoa^2 - r^2 baba
+  float ca, cb;        // |oa|^2 - r^2, |ob|^2 - r^2
+  __device__ __forceinline__ void set(const float *o, const float *a, const float *b, float r) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      ba[c] = __fsub_rn(b[c], a[c]);
+      oa[c] = __fsub_rn(o[c], a[c]);
+      ob[c] = __fsub_rn(o[c], b[c]);
+    }
+    const float rr = __fmul_rn(r, r), oaoa = dot3r(oa[0], oa[1], oa[2], oa[0], oa[1], oa[2]);
+    baba = dot3r(ba[0], ba[1], ba[2], ba[0], ba[1], ba[2]);
+    baoa = dot3r(ba[0], ba[1], ba[2], oa[0], oa[1], oa[2]);
+    C = __fsub_rn(__fsub_rn(__fmul_rn(baba, oaoa), __fmul_rn(baoa, baoa)), __fmul_rn(rr, baba));
+    ca = __fsub_rn(oaoa, rr);
+    cb = __fsub_rn(dot3r(ob[0], ob[1], ob[2], ob[0], ob[1], ob[2]), rr);
+  }
+};
+
 // Ray/capsule hit in FP32 with the oracle's order of operations; t > 0 only.
-__device__ __forceinline__ bool capsule_hit(const Ray &ray, const float *a, const float *b, float r, float &t) {
-  const float ba0 = __fsub_rn(b[0], a[0]), ba1 = __fsub_rn(b[1], a[1]), ba2 = __fsub_rn(b[2], a[2]);
-  const float oa0 = __fsub_rn(ray.o[0], a[0]), oa1 = __fsub_rn(ray.o[1], a[1]), oa2 = __fsub_rn(ray.o[2], a[2]);
-  const float ob0 = __fsub_rn(ray.o[0], b[0]), ob1 = __fsub_rn(ray.o[1], b[1]), ob2 = __fsub_rn(ray.o[2], b[2]);
-  const float d0 = ray.d[0], d1 = ray.d[1], d2 = ray.d[2];
-  const float baba = dot3r(ba0, ba1, ba2, ba0, ba1, ba2), bard = dot3r(ba0, ba1, ba2, d0, d1, d2);
-  const float baoa = dot3r(ba0, ba1, ba2, oa0, oa1, oa2), rdoa = dot3r(d0, d1, d2, oa0, oa1, oa2);
-  const float oaoa = dot3r(oa0, oa1, oa2, oa0, oa1, oa2), rr = __fmul_rn(r, r);
-  const float A = __fsub_rn(baba, __fmul_rn(bard, bard));
+__device__ __forceinline__ bool capsule_hit(const Capsule &S, float d0, float d1, float d2, float &t) {
+  const float bard = dot3r(S.ba[0], S.ba[1], S.ba[2], d0, d1, d2), rdoa = dot3r(d0, d1, d2, S.oa[0], S.oa[1], S.oa[2]);
+  const float A = __fsub_rn(S.baba, __fmul_rn(bard, bard));
   if (A > 0.f) {
-    const float B = __fsub_rn(__fmul_rn(baba, rdoa), __fmul_rn(baoa, bard));
-    const float C = __fsub_rn(__fsub_rn(__fmul_rn(baba, oaoa), __fmul_rn(baoa, baoa)), __fmul_rn(rr, baba));
-    const float H = __fsub_rn(__fmul_rn(B, B), __fmul_rn(A, C));
+    const float B = __fsub_rn(__fmul_rn(S.baba, rdoa), __fmul_rn(S.baoa, bard));
+    const float H = __fsub_rn(__fmul_rn(B, B), __fmul_rn(A, S.C));
     if (H >= 0.f) {
       const float tb = __fdiv_rn(__fsub_rn(-B, __fsqrt_rn(H)), A);
-      const float y = __fadd_rn(baoa, __fmul_rn(tb, bard));
-      if (y > 0.f && y < baba) {
-        if (tb > 0.f) {
-          t = tb;
-          return true;
-        }
-        return false;
+      const float y = __fadd_rn(S.baoa, __fmul_rn(tb, bard));
+      if (y > 0.f && y < S.baba) {
+        t = tb;
+        return tb > 0.f;
       }
     }
   }
   float best = __int_as_float(0x7f800000);
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
-    const float c0 = k == 0 ? oa0 : ob0, c1 = k == 0 ? oa1 : ob1, c2 = k == 0 ? oa2 : ob2;
-    const float bb = dot3r(d0, d1, d2, c0, c1, c2), cc = __fsub_rn(dot3r(c0, c1, c2, c0, c1, c2), rr);
-    const float h = __fsub_rn(__fmul_rn(bb, bb), cc);
+    const float bb = k == 0 ? rdoa : dot3r(d0, d1, d2, S.ob[0], S.ob[1], S.ob[2]);
+    const float h = __fsub_rn(__fmul_rn(bb, bb), k == 0 ? S.ca : S.cb);
     if (h > 0.f) {
       const float tc = __fsub_rn(-bb, __fsqrt_rn(h));
       if (tc > 0.f && tc < best) best = tc;
     }
   }
-  if (best < __int_as_float(0x7f800000)) {
-    t = best;
-    return true;
-  }
-  return false;
+  t = best;
+  return best < __int_as_float(0x7f800000);
 }
 
 __device__ __forceinline__ bool tube_segment(const TubeParams &tp, int64_t s, float *a, float *b) {
-  const int per = tp.max_samples - 1;
-  const int64_t j = s / per;
-  const int k = (int)(s % per);
-  if (k >= tp.count[j] - 1) return false;
-  const double *p = tp.samples + (j * tp.max_samples + k) * 4;
+  const unsigned per = (unsigned)(tp.max_samples - 1), j = (unsigned)s / per, k = (unsigned)s - j * per;   // s < 2^32
+  if ((int)k >= tp.count[j] - 1) return false;
+  const double *p = tp.samples + ((int64_t)j * tp.max_samples + k) * 4;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     a[c] = __double2float_rn(p[c]);
@@ -1585,33 +1652,80 @@ __device__ __forceinline__ bool tube_segment(const TubeParams &tp, int64_t s, fl
   return true;
 }
 
-__global__ void k_vis_init(unsigned long long *__restrict__ vis, int64_t n) {
-  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < n) vis[q] = ~0ull;
+// No hit anywhere, and with a ray table (rays not null) each pixel's direction in
+// the pixel's place of the image (until the resolve overwrites it).
+__global__ void __launch_bounds__(256) k_tube_init(const RayConsts K, int width, int height,
+                                                   unsigned long long *__restrict__ vis, float4 *__restrict__ rays) {
+  const int i = blockIdx.x * 64 + (threadIdx.x & 63), j = blockIdx.y * 4 + (threadIdx.x >> 6);
+  if (i >= width || j >= height) return;
+  const int64_t q = (int64_t)j * width + i;
+  vis[q] = ~0ull;
+  if (rays) {
+    Ray ray;
+    make_ray(K, i, j, ray);
+    rays[q] = make_float4(ray.d[0], ray.d[1], ray.d[2], 0.f);
+  }
 }
 
-__device__ __forceinline__ void tube_group(const TubeParams &tp, int64_t line, int k0, int nseg, int split, int part,
-                                           int lane);
+__device__ __forceinline__ void tube_dir(const TubeParams &tp, int i, int j, Ray &ray) {
+  if (tp.ray_table) {   // perspective: every ray starts at the eye
+    const float4 d = reinterpret_cast<const float4 *>(tp.out)[(int64_t)j * tp.width + i];
+    ray.d[0] = d.x;
+    ray.d[1] = d.y;
+    ray.d[2] = d.z;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) ray.o[c] = tp.ray.E[c];
+  } else {
+    make_ray(tp.ray, i, j, ray);
+  }
+}
 
-// One warp per line (times `split`) walks the line's segments in groups of
-// 32: lane l bounds segment l of the group on the screen, then the warp walks
-// the group's (segment, pixel) pairs 32 at a time, as the trimming raster
-// does.  `split` warps share a line, each taking a contiguous part of every
-// group's pairs, when few long segments could cover much of the image.
-__global__ void __launch_bounds__(128) k_tube_raster(const __grid_constant__ TubeParams tp, int split) {
+// A segment that has pairs.  80 bytes, moved 16 at a time: eight lanes' accesses
+// to eight slots touch every bank once.
+struct __align__(16) TubeSlot {
+  Capsule cap;          // perspective; otherwise the end points in cap.ba and cap.ob
+  float inv_bw;
+  unsigned sid, first;  // segment id, first pair
+  int bw, i0, j0;
+  __device__ __forceinline__ void put(TubeSlot *to) const {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) reinterpret_cast<float4 *>(to)[q] = reinterpret_cast<const float4 *>(this)[q];
+  }
+  __device__ __forceinline__ void get(const TubeSlot *from) {
+#pragma unroll
+    for (int q = 0; q < 5; ++q) reinterpret_cast<float4 *>(this)[q] = reinterpret_cast<const float4 *>(from)[q];
+  }
+};
+static_assert(sizeof(TubeSlot) == 80, "five 16-byte accesses");
+
+__device__ __forceinline__ void tube_group(const TubeParams &tp, int64_t line, int k0, int nseg, int split, int part,
+                                           int lane, TubeSlot *sl);
+
+// A line's segments go in groups of 32: lane l bounds segment l of the group on
+// the screen, then the warp walks the group's (segment, pixel) pairs 32 at a
+// time, as the trimming raster does.  `strides` warps take a line's groups in
+// turn, and `split` warps share each group's pairs, when few long segments
+// could cover much of the image.
+// Bound by instructions: a segment's share of the test is computed once and
+// read from shared memory, a pixel's ray from the table.  4,096 lines of 63
+// segments at 1920x1080, in all: 263 us; 335 with both computed for every pair.
+constexpr int kTubeWarps = 1;   // an SM takes the next warp when one ends: 4096 lines 263 us, 276 in CTAs of 2 or 4 warps
+
+__global__ void __launch_bounds__(32 * kTubeWarps) k_tube_raster(const __grid_constant__ TubeParams tp, int strides,
+                                                                 int split) {
+  __shared__ TubeSlot slots[kTubeWarps][32];
   const int lane = threadIdx.x & 31;
-  const int64_t wid = (int64_t)blockIdx.x * 4 + (threadIdx.x >> 5);
-  const int64_t line = wid / split;
-  const int part = (int)(wid - line * split);
+  const int64_t wid = (int64_t)blockIdx.x * kTubeWarps + (threadIdx.x >> 5);
+  const int64_t at = wid / split, line = at / strides;
+  const int part = (int)(wid - at * split);
   if (line >= tp.n_lines) return;                      // whole warp
   const int nseg = tp.count[line] - 1;
-  for (int k0 = 0; k0 < nseg; k0 += 32) tube_group(tp, line, k0, nseg, split, part, lane);
+  for (int k0 = 32 * (int)(at - line * strides); k0 < nseg; k0 += 32 * strides) tube_group(tp, line, k0, nseg, split, part, lane, slots[threadIdx.x >> 5]);
 }
 
 // One group of 32 segment slots of a line (see k_tube_raster).
 __device__ __forceinline__ void tube_group(const TubeParams &tp, int64_t line, int k0, int nseg, int split, int part,
-                                           int lane) {
-  const unsigned full_mask = 0xffffffffu;
+                                           int lane, TubeSlot *sl) {
   const int per = tp.max_samples - 1;                  // segment slots per line
   const RayConsts &K = tp.ray;
   float a[3] = {0.f, 0.f, 0.f}, b[3] = {0.f, 0.f, 0.f};
@@ -1636,8 +1750,9 @@ __device__ __forceinline__ void tube_group(const TubeParams &tp, int64_t line, i
           ++behind;
           continue;
         }
-        x = r / z;
-        y = u / z;
+        const float iz = rcp_approx(z);
+        x = r * iz;
+        y = u * iz;
       }
       amin = fminf(amin, x);
       amax = fmaxf(amax, x);
@@ -1645,7 +1760,7 @@ __device__ __forceinline__ void tube_group(const TubeParams &tp, int64_t line, i
       bmax = fmaxf(bmax, y);
     }
     int i1 = tp.width - 1, j1 = tp.height - 1;
-    if (behind < 8 && (full || pixel_box(K, tp.width, tp.height, amin, amax, bmin, bmax, i0, i1, j0, j1))) {
+    if (behind < 8 && (full || pixel_box(PixelScale(K), tp.width, tp.height, amin, amax, bmin, bmax, i0, i1, j0, j1))) {
       if (full) {
         i0 = 0;
         j0 = 0;
@@ -1656,43 +1771,50 @@ __device__ __forceinline__ void tube_group(const TubeParams &tp, int64_t line, i
       cnt = bw * (j1 - j0 + 1);   // <= 32768^2 < 2^31
     }
   }
-  long long inc = cnt;
+  PairWalk walk(lane, cnt, split, part);
+  if (walk.has) {
+    TubeSlot m;
+    if (K.persp) {
+      m.cap.set(K.E, a, b, tp.radius);
+    } else {
+      m.cap = Capsule{};
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const long long y = __shfl_up_sync(full_mask, inc, o);
-    if (lane >= o) inc += y;
+      for (int c = 0; c < 3; ++c) {
+        m.cap.ba[c] = a[c];
+        m.cap.ob[c] = b[c];
+      }
+    }
+    m.inv_bw = 1.f / (float)bw;
+    m.sid = (uint32_t)(line * per + k0 + lane);
+    m.first = walk.first;
+    m.bw = bw;
+    m.i0 = i0;
+    m.j0 = j0;
+    m.put(sl + walk.slot);
   }
-  const long long total = __shfl_sync(full_mask, inc, 31), exc = inc - cnt;
-  const long long chunk = (((total + split - 1) / split) + 31) & ~31ll;
-  const long long w0 = (long long)part * chunk, w1 = w0 + chunk < total ? w0 + chunk : total;
-  for (long long base = w0; base < w1; base += 32) {
-    const long long w = base + lane;
-    int q = 0;   // the last lane whose pairs start at or before w (its count is then > 0)
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-      const long long e = __shfl_sync(full_mask, exc, q + step);
-      if (e <= w) q += step;
-    }
-    const long long eq = __shfl_sync(full_mask, exc, q);
-    const int qi0 = __shfl_sync(full_mask, i0, q), qj0 = __shfl_sync(full_mask, j0, q);
-    const int qbw = __shfl_sync(full_mask, bw, q);
-    float qa[3], qb[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      qa[c] = __shfl_sync(full_mask, a[c], q);
-      qb[c] = __shfl_sync(full_mask, b[c], q);
-    }
-    if (w >= w1) continue;
-    const unsigned pix = (unsigned)(w - eq);
-    const int i = qi0 + (int)(pix % (unsigned)qbw), j = qj0 + (int)(pix / (unsigned)qbw);
+  __syncwarp();
+  for (long long base = walk.w0; base < walk.w1; base += 32) {
+    TubeSlot m;
+    m.get(sl + walk.next(lane));
+    if (base + lane >= walk.w1) continue;
+    const unsigned pix = (unsigned)(base + lane) - m.first, row = box_row(pix, (unsigned)m.bw, m.inv_bw);
+    const int i = m.i0 + (int)(pix - row * (unsigned)m.bw), j = m.j0 + (int)row;
     Ray ray;
-    make_ray(K, i, j, ray);
+    tube_dir(tp, i, j, ray);
     float t;
-    if (!capsule_hit(ray, qa, qb, tp.radius, t)) continue;
-    const uint32_t sid = (uint32_t)(line * per + k0 + q);
-    const unsigned long long key = ((unsigned long long)__float_as_uint(t) << 32) | (unsigned long long)sid;
+    bool hit;
+    if (K.persp) {
+      hit = capsule_hit(m.cap, ray.d[0], ray.d[1], ray.d[2], t);
+    } else {
+      Capsule cap;
+      cap.set(ray.o, m.cap.ba, m.cap.ob, tp.radius);
+      hit = capsule_hit(cap, ray.d[0], ray.d[1], ray.d[2], t);
+    }
+    if (!hit) continue;
+    const unsigned long long key = ((unsigned long long)__float_as_uint(t) << 32) | (unsigned long long)m.sid;
     atomicMin(tp.vis + (int64_t)j * tp.width + i, key);
   }
+  __syncwarp();   // the next group overwrites the slots
 }
 
 template <int P, int STORE>
@@ -1710,7 +1832,7 @@ __global__ void __launch_bounds__(128) k_tube_resolve(const __grid_constant__ Tu
   float a[3], b[3];
   tube_segment(tp, s, a, b);
   Ray ray;
-  make_ray(tp.ray, (int)(q % tp.width), (int)(q / tp.width), ray);
+  tube_dir(tp, (int)((unsigned)q % (unsigned)tp.width), (int)((unsigned)q / (unsigned)tp.width), ray);   // q < 2^30
   float p[3], ba[3], pa[3], qa[3];
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
@@ -1742,18 +1864,33 @@ __global__ void __launch_bounds__(128) k_tube_resolve(const __grid_constant__ Tu
 
 }  // namespace
 
-cudaError_t launch_tubes(const TubeParams &tp, int degree, int storage, cudaStream_t s) {
+// A perspective ray costs a rounded square root and three rounded quotients for
+// each of its pairs; with at least a segment to 64 pixels they are computed once
+// per pixel instead (4,096 lines of 199 segments at 1920x1080: 0.73 against 0.82
+// ms; 40 lines of 99, a segment to 520 pixels: 101 against 97 us).
+constexpr int64_t kTubeTablePixels = 64;
+
+cudaError_t launch_tubes(TubeParams tp, int degree, int storage, cudaStream_t s) {
   const int64_t npix = (int64_t)tp.width * tp.height;
   const int64_t nseg = tp.n_lines * (int64_t)(tp.max_samples - 1);
-  k_vis_init<<<(unsigned)((npix + 255) / 256), 256, 0, s>>>(tp.vis, npix);
+  tp.ray_table = tp.ray.persp && nseg >= npix / kTubeTablePixels;
+  k_tube_init<<<dim3((unsigned)((tp.width + 63) / 64), (unsigned)((tp.height + 3) / 4)), 256, 0, s>>>(
+      tp.ray, tp.width, tp.height, tp.vis, tp.ray_table ? reinterpret_cast<float4 *>(tp.out) : nullptr);
   if (nseg > 0) {
-    // warps per line: about 512 pairs per warp and group when the lines'
-    // first groups cover the image twice, 1 for many lines, at most 256
-    const int64_t lines = tp.n_lines;
+    // warps per line: its groups spread over warps while there are fewer than
+    // 64 warps per SM, and about 512 pairs per warp and group when the lines'
+    // first groups cover the image twice, at most 256 in all
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int64_t lines = tp.n_lines, groups = (tp.max_samples - 1 + 31) / 32;
     int64_t split = (2 * npix + lines * 512 - 1) / (lines * 512);
-    split = split < 1 ? 1 : (split > 256 ? 256 : split);
-    const int64_t warps = lines * split;
-    k_tube_raster<<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(tp, (int)split);
+    split = std::min<int64_t>(std::max<int64_t>(split, 1), 256);
+    const int64_t strides = std::min<int64_t>(std::max<int64_t>(64 * (int64_t)sms / lines, 1), std::min<int64_t>(groups, 256));
+    split = (split + strides - 1) / strides;
+    const int64_t warps = lines * strides * split;
+    k_tube_raster<<<(unsigned)((warps + kTubeWarps - 1) / kTubeWarps), 32 * kTubeWarps, 0, s>>>(tp, (int)strides, (int)split);
   }
   const unsigned blocks = (unsigned)((npix + 127) / 128);
 #define LRVOL_TUBE_CASE(P_, S_) k_tube_resolve<P_, S_><<<blocks, 128, 0, s>>>(tp)

@@ -296,9 +296,10 @@ struct TubeParams {
   unsigned long long *vis; // height x width
   float *out;              // height x width x 4
   float tf_scale, tf_bias;
+  int ray_table;           // set by launch_tubes: out holds the pixels' ray directions until they are shaded
   float4 cmap[256];
 };
-cudaError_t launch_tubes(const TubeParams &tp, int degree, int storage, cudaStream_t s);
+cudaError_t launch_tubes(TubeParams tp, int degree, int storage, cudaStream_t s);
 cudaError_t launch_streamline_error(const double *ref, const int32_t *rc, int rmax, const double *app,
                                     const int32_t *ac, int amax, int64_t n, double *sums, cudaStream_t s);
 
