@@ -23,9 +23,10 @@ __device__ __forceinline__ void set_status(uint32_t *status, uint32_t code) { at
 // look-up (Alg. 1)
 // ----------------------------------------------------------------------------
 
-// Element holding the FP32 point (x, y, z), each coordinate in [0, 1] (every
-// caller clamps or checks first): head word of its block, then the tree walk.
-__device__ __forceinline__ uint32_t forest_lookup(const ForestView &f, float x, float y, float z, uint32_t *status) {
+// Head word of the block holding the FP32 point (x, y, z), each coordinate in
+// [0, 1] (every caller clamps or checks first): the block's one element, with
+// kLeaf, or the root of its tree.
+__device__ __forceinline__ uint32_t forest_head(const ForestView &f, float x, float y, float z) {
   // block index floor(p * blocks) (blocks a power of two <= 1024, so the
   // product is exact) as the low bits of 2^23 + floor by a round-down FMA; the
   // index of p = 1 falls on the table's last, repeated layer.  The three
@@ -33,18 +34,45 @@ __device__ __forceinline__ uint32_t forest_lookup(const ForestView &f, float x, 
   const uint32_t hx = __float_as_uint(__fmaf_rd(x, f.fbx, 8388608.f));
   const uint32_t hy = __float_as_uint(__fmaf_rd(y, f.fby, 8388608.f));
   const uint32_t hz = __float_as_uint(__fmaf_rd(z, f.fbz, 8388608.f));
-  uint32_t w = __ldg(f.head + (hz * f.head_sz + (hy * f.head_sy + (hx - f.head_bias))));
+  return __ldg(f.head + (hz * f.head_sz + (hy * f.head_sy + (hx - f.head_bias))));
+}
+
+// The leaf of a grid of cells (GridUnit).
+__device__ __forceinline__ uint32_t grid_cell(const float4 *grid, float x, float y, float z) {
+  const float4 gx = __ldg(grid), gy = __ldg(grid + 1), gz = __ldg(grid + 2);
+  const uint32_t cx = (x >= gx.x) + (x >= gx.y) + (x >= gx.z);
+  const uint32_t cy = (y >= gy.x) + (y >= gy.y) + (y >= gy.z);
+  const uint32_t cz = (z >= gz.x) + (z >= gz.y) + (z >= gz.z);
+  return __ldg(reinterpret_cast<const uint32_t *>(grid + 3) + cx + cy * __float_as_uint(gy.w) + cz * __float_as_uint(gz.w));
+}
+__device__ __noinline__ uint32_t grid_cell_call(const float4 *grid, float x, float y, float z) {
+  return grid_cell(grid, x, y, z);
+}
+
+// The tree walk from a head word: the element, or kNone with the status set.
+// CALL: the grid as a call, for code that inlines the walk many times.
+template <bool CALL = false>
+__device__ __forceinline__ uint32_t forest_walk(const ForestView &f, uint32_t w, float x, float y, float z,
+                                                uint32_t *status) {
   // one exit: a leaf and a word outside the tree both compare >= n_nodes < 2^31
   for (int depth = 0; w < f.n_nodes && depth < kMaxDepth; ++depth) {
     const uint4 n = __ldg(f.nodes + w);
     const float pa = n.y == 0 ? x : (n.y == 1 ? y : z);
     w = pa < __uint_as_float(n.x) ? n.z : n.w;
   }
+  const uint32_t g = w - f.n_nodes;
+  if (g < f.n_grid_units) w = CALL ? grid_cell_call(f.grids + g, x, y, z) : grid_cell(f.grids + g, x, y, z);
   if (!(w & kLeaf)) {
     set_status(status, kStatusBounds);
     return kNone;
   }
   return w & ~kLeaf;
+}
+
+// Element holding the point (Alg. 1).
+template <bool CALL = false>
+__device__ __forceinline__ uint32_t forest_lookup(const ForestView &f, float x, float y, float z, uint32_t *status) {
+  return forest_walk<CALL>(f, forest_head(f, x, y, z), x, y, z, status);
 }
 
 // ----------------------------------------------------------------------------
@@ -141,6 +169,27 @@ __device__ __forceinline__ float fma_sat(float a, float b, float c) {
   return d;
 }
 
+// ---- packed two-lane FP32 (fma.rn.f32x2 and friends; lane "lo" first) ----
+typedef unsigned long long f2;
+
+__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
+  f2 d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void f2_unpack(f2 a, float &lo, float &hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+}
+__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
+  f2 d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
+  f2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
 struct Ray {
   float o[3], d[3], tin, tout;
 };
@@ -204,7 +253,9 @@ __device__ __forceinline__ float tf_coord(const RenderParams &prm, float v) {
 // The coordinate that reads the table's extra entry: no opacity, no colour.
 constexpr float kTfNothing = 256.5f / 255.f;
 
-// The transfer function at coordinate x: colour, and log2(1 - alpha) in w.
+// The transfer function at coordinate x: colour, and log2(1 - alpha) in w.  With
+// PACKED the four interpolations are two packed operations (the same results).
+template <bool PACKED = false>
 __device__ __forceinline__ float4 tf_sample(const float4 *tfb, const float4 *tfd, float x) {
   // entry floor(255 x) without a float-int conversion (those issue on the
   // narrow XU pipe): 255 x + 2^23 rounded down is 2^23 + floor(255 x) exactly;
@@ -212,18 +263,27 @@ __device__ __forceinline__ float4 tf_sample(const float4 *tfb, const float4 *tfd
   const float r = __fmaf_rd(x, 255.f, 8388608.f);
   const int q = __float_as_int(r) - 0x4b000000;
   const float fr = __fmaf_rn(x, 255.f, __fsub_rn(8388608.f, r));
-  const float4 e0 = tfb[q], de = tfd[q];
-  const float sa = fmaf(fr, de.w, e0.w);
-  return make_float4(fmaf(fr, de.x, e0.x), fmaf(fr, de.y, e0.y), fmaf(fr, de.z, e0.z), lg2_approx(fmaxf(1.f - sa, 0.f)));
+  float4 c;
+  if constexpr (PACKED) {
+    const ulonglong2 e0 = reinterpret_cast<const ulonglong2 *>(tfb)[q], de = reinterpret_cast<const ulonglong2 *>(tfd)[q];
+    const f2 f = f2_pack(fr, fr);
+    f2_unpack(f2_fma(f, de.x, e0.x), c.x, c.y);
+    f2_unpack(f2_fma(f, de.y, e0.y), c.z, c.w);
+  } else {
+    const float4 e0 = tfb[q], de = tfd[q];
+    c = make_float4(fmaf(fr, de.x, e0.x), fmaf(fr, de.y, e0.y), fmaf(fr, de.z, e0.z), fmaf(fr, de.w, e0.w));
+  }
+  c.w = lg2_approx(fmaxf(1.f - c.w, 0.f));
+  return c;
 }
 
 // One Alg. 2 update in transmittance form (Tr = 1 - alpha_dst) for a sample of
 // TF coordinate x: w = (1 - T) Tr, C += w C_src, Tr *= T; with SHADE, C_src is
 // multiplied by the intensity sh (Sec. 4.1).
-template <bool SHADE>
+template <bool SHADE, bool PACKED = false>
 __device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, float x, float seg, float sh,
                                           const RenderParams &prm, float &C0, float &C1, float &C2, float &Tr) {
-  const float4 src = tf_sample(tfb, tfd, x);
+  const float4 src = tf_sample<PACKED>(tfb, tfd, x);
   const float T = ex2_approx(src.w * (seg * prm.inv_xi));
   const float w = SHADE ? fmaf(-Tr, T, Tr) * sh : fmaf(-Tr, T, Tr);
   C0 = fmaf(w, src.x, C0);
@@ -232,27 +292,6 @@ __device__ __forceinline__ void composite(const float4 *tfb, const float4 *tfd, 
   Tr *= T;
 }
 
-// ---- packed two-lane FP32 (fma.rn.f32x2 and friends; lane "lo" first) ----
-typedef unsigned long long f2;
-
-__device__ __forceinline__ f2 f2_pack(float lo, float hi) {
-  f2 d;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-  return d;
-}
-__device__ __forceinline__ void f2_unpack(f2 a, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
-}
-__device__ __forceinline__ f2 f2_mul(f2 a, f2 b) {
-  f2 d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
-  f2 d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
 // 256-bit read-only load (32-byte aligned address)
 __device__ __forceinline__ void ld256(const void *p, f2 &a, f2 &b, f2 &c, f2 &d) {
   asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));

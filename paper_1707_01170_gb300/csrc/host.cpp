@@ -205,6 +205,119 @@ struct TreeBuilder {
 
 };
 
+// The trees as the device walks them.  A look-up waits for every node on its
+// way, so a subtree whose splits lie on at most three planes per axis, and that
+// is at least kGridDepth levels deep, becomes a grid: its planes and the element
+// of each of its cells, two dependent reads whatever its depth.  A point is in
+// cell c of an axis if it is on the >= side of c planes, which decides every
+// split of the subtree as the walk does.
+// References while compiling: kLeaf | element; kGridRef | offset into grids;
+// else an index into nodes.
+constexpr uint32_t kGridRef = 0x40000000u;
+constexpr int kGridDepth = 3, kGridPlanes = 3;
+
+struct Compiled {
+  std::vector<Node> nodes;
+  std::vector<GridUnit> grids;   // per grid three units of planes, then its cells, four to a unit
+
+  // A subtree not yet emitted: its planes and depth (wide: more than kGridPlanes on an axis).
+  struct Sub {
+    float plane[3][kGridPlanes];
+    int n[3], depth;
+    bool wide;
+    uint32_t ref;                // in the source tree; once wide, in this one
+  };
+
+  static void add_plane(Sub &s, int a, float x) {
+    if (s.wide) return;
+    int k = 0;
+    while (k < s.n[a] && s.plane[a][k] < x) ++k;
+    if (k < s.n[a] && s.plane[a][k] == x) return;
+    if (s.n[a] == kGridPlanes) {
+      s.wide = true;
+      return;
+    }
+    for (int q = s.n[a]++; q > k; --q) s.plane[a][q] = s.plane[a][q - 1];
+    s.plane[a][k] = x;
+  }
+
+  Sub scan(const std::vector<Node> &src, uint32_t ref) {
+    Sub s{};
+    s.ref = ref;
+    if (ref & kLeaf) return s;
+    const Node &nd = src[ref];
+    Sub c[2] = {scan(src, nd.child[0]), scan(src, nd.child[1])};
+    s.wide = c[0].wide || c[1].wide;
+    s.depth = 1 + std::max(c[0].depth, c[1].depth);
+    float x;
+    std::memcpy(&x, &nd.split_bits, 4);
+    add_plane(s, (int)nd.axis, x);
+    for (const Sub &k : c)
+      for (int a = 0; a < 3; ++a)
+        for (int q = 0; q < k.n[a]; ++q) add_plane(s, a, k.plane[a][q]);
+    if (!s.wide) return s;
+    Node out = nd;
+    for (int k = 0; k < 2; ++k) out.child[k] = c[k].wide ? c[k].ref : emit(src, c[k]);
+    s.ref = (uint32_t)nodes.size();
+    nodes.push_back(out);
+    return s;
+  }
+
+  uint32_t copy(const std::vector<Node> &src, uint32_t ref) {
+    if (ref & kLeaf) return ref;
+    const uint32_t me = (uint32_t)nodes.size();
+    nodes.push_back(src[ref]);
+    const uint32_t a = copy(src, src[ref].child[0]), b = copy(src, src[ref].child[1]);
+    nodes[me].child[0] = a;
+    nodes[me].child[1] = b;
+    return me;
+  }
+
+  void fill(const std::vector<Node> &src, uint32_t ref, const Sub &s, uint32_t *cells, const int *lo, const int *hi) {
+    const int sy = s.n[0] + 1, sz = sy * (s.n[1] + 1);
+    if (ref & kLeaf) {
+      for (int z = lo[2]; z < hi[2]; ++z)
+        for (int y = lo[1]; y < hi[1]; ++y)
+          for (int x = lo[0]; x < hi[0]; ++x) cells[z * sz + y * sy + x] = ref;
+      return;
+    }
+    const Node &nd = src[ref];
+    const int a = (int)nd.axis;
+    float x;
+    std::memcpy(&x, &nd.split_bits, 4);
+    int k = 0;
+    while (s.plane[a][k] != x) ++k;
+    int mid[3] = {hi[0], hi[1], hi[2]};
+    mid[a] = k + 1;
+    fill(src, nd.child[0], s, cells, lo, mid);
+    for (int c = 0; c < 3; ++c) mid[c] = lo[c];
+    mid[a] = k + 1;
+    fill(src, nd.child[1], s, cells, mid, hi);
+  }
+
+  uint32_t emit(const std::vector<Node> &src, const Sub &s) {
+    if (s.depth < kGridDepth) return copy(src, s.ref);
+    const int dim[3] = {s.n[0] + 1, s.n[1] + 1, s.n[2] + 1}, zero[3] = {0, 0, 0};
+    const size_t at = grids.size();
+    grids.resize(at + 3 + (dim[0] * dim[1] * dim[2] + 3) / 4, GridUnit{{kLeaf, kLeaf, kLeaf, kLeaf}});
+    for (int a = 0; a < 3; ++a) {
+      for (int q = 0; q < kGridPlanes; ++q) {
+        const float x = q < s.n[a] ? s.plane[a][q] : INFINITY;
+        std::memcpy(&grids[at + a].w[q], &x, 4);
+      }
+      grids[at + a].w[3] = a == 0 ? 1 : (a == 1 ? dim[0] : dim[0] * dim[1]);
+    }
+    fill(src, s.ref, s, grids[at + 3].w, zero, dim);
+    return kGridRef | (uint32_t)at;
+  }
+
+  // The tree at `ref` of src, compiled; its new reference.
+  uint32_t add(const std::vector<Node> &src, uint32_t ref) {
+    const Sub s = scan(src, ref);
+    return s.wide ? s.ref : emit(src, s);
+  }
+};
+
 // fn(k) for k = 0 .. n - 1 on up to 16 threads, the caller's among them; false
 // if a call returned false or threw.
 template <class Fn>
@@ -232,6 +345,8 @@ bool parallel_for(int n, Fn fn) {
 
 struct ForestBuilder : TreeBuilder {
   std::vector<uint32_t> head;  // as ForestView::head
+  std::vector<GridUnit> grids;
+  int64_t n_tree_nodes = 0;    // nodes of the trees before subtrees became grids
   std::vector<int32_t> depth;  // per block
   int B[3];
 
@@ -273,7 +388,8 @@ struct ForestBuilder : TreeBuilder {
         }))
       return false;
     const int n_slabs = std::min(B[2], 64), thick = B[2] / n_slabs;   // powers of two
-    std::vector<std::vector<Node>> slab_nodes(n_slabs);
+    std::vector<Compiled> slab(n_slabs);
+    std::vector<int64_t> slab_nodes(n_slabs, 0);                      // of the trees as built
     std::vector<std::vector<int64_t>> slab_trees(n_slabs);            // blocks with a tree, as offsets into `depth`
     const size_t plane = (size_t)B[0] * B[1];
     auto at = [&](int64_t q) { return head_at((int)(q % B[0]), (int)(q / B[0] % B[1]), (int)(q / plane)); };
@@ -312,6 +428,7 @@ struct ForestBuilder : TreeBuilder {
           tb.v = v;
           tb.midpoint = midpoint;
           for (size_t k = 0; k < trees.size(); ++k) {
+            tb.nodes.clear();
             const int64_t q = trees[k];
             const int b[3] = {(int)(q % B[0]), (int)(q / B[0] % B[1]), (int)(q / plane)};
             double lo[3], hi[3];
@@ -323,29 +440,59 @@ struct ForestBuilder : TreeBuilder {
             int maxd = 0;
             const uint32_t r = tb.build(mine, lo, hi, 0, &maxd);
             if (r == kNone) return false;
-            head[at(q)] = r;
+            slab_nodes[s] += (int64_t)tb.nodes.size();
+            if (slab[s].nodes.size() + tb.nodes.size() >= kGridRef || slab[s].grids.size() >= kGridRef / 2) return false;
+            head[at(q)] = slab[s].add(tb.nodes, r);
             depth[q] = maxd;
           }
-          slab_nodes[s] = std::move(tb.nodes);
           return true;
         }))
       return false;
-    size_t total = 0;
-    for (const auto &n : slab_nodes) total += n.size();
-    if (total >= kLeaf) return false;
-    nodes.clear();
-    nodes.reserve(total);
+    // the slabs one after the other: nodes, then grids
+    size_t n_split = 0, n_units = 0;
+    n_tree_nodes = 0;
     for (int s = 0; s < n_slabs; ++s) {
-      const uint32_t base = (uint32_t)nodes.size();
-      auto shift = [&](uint32_t r) { return r & kLeaf ? r : r + base; };
-      for (Node n : slab_nodes[s]) {
+      n_split += slab[s].nodes.size();
+      n_units += slab[s].grids.size();
+      n_tree_nodes += slab_nodes[s];
+    }
+    if (n_split + n_units >= kLeaf || n_tree_nodes >= (int64_t)kLeaf) return false;
+    nodes.clear();
+    nodes.reserve(n_split);
+    grids.clear();
+    grids.reserve(n_units);
+    for (int s = 0; s < n_slabs; ++s) {
+      const uint32_t base = (uint32_t)nodes.size(), grid_base = (uint32_t)(n_split + grids.size());
+      auto shift = [&](uint32_t r) { return r & kLeaf ? r : (r & kGridRef ? (r & ~kGridRef) + grid_base : r + base); };
+      for (Node n : slab[s].nodes) {
         n.child[0] = shift(n.child[0]);
         n.child[1] = shift(n.child[1]);
         nodes.push_back(n);
       }
       for (int64_t q : slab_trees[s]) head[at(q)] = shift(head[at(q)]);
+      grids.insert(grids.end(), slab[s].grids.begin(), slab[s].grids.end());
+      slab[s] = Compiled();
     }
     return true;
+  }
+
+  // region()'s trees as layers() leaves its own (too large a forest stays as
+  // built; blocks without an element, kNone, read as leaves here).
+  void compile() {
+    n_tree_nodes = (int64_t)nodes.size();
+    Compiled c;
+    std::vector<uint32_t> refs(head.size());
+    for (size_t q = 0; q < head.size(); ++q) {
+      if (c.nodes.size() + nodes.size() >= kGridRef || c.grids.size() >= kGridRef / 2) return;
+      refs[q] = head[q] & kLeaf ? head[q] : c.add(nodes, head[q]);
+    }
+    const uint32_t base = (uint32_t)c.nodes.size();
+    auto shift = [&](uint32_t r) { return !(r & kLeaf) && (r & kGridRef) ? (r & ~kGridRef) + base : r; };
+    for (Node &n : c.nodes)
+      for (uint32_t &r : n.child) r = shift(r);
+    for (size_t q = 0; q < head.size(); ++q) head[q] = shift(refs[q]);
+    nodes = std::move(c.nodes);
+    grids = std::move(c.grids);
   }
 
   // Recursive region subdivision over blocks [b0, b1) with the elements meeting it.
@@ -433,6 +580,8 @@ ForestView forest_view(const lrvol_s *v) {
   f.head = v->d_head;
   f.nodes = v->d_nodes;
   f.n_nodes = (uint32_t)v->n_nodes;
+  f.grids = reinterpret_cast<const float4 *>(v->d_grids);
+  f.n_grid_units = (uint32_t)v->n_grid_units;
   f.head_sy = (uint32_t)v->blocks[0] + 1;
   f.head_sz = f.head_sy * ((uint32_t)v->blocks[1] + 1);
   f.head_bias = 0x4b000000u * (1u + f.head_sy + f.head_sz);
@@ -652,6 +801,7 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
         return fail(LRVOL_ERR_UNSUPPORTED, "midpoint splits do not resolve this mesh (faces at non-dyadic coordinates)");
       return fail(LRVOL_ERR_ARG, "elements do not form a box partition of [0,1]^3");
     }
+    fb.compile();
   }
   fb.pad_head();
   for (uint32_t h : fb.head)
@@ -672,14 +822,20 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   // the handle has none (a failed host build above left the previous one)
   v->have_accel = false;
   if ((rc = dev_alloc(v, &v->d_head, fb.head.size(), "alloc forest head")) ||
-      (rc = dev_alloc(v, &v->d_nodes, fb.nodes.size(), "alloc forest nodes")))
+      (rc = dev_alloc(v, &v->d_nodes, fb.nodes.size(), "alloc forest nodes")) ||
+      (rc = dev_alloc(v, &v->d_grids, fb.grids.size(), "alloc forest grids")))
     return rc;
   CU(cudaMemcpyAsync(v->d_head, fb.head.data(), sizeof(uint32_t) * fb.head.size(), cudaMemcpyHostToDevice, st), "upload head");
   if (!fb.nodes.empty())
     CU(cudaMemcpyAsync(v->d_nodes, fb.nodes.data(), sizeof(Node) * fb.nodes.size(), cudaMemcpyHostToDevice, st),
        "upload nodes");
+  if (!fb.grids.empty())
+    CU(cudaMemcpyAsync(v->d_grids, fb.grids.data(), sizeof(GridUnit) * fb.grids.size(), cudaMemcpyHostToDevice, st),
+       "upload grids");
   CU(cudaStreamSynchronize(st), "build_accel sync");  // host vectors go out of scope
+  v->n_tree_nodes = fb.n_tree_nodes;
   v->n_nodes = (int64_t)fb.nodes.size();
+  v->n_grid_units = (int64_t)fb.grids.size();
   for (int a = 0; a < 3; ++a) v->blocks[a] = blocks[a];
   v->depth_min = dmin;
   v->depth_max = dmax;
@@ -1053,7 +1209,7 @@ int lrvol_stats(lrvol_t v, lrvol_stats_t *out) {
   std::memset(out, 0, sizeof(*out));
   out->n_elem = v->n_elem;
   out->n_basis = v->n_basis;
-  out->n_nodes = v->n_nodes;
+  out->n_nodes = v->n_tree_nodes;
   for (int a = 0; a < 3; ++a) out->blocks[a] = v->blocks[a];
   out->depth_min = v->depth_min;
   out->depth_max = v->depth_max;
@@ -1078,7 +1234,7 @@ void lrvol_destroy(lrvol_t v) {
   if (!v) return;
   cudaDeviceSynchronize();
   void *ptrs[] = {v->d_box,   v->d_knots, v->d_coef,  v->d_weight, v->d_inc_ptr,  v->d_inc_idx, v->d_bez64,
-                  v->d_bez,   v->d_bezc,  v->d_elem,  v->d_head,  v->d_nodes, v->d_counters, v->d_status,
+                  v->d_bez,   v->d_bezc,  v->d_elem,  v->d_head,  v->d_nodes, v->d_grids, v->d_counters, v->d_status,
                   v->d_range};
   for (void *p : ptrs)
     if (p) cudaFree(p);

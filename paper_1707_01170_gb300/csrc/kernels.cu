@@ -1292,7 +1292,7 @@ __device__ __forceinline__ void trace_line_group(const SLParams &sp, const doubl
     const float above = max3_nan(px - rb.x, py - rb.y, pz - rb.z);
     if (below >= 0.f && above < 0.f) return true;
     if (!in_cube(px, py, pz)) return false;
-    const uint32_t e = forest_lookup(sp.forest, px, py, pz, sp.status);
+    const uint32_t e = forest_lookup<true>(sp.forest, px, py, pz, sp.status);
     if (e >= (uint32_t)sp.n_elem) {   // kNone included
       set_status(sp.status, kStatusBounds);
       return false;

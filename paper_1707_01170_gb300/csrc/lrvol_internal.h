@@ -52,12 +52,21 @@ struct Node {
   uint32_t child[2];
 };
 
+// A grid of cells that stands for a subtree: units 0..2 hold an axis' planes
+// (three, +inf where there are fewer) and its cells' stride, the rest the cells'
+// elements (kLeaf | id), x fastest.
+struct GridUnit {
+  uint32_t w[4];
+};
+
 struct ForestView {
   // One word per block, x fastest, and each axis' last layer once more (what
   // p = 1 finds without a clamp): (blocks[0]+1) x (blocks[1]+1) x (blocks[2]+1).
   const uint32_t *head;
   const uint4 *nodes;
-  uint32_t n_nodes;              // < 2^31
+  uint32_t n_nodes;              // < 2^31; references from n_nodes on are units of grids
+  const float4 *grids;           // GridUnit
+  uint32_t n_grid_units;
   uint32_t head_sy, head_sz;     // strides of y and z
   uint32_t head_bias;            // 0x4b000000 (1 + head_sy + head_sz) mod 2^32, see forest_lookup
   float fbx, fby, fbz;           // block counts (powers of two)
@@ -167,7 +176,9 @@ struct lrvol_s {
   // forest
   uint32_t *d_head = nullptr;
   uint4 *d_nodes = nullptr;
-  int64_t n_nodes = 0;
+  lrvol::GridUnit *d_grids = nullptr;
+  int64_t n_nodes = 0, n_grid_units = 0;
+  int64_t n_tree_nodes = 0;   // of the trees as built, before subtrees became grids
   int blocks[3] = {0, 0, 0};
   int depth_min = 0, depth_max = 0;
   double depth_mean = 0, depth_var = 0;
@@ -212,6 +223,10 @@ cudaError_t launch_lookup(const lrvol_s *v, const float *pts, int64_t n, uint32_
 cudaError_t launch_eval_grad(const lrvol_s *v, const float *pts, int64_t n, float *out, cudaStream_t s);
 cudaError_t launch_eval(const lrvol_s *v, const float *pts, int64_t n, float *out, cudaStream_t s);
 cudaError_t launch_render(const RenderParams &prm, int degree, int field, int storage, cudaStream_t s);
+// f: 0 scalar, 1 |v|, 2 component, 3 shaded scalar
+cudaError_t launch_render_f32(const RenderParams &prm, int degree, int f, bool trace, cudaStream_t s);
+cudaError_t launch_render_f16(const RenderParams &prm, int degree, int f, bool trace, cudaStream_t s);
+cudaError_t launch_render_bf16(const RenderParams &prm, int degree, int f, bool trace, cudaStream_t s);
 cudaError_t launch_render_trace(const RenderParams &prm, int degree, int field, int storage, cudaStream_t s);
 cudaError_t launch_render_static(RenderParams prm, int degree, int field, int storage, cudaStream_t s,
                                  unsigned long long *counters_out);
