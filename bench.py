@@ -233,7 +233,7 @@ def cpu_baseline(vol, tf, cam, step, samples_per_frame=None, target_s: float = 1
     return out
 
 
-RENDER_SOURCES = ("render.cu", "device_common.cuh", "lrvol_internal.h")
+RENDER_SOURCES = ("render.cu", "render_kernel.cuh", "device_common.cuh", "lrvol_internal.h")
 
 
 def render_source_hash(root: str | None = None) -> str:

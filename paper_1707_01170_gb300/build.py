@@ -1,5 +1,5 @@
 """Build liblrvol.so in place with nvcc for sm_103a (one -gencode, translation
-units compiled in parallel).  No CMake; a few seconds on the build host."""
+units compiled in parallel).  No CMake; under a minute on the build host."""
 from __future__ import annotations
 
 import os
@@ -19,8 +19,9 @@ FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-I", INCLUDE, "-I", CSRC,
          # host code: no FMA contraction (the camera constants are FP64 algebra
          # with a fixed order of operations, shared by the ray definition)
          "-Xcompiler", "-fPIC,-ffp-contract=off,-fno-fast-math"]
-SOURCES = ["kernels.cu", "render.cu", "train.cu", "points.cu", "setup.cu", "host.cpp", "server.cpp"]
-HEADERS = ["lrvol_internal.h", "device_common.cuh"]
+SOURCES = ["kernels.cu", "render.cu", "render_f32.cu", "render_f16.cu", "render_bf16.cu", "train.cu", "points.cu",
+           "setup.cu", "host.cpp", "server.cpp"]
+HEADERS = ["lrvol_internal.h", "device_common.cuh", "render_kernel.cuh"]
 
 
 def nvcc() -> str:

@@ -1,277 +1,19 @@
-// liblrvol render kernel for sm_103a (Sec. 4, Alg. 2, Eq. 4).
-//
-//   k_render<P, FIELD, STORE, FIXED, TRACE>
-//       per-pixel ray casting with element reuse, Eq. 4 (or fixed, or learned)
-//       steps, transfer function and Alg. 2 compositing, and gradient shading
-//       (Sec. 4.1).  TRACE = false is the product kernel; TRACE = true is the
-//       same template over a pixel list, writing every sample it composites.
-//   launch_render, launch_render_trace, launch_render_static
-//       the launches of lrvol_render, lrvol_render_trace and
-//       lrvol_render_noalloc (the last with the library's static scratch).
+// liblrvol renders: the launches of lrvol_render, lrvol_render_trace and
+// lrvol_render_noalloc (the last with the library's static scratch).  The kernel
+// is in render_kernel.cuh.
 #include <mutex>
 
-#include "device_common.cuh"
-
-static_assert(LRVOL_BAND_ROWS == 8, "a CTA renders 8 rows: one interleaved band");
+#include "lrvol_internal.h"
 
 namespace lrvol {
 namespace {
 
-// One CTA of 4 warps renders a 16x8-pixel tile, so the warps sharing an SM's
-// L1 march through neighbouring elements; one lane traces one ray.  A warp
-// covers an 8x4 patch for scalar fields and a 4x8 patch for 3-vector fields
-// (the shapes that measured fastest for each).  The element-change branch (look-up and block loads) is kept
-// minimal: a warp runs it whenever any of its lanes changes element, which
-// happens almost every iteration.
-//
-// In the sample loop the Alg. 2 update of sample k is issued together with
-// the evaluation of sample k+1 (they are independent), so the scheduler can
-// overlap their latencies; a ray that terminates after sample k discards the
-// already evaluated sample k+1.  Sample "-1" is a transfer-function entry of
-// zeros, so the loop has one path.
-//
-// A warp's iteration waits about as long for its instructions as for the loads
-// of an element change, so both the sample's and the change's instructions
-// count: clamps fused into the multiply-add (.sat), no branch besides the
-// element change, block sizes and step rule known to the compiler, a head
-// table that needs no clamped index.  182 instructions an iteration became
-// about 160: the 1080p Eq. 4 frame of a tricubic FP32 volume 2.51 -> 2.33 ms,
-// a 256 x 256 fixed-step frame 145 -> 125 us, the 4K learned FP16 frame 4.77 ->
-// 4.33 ms, 3-vector speed with FP16 blocks 0.80 -> 0.73 ms.
-//
-// TRACE (a compile-time flag; false in every product launch, where the trace
-// code compiles out) runs the same march for a list of pixels, one thread per
-// listed pixel, and also writes each sample's (t, element id, field value,
-// segment length), the composited sample count and the pixel's RGBA.  It is
-// the parity hook that compares this kernel's own samples with the oracle.
-//
-// FIELD 3 renders a scalar volume with gradient shading (Sec. 4.1): each
-// sample also evaluates the block's gradient, and C_src is scaled by
-// I = max(0.4, |l . g| / max(|g|, eps)).
-// CTAs per SM the register budget allows: the tricubic FP32/BF16 block takes
-// 64 registers a lane (4 CTAs of 128 threads), 16-bit pairs of an FP16 block
-// 32 (5 CTAs); the triquadratic 3-vector FP16 block (42 registers instead of
-// 83) also fits 5.  The shaded tricubic kernel keeps the gradient's partial
-// sums too: at 4 CTAs it spills 88 bytes and still beats 3 CTAs without
-// spills by 5 % (measured); forcing 5 CTAs on the FP32 kernels spills
-// inside the sample loop and costs 37-51 %.
-template <int P, int FIELD, int STORE>
-constexpr int render_min_ctas() {
-  if (STORE == LRVOL_STORE_F16) {
-    if (P == 3 && FIELD == 0) return 5;
-    if (P == 2 && (FIELD == 1 || FIELD == 2)) return 5;
-  }
-  return 4;
-}
-
-template <int P, int FIELD, int STORE, bool FIXED, bool TRACE>
-__global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_render(const __grid_constant__ RenderParams prm) {
-  constexpr int N = P + 1;
-  constexpr bool SHADE = FIELD == 3;
-  constexpr int BF = SHADE ? 0 : FIELD;
-  __shared__ float4 tfb[kTfEntries], tfd[kTfEntries];
-  load_tf(prm, tfb, tfd);
-  __syncthreads();
-
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int i, j;
-  bool active;
-  int64_t g = 0;               // TRACE: position in the pixel list
-  uint32_t cur_e = kNone;      // TRACE: element of the current sample
-  if constexpr (TRACE) {
-    g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    active = g < prm.trace_n;
-    i = active ? __ldg(prm.trace_pix + 2 * g) : 0;
-    j = active ? __ldg(prm.trace_pix + 2 * g + 1) : 0;
-    if (active && (i < 0 || i >= prm.width || j < 0 || j >= prm.height)) {
-      set_status(prm.status, kStatusBounds);
-      prm.trace_count[g] = 0;
-      prm.trace_rgba[g] = make_float4(0.f, 0.f, 0.f, 0.f);
-      active = false;
-    }
-  } else {
-    if constexpr (BF == 1 || BF == 2) {   // 3-vector fields: four 4x8 patches side by side
-      i = blockIdx.x * 16 + warp * 4 + (lane & 3);
-      j = prm.row_begin + (blockIdx.y * prm.band_count + prm.band_index) * 8 + (lane >> 2);
-    } else {                              // scalar fields: 2x2 patches of 8x4
-      i = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
-      j = prm.row_begin + (blockIdx.y * prm.band_count + prm.band_index) * 8 + (warp >> 1) * 4 + (lane >> 3);
-    }
-    active = i < prm.width && j < prm.row_end;
-  }
-  unsigned nsamp = 0, nlook = 0, nhit = 0;
-
-  Ray ray;
-  if (active) {
-    float C0 = 0.f, C1 = 0.f, C2 = 0.f, Tr = 1.f;
-    if (make_ray(prm.ray, i, j, ray) &&
-        (prm.trim == nullptr || trim_cut(__ldg(prm.trim + (int64_t)j * prm.width + i), ray.tin, ray.tout))) {
-      ++nhit;
-      const float tr_stop = 1.f - prm.alpha_stop;
-      float4 ra = make_float4(0.f, 0.f, 0.f, 0.f), rb = ra, rc = ra, rd = ra;
-      float dsv = 0.f;       // step inside the current element (Eq. 4, or Eq. 4 x learned multiplier)
-      Block<P, BF, STORE> blk;
-      float t = ray.tin + 0.f;   // not -0
-      float kf = 0.f;        // FIXED: k + 1 (exact up to kMaxSamplesPerRay)
-      int k = 0;             // samples evaluated; sample k - 1 is not yet composited
-      // sample k - 1: TF coordinate, segment, shading; at k = 0 a sample of no opacity
-      float pcoord = kTfNothing, pseg = 0.f, psh = 1.f;
-      float lx = 0.f, ly = 0.f, lz = 0.f;   // towards the light (shading)
-      if constexpr (SHADE) {
-        lx = prm.light_set ? prm.light[0] : -ray.d[0];
-        ly = prm.light_set ? prm.light[1] : -ray.d[1];
-        lz = prm.light_set ? prm.light[2] : -ray.d[2];
-      }
-      bool stopped = false;  // opaque: sample k is not composited
-      do {
-        const float px = fma_sat(t, ray.d[0], ray.o[0]);
-        const float py = fma_sat(t, ray.d[1], ray.o[1]);
-        const float pz = fma_sat(t, ray.d[2], ray.o[2]);
-        const bool inside = px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z;
-        if (!inside) {
-          uint32_t cur = forest_lookup(prm.forest, px, py, pz, prm.status);
-          if (cur >= (uint32_t)prm.n_elem) {   // kNone included: the ray ends, its pixel means nothing
-            set_status(prm.status, kStatusBounds);
-            ray.tout = 0.f;
-            cur = 0;
-          }
-          ++nlook;
-          if constexpr (TRACE) cur_e = cur;
-          load_record(prm.elem + cur, ra, rb, rc, rd);
-          if constexpr (!FIXED)
-            dsv = prm.mode == LRVOL_STEP_LEARNED ? __fmul_rn(ra.w, __ldg(prm.mult + cur)) : ra.w;
-          if constexpr (BF == 2)
-            blk.load(prm.bezc + (int64_t)cur * blk.BYTES, prm.comp);
-          else
-            blk.load(prm.bez + (int64_t)cur * blk.BYTES, 0);
-        }
-        float tn;
-        if constexpr (FIXED) {
-          kf += 1.f;
-          tn = __fmaf_rn(kf, prm.h, ray.tin);
-        } else {
-          tn = __fadd_rn(t, dsv);
-        }
-        // the next float where a step does not advance (t >= 0, so its bits order like it)
-        tn = tn > t ? tn : __int_as_float(__float_as_int(t) + 1);
-        const float seg = __fsub_rn(fminf(tn, ray.tout), t);
-        // evaluate sample k ...
-        float bx[N], by[N], bz[N];
-        const float ux = local_u(px, ra.x, rc.x, rd.x);
-        const float uy = local_u(py, ra.y, rc.y, rd.y);
-        const float uz = local_u(pz, ra.z, rc.z, rd.z);
-        monomials<P>(ux, bx);
-        monomials<P>(uy, by);
-        monomials<P>(uz, bz);
-        float v, sh = 1.f;
-        if constexpr (SHADE) {
-          float dx[N], dy[N], dz[N], gu, gv, gw;
-          dmonomials<P>(ux, dx);
-          dmonomials<P>(uy, dy);
-          dmonomials<P>(uz, dz);
-          v = blk.eval_grad(bx, by, bz, dx, dy, dz, gu, gv, gw);
-          const float gx = gu * rd.x, gy = gv * rd.y, gz = gw * rd.z;   // world gradient: d/dx = iw d/du
-          const float gl = fmaf(gx, lx, fmaf(gy, ly, gz * lz));
-          const float gn = fmaxf(sqrtf(fmaf(gx, gx, fmaf(gy, gy, gz * gz))), prm.grad_eps);
-          sh = fmaxf(0.4f, fabsf(gl) / gn);
-        } else {
-          v = blk.eval(bx, by, bz);
-        }
-        if constexpr (TRACE) {
-          if (k < prm.trace_max) prm.trace_rec[g * prm.trace_max + k] = make_float4(t, __uint_as_float(cur_e), v, seg);
-        }
-        // ... while compositing sample k-1
-        composite<SHADE>(tfb, tfd, pcoord, pseg, psh, prm, C0, C1, C2, Tr);
-        stopped = Tr <= tr_stop && k > 0;
-        pcoord = tf_coord(prm, v);
-        psh = sh;
-        pseg = seg;
-        t = tn;
-        ++k;
-      } while (!stopped && t < ray.tout && k < kMaxSamplesPerRay);
-      if (stopped || k >= kMaxSamplesPerRay) {
-        if (!stopped) set_status(prm.status, kStatusTimeout);
-        nsamp = k - 1;
-      } else {
-        composite<SHADE>(tfb, tfd, pcoord, pseg, psh, prm, C0, C1, C2, Tr);
-        nsamp = k;
-      }
-    }
-    if constexpr (TRACE) {
-      prm.trace_rgba[g] = make_float4(C0, C1, C2, 1.f - Tr);
-      prm.trace_count[g] = (int32_t)nsamp;
-    } else {
-      reinterpret_cast<float4 *>(prm.out)[(int64_t)j * prm.width + i] = make_float4(C0, C1, C2, 1.f - Tr);
-    }
-  }
-  // per-warp counters
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    nsamp += __shfl_down_sync(0xffffffffu, nsamp, o);
-    nlook += __shfl_down_sync(0xffffffffu, nlook, o);
-    nhit += __shfl_down_sync(0xffffffffu, nhit, o);
-  }
-  if (lane == 0) {
-    atomicAdd(prm.counters + kCntSamples, (unsigned long long)nsamp);
-    atomicAdd(prm.counters + kCntLookups, (unsigned long long)nlook);
-    atomicAdd(prm.counters + kCntRays, (unsigned long long)nhit);
-  }
-}
-
-template <int P, int FIELD, int STORE, bool FIXED, bool TRACE>
-cudaError_t launch_render_f(const RenderParams &prm, cudaStream_t s) {
-  if constexpr (TRACE) {
-    k_render<P, FIELD, STORE, FIXED, true><<<(unsigned)((prm.trace_n + 127) / 128), 128, 0, s>>>(prm);
-  } else {
-    // this call's bands: band_index, band_index + band_count, ... of the 8-row bands
-    const int n_bands = (prm.row_end - prm.row_begin + 7) / 8;
-    const int mine = (n_bands - prm.band_index + prm.band_count - 1) / prm.band_count;
-    const dim3 grid((unsigned)((prm.width + 15) / 16), (unsigned)mine);
-    k_render<P, FIELD, STORE, FIXED, false><<<grid, 128, 0, s>>>(prm);
-  }
-  return cudaGetLastError();
-}
-
-// Fixed steps have kernels of their own: which step rule a frame takes is the
-// same for every sample, and a test of it costs a sample two instructions and
-// the registers of both rules.
-template <int P, int FIELD, int STORE, bool TRACE>
-cudaError_t launch_render_t(const RenderParams &prm, cudaStream_t s) {
-  if (prm.mode == LRVOL_STEP_FIXED) return launch_render_f<P, FIELD, STORE, true, TRACE>(prm, s);
-  return launch_render_f<P, FIELD, STORE, false, TRACE>(prm, s);
-}
-
-template <int STORE, bool TRACE>
-cudaError_t launch_render_s(const RenderParams &prm, int degree, int f, cudaStream_t s) {
-  if (f == 3) {  // scalar with gradient shading
-    switch (degree) {
-      case 1: return launch_render_t<1, 3, STORE, TRACE>(prm, s);
-      case 2: return launch_render_t<2, 3, STORE, TRACE>(prm, s);
-      case 3: return launch_render_t<3, 3, STORE, TRACE>(prm, s);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  switch (degree * 3 + f) {
-    case 3: return launch_render_t<1, 0, STORE, TRACE>(prm, s);
-    case 4: return launch_render_t<1, 1, STORE, TRACE>(prm, s);
-    case 5: return launch_render_t<1, 2, STORE, TRACE>(prm, s);
-    case 6: return launch_render_t<2, 0, STORE, TRACE>(prm, s);
-    case 7: return launch_render_t<2, 1, STORE, TRACE>(prm, s);
-    case 8: return launch_render_t<2, 2, STORE, TRACE>(prm, s);
-    case 9: return launch_render_t<3, 0, STORE, TRACE>(prm, s);
-    case 10: return launch_render_t<3, 1, STORE, TRACE>(prm, s);
-    case 11: return launch_render_t<3, 2, STORE, TRACE>(prm, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-template <bool TRACE>
-cudaError_t launch_render_any(const RenderParams &prm, int degree, int field, int storage, cudaStream_t s) {
+cudaError_t launch_render_any(const RenderParams &prm, int degree, int field, int storage, bool trace, cudaStream_t s) {
   const int f = field == kFieldShaded ? 3 : (field == LRVOL_FIELD_MAGNITUDE ? 1 : (field == LRVOL_FIELD_COMPONENT ? 2 : 0));
   switch (storage) {
-    case LRVOL_STORE_F32: return launch_render_s<LRVOL_STORE_F32, TRACE>(prm, degree, f, s);
-    case LRVOL_STORE_F16: return launch_render_s<LRVOL_STORE_F16, TRACE>(prm, degree, f, s);
-    case LRVOL_STORE_BF16: return launch_render_s<LRVOL_STORE_BF16, TRACE>(prm, degree, f, s);
+    case LRVOL_STORE_F32: return launch_render_f32(prm, degree, f, trace, s);
+    case LRVOL_STORE_F16: return launch_render_f16(prm, degree, f, trace, s);
+    case LRVOL_STORE_BF16: return launch_render_bf16(prm, degree, f, trace, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -279,14 +21,14 @@ cudaError_t launch_render_any(const RenderParams &prm, int degree, int field, in
 }  // namespace
 
 cudaError_t launch_render(const RenderParams &prm, int degree, int field, int storage, cudaStream_t s) {
-  return launch_render_any<false>(prm, degree, field, storage, s);
+  return launch_render_any(prm, degree, field, storage, false, s);
 }
 
 // The same kernel template with the trace compiled in, over the pixel list in
 // prm.trace_pix (prm.trace_n entries).
 cudaError_t launch_render_trace(const RenderParams &prm, int degree, int field, int storage, cudaStream_t s) {
   if (prm.trace_n == 0) return cudaSuccess;
-  return launch_render_any<true>(prm, degree, field, storage, s);
+  return launch_render_any(prm, degree, field, storage, true, s);
 }
 
 // ----------------------------------------------------------------------------

@@ -1,0 +1,11 @@
+// k_render for BF16 blocks.
+#include "render_kernel.cuh"
+
+namespace lrvol {
+
+cudaError_t launch_render_bf16(const RenderParams &prm, int degree, int f, bool trace, cudaStream_t s) {
+  return trace ? launch_render_s<LRVOL_STORE_BF16, true>(prm, degree, f, s)
+               : launch_render_s<LRVOL_STORE_BF16, false>(prm, degree, f, s);
+}
+
+}  // namespace lrvol
