@@ -234,35 +234,38 @@ __device__ __forceinline__ bool make_ray(const RayConsts &K, int i, int j, Ray &
   return hit && tin < tout;
 }
 
-// The TF in shared memory: entry i and the difference to entry i + 1 (0 at the
-// last), and entry 256 of zeros (kTfNothing).
+// The TF in shared memory: entry i and the difference to entry i + 1; entry 255 is
+// what 254 and its difference give, with no difference (x = 255 needs no clamped
+// index); entry 256 is zeros (kTfNothing).
 constexpr int kTfEntries = 257;
 __device__ __forceinline__ void load_tf(const RenderParams &prm, float4 *tfb, float4 *tfd) {
   for (int q = threadIdx.x; q < 256; q += blockDim.x) {
-    const float4 e0 = prm.tf[q], e1 = prm.tf[q < 255 ? q + 1 : 255];
-    tfb[q] = e0;
-    tfd[q] = make_float4(e1.x - e0.x, e1.y - e0.y, e1.z - e0.z, e1.w - e0.w);
+    const float4 e0 = prm.tf[min(q, 254)], e1 = prm.tf[min(q, 254) + 1];
+    const float4 de = make_float4(e1.x - e0.x, e1.y - e0.y, e1.z - e0.z, e1.w - e0.w);
+    tfb[q] = q < 255 ? e0 : make_float4(e0.x + de.x, e0.y + de.y, e0.z + de.z, e0.w + de.w);
+    tfd[q] = q < 255 ? de : make_float4(0.f, 0.f, 0.f, 0.f);
   }
   if (threadIdx.x == 0) tfb[256] = tfd[256] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// TF coordinate of a field value, in [0, 1].
+// TF coordinate of a field value, in entries: [0, 255].  (In [0, 1] the clamp is
+// free, but its scale is rounded where 255 / range often is not: with it one to
+// seven rays of 65,536 ended a sample earlier or later.)
 __device__ __forceinline__ float tf_coord(const RenderParams &prm, float v) {
-  return fma_sat(v, prm.tf_scale, prm.tf_bias);
+  return fminf(fmaxf(fmaf(v, prm.tf_scale, prm.tf_bias), 0.f), 255.f);
 }
 // The coordinate that reads the table's extra entry: no opacity, no colour.
-constexpr float kTfNothing = 256.5f / 255.f;
+constexpr float kTfNothing = 256.5f;
 
 // The transfer function at coordinate x: colour, and log2(1 - alpha) in w.  With
 // PACKED the four interpolations are two packed operations (the same results).
 template <bool PACKED = false>
 __device__ __forceinline__ float4 tf_sample(const float4 *tfb, const float4 *tfd, float x) {
-  // entry floor(255 x) without a float-int conversion (those issue on the
-  // narrow XU pipe): 255 x + 2^23 rounded down is 2^23 + floor(255 x) exactly;
-  // x = 1 reads entry 255, whose difference is 0
-  const float r = __fmaf_rd(x, 255.f, 8388608.f);
+  // entry floor(x) without a float-int conversion (those issue on the narrow XU
+  // pipe): x + 2^23 rounded down is 2^23 + floor(x) exactly
+  const float r = __fadd_rd(x, 8388608.f);
   const int q = __float_as_int(r) - 0x4b000000;
-  const float fr = __fmaf_rn(x, 255.f, __fsub_rn(8388608.f, r));
+  const float fr = __fsub_rn(x, __fsub_rn(r, 8388608.f));
   float4 c;
   if constexpr (PACKED) {
     const ulonglong2 e0 = reinterpret_cast<const ulonglong2 *>(tfb)[q], de = reinterpret_cast<const ulonglong2 *>(tfd)[q];

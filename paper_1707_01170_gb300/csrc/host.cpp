@@ -653,8 +653,8 @@ int prepare_render(const lrvol_s *v, const lrvol_camera *cam, const lrvol_tf *tf
   prm->h = (float)step->h;
   prm->inv_xi = (float)(1.0 / step->xi);
   prm->alpha_stop = (float)step->alpha_stop;
-  prm->tf_scale = (float)(1.0 / (tf->vmax - tf->vmin));
-  prm->tf_bias = (float)(-tf->vmin / (tf->vmax - tf->vmin));
+  prm->tf_scale = (float)(255.0 / (tf->vmax - tf->vmin));
+  prm->tf_bias = (float)(-tf->vmin * 255.0 / (tf->vmax - tf->vmin));
   for (int q = 0; q < 256; ++q) prm->tf[q] = make_float4(tf->rgba[q][0], tf->rgba[q][1], tf->rgba[q][2], tf->rgba[q][3]);
   prm->trim = reinterpret_cast<const float2 *>(step->trim);
   if (step->shading == LRVOL_SHADE_GRADIENT) {
@@ -1064,8 +1064,8 @@ int lrvol_labels(lrvol_t v, const lrvol_camera *cam, const lrvol_tf *tf, const l
   prm.mode = LRVOL_STEP_HEURISTIC;
   prm.inv_xi = (float)(1.0 / step->xi);
   prm.alpha_stop = (float)step->alpha_stop;
-  prm.tf_scale = (float)(1.0 / (tf->vmax - tf->vmin));
-  prm.tf_bias = (float)(-tf->vmin / (tf->vmax - tf->vmin));
+  prm.tf_scale = (float)(255.0 / (tf->vmax - tf->vmin));
+  prm.tf_bias = (float)(-tf->vmin * 255.0 / (tf->vmax - tf->vmin));
   prm.counters = v->d_counters;
   prm.status = v->d_status;
   for (int q = 0; q < 256; ++q) prm.tf[q] = make_float4(tf->rgba[q][0], tf->rgba[q][1], tf->rgba[q][2], tf->rgba[q][3]);

@@ -130,7 +130,7 @@ struct RenderParams {
   int mode;               // LRVOL_STEP_*
   const float *mult;      // LEARNED: per-element step multipliers
   float h, inv_xi, alpha_stop;
-  float tf_scale, tf_bias; // x = v * tf_scale + tf_bias, clamped to [0, 1]
+  float tf_scale, tf_bias; // x = v * tf_scale + tf_bias, clamped to [0, 255]
   const float2 *trim;     // NULL or per pixel (t_front, t_back), row major over the full image
   int light_set;          // shading: 1 = light[] (unit), 0 = towards the eye along the ray
   float light[3];
