@@ -1,7 +1,7 @@
 // liblrvol render kernel for sm_103a (Sec. 4, Alg. 2, Eq. 4), compiled once per
 // block storage (render_f32.cu, render_f16.cu, render_bf16.cu).
 //
-//   k_render<P, FIELD, STORE, FIXED, TREES, TRACE>
+//   k_render<P, FIELD, STORE, FIXED, TREES, PAIR, TRACE>
 //       per-pixel ray casting with element reuse, Eq. 4 (or fixed, or learned)
 //       steps, transfer function and Alg. 2 compositing, and gradient shading
 //       (Sec. 4.1).  TRACE = false is the product kernel; TRACE = true is the
@@ -27,6 +27,11 @@ namespace {
 // its head word: the two are independent, so their latencies overlap.  A ray
 // that terminates after sample k discards the sample k+1 evaluated with it.
 // Sample "-1" is a transfer-function entry of zeros, so the loop has one path.
+//
+// With PAIR a pass of the loop also evaluates the ray's next sample and keeps it
+// where it lies in the box of the pass' element: the wait for an element's loads,
+// and their way through L1, then comes once for two samples.  The samples, their
+// order and their arithmetic are those of one a pass.
 //
 // A warp's iteration waits about as long for its instructions as for the loads
 // of an element change, so both the sample's and the change's instructions
@@ -64,8 +69,9 @@ constexpr int render_min_ctas() {
   return 4;
 }
 
-template <int P, int FIELD, int STORE, bool FIXED, bool TREES, bool TRACE>
+template <int P, int FIELD, int STORE, bool FIXED, bool TREES, bool PAIR, bool TRACE>
 __global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_render(const __grid_constant__ RenderParams prm) {
+  static_assert(!(PAIR && TRACE), "the traced march takes one sample a pass");
   constexpr int N = P + 1;
   constexpr bool SHADE = FIELD == 3;
   // packed colours pay where the blocks are FP32 (1080p Eq. 4 frame 2.81 -> 2.75
@@ -116,9 +122,11 @@ __global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_r
       Block<P, BF, STORE> blk;
       float t = ray.tin + 0.f;   // not -0
       float kf = 0.f;        // FIXED: k + 1 (exact up to kMaxSamplesPerRay)
-      int k = 0;             // samples evaluated; sample k - 1 is not yet composited
-      // sample k - 1: TF coordinate, segment, shading; at k = 0 a sample of no opacity
+      int k = 0;             // samples evaluated; the last pass' are not yet composited
+      int pending = 0;       // how many those are
+      // their TF coordinates, segments, shading; kTfNothing: a sample of no opacity
       float pcoord = kTfNothing, pseg = 0.f, psh = 1.f;
+      float qcoord = kTfNothing, qseg = 0.f, qsh = 1.f;
       float lx = 0.f, ly = 0.f, lz = 0.f;   // towards the light (shading)
       if constexpr (SHADE) {
         lx = prm.light_set ? prm.light[0] : -ray.d[0];
@@ -142,6 +150,13 @@ __global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_r
           head = forest_head(prm.forest, px, py, pz);
         composite<SHADE, PACKED>(tfb, tfd, pcoord, pseg, psh, prm, C0, C1, C2, Tr);
         stopped = Tr <= tr_stop && k > 0;
+        bool first = false;   // stopped at the first of two
+        if constexpr (PAIR) {
+          first = stopped && pending == 2;
+          composite<SHADE, PACKED>(tfb, tfd, first ? kTfNothing : qcoord, qseg, qsh, prm, C0, C1, C2, Tr);
+          stopped = Tr <= tr_stop && k > 0;
+          k -= first;
+        }
         if constexpr (!TREES) changed = head != word;
         if (changed) {
           uint32_t cur;
@@ -156,7 +171,7 @@ __global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_r
             ray.tout = 0.f;
             cur = 0;
           }
-          ++nlook;
+          nlook += !first;
           if constexpr (TRACE) cur_e = cur;
           load_record(prm.elem + cur, ra, rb, rc, rd);
           if constexpr (!FIXED)
@@ -166,52 +181,74 @@ __global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_r
           else
             blk.load(prm.bez + (int64_t)cur * blk.BYTES, 0);
         }
-        float tn;
-        if constexpr (FIXED) {
-          kf += 1.f;
-          tn = __fmaf_rn(kf, prm.h, ray.tin);
-        } else {
-          tn = __fadd_rn(t, dsv);
-        }
         // the next float where a step does not advance (t >= 0, so its bits order like it)
-        tn = tn > t ? tn : __int_as_float(__float_as_int(t) + 1);
-        const float seg = __fsub_rn(fminf(tn, ray.tout), t);
-        // evaluate sample k ...
-        float bx[N], by[N], bz[N];
-        const float ux = local_u(px, ra.x, rc.x, rd.x);
-        const float uy = local_u(py, ra.y, rc.y, rd.y);
-        const float uz = local_u(pz, ra.z, rc.z, rd.z);
-        monomials<P>(ux, bx);
-        monomials<P>(uy, by);
-        monomials<P>(uz, bz);
-        float v, sh = 1.f;
-        if constexpr (SHADE) {
-          float dx[N], dy[N], dz[N], gu, gv, gw;
-          dmonomials<P>(ux, dx);
-          dmonomials<P>(uy, dy);
-          dmonomials<P>(uz, dz);
-          v = blk.eval_grad(bx, by, bz, dx, dy, dz, gu, gv, gw);
-          const float gx = gu * rd.x, gy = gv * rd.y, gz = gw * rd.z;   // world gradient: d/dx = iw d/du
-          const float gl = fmaf(gx, lx, fmaf(gy, ly, gz * lz));
-          const float gn = fmaxf(sqrtf(fmaf(gx, gx, fmaf(gy, gy, gz * gz))), prm.grad_eps);
-          sh = fmaxf(0.4f, fabsf(gl) / gn);
-        } else {
-          v = blk.eval(bx, by, bz);
-        }
+        auto advance = [&](float from, float steps) -> float {
+          const float to = FIXED ? __fmaf_rn(steps, prm.h, ray.tin) : __fadd_rn(from, dsv);
+          return to > from ? to : __int_as_float(__float_as_int(from) + 1);
+        };
+        auto evaluate = [&](float x, float y, float z, float &sh) -> float {
+          float bx[N], by[N], bz[N];
+          const float ux = local_u(x, ra.x, rc.x, rd.x);
+          const float uy = local_u(y, ra.y, rc.y, rd.y);
+          const float uz = local_u(z, ra.z, rc.z, rd.z);
+          monomials<P>(ux, bx);
+          monomials<P>(uy, by);
+          monomials<P>(uz, bz);
+          sh = 1.f;
+          if constexpr (SHADE) {
+            float dx[N], dy[N], dz[N], gu, gv, gw;
+            dmonomials<P>(ux, dx);
+            dmonomials<P>(uy, dy);
+            dmonomials<P>(uz, dz);
+            const float v = blk.eval_grad(bx, by, bz, dx, dy, dz, gu, gv, gw);
+            const float gx = gu * rd.x, gy = gv * rd.y, gz = gw * rd.z;   // world gradient: d/dx = iw d/du
+            const float gl = fmaf(gx, lx, fmaf(gy, ly, gz * lz));
+            const float gn = fmaxf(sqrtf(fmaf(gx, gx, fmaf(gy, gy, gz * gz))), prm.grad_eps);
+            sh = fmaxf(0.4f, fabsf(gl) / gn);
+            return v;
+          } else {
+            return blk.eval(bx, by, bz);
+          }
+        };
+        float tn = advance(t, kf + 1.f);
+        const float te = fminf(tn, ray.tout);
+        pseg = __fsub_rn(te, t);
+        const float v = evaluate(px, py, pz, psh);
         if constexpr (TRACE) {
-          if (k < prm.trace_max) prm.trace_rec[g * prm.trace_max + k] = make_float4(t, __uint_as_float(cur_e), v, seg);
+          if (k < prm.trace_max) prm.trace_rec[g * prm.trace_max + k] = make_float4(t, __uint_as_float(cur_e), v, pseg);
         }
         pcoord = tf_coord(prm, v);
-        psh = sh;
-        pseg = seg;
+        bool two = false;
+        if constexpr (PAIR) {
+          const float qx = fma_sat(tn, ray.d[0], ray.o[0]);
+          const float qy = fma_sat(tn, ray.d[1], ray.o[1]);
+          const float qz = fma_sat(tn, ray.d[2], ray.o[2]);
+          two = qx >= ra.x && qy >= ra.y && qz >= ra.z && qx < rb.x && qy < rb.y && qz < rb.z && tn < ray.tout &&
+                k + 2 < kMaxSamplesPerRay;
+          const float t2 = advance(tn, kf + 2.f);
+          qseg = __fsub_rn(fminf(t2, ray.tout), te);   // finite also where the sample is dropped
+          const float v2 = evaluate(qx, qy, qz, qsh);
+          qcoord = two ? tf_coord(prm, v2) : kTfNothing;
+          tn = two ? t2 : tn;
+        }
+        pending = two ? 2 : 1;
+        if constexpr (FIXED) kf += two ? 2.f : 1.f;
         t = tn;
-        ++k;
+        k += pending;
       } while (!stopped && t < ray.tout && k < kMaxSamplesPerRay);
       if (stopped || k >= kMaxSamplesPerRay) {
         if (!stopped) set_status(prm.status, kStatusTimeout);
-        nsamp = k - 1;
+        nsamp = k - pending;
       } else {
         composite<SHADE, PACKED>(tfb, tfd, pcoord, pseg, psh, prm, C0, C1, C2, Tr);
+        if constexpr (PAIR) {
+          if (pending == 2) {
+            if (Tr <= tr_stop)
+              --k;
+            else
+              composite<SHADE, PACKED>(tfb, tfd, qcoord, qseg, qsh, prm, C0, C1, C2, Tr);
+          }
+        }
         nsamp = k;
       }
     }
@@ -236,18 +273,47 @@ __global__ void __launch_bounds__(128, (render_min_ctas<P, FIELD, STORE>())) k_r
   }
 }
 
-template <int P, int FIELD, int STORE, bool FIXED, bool TREES, bool TRACE>
+// This call's 8-row bands: band_index, band_index + band_count, ...
+inline dim3 render_grid(const RenderParams &prm) {
+  const int n_bands = (prm.row_end - prm.row_begin + 7) / 8;
+  const int mine = (n_bands - prm.band_index + prm.band_count - 1) / prm.band_count;
+  return dim3((unsigned)((prm.width + 15) / 16), (unsigned)mine);
+}
+
+template <int P, int FIELD, int STORE, bool FIXED, bool TREES, bool PAIR, bool TRACE>
 cudaError_t launch_render_f(const RenderParams &prm, cudaStream_t s) {
   if constexpr (TRACE) {
-    k_render<P, FIELD, STORE, FIXED, TREES, true><<<(unsigned)((prm.trace_n + 127) / 128), 128, 0, s>>>(prm);
+    k_render<P, FIELD, STORE, FIXED, TREES, PAIR, true><<<(unsigned)((prm.trace_n + 127) / 128), 128, 0, s>>>(prm);
   } else {
-    // this call's bands: band_index, band_index + band_count, ... of the 8-row bands
-    const int n_bands = (prm.row_end - prm.row_begin + 7) / 8;
-    const int mine = (n_bands - prm.band_index + prm.band_count - 1) / prm.band_count;
-    const dim3 grid((unsigned)((prm.width + 15) / 16), (unsigned)mine);
-    k_render<P, FIELD, STORE, FIXED, TREES, false><<<grid, 128, 0, s>>>(prm);
+    const dim3 grid = render_grid(prm);
+    k_render<P, FIELD, STORE, FIXED, TREES, PAIR, false><<<grid, 128, 0, s>>>(prm);
   }
   return cudaGetLastError();
+}
+
+// Two samples a pass (PAIR) or one.  Two cost their instructions also where the
+// second lies in another element, one waits for an element's loads once a sample.
+// Few warps an SM leave that wait bare, so frames of up to 12 CTAs for each of
+// the 152 SMs (640x360) take two: 256x256 and 640x360 frames, one / two a pass,
+// Eq. 4 tricubic FP32 408 / 351 and 545 / 476 us, learned FP16 185 / 175 and 262 /
+// 242, fixed FP32 296 / 270 and 394 / 382, triquadratic speed FP16 342 / 318 and
+// 342 / 338, component FP16 480 / 402 and 441 / 403.  Larger frames pay for the
+// second (1080p: learned FP32 1675 / 1745 us, fixed 1813 / 2042, speed FP16 653 /
+// 690) except Eq. 4 steps of tricubic scalar volumes, where an element holds 5.5
+// samples (FP32 2744 / 2599, BF16 2483 / 2337, FP16 2107 / 2061).  Never: shaded
+// frames (515 / 532 at 256x256, 3920 / 4351 at 1080p), and scalar volumes of degree
+// 2 and 1, whose elements hold fewer samples and load less (182 / 180, 215 / 228
+// and 256 / 242 at 256x256, 512x288 and 640x360; 89 / 93 at 512x288).
+constexpr unsigned kPairCtas = 12 * 152;
+
+template <int P, int FIELD, int STORE, bool FIXED, bool TREES, bool TRACE>
+cudaError_t launch_render_p(const RenderParams &prm, cudaStream_t s) {
+  if constexpr ((P == 3 || (P == 2 && FIELD != 0)) && FIELD != 3 && !TRACE) {
+    const dim3 grid = render_grid(prm);
+    if ((P == 3 && FIELD == 0 && prm.mode == LRVOL_STEP_HEURISTIC) || grid.x * grid.y <= kPairCtas)
+      return launch_render_f<P, FIELD, STORE, FIXED, TREES, true, TRACE>(prm, s);
+  }
+  return launch_render_f<P, FIELD, STORE, FIXED, TREES, false, TRACE>(prm, s);
 }
 
 // Fixed steps, and forests without a tree, have kernels of their own: which step
@@ -259,10 +325,10 @@ template <int P, int FIELD, int STORE, bool TRACE>
 cudaError_t launch_render_t(const RenderParams &prm, cudaStream_t s) {
   const bool trees = prm.forest.n_nodes > 0 || prm.forest.n_grid_units > 0;
   if (prm.mode == LRVOL_STEP_FIXED)
-    return trees ? launch_render_f<P, FIELD, STORE, true, true, TRACE>(prm, s)
-                 : launch_render_f<P, FIELD, STORE, true, false, TRACE>(prm, s);
-  return trees ? launch_render_f<P, FIELD, STORE, false, true, TRACE>(prm, s)
-               : launch_render_f<P, FIELD, STORE, false, false, TRACE>(prm, s);
+    return trees ? launch_render_p<P, FIELD, STORE, true, true, TRACE>(prm, s)
+                 : launch_render_p<P, FIELD, STORE, true, false, TRACE>(prm, s);
+  return trees ? launch_render_p<P, FIELD, STORE, false, true, TRACE>(prm, s)
+               : launch_render_p<P, FIELD, STORE, false, false, TRACE>(prm, s);
 }
 
 template <int STORE, bool TRACE>
