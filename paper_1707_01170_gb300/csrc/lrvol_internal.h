@@ -200,7 +200,8 @@ struct Incidence {
   int64_t n_elem = 0;
   int R = 1;
   unsigned char *base = nullptr;
-  int64_t o_ptr = 0, o_cell_ptr = 0, o_sums = 0, o_cell_count = 0, o_cell_of = 0, o_cell_el = 0, o_count = 0, o_empty = 0;
+  int64_t o_ptr = 0, o_cell_ptr = 0, o_sums = 0, o_cell_count = 0, o_cell_of = 0, o_cell_el = 0, o_cell_ends = 0,
+          o_count = 0, o_empty = 0;
   int64_t plan(int64_t n_elem);
   cudaError_t count(const lrvol_s *v, unsigned char *scratch, cudaStream_t s);
   cudaError_t fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, cudaStream_t s);
@@ -212,6 +213,7 @@ struct Incidence {
   uint32_t *cell_count() const { return at<uint32_t>(o_cell_count); }
   int32_t *cell_of() const { return at<int32_t>(o_cell_of); }
   int32_t *cell_el() const { return at<int32_t>(o_cell_el); }
+  longlong2 *cell_ends() const { return at<longlong2>(o_cell_ends); }
   uint32_t *counts() const { return at<uint32_t>(o_count); }
   uint32_t *empty() const { return at<uint32_t>(o_empty); }
 };

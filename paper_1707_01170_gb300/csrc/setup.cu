@@ -20,11 +20,15 @@ namespace {
 // incidence.  Elements are bucketed by their centres on a grid of R^3 cells, so
 // a B-spline's candidates are the buckets its support meets: for each (y, z)
 // one contiguous run of elements.  A warp takes a B-spline and its lanes the
-// run's elements; a pass counts the elements' B-splines, the other fills their
-// lists.  The lists are filled in no fixed order and sorted afterwards, since
-// k_to_bezier adds in the list's order.  Bound by the candidates' box reads
-// from the L2: about 1 ms for 174,000 elements and 11.45 M entries, where one
-// host thread took 145 ms (388,016 elements, 10.56 M entries: 365 ms).
+// run's elements, 16 to a run (about 16 elements); a pass counts the elements'
+// B-splines, the other fills their lists.  The lists are filled in no fixed order
+// and sorted afterwards, since k_to_bezier adds in the list's order.  An FP64
+// comparison occupies an SM for 16 cycles whatever lanes take part, so FP64 values
+// are compared by their bits as integers, and the support's six cells are
+// computed by six lanes at once; the boxes are copied into the buckets' order,
+// so that a run is read in whole lines.  179,768 elements and 11.8 M entries: 240 us
+// to count and 325 to fill; 677 each with the boxes read where they are, 865 with
+// FP64 comparisons and a warp to a run.  (One host thread took 145 ms for it all.)
 // ----------------------------------------------------------------------------
 struct CellGrid {
   int R;
@@ -43,13 +47,27 @@ __global__ void __launch_bounds__(256) k_cell_count(const double *__restrict__ b
   atomicAdd(count + c, 1u);
 }
 
-__global__ void __launch_bounds__(256) k_cell_fill(const int32_t *__restrict__ cell_of, int64_t n_elem,
+// Integers in the order of the numbers (no NaN; both zeros are 0).
+__device__ __forceinline__ int64_t order_key(double x) {
+  const int64_t b = __double_as_longlong(x);
+  return b >= 0 ? b : (b == INT64_MIN ? 0 : b ^ INT64_MAX);
+}
+__device__ __forceinline__ double from_order_key(int64_t k) { return __longlong_as_double(k >= 0 ? k : k ^ INT64_MAX); }
+__device__ __forceinline__ int64_t order_key_01(double x) { return __double_as_longlong(x) & INT64_MAX; }   // x >= 0 or -0
+
+// The elements of a cell side by side: their numbers, and for each axis the keys of
+// their lower and upper ends.
+__global__ void __launch_bounds__(256) k_cell_fill(const double *__restrict__ box, const int32_t *__restrict__ cell_of, int64_t n_elem,
                                                    const int64_t *__restrict__ cell_ptr, uint32_t *__restrict__ cursor,
-                                                   int32_t *__restrict__ cell_el) {
+                                                   int32_t *__restrict__ cell_el, longlong2 *__restrict__ ends) {
   const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= n_elem) return;
   const int32_t c = cell_of[e];
-  cell_el[cell_ptr[c] + atomicAdd(cursor + c, 1u)] = (int32_t)e;
+  const int64_t slot = cell_ptr[c] + atomicAdd(cursor + c, 1u);
+  cell_el[slot] = (int32_t)e;
+  const double *b = box + 6 * e;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) ends[a * n_elem + slot] = make_longlong2(order_key_01(b[a]), order_key_01(b[3 + a]));
 }
 
 constexpr int kSetupWarps = 8;
@@ -58,26 +76,33 @@ constexpr int kSetupWarps = 8;
 // true: their indices from list[ptr[e]] on, count as the cursors (zeroed).
 template <bool FILL>
 __global__ void __launch_bounds__(32 * kSetupWarps) k_incident(
-    const double *__restrict__ box, const double *__restrict__ knots, int64_t n_basis, int p0, int p1, int p2, int kw,
-    CellGrid g, const int64_t *__restrict__ cell_ptr, const int32_t *__restrict__ cell_el,
+    const longlong2 *__restrict__ ends, int64_t n_elem, const double *__restrict__ knots, int64_t n_basis, int p0,
+    int p1, int p2, int kw, CellGrid g, const int64_t *__restrict__ cell_ptr, const int32_t *__restrict__ cell_el,
     uint32_t *__restrict__ count, const int64_t *__restrict__ ptr, int32_t *__restrict__ list) {
   const int64_t i = (int64_t)blockIdx.x * kSetupWarps + (threadIdx.x >> 5);
   if (i >= n_basis) return;
   const int lane = threadIdx.x & 31;
-  const double *k = knots + i * kw;
-  const double lx = k[0], hx = k[p0 + 1], ly = k[p0 + 2], hy = k[p0 + 3 + p1], lz = k[p0 + p1 + 4],
-               hz = k[p0 + p1 + p2 + 5];
-  const int cx0 = g.coord(lx), cx1 = g.coord(hx);
-  const int cy0 = g.coord(ly), ny = g.coord(hy) - cy0 + 1;
-  const int cz0 = g.coord(lz), rows = ny * (g.coord(hz) - cz0 + 1);
-  for (int r = 0; r < rows; ++r) {
-    const int64_t row = ((int64_t)(cz0 + r / ny) * g.R + cy0 + r % ny) * g.R;
-    const int64_t end = cell_ptr[row + cx1 + 1];
-    for (int64_t q = cell_ptr[row + cx0] + lane; q < end; q += 32) {
-      const int32_t e = cell_el[q];
-      const double2 *b2 = reinterpret_cast<const double2 *>(box + 6 * (int64_t)e);   // 48 bytes an element
-      const double2 a = __ldg(b2), b = __ldg(b2 + 1), c = __ldg(b2 + 2);             // lo x y | lo z, hi x | hi y z
-      if (lx <= a.x && ly <= a.y && lz <= b.x && b.y <= hx && c.x <= hy && c.y <= hz) {
+  // lane 2a: lower end of the support on axis a, lane 2a + 1: its upper end
+  const int axis = (lane >> 1) % 3;
+  const int at = (axis > 0 ? p0 + 2 : 0) + (axis > 1 ? p1 + 2 : 0) + (lane & 1) * ((axis == 0 ? p0 : axis == 1 ? p1 : p2) + 1);
+  const double knot = knots[i * kw + at];
+  const int64_t key = order_key(knot);
+  const int cell = g.coord(knot);
+  int64_t end[6];
+  int c[6];
+#pragma unroll
+  for (int t = 0; t < 6; ++t) {
+    end[t] = __shfl_sync(0xffffffffu, key, t);
+    c[t] = __shfl_sync(0xffffffffu, cell, t);
+  }
+  const int ny = c[3] - c[2] + 1, rows = ny * (c[5] - c[4] + 1);
+  for (int r = lane >> 4; r < rows; r += 2) {
+    const int64_t row = ((int64_t)(c[4] + r / ny) * g.R + c[2] + r % ny) * g.R;
+    const int64_t stop = cell_ptr[row + c[1] + 1];
+    for (int64_t q = cell_ptr[row + c[0]] + (lane & 15); q < stop; q += 16) {
+      const longlong2 x = __ldg(ends + q), y = __ldg(ends + n_elem + q), z = __ldg(ends + 2 * n_elem + q);
+      if (end[0] <= x.x && end[2] <= y.x && end[4] <= z.x && x.y <= end[1] && y.y <= end[3] && z.y <= end[5]) {
+        const int32_t e = cell_el[q];
         const uint32_t n = atomicAdd(count + e, 1u);
         if constexpr (FILL) list[ptr[e] + n] = (int32_t)i;
       }
@@ -468,7 +493,10 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
 // Render copy of the FP64 blocks (layout and storage in lrvol_internal.h):
 // binomials folded in; for 16-bit storage a per-element, per-component offset
 // o = (max+min)/2 and scale s = (max-min)/2 of the FP64 coefficients, and
-// q' = binomial*(c - o)/s rounded once from FP64.  One warp per element.
+// q' = binomial*(c - o)/s rounded once from FP64.  One warp per element.  Bound by
+// FP64 operations (16 cycles of an SM each), so the range is found on integers:
+// 179,768 tricubic elements, FP32 187 us (291 with FP64 minima and maxima),
+// FP16 378 (549), of which the division is most.
 __device__ __forceinline__ void store_slot(unsigned char *base, int storage, int slot, double x) {
   if (storage == LRVOL_STORE_F32) {
     reinterpret_cast<float *>(base)[slot] = (float)x;
@@ -491,15 +519,20 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_pack(const double *__restric
   double o[3] = {0.0, 0.0, 0.0}, sc[3] = {1.0, 1.0, 1.0};
   for (int c = 0; c < nc; ++c) {
     // coefficient range (the block's convex hull bounds the field on the element)
-    double mn = __longlong_as_double(0x7ff0000000000000ll), mx = -mn;
+    constexpr int64_t kInf = 0x7ff0000000000000ll;
+    int64_t kmn = kInf, kmx = kInf ^ INT64_MIN ^ INT64_MAX;   // inf and -inf
     for (int q = lane; q < nb; q += 32) {
-      mn = fmin(mn, be[c * nb + q]);
-      mx = fmax(mx, be[c * nb + q]);
+      const double x = be[c * nb + q];
+      if (order_key_01(x) <= kInf) {   // no NaN
+        kmn = min(kmn, order_key(x));
+        kmx = max(kmx, order_key(x));
+      }
     }
     for (int off = 16; off > 0; off >>= 1) {
-      mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, off));
-      mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+      kmn = min(kmn, __shfl_xor_sync(0xffffffffu, kmn, off));
+      kmx = max(kmx, __shfl_xor_sync(0xffffffffu, kmx, off));
     }
+    const double mn = from_order_key(kmn), mx = from_order_key(kmx);
     if (lane == 0) range[e * nc + c] = make_float2(__double2float_rd(mn), __double2float_ru(mx));
     if (storage != LRVOL_STORE_F32) {
       o[c] = 0.5 * (mx + mn);
@@ -518,8 +551,8 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_pack(const double *__restric
     const int ix = q % n0, iy = (q / n0) % n1, iz = q / (n0 * n1);
     const double binom = (double)(binomial(p0, ix) * binomial(p1, iy) * binomial(p2, iz));
     for (int c = 0; c < nc; ++c) {
-      const double d = be[c * nb + q] - o[c];   // o = 0 and s = 1 for FP32 storage
-      const double x = storage == LRVOL_STORE_F32 ? binom * d : binom * d / sc[c];
+      const double b = be[c * nb + q];
+      const double x = storage == LRVOL_STORE_F32 ? binom * b : binom * (b - o[c]) / sc[c];
       store_slot(out + e * ebytes, storage, render_slot(nc, n0, nb, iz * n1 + iy, ix, c), x);
       if (outc) store_slot(outc + e * ecbytes, storage, c * roundup8(nb) + q, x);
     }
@@ -568,6 +601,7 @@ int64_t Incidence::plan(int64_t n_elem_) {
   o_cell_count = take(4 * cells);
   o_cell_of = take(4 * n_elem);
   o_cell_el = take(4 * n_elem);
+  o_cell_ends = take(48 * n_elem);
   o_count = take(4 * n_elem);
   o_empty = take(4);
   return at;
@@ -585,17 +619,17 @@ cudaError_t Incidence::count(const lrvol_s *v, unsigned char *scratch, cudaStrea
   k_cell_count<<<eb, 256, 0, s>>>(v->d_box, n_elem, g, cell_of(), cell_count());
   if ((e = exclusive_scan(cell_count(), cells, cell_ptr(), sums(), nullptr, s)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(cell_count(), 0, 4 * cells, s)) != cudaSuccess) return e;
-  k_cell_fill<<<eb, 256, 0, s>>>(cell_of(), n_elem, cell_ptr(), cell_count(), cell_el());
-  k_incident<false><<<wb, 32 * kSetupWarps, 0, s>>>(v->d_box, v->d_knots, v->n_basis, v->p[0], v->p[1], v->p[2], v->kw,
-                                                   g, cell_ptr(), cell_el(), counts(), nullptr, nullptr);
+  k_cell_fill<<<eb, 256, 0, s>>>(v->d_box, cell_of(), n_elem, cell_ptr(), cell_count(), cell_el(), cell_ends());
+  k_incident<false><<<wb, 32 * kSetupWarps, 0, s>>>(cell_ends(), n_elem, v->d_knots, v->n_basis, v->p[0], v->p[1],
+                                                   v->p[2], v->kw, g, cell_ptr(), cell_el(), counts(), nullptr, nullptr);
   if ((e = exclusive_scan(counts(), n_elem, ptr(), sums(), empty(), s)) != cudaSuccess) return e;
   return cudaMemsetAsync(counts(), 0, 4 * n_elem, s);   // from here the fill's cursors
 }
 
 cudaError_t Incidence::fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, cudaStream_t s) {
   const unsigned wb = (unsigned)((v->n_basis + kSetupWarps - 1) / kSetupWarps);
-  k_incident<true><<<wb, 32 * kSetupWarps, 0, s>>>(v->d_box, v->d_knots, v->n_basis, v->p[0], v->p[1], v->p[2], v->kw,
-                                                  CellGrid{R}, cell_ptr(), cell_el(), counts(), ptr(), unsorted);
+  k_incident<true><<<wb, 32 * kSetupWarps, 0, s>>>(cell_ends(), n_elem, v->d_knots, v->n_basis, v->p[0], v->p[1],
+                                                  v->p[2], v->kw, CellGrid{R}, cell_ptr(), cell_el(), counts(), ptr(), unsorted);
   k_sort_lists<<<(unsigned)((n_elem + kSetupWarps - 1) / kSetupWarps), 32 * kSetupWarps, 0, s>>>(ptr(), n_elem, unsorted,
                                                                                               list);
   return cudaGetLastError();

@@ -136,3 +136,24 @@ def test_element_without_a_spline_is_refused():
     with pytest.raises(lv.LrvolError):
         gv.get_bezier()
     gv.close()
+
+
+def test_signed_zeros_and_knots_below_zero():
+    """-0 in boxes, knots and coefficients is 0, and knots below 0 lie below it: the same lists and blocks."""
+    k = np.array([[-2.0, -1.0, 0.0, 1.0], [-1.0, 0.0, 1.0, 2.0], [0.0, 1.0, 2.0, 3.0]])
+    q = np.stack(np.meshgrid(*[np.arange(3)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    coef = np.sin(np.arange(27.0))[:, None]
+    coef[::4] = 0.0
+    vol = LRVolume(deg=np.array([2, 2, 2]), elem_box=np.array([[0.0, 0, 0, 1, 1, 1]]), knots=k[q].reshape(27, 12), coef=coef,
+                   weight=np.ones(27), grid=np.array([1, 1, 1]))
+    out = []
+    for zero in (0.0, -0.0):
+        for a in (vol.elem_box, vol.knots, vol.coef):
+            a[a == 0] = zero
+        gv = lv.Volume(vol).to_bezier()
+        f = torch.rand((64, 3), generator=torch.Generator().manual_seed(2)).cuda()
+        out.append((gv.stats()["incidence_entries"], gv.get_bezier(), gv.build_accel((1, 1, 1)).eval(f).cpu(),
+                    gv.to_bezier(lv.STORE_F16).eval(f).cpu()))
+        gv.close()
+    assert out[0][0] == out[1][0] == 27 == _incidence(vol)
+    assert all(np.array_equal(a, b) for a, b in zip(out[0][1:], out[1][1:]))
