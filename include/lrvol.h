@@ -154,7 +154,8 @@ int lrvol_create(const int32_t deg[3], int32_t ncomp, int64_t n_elem, const doub
  * regular blocks (each a power of two, at most 1024), one depth-balanced k-d
  * tree per block over the elements meeting it; split planes are element
  * faces rounded up to FP32 so that FP32 queries decide exactly as in FP64.
- * The tree is built on the host and uploaded on `stream`.
+ * The trees are built on the host, by several threads where there are many
+ * elements, and uploaded on `stream`.
  * Errors: LRVOL_ERR_ARG (blocks not powers of two), LRVOL_ERR_OOM, LRVOL_ERR_CUDA. */
 int lrvol_build_accel(lrvol_t vol, const int32_t blocks[3], void *stream);
 
@@ -205,7 +206,8 @@ int lrvol_render(lrvol_t vol, const lrvol_camera *cam, const lrvol_tf *tf, const
  * flag that is off in every lrvol_render launch; every per-ray decision and
  * value is the same as in lrvol_render's image (one thread per listed pixel
  * instead of per tile position; a ray's work does not depend on its
- * neighbours).
+ * neighbours, nor on whether a pass of its loop takes one sample, as here,
+ * or two).
  *   pix_dev      n_pix x 2 int32 (i, j) pixel coordinates (device); the
  *                camera's row range is ignored.  A pixel outside the image
  *                gets count 0, RGBA 0 and sets the status word (LRVOL_ERR_BOUNDS
@@ -414,7 +416,8 @@ int lrvol_trim(const lrvol_camera *cam, const float *tri_dev, int64_t n_tri, flo
  * A streamline stops at t_end (status 0), when a stage point or the next
  * point leaves [0,1]^3 (status 1; the point before is the last sample),
  * after max_samples samples (2), or when the step control gives up (3).
- * One thread traces one line at a time; a grid that fits on the GPU at once
+ * One thread, or four lanes together while there are few lines, trace one
+ * line at a time; a grid that fits on the GPU at once
  * takes the seeds from a counter in the handle, so concurrent streamline
  * calls on one handle are not allowed (as for every call on a handle).
  * With fewer seeds than the GPU holds warps, each warp traces fewer than 32

@@ -18,9 +18,9 @@ namespace {
 // One CTA of 4 warps renders a 16x8-pixel tile, so the warps sharing an SM's
 // L1 march through neighbouring elements; one lane traces one ray.  A warp
 // covers an 8x4 patch for scalar fields and a 4x8 patch for 3-vector fields
-// (the shapes that measured fastest for each).  The element-change branch (look-up and block loads) is kept
-// minimal: a warp runs it whenever any of its lanes changes element, which
-// happens almost every iteration.
+// (the shapes that measured fastest for each).  The element-change branch
+// (look-up and block loads) is kept minimal: a warp runs it whenever any of its
+// lanes changes element, which happens almost every iteration.
 //
 // In the sample loop the Alg. 2 update of sample k comes after the position of
 // sample k+1 and, where no block of the forest holds a tree, after the load of
@@ -35,14 +35,15 @@ namespace {
 //
 // A warp's iteration waits about as long for its instructions as for the loads
 // of an element change, so both the sample's and the change's instructions
-// count: clamps fused into the multiply-add (.sat), no branch besides the
-// element change, block sizes and step rule known to the compiler, a head
+// count: the position's clamps fused into its multiply-add (.sat), no branch
+// besides the element change, block sizes and step rule known to the compiler, a head
 // table that needs no clamped index, and without trees (TREES false) no box test.
 // 1920x1080 frames of a 174,000-element tricubic volume, Eq. 4 steps, with
 // FP32 / BF16 / FP16 blocks: 3.05 / 2.98 / 2.45 ms before these, 2.75 / 2.49 /
-// 2.10 now; FP32 gradient-shaded 4.51 -> 3.92; learned FP16 at 3840x2160 4.27 ->
-// 3.74; 3-vector speed of 388,016 triquadratic elements in a forest with trees,
-// FP32 / FP16: 0.93 / 0.79 -> 0.77 / 0.67 (grids for subtrees among it).
+// 2.10 with them, 2.60 / 2.34 / 2.08 with two samples a pass as well; FP32
+// gradient-shaded 4.51 -> 3.92; learned FP16 at 3840x2160 4.27 -> 3.76; 3-vector
+// speed of 388,016 triquadratic elements in a forest with trees, FP32 / FP16:
+// 0.93 / 0.79 -> 0.77 / 0.67 (grids for subtrees among it).
 //
 // TRACE (a compile-time flag; false in every product launch, where the trace
 // code compiles out) runs the same march for a list of pixels, one thread per
