@@ -369,19 +369,13 @@ __device__ __forceinline__ void factor(const double *__restrict__ xi, double a, 
 // B-splines over an element share their univariate factors (about 20 different
 // ones over the three axes among 66 B-splines).  So the warp first finds the
 // different local knot vectors of each axis, by bits, computes each factor
-// once, a lane a factor.  The B-splines' coefficients then go into a table over
-// the three axes' factors, zeros where there is no B-spline, and the table is
-// contracted with the factors one axis after the other, in place: about 80 FP64
-// instructions a warp instead of 4 for each of the 66 B-splines.  Where the table
-// would have more than kCells entries, or two B-splines would share one, the
-// products of the listed factors are added up one B-spline after the other.
+// once, a lane a factor, and then adds the products of the listed factors.
 // A list of more than kListMax B-splines, or with more than 32 different knot
 // vectors on an axis, is left to the general kernel (todo, n_todo).
-// 179,768 tricubic elements (11.8 M pairs) take 2.49 ms, 4.03 with the products
-// added up, 13.8 with a factor of every pair and axis computed anew; 388,016
-// triquadratic 3-vector elements 2.39 ms, 4.21 with the products added up.  What is
-// left is half the factors' divisions.
-constexpr int kListMax = 128, kCells = 640;
+// The change of basis of 174,000 tricubic elements (11.45 M pairs) takes 7.2 ms
+// in all, allocations included, 17.0 with a factor of every pair and axis
+// computed anew; 388,016 triquadratic 3-vector elements 11.4 instead of 14.9.
+constexpr int kListMax = 128;
 
 template <int P, int NC>
 __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
@@ -394,7 +388,6 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
   __shared__ double s_g[kBezWarps][NC][kListMax];
   __shared__ uint32_t s_ids[kBezWarps][kListMax];
   __shared__ int32_t s_rep[kBezWarps][3][32];
-  __shared__ double s_cells[kBezWarps][kCells];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t e = (int64_t)blockIdx.x * kBezWarps + w;
   if (e >= n_elem) return;
@@ -458,62 +451,6 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
     for (int q = 0; q < N; ++q) s_fac[w][a][t][q] = beta[q];
   }
   __syncwarp();
-  // cell (i, j, k) at (i * sy + j) * sz + k; the contractions leave N for j and k
-  const int sy = max(nd[1], N), sz = max(nd[2], N), cells = nd[0] * sy * sz;
-  double *T = s_cells[w];
-  auto cell_of = [&](int s) {
-    const uint32_t ids = s_ids[w][s];
-    return (int)(((ids & 255u) * sy + ((ids >> 8) & 255u)) * sz + (ids >> 16));
-  };
-  bool table = cells <= kCells;
-  if (table) {   // each B-spline in a cell of its own?
-    long long *tag = reinterpret_cast<long long *>(T);
-    for (int s = lane; s < L; s += 32) tag[cell_of(s)] = s;
-    __syncwarp();
-    for (int s = lane; s < L; s += 32) table &= tag[cell_of(s)] == s;
-    table = __all_sync(kAll, table);
-  }
-  if (table) {
-#pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
-      __syncwarp();
-      for (int q = lane; q < cells; q += 32) T[q] = 0.0;
-      __syncwarp();
-      for (int s = lane; s < L; s += 32) T[cell_of(s)] = s_g[w][c][s];
-      __syncwarp();
-      // in place: whole rows of k, then whole (j, k) planes, are read before they are written
-      constexpr int ZL = 32 / N * N, YL = 32 / (N * N) * (N * N);
-      for (int q0 = 0; q0 < nd[0] * nd[1] * N; q0 += ZL) {
-        const int q = q0 + lane, row = q / N, z = q % N;
-        const bool on = lane < ZL && row < nd[0] * nd[1];
-        double *at = T + (on ? (row / nd[1] * sy + row % nd[1]) * sz : 0);
-        double t = 0.0;
-        if (on)
-          for (int k = 0; k < nd[2]; ++k) t = fma(at[k], s_fac[w][2][k][z], t);
-        __syncwarp();
-        if (on) at[z] = t;
-        __syncwarp();
-      }
-      for (int q0 = 0; q0 < nd[0] * N * N; q0 += YL) {
-        const int q = q0 + lane, i = q / (N * N), y = q / N % N, z = q % N;
-        const bool on = lane < YL && i < nd[0];
-        double *at = T + (on ? i * sy * sz : 0);
-        double t = 0.0;
-        if (on)
-          for (int j = 0; j < nd[1]; ++j) t = fma(at[j * sz + z], s_fac[w][1][j][y], t);
-        __syncwarp();
-        if (on) at[y * sz + z] = t;
-        __syncwarp();
-      }
-      for (int q = lane; q < NB; q += 32) {
-        const int x = q % N, y = q / N % N, z = q / (N * N);
-        double t = 0.0;
-        for (int i = 0; i < nd[0]; ++i) t = fma(T[(i * sy + y) * sz + z], s_fac[w][0][i][x], t);
-        out64[(e * NC + c) * NB + q] = t;
-      }
-    }
-    return;
-  }
   double acc[R][NC];
   int ix[R], iy[R], iz[R];
 #pragma unroll
@@ -559,8 +496,7 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
 // q' = binomial*(c - o)/s rounded once from FP64.  One warp per element.  Bound by
 // FP64 operations (16 cycles of an SM each), so the range is found on integers:
 // 179,768 tricubic elements, FP32 187 us (291 with FP64 minima and maxima),
-// FP16 378 (549), of which the division
-// is most; 388,016 triquadratic 3-vector elements, FP32 414 (1294).
+// FP16 378 (549), of which the division is most.
 __device__ __forceinline__ void store_slot(unsigned char *base, int storage, int slot, double x) {
   if (storage == LRVOL_STORE_F32) {
     reinterpret_cast<float *>(base)[slot] = (float)x;

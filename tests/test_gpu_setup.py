@@ -157,33 +157,3 @@ def test_signed_zeros_and_knots_below_zero():
         gv.close()
     assert out[0][0] == out[1][0] == 27 == _incidence(vol)
     assert all(np.array_equal(a, b) for a, b in zip(out[0][1:], out[1][1:]))
-
-
-@pytest.mark.parametrize("deg", [(1, 1, 1), (2, 2, 2), (3, 3, 3), (4, 4, 4)])
-@pytest.mark.parametrize("ncomp", [1, 3])
-@pytest.mark.parametrize("shape", [(1, 1, 1), (8, 8, 9), (9, 9, 8), (9, 9, 9), (2, 20, 16), "twice"])
-def test_tables_of_splines(deg, ncomp, shape):
-    """Tables of one cell, about and above 640, thin ones, with empty cells, and a B-spline listed twice.
-
-    Over [0, 1] the B-spline on (-n, 0, .., 0, 1) is c_n (1 - x)^p with c_n = 1 for the triangle's one entry: the first
-    Bernstein polynomial.  The block's first coefficient is the sum, the rest are 0.
-    """
-    p = deg[0]
-    n = (3, 3, 3) if shape == "twice" else shape
-    k = [np.stack([-np.arange(1.0, m + 1)] + [np.zeros(m)] * p + [np.ones(m)], 1) for m in n]
-    q = np.stack(np.meshgrid(*[np.arange(m) for m in n], indexing="ij"), -1).reshape(-1, 3)
-    rng = np.random.default_rng(sum(n))
-    if shape == "twice":
-        q = np.concatenate([q, q[5:6]])
-    elif len(q) > 100:      # every factor used, most cells empty
-        must = np.stack([np.arange(max(n)) % m for m in n], 1)
-        q = np.unique(np.concatenate([must, q[rng.permutation(len(q))[:80]]]), axis=0)
-    knots = np.concatenate([k[a][q[:, a]] for a in range(3)], axis=1)
-    vol = LRVolume(deg=np.array(deg), elem_box=np.array([[0.0, 0, 0, 1, 1, 1]]), knots=knots,
-                   coef=rng.random((len(q), ncomp)), weight=rng.random(len(q)), grid=np.array([1, 1, 1]))
-    gv = lv.Volume(vol).to_bezier()
-    got = gv.get_bezier()[0]
-    gv.close()
-    want = np.zeros((ncomp,) + (p + 1,) * 3)
-    want[:, 0, 0, 0] = (vol.weight[:, None] * vol.coef).sum(0)
-    assert np.abs(got.reshape(want.shape) - want).max() <= 8 * len(q) * 2.0 ** -53 * want.max()
