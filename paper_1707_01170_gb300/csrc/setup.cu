@@ -466,21 +466,13 @@ __global__ void __launch_bounds__(32 * kBezWarps) k_to_bezier_shared(
   for (int s = 0; s < L; ++s) {
     const uint32_t ids = s_ids[w][s];
     const double *fx = s_fac[w][0][ids & 255u], *fy = s_fac[w][1][(ids >> 8) & 255u], *fz = s_fac[w][2][ids >> 16];
-    if constexpr (N == 4) {   // the lane's coefficients differ in z only
-      const double xy = fx[ix[0]] * fy[iy[0]];
+    // the products in this order: the blocks' last bits decide whether a constant
+    // element's range is one value, and with it the bins of its features
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const double gxy = s_g[w][c][s] * xy;
+    for (int r = 0; r < R; ++r) {
+      const double prod = fx[ix[r]] * fy[iy[r]] * fz[iz[r]];
 #pragma unroll
-        for (int r = 0; r < R; ++r) acc[r][c] = fma(gxy, fz[iz[r]], acc[r][c]);
-      }
-    } else {
-#pragma unroll
-      for (int r = 0; r < R; ++r) {
-        const double prod = fx[ix[r]] * fy[iy[r]] * fz[iz[r]];
-#pragma unroll
-        for (int c = 0; c < NC; ++c) acc[r][c] = fma(s_g[w][c][s], prod, acc[r][c]);
-      }
+      for (int c = 0; c < NC; ++c) acc[r][c] = fma(s_g[w][c][s], prod, acc[r][c]);
     }
   }
 #pragma unroll
