@@ -11,6 +11,7 @@ of incidence entries against a direct test of supports, and two conversions bit
 for bit (the lists are filled in no fixed order and sorted).
 """
 import math
+import time
 
 import numpy as np
 import pytest
@@ -86,6 +87,23 @@ def test_forest_accepts_and_refuses_as_it_did():
         with pytest.raises(lv.LrvolError) as err:
             gv.build_accel(blocks)
         assert err.value.status == lv.ERR_ARG
+    gv.close()
+
+
+def _boxes(lo, hi, n):
+    v = _half_box()
+    v.elem_box = np.tile(np.array([[*lo, *hi]], dtype=np.float64), (n, 1))
+    return v
+
+
+@pytest.mark.parametrize("name,lo,hi,n", [("cubes", (0, 0, 0), (1, 1, 1), 8000), ("sheets", (0, 0, 0.5), (1, 1, 0.500001), 20000)])
+def test_overlapping_boxes_are_refused_at_once(name, lo, hi, n):
+    """Boxes that all meet thousands of blocks (in all 2.1e9 and 8.2e7): refused without visiting those."""
+    gv = lv.Volume(_boxes(lo, hi, n))
+    t = time.perf_counter()
+    with pytest.raises(lv.LrvolError) as err:
+        gv.build_accel((64, 64, 64))
+    assert err.value.status == lv.ERR_ARG and time.perf_counter() - t < 0.1
     gv.close()
 
 
