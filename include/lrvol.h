@@ -154,8 +154,8 @@ int lrvol_create(const int32_t deg[3], int32_t ncomp, int64_t n_elem, const doub
  * regular blocks (each a power of two, at most 1024), one depth-balanced k-d
  * tree per block over the elements meeting it; split planes are element
  * faces rounded up to FP32 so that FP32 queries decide exactly as in FP64.
- * The trees are built on the host, by several threads where there are many
- * elements, and uploaded on `stream`.
+ * The trees are built on the host, by up to 16 threads where the work is worth
+ * starting them, and uploaded on `stream`.
  * Errors: LRVOL_ERR_ARG (blocks not powers of two), LRVOL_ERR_OOM, LRVOL_ERR_CUDA. */
 int lrvol_build_accel(lrvol_t vol, const int32_t blocks[3], void *stream);
 

@@ -92,19 +92,74 @@ struct TreeBuilder {
   bool unresolved = false;     // a midpoint tree reached kMaxDepth
 
   const double *box(int32_t e) const { return &v->box[6 * (size_t)e]; }
+
   // Build a tree over `els` inside region [rlo, rhi); returns a reference.
-  uint32_t build(std::vector<int32_t> &els, const double *rlo, const double *rhi, int d, int *maxd) {
+  uint32_t build(const int32_t *els, size_t n, const double *rlo, const double *rhi, int *maxd) {
+    pool.assign(els, els + n);
+    return subtree(0, n, rlo, rhi, 0, maxd);
+  }
+
+ private:
+  // Element lists of the subtrees under way, on one stack: a node puts its
+  // children's lists on top and takes them off when both are built.  (4,096
+  // elements in one tree, the whole call: 583 us by midpoints and 2,148 balanced
+  // with a vector for each list, 349 and 1,698 so.)
+  std::vector<int32_t> pool;
+  std::vector<double> cand;
+
+  // The elements of pool[beg, end) on either side of the plane t, on top of the
+  // pool: the low ones, and from the returned place on the high ones.
+  size_t divide(size_t beg, size_t end, int a, double t) {
+    size_t to = pool.size();
+    pool.resize(to + 2 * (end - beg));
+    for (size_t q = beg; q < end; ++q) {
+      pool[to] = pool[q];
+      to += box(pool[q])[a] < t;
+    }
+    const size_t mid = to;
+    for (size_t q = beg; q < end; ++q) {
+      pool[to] = pool[q];
+      to += box(pool[q])[3 + a] > t;
+    }
+    pool.resize(to);
+    return mid;
+  }
+
+  // The node that splits region [rlo, rhi) at t, its children from the lists on top of the pool.
+  uint32_t node(size_t low, size_t mid, int a, double t, const double *rlo, const double *rhi, int d, int *maxd) {
+    const uint32_t me = (uint32_t)nodes.size();
+    nodes.push_back(Node{0, 0, {0, 0}});
+    Node nd;
+    const float s = round_up_f32(t);
+    std::memcpy(&nd.split_bits, &s, 4);
+    nd.axis = (uint32_t)a;
+    double lhi[3], hlo[3];
+    for (int c = 0; c < 3; ++c) {
+      lhi[c] = c == a ? t : rhi[c];
+      hlo[c] = c == a ? t : rlo[c];
+    }
+    const size_t top = pool.size();
+    nd.child[0] = subtree(low, mid, rlo, lhi, d + 1, maxd);
+    if (nd.child[0] == kNone) return kNone;
+    nd.child[1] = subtree(mid, top, hlo, rhi, d + 1, maxd);
+    if (nd.child[1] == kNone) return kNone;
+    pool.resize(low);
+    nodes[me] = nd;
+    return me;
+  }
+
+  uint32_t subtree(size_t beg, size_t end, const double *rlo, const double *rhi, int d, int *maxd) {
     *maxd = std::max(*maxd, d);
-    if (els.size() == 1) return kLeaf | (uint32_t)els[0];
-    if (midpoint) return build_mid(els, rlo, rhi, d, maxd);
+    const size_t n = end - beg;
+    if (n == 1) return kLeaf | (uint32_t)pool[beg];
+    if (midpoint) return subtree_mid(beg, end, rlo, rhi, d, maxd);
     int best_axis = -1;
     double best_t = 0;
     size_t best_score = SIZE_MAX;
-    std::vector<double> cand;
     for (int a = 0; a < 3; ++a) {
       cand.clear();
-      for (int32_t e : els) {
-        const double *b = box(e);
+      for (size_t q = beg; q < end; ++q) {
+        const double *b = box(pool[q]);
         if (b[a] > rlo[a] && b[a] < rhi[a]) cand.push_back(b[a]);
         if (b[3 + a] > rlo[a] && b[3 + a] < rhi[a]) cand.push_back(b[3 + a]);
       }
@@ -118,8 +173,8 @@ struct TreeBuilder {
       for (double c : cand)
         if (std::fabs(c - mean) < std::fabs(t - mean)) t = c;
       size_t nl = 0, nr = 0;
-      for (int32_t e : els) {
-        const double *b = box(e);
+      for (size_t q = beg; q < end; ++q) {
+        const double *b = box(pool[q]);
         nl += b[a] < t;
         nr += b[3 + a] > t;
       }
@@ -131,33 +186,9 @@ struct TreeBuilder {
       }
     }
     if (best_axis < 0) return kNone;  // cannot happen for a valid box partition
-    std::vector<int32_t> L, R;
-    for (int32_t e : els) {
-      const double *b = box(e);
-      if (b[best_axis] < best_t) L.push_back(e);
-      if (b[3 + best_axis] > best_t) R.push_back(e);
-    }
-    if (L.size() >= els.size() || R.size() >= els.size() || L.empty() || R.empty()) return kNone;
-    uint32_t me = (uint32_t)nodes.size();
-    nodes.push_back(Node{0, 0, {0, 0}});
-    Node nd;
-    float s = round_up_f32(best_t);
-    std::memcpy(&nd.split_bits, &s, 4);
-    nd.axis = (uint32_t)best_axis;
-    double llo[3], lhi[3], hlo[3], hhi[3];
-    for (int a = 0; a < 3; ++a) {
-      llo[a] = hlo[a] = rlo[a];
-      lhi[a] = hhi[a] = rhi[a];
-    }
-    lhi[best_axis] = best_t;
-    hlo[best_axis] = best_t;
-    els.clear();
-    els.shrink_to_fit();
-    nd.child[0] = build(L, llo, lhi, d + 1, maxd);
-    nd.child[1] = build(R, hlo, hhi, d + 1, maxd);
-    if (nd.child[0] == kNone || nd.child[1] == kNone) return kNone;
-    nodes[me] = nd;
-    return me;
+    const size_t low = pool.size(), mid = divide(beg, end, best_axis, best_t), nl = mid - low, nr = pool.size() - mid;
+    if (nl >= n || nr >= n || nl == 0 || nr == 0) return kNone;
+    return node(low, mid, best_axis, best_t, rlo, rhi, d, maxd);
   }
 
   // Octree-style tree: the region's midpoint on axes x, y, z in turn (three
@@ -166,43 +197,17 @@ struct TreeBuilder {
   // faces are reached exactly (midpoints of dyadic regions are dyadic, and
   // exact in FP32 down to 2^-149); a face at a non-dyadic coordinate never
   // is, and the tree is abandoned at kMaxDepth.
-  uint32_t build_mid(std::vector<int32_t> &els, const double *rlo, const double *rhi, int d, int *maxd) {
+  uint32_t subtree_mid(size_t beg, size_t end, const double *rlo, const double *rhi, int d, int *maxd) {
     if (d >= kMaxDepth - 1) {
       unresolved = true;
       return kNone;
     }
     const int a = d % 3;
     const double t = 0.5 * (rlo[a] + rhi[a]);
-    std::vector<int32_t> L, R;
-    for (int32_t e : els) {
-      const double *b = box(e);
-      if (b[a] < t) L.push_back(e);
-      if (b[3 + a] > t) R.push_back(e);
-    }
-    if (L.empty() || R.empty()) return kNone;   // not a box partition
-    uint32_t me = (uint32_t)nodes.size();
-    nodes.push_back(Node{0, 0, {0, 0}});
-    Node nd;
-    float s = round_up_f32(t);
-    std::memcpy(&nd.split_bits, &s, 4);
-    nd.axis = (uint32_t)a;
-    double llo[3], lhi[3], hlo[3], hhi[3];
-    for (int c = 0; c < 3; ++c) {
-      llo[c] = hlo[c] = rlo[c];
-      lhi[c] = hhi[c] = rhi[c];
-    }
-    lhi[a] = t;
-    hlo[a] = t;
-    els.clear();
-    els.shrink_to_fit();
-    nd.child[0] = build(L, llo, lhi, d + 1, maxd);
-    if (nd.child[0] == kNone) return kNone;
-    nd.child[1] = build(R, hlo, hhi, d + 1, maxd);
-    if (nd.child[1] == kNone) return kNone;
-    nodes[me] = nd;
-    return me;
+    const size_t low = pool.size(), mid = divide(beg, end, a, t);
+    if (mid == low || mid == pool.size()) return kNone;   // not a box partition
+    return node(low, mid, a, t, rlo, rhi, d, maxd);
   }
-
 };
 
 // The trees as the device walks them.  A look-up waits for every node on its
@@ -318,10 +323,19 @@ struct Compiled {
   }
 };
 
-// fn(k) for k = 0 .. n - 1 on up to 16 threads, the caller's among them; false
-// if a call returned false or threw.
+// Threads for work of about `ns` nanoseconds on one.  Starting a thread takes
+// the caller 50 us, so k threads finish after ns / k + 50 us (k - 1).  (8 elements
+// in 16^3 blocks: 780 us with 15 threads started, 37 with none.)
+int threads_for(double ns) {
+  const double k = std::sqrt(ns / 50e3);
+  if (k < 2) return 1;
+  return (int)std::min<double>(k, std::min(16u, std::max(1u, std::thread::hardware_concurrency())));
+}
+
+// fn(k) for k = 0 .. n - 1 on up to `n_threads` threads, the caller's among them;
+// false if a call returned false or threw.
 template <class Fn>
-bool parallel_for(int n, Fn fn) {
+bool parallel_for(int n, int n_threads, Fn fn) {
   std::atomic<int> next{0};
   std::atomic<bool> ok{true};
   auto work = [&]() {
@@ -333,7 +347,7 @@ bool parallel_for(int n, Fn fn) {
     }
   };
   std::vector<std::thread> threads;
-  const int extra = std::min<int>({n, 16, (int)std::max(1u, std::thread::hardware_concurrency())}) - 1;
+  const int extra = std::min(n, n_threads) - 1;
   try {
     for (int t = 0; t < extra; ++t) threads.emplace_back(work);
   } catch (...) {   // fewer threads than wanted
@@ -363,8 +377,9 @@ struct ForestBuilder : TreeBuilder {
 
   // The forest by layers of blocks: each element is painted over the blocks it
   // meets, a block that one element meets names it, and the others get their
-  // trees.  Layers are independent and run on several threads; their nodes
-  // follow one another in layer order.  Gives the trees of region(), and false
+  // trees.  Layers (runs of consecutive blocks) are independent and run on
+  // several threads where the work is worth their start; their nodes follow one
+  // another in the blocks' order, however many layers there are.  Gives the trees of region(), and false
   // wherever a block meets no element or a tree fails: region() then decides
   // (it accepts some meshes with gaps, and names the error).  Also false, before
   // anything is painted, where the boxes' volumes add up to more than the cube's
@@ -373,8 +388,8 @@ struct ForestBuilder : TreeBuilder {
   // (8,000 boxes that all cover the cube, 64^3 blocks: 1 ms; painted, 4.4 s and
   // 1.2 GB), and what layers() keeps stays within 64 MB and 64 bytes a block and
   // element.  (1,000 sheets across 64^3 blocks are 4.4 M meetings, 16 a block.)
-  // 174,000 elements in 64^3 blocks (no trees): 19.3 ms by region(), 2.7 ms so;
-  // 388,016 elements and 562,882 nodes: 145 and 18 ms.
+  // The whole call, 174,000 elements in 64^3 blocks (no trees): 18.8 ms by region(),
+  // 1.9 ms so; 388,016 elements and 562,882 nodes: 144 and 11.3 ms.
   bool layers() {
     const int64_t N = v->n_elem;
     struct Range {
@@ -387,7 +402,7 @@ struct ForestBuilder : TreeBuilder {
       double volume = 0, visits = 0;   // of the boxes; blocks that their elements meet
     };
     std::vector<Sums> sums(n_parts);
-    if (!parallel_for(n_parts, [&](int k) {
+    if (!parallel_for(n_parts, threads_for(10. * N), [&](int k) {
           for (int64_t e = k * part; e < std::min(N, (k + 1) * part); ++e) {
             const double *b = box((int32_t)e);
             double volume = 1, visits = 1;
@@ -411,28 +426,38 @@ struct ForestBuilder : TreeBuilder {
     // a partition's volumes add up to 1, rounded five times each and once a sum (2^-53 relative)
     if (all.volume > 1 + (N + 8) * 0x1p-52 || all.visits > 0x1p24 + 16. * ((double)N + (double)depth.size()))
       return false;
-    const int n_slabs = std::min(B[2], 64), thick = B[2] / n_slabs;   // powers of two
+    // about: 1 ns a block, 1.5 a meeting, and 400 (or 100, by midpoints) for an element in a tree
+    const int64_t n_blocks = (int64_t)depth.size(), plane = (int64_t)B[0] * B[1];
+    const int n_threads = threads_for(1. * n_blocks + 1.5 * all.visits +
+                                      std::max(0., all.visits - (double)n_blocks) * (midpoint ? 100. : 400.));
+    const int n_slabs = n_threads == 1 ? 1 : (int)std::min<int64_t>(n_blocks, 4 * n_threads);
     std::vector<Compiled> slab(n_slabs);
     std::vector<int64_t> slab_nodes(n_slabs, 0);                      // of the trees as built
     std::vector<std::vector<int64_t>> slab_trees(n_slabs);            // blocks with a tree, as offsets into `depth`
-    const size_t plane = (size_t)B[0] * B[1];
     auto at = [&](int64_t q) { return head_at((int)(q % B[0]), (int)(q / B[0] % B[1]), (int)(q / plane)); };
-    if (!parallel_for(n_slabs, [&](int s) {
-          const int z0 = s * thick, z1 = z0 + thick;
-          auto paint = [&](auto block) {   // block(element, offset into depth) for every block of the slab it meets
+    if (!parallel_for(n_slabs, n_threads, [&](int s) {
+          const int64_t q0 = n_blocks * s / n_slabs, q1 = n_blocks * (s + 1) / n_slabs;
+          const int64_t r0 = q0 / B[0], r1 = (q1 - 1) / B[0] + 1;        // its rows of blocks along x
+          const int z0 = (int)(q0 / plane), z1 = (int)((q1 - 1) / plane) + 1;
+          auto paint = [&](auto block) {   // block(element, offset into depth, into head) for every block of the slab it meets
             for (int64_t e = 0; e < N; ++e) {
               const Range &r = range[e];
-              for (int z = std::max<int>(z0, r.lo[2]); z < std::min<int>(z1, r.hi[2]); ++z)
-                for (int y = r.lo[1]; y < r.hi[1]; ++y)
-                  for (int x = r.lo[0]; x < r.hi[0]; ++x) block((int32_t)e, ((int64_t)z * B[1] + y) * B[0] + x);
+              for (int z = std::max<int>(z0, r.lo[2]); z < std::min<int>(z1, r.hi[2]); ++z) {
+                const int64_t row = (int64_t)z * B[1], y1 = std::min<int64_t>(r.hi[1], r1 - row);
+                for (int64_t y = std::max<int64_t>(r.lo[1], r0 - row); y < y1; ++y) {
+                  const int64_t q = (row + y) * B[0], h = (int64_t)head_at(0, (int)y, z);
+                  const int64_t x1 = std::min<int64_t>(r.hi[0], q1 - q);
+                  for (int64_t x = std::max<int64_t>(r.lo[0], q0 - q); x < x1; ++x) block((int32_t)e, q + x, h + x);
+                }
+              }
             }
           };
-          paint([&](int32_t e, int64_t q) {   // depth counts the elements here
-            if (depth[q]++ == 0) head[at(q)] = kLeaf | (uint32_t)e;
+          paint([&](int32_t e, int64_t q, int64_t h) {   // depth counts the elements here
+            if (depth[q]++ == 0) head[h] = kLeaf | (uint32_t)e;
           });
           std::vector<int64_t> &trees = slab_trees[s];
           std::vector<size_t> off(1, 0);
-          for (int64_t q = z0 * (int64_t)plane; q < z1 * (int64_t)plane; ++q) {
+          for (int64_t q = q0; q < q1; ++q) {
             if (depth[q] == 0) return false;
             if (depth[q] == 1) {
               depth[q] = 0;
@@ -445,8 +470,8 @@ struct ForestBuilder : TreeBuilder {
           if (trees.empty()) return true;
           std::vector<int32_t> els(off.back());
           std::vector<size_t> cur(off.begin(), off.end() - 1);
-          paint([&](int32_t e, int64_t q) {
-            if (depth[q] > 0) els[cur[head[at(q)]]++] = e;
+          paint([&](int32_t e, int64_t q, int64_t h) {
+            if (depth[q] > 0) els[cur[head[h]]++] = e;
           });
           TreeBuilder tb;
           tb.v = v;
@@ -460,9 +485,8 @@ struct ForestBuilder : TreeBuilder {
               lo[a] = (double)b[a] / B[a];
               hi[a] = (double)(b[a] + 1) / B[a];
             }
-            std::vector<int32_t> mine(els.begin() + off[k], els.begin() + off[k + 1]);
             int maxd = 0;
-            const uint32_t r = tb.build(mine, lo, hi, 0, &maxd);
+            const uint32_t r = tb.build(&els[off[k]], off[k + 1] - off[k], lo, hi, &maxd);
             if (r == kNone) return false;
             slab_nodes[s] += (int64_t)tb.nodes.size();
             if (slab[s].nodes.size() + tb.nodes.size() >= kGridRef || slab[s].grids.size() >= kGridRef / 2) return false;
@@ -539,7 +563,7 @@ struct ForestBuilder : TreeBuilder {
         hi[a] = (double)b1[a] / B[a];
       }
       int maxd = 0;
-      uint32_t r = build(els, lo, hi, 0, &maxd);
+      uint32_t r = build(els.data(), els.size(), lo, hi, &maxd);
       if (r == kNone) return false;
       head[head_at(b0[0], b0[1], b0[2])] = r;
       depth[((size_t)b0[2] * B[1] + b0[1]) * B[0] + b0[0]] = maxd;
@@ -604,7 +628,7 @@ ForestView forest_view(const lrvol_s *v) {
   f.head = v->d_head;
   f.nodes = v->d_nodes;
   f.n_nodes = (uint32_t)v->n_nodes;
-  f.grids = reinterpret_cast<const float4 *>(v->d_grids);
+  f.grids = reinterpret_cast<const float4 *>(v->d_nodes + v->n_nodes);
   f.n_grid_units = (uint32_t)v->n_grid_units;
   f.head_sy = (uint32_t)v->blocks[0] + 1;
   f.head_sz = f.head_sy * ((uint32_t)v->blocks[1] + 1);
@@ -832,11 +856,11 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
     if (h == kNone) return fail(LRVOL_ERR_ARG, "a forest block holds no element");
   if (fb.nodes.size() >= kLeaf) return fail(LRVOL_ERR_ARG, "forest too large");
   // depth statistics over blocks
-  double s = 0, s2 = 0;
+  int64_t s = 0, s2 = 0;
   int dmin = INT32_MAX, dmax = 0;
   for (int32_t d : fb.depth) {
     s += d;
-    s2 += (double)d * d;
+    s2 += (int64_t)d * d;
     dmin = std::min(dmin, d);
     dmax = std::max(dmax, d);
   }
@@ -846,16 +870,15 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   // the handle has none (a failed host build above left the previous one)
   v->have_accel = false;
   if ((rc = dev_alloc(v, &v->d_head, fb.head.size(), "alloc forest head")) ||
-      (rc = dev_alloc(v, &v->d_nodes, fb.nodes.size(), "alloc forest nodes")) ||
-      (rc = dev_alloc(v, &v->d_grids, fb.grids.size(), "alloc forest grids")))
+      (rc = dev_alloc(v, &v->d_nodes, fb.nodes.size() + fb.grids.size(), "alloc forest nodes")))
     return rc;
   CU(cudaMemcpyAsync(v->d_head, fb.head.data(), sizeof(uint32_t) * fb.head.size(), cudaMemcpyHostToDevice, st), "upload head");
   if (!fb.nodes.empty())
     CU(cudaMemcpyAsync(v->d_nodes, fb.nodes.data(), sizeof(Node) * fb.nodes.size(), cudaMemcpyHostToDevice, st),
        "upload nodes");
   if (!fb.grids.empty())
-    CU(cudaMemcpyAsync(v->d_grids, fb.grids.data(), sizeof(GridUnit) * fb.grids.size(), cudaMemcpyHostToDevice, st),
-       "upload grids");
+    CU(cudaMemcpyAsync(v->d_nodes + fb.nodes.size(), fb.grids.data(), sizeof(GridUnit) * fb.grids.size(),
+                       cudaMemcpyHostToDevice, st), "upload grids");
   CU(cudaStreamSynchronize(st), "build_accel sync");  // host vectors go out of scope
   v->n_tree_nodes = fb.n_tree_nodes;
   v->n_nodes = (int64_t)fb.nodes.size();
@@ -863,8 +886,8 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   for (int a = 0; a < 3; ++a) v->blocks[a] = blocks[a];
   v->depth_min = dmin;
   v->depth_max = dmax;
-  v->depth_mean = s / (double)nblk;
-  v->depth_var = std::max(0.0, s2 / (double)nblk - v->depth_mean * v->depth_mean);
+  v->depth_mean = (double)s / (double)nblk;
+  v->depth_var = std::max(0.0, (double)s2 / (double)nblk - v->depth_mean * v->depth_mean);
   v->have_accel = true;
   return LRVOL_OK;
 }
@@ -1258,7 +1281,7 @@ void lrvol_destroy(lrvol_t v) {
   if (!v) return;
   cudaDeviceSynchronize();
   void *ptrs[] = {v->d_box,   v->d_knots, v->d_coef,  v->d_weight, v->d_inc_ptr,  v->d_inc_idx, v->d_bez64,
-                  v->d_bez,   v->d_bezc,  v->d_elem,  v->d_head,  v->d_nodes, v->d_grids, v->d_counters, v->d_status,
+                  v->d_bez,   v->d_bezc,  v->d_elem,  v->d_head,  v->d_nodes, v->d_counters, v->d_status,
                   v->d_range};
   for (void *p : ptrs)
     if (p) cudaFree(p);

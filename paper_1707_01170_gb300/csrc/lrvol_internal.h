@@ -175,8 +175,7 @@ struct lrvol_s {
   bool have_bezier = false;
   // forest
   uint32_t *d_head = nullptr;
-  uint4 *d_nodes = nullptr;
-  lrvol::GridUnit *d_grids = nullptr;
+  uint4 *d_nodes = nullptr;   // the nodes, then the units of the grids
   int64_t n_nodes = 0, n_grid_units = 0;
   int64_t n_tree_nodes = 0;   // of the trees as built, before subtrees became grids
   int blocks[3] = {0, 0, 0};

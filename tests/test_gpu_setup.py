@@ -107,6 +107,22 @@ def test_overlapping_boxes_are_refused_at_once(name, lo, hi, n):
     gv.close()
 
 
+def test_small_forests_start_no_threads():
+    """Starting the threads of a large mesh takes ten times as long as a small mesh's forest."""
+    gv = lv.Volume(V.tensor_product((1, 1, 1), (2, 2, 2)))
+
+    def best(blocks):
+        t = []
+        for _ in range(30):
+            t0 = time.perf_counter()
+            gv.build_accel(blocks)
+            t.append(time.perf_counter() - t0)
+        return min(t)
+    one, many = best((1, 1, 1)), best((16, 16, 16))
+    gv.close()
+    assert many < 4 * one
+
+
 @pytest.mark.parametrize("name", list(VOLS))
 def test_blocks_and_incidence(name):
     vol = VOLS[name]()
