@@ -892,46 +892,77 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
   return LRVOL_OK;
 }
 
+// Pairs of an element and a B-spline up to which lrvol_to_bezier's incidence goes
+// pair by pair, and up to which its lists get room for every pair (2^17 integers,
+// 512 KB: larger allocations cost more than the wait for the lists' size).
+constexpr int64_t kDirectPairs = (int64_t)1 << 20, kRoomPairs = (int64_t)1 << 17;
+
 int lrvol_to_bezier(lrvol_t v, int32_t storage, void *stream) {
   if (!v) return fail(LRVOL_ERR_ARG, "null handle");
   if (storage != LRVOL_STORE_F32 && storage != LRVOL_STORE_F16 && storage != LRVOL_STORE_BF16)
     return fail(LRVOL_ERR_ARG, "bad storage");
   cudaStream_t st = (cudaStream_t)stream;
   int rc;
+  // Small volumes go pair by pair of an element and a B-spline: the buckets' scratch
+  // and launches take longer (a volume made, with its forest, converted and closed:
+  // 8 trilinear elements 251 us through the buckets, 135 so; 512 tricubic ones 384 and
+  // 316).  With few pairs the lists get room for all of them and nothing waits for
+  // their size.
+  const bool direct = v->n_basis <= kDirectPairs / v->n_elem, room = v->n_basis <= kRoomPairs / v->n_elem;
+  int64_t size[2] = {0, 0};   // entries of all lists, whether one is empty
   Incidence inc;
   DeviceBuffer scratch, unsorted;
-  if ((rc = scratch.alloc(inc.plan(v->n_elem), "alloc incidence scratch"))) return rc;
-  CU(inc.count(v, scratch.p, st), "incidence count kernels");
-  int64_t entries = 0;
-  uint32_t empty = 0;
-  CU(cudaMemcpyAsync(&entries, inc.ptr() + v->n_elem, sizeof entries, cudaMemcpyDeviceToHost, st), "read incidence size");
-  CU(cudaMemcpyAsync(&empty, inc.empty(), sizeof empty, cudaMemcpyDeviceToHost, st), "read incidence check");
-  CU(cudaStreamSynchronize(st), "incidence sync");
-  if (empty) return fail(LRVOL_ERR_ARG, "an element lies in no B-spline support");
-  if ((rc = unsorted.alloc(4 * entries, "alloc incidence lists"))) return rc;
+  if (!direct) {
+    if ((rc = scratch.alloc(inc.plan(v->n_elem), "alloc incidence scratch"))) return rc;
+    CU(inc.count(v, scratch.p, st), "incidence count kernels");
+    uint32_t empty = 0;
+    CU(cudaMemcpyAsync(size, inc.ptr() + v->n_elem, sizeof size[0], cudaMemcpyDeviceToHost, st), "read incidence size");
+    CU(cudaMemcpyAsync(&empty, inc.empty(), sizeof empty, cudaMemcpyDeviceToHost, st), "read incidence check");
+    CU(cudaStreamSynchronize(st), "incidence sync");
+    if (empty) return fail(LRVOL_ERR_ARG, "an element lies in no B-spline support");
+    if ((rc = unsorted.alloc(4 * size[0], "alloc incidence lists"))) return rc;
+  }
   const int n0 = v->p[0] + 1, n1 = v->p[1] + 1, n2 = v->p[2] + 1, nb = n0 * n1 * n2;
   v->have_bezier = false;   // the blocks are replaced: none until the new ones are complete
   v->storage = storage;
   v->elem_bytes = elem_bytes(storage, render_slots(v->nc, n0, n1, n2));
   v->elemc_bytes = v->nc == 3 ? elem_bytes(storage, 3 * roundup8(nb)) : 0;
-  if ((rc = dev_alloc(v, &v->d_inc_ptr, (size_t)v->n_elem + 1, "alloc incidence ptr")) ||
-      (rc = dev_alloc(v, &v->d_inc_idx, (size_t)entries, "alloc incidence")) ||
+  if ((rc = dev_alloc(v, &v->d_inc_ptr, (size_t)v->n_elem + 2, "alloc incidence ptr"))) return rc;
+  if (direct) {
+    CU(launch_incidence_direct(v, false, st), "incidence count kernels");
+    if (!room) {
+      CU(cudaMemcpyAsync(size, v->d_inc_ptr + v->n_elem, sizeof size, cudaMemcpyDeviceToHost, st), "read incidence size");
+      CU(cudaStreamSynchronize(st), "incidence sync");
+    }
+  }
+  // the lists, and behind them what k_to_bezier needs besides (the buckets' scratch has that)
+  const int64_t entries = room ? v->n_elem * v->n_basis : size[0];
+  if ((rc = dev_alloc(v, &v->d_inc_idx, (size_t)(entries + (direct ? v->n_elem + 1 : 0)), "alloc incidence")) ||
       (rc = dev_alloc(v, &v->d_bez64, (size_t)v->n_elem * v->nc * nb, "alloc bezier64")) ||
       (rc = dev_alloc(v, &v->d_bez, (size_t)v->n_elem * v->elem_bytes, "alloc render blocks")) ||
       (v->nc == 3 && (rc = dev_alloc(v, &v->d_bezc, (size_t)v->n_elem * v->elemc_bytes, "alloc render copy"))) ||
       (rc = dev_alloc(v, &v->d_elem, (size_t)v->n_elem, "alloc element records")) ||
       (rc = dev_alloc(v, &v->d_range, (size_t)v->n_elem * v->nc, "alloc coefficient ranges")))
     return rc;
-  CU(cudaMemcpyAsync(v->d_inc_ptr, inc.ptr(), sizeof(int64_t) * (v->n_elem + 1), cudaMemcpyDeviceToDevice, st),
-     "keep incidence ptr");
-  CU(inc.fill(v, reinterpret_cast<int32_t *>(unsorted.p), v->d_inc_idx, st), "incidence list kernels");
+  int32_t *todo = direct ? v->d_inc_idx + entries : inc.cell_of();
+  uint32_t *n_todo = direct ? reinterpret_cast<uint32_t *>(todo + v->n_elem) : inc.empty();
+  if (direct) {
+    CU(launch_incidence_direct(v, true, st), "incidence list kernels");
+  } else {
+    CU(cudaMemcpyAsync(v->d_inc_ptr, inc.ptr(), sizeof(int64_t) * (v->n_elem + 1), cudaMemcpyDeviceToDevice, st),
+       "keep incidence ptr");
+    CU(inc.fill(v, reinterpret_cast<int32_t *>(unsorted.p), v->d_inc_idx, st), "incidence list kernels");
+  }
   CU(cudaMemsetAsync(v->d_bez, 0, (size_t)v->n_elem * v->elem_bytes, st), "clear render blocks");
   if (v->d_bezc) CU(cudaMemsetAsync(v->d_bezc, 0, (size_t)v->n_elem * v->elemc_bytes, st), "clear render copy");
-  CU(launch_to_bezier(v, inc.cell_of(), inc.empty(), st), "to_bezier kernels");   // their scratch: no longer needed there
+  CU(launch_to_bezier(v, todo, n_todo, st), "to_bezier kernels");
   CU(launch_pack(v, st), "pack kernel");
   CU(launch_elem_records(v, st), "element record kernel");
+  if (room)
+    CU(cudaMemcpyAsync(size, v->d_inc_ptr + v->n_elem, sizeof size, cudaMemcpyDeviceToHost, st), "read incidence size");
   CU(cudaStreamSynchronize(st), "to_bezier sync");  // the scratch goes out of scope
-  v->inc_entries = entries;
+  if (size[1]) return fail(LRVOL_ERR_ARG, "an element lies in no B-spline support");
+  v->inc_entries = size[0];
   v->have_bezier = true;
   return LRVOL_OK;
 }

@@ -216,6 +216,9 @@ struct Incidence {
   uint32_t *counts() const { return at<uint32_t>(o_count); }
   uint32_t *empty() const { return at<uint32_t>(o_empty); }
 };
+// The same pair by pair, without scratch: the offsets into v->d_inc_ptr (n_elem + 2
+// entries, in the last whether a list is empty), then with `fill` the lists.
+cudaError_t launch_incidence_direct(const lrvol_s *v, bool fill, cudaStream_t s);
 // todo, n_todo: scratch for n_elem entries and one counter
 cudaError_t launch_to_bezier(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, cudaStream_t s);
 cudaError_t launch_pack(const lrvol_s *v, cudaStream_t s);

@@ -1,6 +1,6 @@
 // liblrvol set-up kernels for sm_103a: what lrvol_to_bezier does once per volume.
 //
-//   k_cell_*, k_incident, k_sort_lists, k_scan_*
+//   k_cell_*, k_incident, k_sort_lists, k_scan_*, k_incident_direct, k_incident_small
 //                  element -> B-spline incidence: the B-splines whose support
 //                  contains the element, in ascending order.
 //   k_to_bezier    Sec. 3.2.3 change of basis, FP64: per element, the Bernstein
@@ -198,6 +198,115 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_add(int64_t *__restrict__
                                                            const int64_t *__restrict__ sums) {
   const int64_t q0 = (int64_t)blockIdx.x * kScanTile, add = sums[blockIdx.x];
   for (int64_t q = q0 + threadIdx.x; q < min(n, q0 + kScanTile); q += kScanThreads) out[q] += add;
+}
+
+// The B-splines over element e out of all of them, by a warp: their number, and
+// with FILL their indices from list[0] on, in ascending order.
+template <bool FILL>
+__device__ __forceinline__ int64_t pairs_of_element(const double *__restrict__ box, int64_t e,
+                                                    const double *__restrict__ knots, int64_t n_basis, int p0, int p1,
+                                                    int p2, int kw, int32_t *__restrict__ list) {
+  const int lane = threadIdx.x & 31, off[3] = {0, p0 + 2, p0 + p1 + 4}, deg[3] = {p0, p1, p2};
+  int64_t lo[3], hi[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = order_key_01(box[6 * e + a]);
+    hi[a] = order_key_01(box[6 * e + 3 + a]);
+  }
+  constexpr int U = 4;   // B-splines a lane has under way
+  int64_t n = 0;
+  for (int64_t i0 = 0; i0 < n_basis; i0 += 32 * U) {
+    bool in[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t i = i0 + 32 * u + lane;
+      const double *k = knots + min(i, n_basis - 1) * kw;
+      in[u] = i < n_basis;
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        in[u] &= order_key(__ldg(k + off[a])) <= lo[a] && hi[a] <= order_key(__ldg(k + off[a] + deg[a] + 1));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const unsigned m = __ballot_sync(0xffffffffu, in[u]);
+      if constexpr (FILL) {
+        if (in[u]) list[n + __popc(m & ((1u << lane) - 1u))] = (int32_t)(i0 + 32 * u + lane);
+      }
+      n += __popc(m);
+    }
+  }
+  return n;
+}
+
+// Incidence of a small volume, a warp an element.  FILL false: ptr[e] = the
+// length of e's list; FILL true: the lists from ptr[e] on.
+template <bool FILL>
+__global__ void __launch_bounds__(32 * kSetupWarps) k_incident_direct(const double *__restrict__ box, int64_t n_elem,
+                                                                     const double *__restrict__ knots, int64_t n_basis,
+                                                                     int p0, int p1, int p2, int kw,
+                                                                     int64_t *__restrict__ ptr, int32_t *__restrict__ list) {
+  const int64_t e = (int64_t)blockIdx.x * kSetupWarps + (threadIdx.x >> 5);
+  if (e >= n_elem) return;
+  const int64_t n = pairs_of_element<FILL>(box, e, knots, n_basis, p0, p1, p2, kw, FILL ? list + ptr[e] : nullptr);
+  if (!FILL && (threadIdx.x & 31) == 0) ptr[e] = n;
+}
+
+// ptr: lengths to offsets in place, the total in ptr[n] and in ptr[n + 1]
+// whether a length is 0.  One CTA.
+__global__ void __launch_bounds__(kScanThreads) k_scan_direct(int64_t *__restrict__ ptr, int64_t n) {
+  int64_t carry = 0;
+  int empty = 0;
+  for (int64_t base = 0; base < n; base += kScanThreads) {
+    const int64_t q = base + threadIdx.x, v = q < n ? ptr[q] : 0;
+    int64_t total;
+    const int64_t at = cta_exclusive(v, total);
+    empty |= q < n && v == 0;
+    if (q < n) ptr[q] = carry + at;
+    carry += total;
+  }
+  empty = __syncthreads_or(empty);
+  if (threadIdx.x == 0) {
+    ptr[n] = carry;
+    ptr[n + 1] = empty;
+  }
+}
+
+// The same three steps in one CTA, for at most kSmallElems elements.
+constexpr int kSmallElems = 64;
+
+__global__ void __launch_bounds__(1024) k_incident_small(const double *__restrict__ box, int n_elem,
+                                                         const double *__restrict__ knots, int n_basis, int p0, int p1,
+                                                         int p2, int kw, int64_t *__restrict__ ptr,
+                                                         int32_t *__restrict__ list) {
+  __shared__ int at[kSmallElems];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int e = w; e < n_elem; e += 32) {
+    const int n = (int)pairs_of_element<false>(box, e, knots, n_basis, p0, p1, p2, kw, nullptr);
+    if (lane == 0) at[e] = n;
+  }
+  __syncthreads();
+  if (w == 0) {
+    int before = 0;
+    bool empty = false;
+    for (int q = lane; q < kSmallElems; q += 32) {   // every lane takes both turns
+      const int v = q < n_elem ? at[q] : 0;
+      int inc = v;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
+      }
+      empty |= q < n_elem && v == 0;
+      if (q < n_elem) ptr[q] = at[q] = before + inc - v;
+      before += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    empty = __any_sync(0xffffffffu, empty);
+    if (lane == 0) {
+      ptr[n_elem] = before;
+      ptr[n_elem + 1] = empty;
+    }
+  }
+  __syncthreads();
+  for (int e = w; e < n_elem; e += 32) pairs_of_element<true>(box, e, knots, n_basis, p0, p1, p2, kw, list + at[e]);
 }
 
 cudaError_t exclusive_scan(const uint32_t *count, int64_t n, int64_t *out, int64_t *sums, uint32_t *empty,
@@ -630,6 +739,27 @@ cudaError_t Incidence::fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, 
   return cudaGetLastError();
 }
 
+// Pair by pair: one CTA's kernel while a warp has one or two elements and a load
+// round for each, then a warp an element over the GPU, counted (fill false) and filled.
+bool incidence_small(const lrvol_s *v) { return v->n_elem <= kSmallElems && v->n_basis <= 8192 / v->n_elem; }
+
+cudaError_t launch_incidence_direct(const lrvol_s *v, bool fill, cudaStream_t s) {
+  const unsigned blocks = (unsigned)((v->n_elem + kSetupWarps - 1) / kSetupWarps);
+  if (fill) {
+    if (incidence_small(v))
+      k_incident_small<<<1, 1024, 0, s>>>(v->d_box, (int)v->n_elem, v->d_knots, (int)v->n_basis, v->p[0], v->p[1],
+                                          v->p[2], v->kw, v->d_inc_ptr, v->d_inc_idx);
+    else
+      k_incident_direct<true><<<blocks, 32 * kSetupWarps, 0, s>>>(v->d_box, v->n_elem, v->d_knots, v->n_basis, v->p[0],
+                                                                 v->p[1], v->p[2], v->kw, v->d_inc_ptr, v->d_inc_idx);
+  } else if (!incidence_small(v)) {
+    k_incident_direct<false><<<blocks, 32 * kSetupWarps, 0, s>>>(v->d_box, v->n_elem, v->d_knots, v->n_basis, v->p[0],
+                                                                v->p[1], v->p[2], v->kw, v->d_inc_ptr, nullptr);
+    k_scan_direct<<<1, kScanThreads, 0, s>>>(v->d_inc_ptr, v->n_elem);
+  }
+  return cudaGetLastError();
+}
+
 template <int P, int NC>
 static void launch_shared(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, cudaStream_t s) {
   k_to_bezier_shared<P, NC><<<(unsigned)((v->n_elem + kBezWarps - 1) / kBezWarps), 32 * kBezWarps, 0, s>>>(
@@ -656,6 +786,7 @@ cudaError_t launch_to_bezier(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, 
       default: return cudaErrorInvalidValue;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (v->n_basis <= 32) return e;   // no list that the kernel leaves over
     blocks = std::min<int64_t>(blocks, 1216);   // usually nothing is left: a grid that strides over the list
   }
   k_to_bezier<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_box, v->d_knots, v->d_coef, v->d_weight, v->d_inc_ptr,

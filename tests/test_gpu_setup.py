@@ -137,6 +137,53 @@ def test_blocks_and_incidence(name):
     assert np.array_equal(got, again)
 
 
+@pytest.mark.parametrize("n", [1, 32, 33, 128, 129, 8192, 8193, 1 << 17, (1 << 17) + 1, 1 << 20])
+def test_incidence_at_the_edges_of_its_routes(n):
+    """One trilinear element among n B-splines, of which every third lies over it."""
+    knots = np.tile([0.0, 0.0, 1.0], (n, 3))
+    knots[np.arange(n) % 3 != 0, 4:6] = 0.25, 0.5      # in y up to 1/2
+    knots[np.arange(n) % 3 != 0, 3] = 0.0
+    rng = np.random.default_rng(n)
+    vol = LRVolume(deg=np.array([1, 1, 1]), elem_box=np.array([[0.0, 0, 0, 1, 1, 1]]), knots=knots, coef=rng.random((n, 1)),
+                   weight=np.ones(n), grid=np.array([1, 1, 1]))
+    gv = lv.Volume(vol).to_bezier()
+    got, entries = gv.get_bezier()[0, 0], gv.stats()["incidence_entries"]
+    gv.close()
+    want = np.zeros((2, 2, 2))
+    want[0, 0, 0] = math.fsum(vol.coef[::3, 0])
+    assert entries == (n + 2) // 3
+    assert np.abs(got - want).max() <= 2 * n * 2.0 ** -53 * want.max()     # a sum of n / 3 numbers, one after the other
+
+
+@pytest.mark.parametrize("n", [4, 5, 8, 10])
+def test_small_routes_refuse_an_element_without_a_spline(n):
+    """n^3 elements (every route) of which the last has no B-spline: refused, and again."""
+    vol = V.tensor_product((1, 1, 1), (n,) * 3)
+    vol.knots[:, :3] = np.minimum(vol.knots[:, :3], 1 - 1 / n)
+    gv = lv.Volume(vol)
+    for _ in range(2):
+        with pytest.raises(lv.LrvolError) as err:
+            gv.to_bezier()
+        assert err.value.status == lv.ERR_ARG
+        with pytest.raises(lv.LrvolError):
+            gv.get_bezier()
+    gv.close()
+
+
+def test_small_volumes_convert_without_the_buckets():
+    """The buckets' launches and waits double the time of a small volume's conversion (130 against 57 us)."""
+    def best(n):
+        gv = lv.Volume(V.tensor_product((1, 1, 1), (n,) * 3))
+        t = []
+        for _ in range(100):
+            t0 = time.perf_counter()
+            gv.to_bezier()
+            t.append(time.perf_counter() - t0)
+        gv.close()
+        return min(t)
+    assert best(2) < 0.7 * best(11)
+
+
 def test_more_knot_vectors_than_lanes():
     """One trilinear element under 40 B-splines that differ in x, and 3 x 50 on three axes."""
     for nx, ny, nz in ((40, 1, 1), (5, 5, 6), (1, 33, 2)):
