@@ -110,15 +110,44 @@ __global__ void __launch_bounds__(32 * kSetupWarps) k_incident(
   }
 }
 
-// out = the lists of `in` in ascending order: a warp per element, every entry
-// placed at the number of smaller ones (the entries are distinct).
+// out = the lists of `in` in ascending order (`in` is lost): a warp per element,
+// every entry placed at the number of smaller ones (the entries are distinct).
+// That is quadratic, and a list may hold every B-spline: past kSortLong entries
+// the warp sorts by one bit after the other instead (n_bits of them hold an
+// entry).  One element with 350,000 entries, the whole conversion: 0.24 s, 60 s
+// by counting.
+constexpr int64_t kSortLong = 4096;
+
 __global__ void __launch_bounds__(32 * kSetupWarps) k_sort_lists(const int64_t *__restrict__ ptr, int64_t n_elem,
-                                                                const int32_t *__restrict__ in,
-                                                                int32_t *__restrict__ out) {
+                                                                int n_bits, int32_t *in, int32_t *out) {
   const int64_t e = (int64_t)blockIdx.x * kSetupWarps + (threadIdx.x >> 5);
   if (e >= n_elem) return;
   const int lane = threadIdx.x & 31;
   const int64_t beg = ptr[e], end = ptr[e + 1];
+  if (end - beg > kSortLong) {
+    int32_t *from = in, *to = out;
+    for (int bit = 0; bit < (n_bits | 1); ++bit) {   // an odd number of passes ends in `out`
+      int64_t zeros = 0;
+      for (int64_t q = beg + lane; q < end; q += 32) zeros += !(from[q] >> bit & 1);
+      for (int o = 16; o > 0; o >>= 1) zeros += __shfl_xor_sync(0xffffffffu, zeros, o);
+      int64_t at[2] = {beg, beg + zeros};
+      int32_t next = beg + lane < end ? from[beg + lane] : 0;
+      for (int64_t q0 = beg; q0 < end; q0 += 32) {
+        const int32_t v = next;
+        if (q0 + 32 + lane < end) next = from[q0 + 32 + lane];
+        const bool valid = q0 + lane < end, one = v >> bit & 1;
+        const unsigned m1 = __ballot_sync(0xffffffffu, valid && one), m0 = __ballot_sync(0xffffffffu, valid && !one);
+        if (valid) to[(one ? at[1] : at[0]) + __popc((one ? m1 : m0) & ((1u << lane) - 1u))] = v;
+        at[0] += __popc(m0);
+        at[1] += __popc(m1);
+      }
+      __syncwarp();
+      int32_t *const t = from;
+      from = to;
+      to = t;
+    }
+    return;
+  }
   for (int64_t q0 = beg; q0 < end; q0 += 32) {
     const int32_t v = q0 + lane < end ? in[q0 + lane] : INT32_MAX;
     int rank = 0;
@@ -734,8 +763,10 @@ cudaError_t Incidence::fill(const lrvol_s *v, int32_t *unsorted, int32_t *list, 
   const unsigned wb = (unsigned)((v->n_basis + kSetupWarps - 1) / kSetupWarps);
   k_incident<true><<<wb, 32 * kSetupWarps, 0, s>>>(cell_ends(), n_elem, v->d_knots, v->n_basis, v->p[0], v->p[1],
                                                   v->p[2], v->kw, CellGrid{R}, cell_ptr(), cell_el(), counts(), ptr(), unsorted);
-  k_sort_lists<<<(unsigned)((n_elem + kSetupWarps - 1) / kSetupWarps), 32 * kSetupWarps, 0, s>>>(ptr(), n_elem, unsorted,
-                                                                                              list);
+  int n_bits = 1;
+  while (v->n_basis > (int64_t)1 << n_bits) ++n_bits;
+  k_sort_lists<<<(unsigned)((n_elem + kSetupWarps - 1) / kSetupWarps), 32 * kSetupWarps, 0, s>>>(ptr(), n_elem, n_bits,
+                                                                                              unsorted, list);
   return cudaGetLastError();
 }
 

@@ -155,6 +155,33 @@ def test_incidence_at_the_edges_of_its_routes(n):
     assert np.abs(got - want).max() <= 2 * n * 2.0 ** -53 * want.max()     # a sum of n / 3 numbers, one after the other
 
 
+@pytest.mark.parametrize("n", [12285, 12291, 150_000, 300_000])
+def test_long_lists_are_sorted(n):
+    """96 trilinear elements under n B-splines each third of which lies over all of them: lists of up to 4,095 and
+    4,097 entries, sorted by counting and by bits, and of 50,000 and 100,000, in much less than a second."""
+    tp = V.tensor_product((1, 1, 1), (4, 4, 6))
+    knots = np.tile([-1.0, 0.0, 1.0], (n, 3))
+    knots[np.arange(n) % 3 != 0, 3:6] = -3.0, -2.0, -1.0
+    rng = np.random.default_rng(n)
+    vol = LRVolume(deg=tp.deg, elem_box=tp.elem_box, knots=knots, coef=rng.random((n, 1)), weight=np.ones(n), grid=tp.grid)
+    gv = lv.Volume(vol)
+    t = time.perf_counter()
+    got = gv.to_bezier().get_bezier()
+    t = time.perf_counter() - t
+    entries = gv.stats()["incidence_entries"]
+    gv.close()
+    # over [0, 1]^3 every B-spline that counts is (1 - x)(1 - y)(1 - z): a corner's value, added in list order
+    lo, hi = tp.elem_box[:, :3], tp.elem_box[:, 3:]
+    x = np.stack([1 - lo, 1 - hi], 1)
+    corner = np.einsum("ei,ej,ek->ekji", x[:, :, 0], x[:, :, 1], x[:, :, 2])
+    want = math.fsum(vol.coef[::3, 0]) * corner[:, None]
+    assert entries == 96 * ((n + 2) // 3) and t < 0.5
+    assert np.abs(got - want).max() <= 2 * n * 2.0 ** -53 * want.max()
+    again = lv.Volume(vol).to_bezier()
+    assert np.array_equal(got, again.get_bezier())     # the order of the sums, and so the bits, do not change
+    again.close()
+
+
 @pytest.mark.parametrize("n", [4, 5, 8, 10])
 def test_small_routes_refuse_an_element_without_a_spline(n):
     """n^3 elements (every route) of which the last has no B-spline: refused, and again."""
