@@ -362,6 +362,7 @@ struct ForestBuilder : TreeBuilder {
   std::vector<GridUnit> grids;
   int64_t n_tree_nodes = 0;    // nodes of the trees before subtrees became grids
   std::vector<int32_t> depth;  // per block
+  LabelCost cost;              // from the boxes (layers())
   int B[3];
 
   size_t head_at(int x, int y, int z) const { return ((size_t)z * (B[1] + 1) + y) * (B[0] + 1) + x; }
@@ -400,19 +401,22 @@ struct ForestBuilder : TreeBuilder {
     const int n_parts = (int)((N + part - 1) / part);
     struct Sums {
       double volume = 0, visits = 0;   // of the boxes; blocks that their elements meet
+      double surface = 0, steps = 0;   // of the boxes; volume / smallest side
     };
     std::vector<Sums> sums(n_parts);
     if (!parallel_for(n_parts, threads_for(10. * N), [&](int k) {
           for (int64_t e = k * part; e < std::min(N, (k + 1) * part); ++e) {
             const double *b = box((int32_t)e);
-            double volume = 1, visits = 1;
+            double visits = 1, s[3];
             for (int a = 0; a < 3; ++a) {   // exact: B is a power of two
               range[e].lo[a] = (uint16_t)(int)(b[a] * B[a]);
               range[e].hi[a] = (uint16_t)(int)std::ceil(b[3 + a] * B[a]);
-              volume *= b[3 + a] - b[a];
+              s[a] = b[3 + a] - b[a];
               visits *= range[e].hi[a] - range[e].lo[a];
             }
-            sums[k].volume += volume;
+            sums[k].volume += s[0] * s[1] * s[2];
+            sums[k].surface += 2 * (s[0] * s[1] + s[1] * s[2] + s[0] * s[2]);
+            sums[k].steps += std::max({s[1] * s[2], s[0] * s[2], s[0] * s[1]});
             sums[k].visits += visits;
           }
           return true;
@@ -422,7 +426,11 @@ struct ForestBuilder : TreeBuilder {
     for (const Sums &k : sums) {
       all.volume += k.volume;
       all.visits += k.visits;
+      all.surface += k.surface;
+      all.steps += k.steps;
     }
+    cost.chord = 4 * all.volume / all.surface;   // a random line's mean chord of a convex body is 4 V / S
+    cost.ds = std::ldexp(all.volume / all.steps, -std::max({v->p[0], v->p[1], v->p[2]}));
     // a partition's volumes add up to 1, rounded five times each and once a sum (2^-53 relative)
     if (all.volume > 1 + (N + 8) * 0x1p-52 || all.visits > 0x1p24 + 16. * ((double)N + (double)depth.size()))
       return false;
@@ -880,6 +888,7 @@ int lrvol_build_accel_split(lrvol_t v, const int32_t blocks[3], int32_t split, v
     CU(cudaMemcpyAsync(v->d_nodes + fb.nodes.size(), fb.grids.data(), sizeof(GridUnit) * fb.grids.size(),
                        cudaMemcpyHostToDevice, st), "upload grids");
   CU(cudaStreamSynchronize(st), "build_accel sync");  // host vectors go out of scope
+  v->label_cost = fb.cost;
   v->n_tree_nodes = fb.n_tree_nodes;
   v->n_nodes = (int64_t)fb.nodes.size();
   v->n_grid_units = (int64_t)fb.grids.size();
@@ -1147,7 +1156,7 @@ int lrvol_labels(lrvol_t v, const lrvol_camera *cam, const lrvol_tf *tf, const l
   prm.counters = v->d_counters;
   prm.status = v->d_status;
   for (int q = 0; q < 256; ++q) prm.tf[q] = make_float4(tf->rgba[q][0], tf->rgba[q][1], tf->rgba[q][2], tf->rgba[q][3]);
-  CU(launch_labels(prm, v->p[0], (float)h_fine, (float)tau, cand, n_cand, label, (cudaStream_t)stream),
+  CU(launch_labels(prm, v->p[0], v->label_cost, (float)h_fine, (float)tau, cand, hc, n_cand, label, (cudaStream_t)stream),
      "labels kernel");
   return LRVOL_OK;
 }

@@ -12,6 +12,7 @@
 //   change of basis in setup.cu, look-up and evaluation at points in points.cu;
 //   the device helpers these files share are in device_common.cuh.)
 #include <algorithm>
+#include <cmath>
 
 #include "device_common.cuh"
 
@@ -466,6 +467,85 @@ __device__ __forceinline__ bool seg_left(const Ray &ray, const float4 &lo, const
          !(px >= lo.x && py >= lo.y && pz >= lo.z && px < hi.x && py < hi.y && pz < hi.z);
 }
 
+// Alg. 2 from transparent over [ta, tb) with samples ta + k*h (each in its element).
+template <int P>
+__device__ void seg_composite(const RenderParams &prm, const Ray &ray, const float4 *tfb, const float4 *tfd, float ta,
+                              float tb, float h, SegState &st, Block<P, 0, LRVOL_STORE_F32> &blk, float &C0, float &C1,
+                              float &C2, float &Tr) {
+  C0 = C1 = C2 = 0.f;
+  Tr = 1.f;
+  for (int k = 0; k < kMaxSamplesPerRay; ++k) {
+    const float t = __fmaf_rn((float)k, h, ta);
+    float4 src;
+    if (!(t < tb) || !seg_sample<P>(prm, ray, tfb, tfd, t, st, blk, src)) break;
+    const float tn = __fmaf_rn((float)(k + 1), h, ta);
+    const float T = ex2_approx(src.w * (__fsub_rn(fminf(tn, tb), t) * prm.inv_xi)), w = fmaf(-Tr, T, Tr);
+    C0 = fmaf(w, src.x, C0);
+    C1 = fmaf(w, src.y, C1);
+    C2 = fmaf(w, src.z, C2);
+    Tr *= T;
+  }
+}
+
+// One lane per ray, one march per composite, candidates until one fails: many
+// rays of few samples a visit (rule in launch_labels).
+template <int P>
+__global__ void __launch_bounds__(128) k_labels_lane(const __grid_constant__ RenderParams prm, float h_fine, float tau,
+                                                     const float *__restrict__ cand, int n_cand,
+                                                     int32_t *__restrict__ label) {
+  __shared__ float4 tfb[kTfEntries], tfd[kTfEntries];
+  load_tf(prm, tfb, tfd);
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int i = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
+  const int j = prm.row_begin + blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
+  if (i >= prm.width || j >= prm.row_end) return;
+  Ray ray;
+  if (!make_ray(prm.ray, i, j, ray)) return;
+  Block<P, 0, LRVOL_STORE_F32> blk;
+  SegState st;
+  st.e = kNone;
+  const float tr_stop = 1.f - prm.alpha_stop;
+  float Tfront = 1.f, t = ray.tin;
+  for (int visit = 0; visit < kMaxSamplesPerRay && t < ray.tout && Tfront > tr_stop; ++visit) {
+    // the visit: element of the heuristic sample at t, up to the first heuristic sample past it
+    if (!seg_locate<P>(prm, st, blk, fma_sat(t, ray.d[0], ray.o[0]), fma_sat(t, ray.d[1], ray.o[1]),
+                       fma_sat(t, ray.d[2], ray.o[2])))
+      return;
+    const uint32_t e = st.e;
+    const float4 lo = st.ra, hi = st.rb;
+    const float ds = lo.w;
+    float tb = t;
+    for (int q = 0; q < kMaxSamplesPerRay; ++q) {
+      tb = __fadd_rn(tb, ds);
+      if (seg_left(ray, lo, hi, tb)) break;
+    }
+    tb = fminf(tb, ray.tout);
+    float R0, R1, R2, RT;
+    seg_composite<P>(prm, ray, tfb, tfd, t, tb, h_fine, st, blk, R0, R1, R2, RT);
+    int best = 0;
+    for (int c = 1; c < n_cand; ++c) {
+      // the candidate's first sample outside e (or the ray's exit)
+      const float sc = __fmul_rn(ds, __ldg(cand + c));
+      float tc = t;
+      for (int k = 1; k < kMaxSamplesPerRay; ++k) {
+        tc = __fmaf_rn((float)k, sc, t);
+        if (seg_left(ray, lo, hi, tc)) break;
+      }
+      tc = fminf(tc, ray.tout);
+      float F0, F1, F2, FT, A0, A1, A2, AT;
+      seg_composite<P>(prm, ray, tfb, tfd, t, tc, h_fine, st, blk, F0, F1, F2, FT);
+      seg_composite<P>(prm, ray, tfb, tfd, t, tc, sc, st, blk, A0, A1, A2, AT);
+      const float err = Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
+      if (!(err <= tau)) break;
+      best = c;
+    }
+    atomicMin(label + e, best);
+    Tfront *= RT;
+    t = tb;
+  }
+}
+
 // One warp per ray.  A visit's fine samples are independent until they are
 // composited, so the lanes take 32 at a time: Alg. 2 over them is a prefix
 // product of transmittances and prefix sums of colours.  Lane 0's end is the
@@ -475,10 +555,10 @@ __device__ __forceinline__ bool seg_left(const Ray &ray, const float4 &lo, const
 // samples, a few each, are spread over the lanes as (candidate, sample) slots
 // and composited by the candidates' lanes.
 //
-// With a thread per ray and a fine march per candidate the kernel evaluated
-// the visit's fine samples up to seven times, with 12 of 32 lanes active and a
-// tail of long rays: 13.0 ms for a 320x180 camera of a 174,000-element tricubic
-// volume, 2.8 ms now.  Held to 128 registers for four CTAs an SM: with the 146 it
+// A lane per ray with a march per composite (k_labels_lane) evaluates the visit's
+// fine samples up to seven times, with 12 of 32 lanes active and a tail of long
+// rays: 12.0 ms for a 320x180 camera of a 174,000-element tricubic volume with
+// seven candidates, 2.8 ms here.  Held to 128 registers for four CTAs an SM: with the 146 it
 // would take, three fit and it is a fifth slower, and five CTAs spill.
 template <int P>
 __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
@@ -575,7 +655,11 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
     // fine composites over [t, te)
     float F0 = 0.f, F1 = 0.f, F2 = 0.f, FT = 1.f;
     bool need = lane < n_cand && t < te;
-    const float te_max = __uint_as_float(__reduce_max_sync(kAll, need ? __float_as_uint(te) : 0u));   // te >= 0
+    auto last_end = [&]() { return __uint_as_float(__reduce_max_sync(kAll, need ? __float_as_uint(te) : 0u)); };   // te >= 0
+    auto error = [&]() {
+      return Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
+    };
+    float te_max = last_end();
     // fine samples before te: a quotient, corrected with the samples' own places
     int nf = 0;
     if (need) {
@@ -584,7 +668,8 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
       while (nf < kMaxSamplesPerRay && __fmaf_rn((float)nf, h_fine, t) < te) ++nf;
     }
     float cT = 1.f, cC0 = 0.f, cC1 = 0.f, cC2 = 0.f;   // composite of the earlier chunks
-    for (int kb = 0; kb < kMaxSamplesPerRay && __any_sync(kAll, need); kb += 32) {
+    unsigned open_ends = __ballot_sync(kAll, need);
+    for (int kb = 0; kb < kMaxSamplesPerRay && open_ends; kb += 32) {
       const float ts = __fmaf_rn((float)(kb + lane), h_fine, t), tn = __fmaf_rn((float)(kb + lane + 1), h_fine, t);
       const bool act = ts < te_max;
       float4 src = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -624,9 +709,20 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
       cC0 += __shfl_sync(kAll, s0, 31);
       cC1 += __shfl_sync(kAll, s1, 31);
       cC2 += __shfl_sync(kAll, s2, 31);
+      const unsigned before_chunk = open_ends;
+      open_ends = __ballot_sync(kAll, need);
+      // candidates ended while others are open: the label is the one before the first
+      // that fails, so those behind a failed one need no end
+      if ((before_chunk & ~open_ends) > 1u && open_ends > 1u) {
+        const unsigned failed = __ballot_sync(kAll, is_cand && fin && !(error() <= tau));
+        if (failed) {
+          need &= lane < __ffs(failed);
+          te_max = last_end();
+          open_ends = __ballot_sync(kAll, need);
+        }
+      }
     }
-    const float err = Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
-    const unsigned bad = __ballot_sync(kAll, is_cand && !(err <= tau));
+    const unsigned bad = __ballot_sync(kAll, is_cand && !(error() <= tau));
     if (lane == 0) atomicMin(label + e, bad ? __ffs(bad) - 2 : n_cand - 1);
     Tfront *= __shfl_sync(kAll, FT, 0);
     t = tb;
@@ -677,15 +773,57 @@ cudaError_t launch_mlp_infer(const float *x, int64_t n, const uint16_t *packed, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_labels(const RenderParams &prm, int degree, float h_fine, float tau, const float *cand, int n_cand,
-                          int32_t *label, cudaStream_t s) {
-  // four rays a CTA, a 2x2 patch
-  const dim3 grid((unsigned)((prm.width + 1) / 2), (unsigned)((prm.row_end - prm.row_begin + 1) / 2));
-  switch (degree) {
-    case 1: k_labels<1><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-    case 2: k_labels<2><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-    case 3: k_labels<3><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-    default: return cudaErrorInvalidValue;
+// Whether a lane a ray is faster than a warp a ray.  A warp wastes lanes on a visit
+// of few samples, lanes need many rays to fill the GPU and march again for every
+// candidate.  Per ray and visit the lane's work is its samples (1 + 0.091 each), the
+// warp's a chunk of 32 fine samples up to the longest candidate's end and the steps of
+// the candidate with most samples (1 + 0.26 and 0.026 each); rays up to 2,500 (lanes)
+// and 85 (warps) per SM are hidden in one another's latency.  An element is crossed
+// in `chord` on average, its Eq. 4 step is ds, and a candidate passes the more often the
+// larger tau is.  The constants are a fit to 5,271 timings (seven volumes of degree 1 to
+// 3, 64x36 to 1280x720 rays, 1 to 16 candidates, h_fine 1/64 to 1/8192, tau 1e-5 to 1e-2),
+// in which the choice is within 5 % of the faster kernel for 97 % and 0.5 % on average.
+// 174,000 tricubic elements, lane / warp: 640x360 rays, one candidate, h_fine 1/256 0.49 /
+// 4.9 ms; 320x180, seven candidates, h_fine 1/2048 12.0 / 2.8 ms.
+static bool labels_by_lane(const LabelCost &cost, int64_t rays, int sms, double h_fine, double tau, const float *cand,
+                           int n_cand) {
+  const double pass = 1 / (1 + std::exp(-2.23 - 0.66 * std::log10(tau / 4e-4)));
+  double samples = cost.chord / h_fine, farthest = cost.chord, steps = 0, reached = 1;
+  for (int c = 1; c < n_cand; ++c) {
+    const double sc = cost.ds * cand[c], length = sc < cost.chord ? cost.chord + 0.5 * sc : sc;
+    reached *= pass;
+    samples += reached * (length / h_fine + length / sc);
+    farthest = std::max(farthest, length);
+    steps = std::max(steps, length / sc);
+  }
+  const double per_sm = (double)rays / sms;
+  return 1.29 * (1 + 0.091 * samples) * (1 + per_sm / 2540) <
+         1.05 * (1 + 0.257 * farthest / (32 * h_fine) + 0.0256 * steps) * (1 + per_sm / 85);
+}
+
+cudaError_t launch_labels(const RenderParams &prm, int degree, const LabelCost &cost, float h_fine, float tau,
+                          const float *cand, const float *cand_host, int n_cand, int32_t *label, cudaStream_t s) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int w = prm.width, h = prm.row_end - prm.row_begin;
+  if (labels_by_lane(cost, (int64_t)w * h, sms, h_fine, tau, cand_host, n_cand)) {
+    const dim3 grid((unsigned)((w + 15) / 16), (unsigned)((h + 7) / 8));
+    switch (degree) {
+      case 1: k_labels_lane<1><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
+      case 2: k_labels_lane<2><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
+      case 3: k_labels_lane<3><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
+      default: return cudaErrorInvalidValue;
+    }
+  } else {
+    const dim3 grid((unsigned)((w + 1) / 2), (unsigned)((h + 1) / 2));   // four rays a CTA, a 2x2 patch
+    switch (degree) {
+      case 1: k_labels<1><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
+      case 2: k_labels<2><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
+      case 3: k_labels<3><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
+      default: return cudaErrorInvalidValue;
+    }
   }
   return cudaGetLastError();
 }

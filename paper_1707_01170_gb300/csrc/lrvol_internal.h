@@ -72,6 +72,12 @@ struct ForestView {
   float fbx, fby, fbz;           // block counts (powers of two)
 };
 
+// What a ray meets on average: the length it crosses an element in and the Eq. 4
+// step there.
+struct LabelCost {
+  double chord = 1, ds = 1;
+};
+
 struct RayConsts {
   float E[3], F[3], R[3], U[3];
   float sxs, sxo, sys, syo;
@@ -158,6 +164,7 @@ struct lrvol_s {
   int64_t n_elem = 0, n_basis = 0;
   int kw = 0;  // knots per B-spline
   std::vector<double> box;  // element boxes (the forest is built on the host)
+  lrvol::LabelCost label_cost;
 
   // device copies of the spline
   double *d_box = nullptr, *d_knots = nullptr, *d_coef = nullptr, *d_weight = nullptr;
@@ -352,7 +359,8 @@ struct AdamStep {
 };
 cudaError_t launch_mlp_grad(const float *x, const float *target, int64_t n, float *p, float *grad, float *loss,
                             float *scratch, const AdamStep *adam, cudaStream_t s);
-cudaError_t launch_labels(const RenderParams &prm, int degree, float h_fine, float tau, const float *cand, int n_cand,
-                          int32_t *label, cudaStream_t s);
+// cand_host: the candidates on the host
+cudaError_t launch_labels(const RenderParams &prm, int degree, const LabelCost &cost, float h_fine, float tau,
+                          const float *cand, const float *cand_host, int n_cand, int32_t *label, cudaStream_t s);
 
 }  // namespace lrvol

@@ -2,6 +2,8 @@
 candidate samples than lanes; visits of fewer and of many more than 32 fine
 samples; images that are not a multiple of a CTA's 2x2 rays; every degree.
 
+Rays by lanes (many rays, few samples a visit) the same way.
+
 A label is the outcome of comparisons err <= tau, FP32 here and FP64 in the
 oracle, whose composites differ by about 1e-3 of tau: labels lie between the
 oracle's at tau (1 -+ 0.02), and 98 % of them (all of fewer than 50) are equal.
@@ -12,6 +14,7 @@ import pytest
 torch = pytest.importorskip("torch")
 
 from oracle.oracle import Oracle
+from paper_1707_01170_gb300 import learned as LS
 from paper_1707_01170_gb300 import lrvol as lv
 from paper_1707_01170_gb300.synth import volumes as V
 from paper_1707_01170_gb300.synth.lrgen import Stream
@@ -21,14 +24,12 @@ pytestmark = pytest.mark.gpu
 CANDS = {"one": (1.0,), "two": (1.0, 8.0), "sixteen": tuple(0.25 * k for k in range(1, 17)), "short": (0.02, 0.05, 1.0)}
 
 
-@pytest.mark.parametrize("cand", sorted(CANDS))
-@pytest.mark.parametrize("deg,h_fine", [(1, 1 / 64), (2, 1 / 512), (3, 1 / 2048)])
-def test_labels(deg, h_fine, cand):
+def _check(deg, h_fine, cand, size):
     vol = V.refined_ball((deg,) * 3, (3, 3, 3), centres=((0.45, 0.5, 0.55),), radii=(0.35,), seed=9)
     orc = Oracle(vol)
     tf = V.seeded_tf(Stream(31), alpha_max=0.05)
     tf.table = tf.table.astype(np.float32).astype(np.float64)
-    cam, tau = V.orbit_camera(Stream(32 + deg), 5, 3), 4e-4
+    cam, tau = V.orbit_camera(Stream(32 + deg), *size), 4e-4
     step = V.StepParams(mode="heuristic", xi=1 / 256, alpha_stop=0.97)
     gv = lv.Volume(vol).build_accel((4, 4, 4)).to_bezier()
     got = lv.labels(gv, cam, tf, step, h_fine, tau, CANDS[cand]).cpu().numpy()
@@ -38,3 +39,37 @@ def test_labels(deg, h_fine, cand):
     assert seen.sum() > 10 and np.array_equal(seen, got < len(CANDS[cand]))
     assert np.all((low <= got) & (got <= high))
     assert (got != want).sum() <= 0.02 * seen.sum()
+
+
+@pytest.mark.parametrize("cand", sorted(CANDS))
+@pytest.mark.parametrize("deg,h_fine", [(1, 1 / 64), (2, 1 / 512), (3, 1 / 2048)])
+def test_labels(deg, h_fine, cand):
+    _check(deg, h_fine, cand, (5, 3))
+
+
+@pytest.mark.parametrize("cand", ["one", "two"])
+@pytest.mark.parametrize("deg", [1, 2, 3])
+def test_labels_by_lanes(deg, cand):
+    """45,000 rays, an odd number a side, and six fine samples a visit: a lane a ray (ratio 0.4 to 0.7 of the rule's
+    limit on 152 SMs)."""
+    _check(deg, 1 / 40, cand, (301, 151))
+
+
+def test_coarse_labels_take_no_warp_a_ray():
+    """One candidate and a fine step of an element's size cost a fraction of seven candidates and 1/2048."""
+    gv = lv.Volume(V.tensor_product((3, 3, 3), (24, 24, 24))).build_accel((32, 32, 32)).to_bezier()
+    cam, tf = V.orbit_camera(Stream(5), 640, 360), V.seeded_tf(Stream(31), alpha_max=0.05)
+    step = V.StepParams(mode="heuristic", xi=1 / 256, alpha_stop=0.99)
+
+    def best(h_fine, cand):
+        t = []
+        for _ in range(4):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            lv.labels(gv, cam, tf, step, h_fine, 4e-4, cand)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+    assert best(1 / 32, (1.0,)) < 0.2 * best(1 / 2048, LS.CAND)
+    gv.close()
