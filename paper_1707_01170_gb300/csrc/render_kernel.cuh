@@ -294,24 +294,45 @@ cudaError_t launch_render_f(const RenderParams &prm, cudaStream_t s) {
 
 // Two samples a pass (PAIR) or one.  Two cost their instructions also where the
 // second lies in another element, one waits for an element's loads once a sample.
-// Few warps an SM leave that wait bare, so frames of up to 12 CTAs for each of
-// the 152 SMs (640x360) take two: 256x256 and 640x360 frames, one / two a pass,
-// Eq. 4 tricubic FP32 408 / 351 and 545 / 476 us, learned FP16 185 / 175 and 262 /
-// 242, fixed FP32 296 / 270 and 394 / 382, triquadratic speed FP16 342 / 318 and
-// 342 / 338, component FP16 480 / 402 and 441 / 403.  Larger frames pay for the
-// second (1080p: learned FP32 1675 / 1745 us, fixed 1813 / 2042, speed FP16 653 /
-// 690) except Eq. 4 steps of tricubic scalar volumes, where an element holds 5.5
-// samples (FP32 2744 / 2599, BF16 2483 / 2337, FP16 2107 / 2061).  Never: shaded
-// frames (515 / 532 at 256x256, 3920 / 4351 at 1080p), and scalar volumes of degree
-// 2 and 1, whose elements hold fewer samples and load less (182 / 180, 215 / 228
-// and 256 / 242 at 256x256, 512x288 and 640x360; 89 / 93 at 512x288).
-constexpr unsigned kPairCtas = 12 * 152;
+// Two / one a pass, time of the frame (a 174,000-element volume with scalar and
+// 3-vector blocks of degree 3, the 388,016-element flow of degree 2, and two small
+// volumes of degree 3 and 2 behind the comma; FP32, FP16 and BF16 blocks):
+//   Eq. 4, tricubic scalar      0.89..0.95 at 256x256, 0.95..1.00 at 960x540, 0.94..0.98
+//                               at 1080p, 0.91..1.04: always two
+//   other frames                one above 12 CTAs an SM (640x360): 1.04 (learned scalar),
+//                               1.06 (FP16 speed) at 1080p
+//   learned                     0.82..0.92 at 256x256, 0.78..0.94 at 640x360: two
+//   Eq. 4, 3-vectors            0.81..1.01 and 0.84..1.05, 0.85..1.06: two, but the speed of a
+//                               degree-2 volume that caches hold 1.03..1.12: one
+//   fixed, scalar or component  0.91..1.06 at 256x256; 0.96..1.16 at 640x360, BF16
+//                               0.89..1.03: two up to 4 CTAs an SM, BF16 12
+//   fixed, speed                0.99..1.14 at 256x256: one, but tricubic BF16 0.90..0.99
+// Never: shaded frames (1.03 at 256x256, 1.11 at 1080p), and scalar volumes of degree 2
+// and 1, whose elements hold fewer samples and load less (0.95..1.06).
+constexpr int64_t kPairBytes = (int64_t)16 << 20;
+
+template <int P, int FIELD, int STORE, bool FIXED>
+constexpr bool pairs_exist() {
+  if (FIXED && FIELD == 1) return P == 3 && STORE == LRVOL_STORE_BF16;
+  return (P == 3 || (P == 2 && FIELD != 0)) && FIELD != 3;
+}
+
+template <int P, int FIELD, int STORE, bool FIXED>
+bool take_pairs(const RenderParams &prm, int64_t ctas, int sms) {
+  if (P == 3 && FIELD == 0 && prm.mode == LRVOL_STEP_HEURISTIC) return true;
+  if (ctas > (FIXED && STORE != LRVOL_STORE_BF16 ? 4 : 12) * (int64_t)sms) return false;
+  return !(P == 2 && FIELD == 1 && prm.mode == LRVOL_STEP_HEURISTIC && prm.n_elem * Block<P, FIELD, STORE>::BYTES < kPairBytes);
+}
 
 template <int P, int FIELD, int STORE, bool FIXED, bool TREES, bool TRACE>
 cudaError_t launch_render_p(const RenderParams &prm, cudaStream_t s) {
-  if constexpr ((P == 3 || (P == 2 && FIELD != 0)) && FIELD != 3 && !TRACE) {
+  if constexpr (pairs_exist<P, FIELD, STORE, FIXED>() && !TRACE) {
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
     const dim3 grid = render_grid(prm);
-    if ((P == 3 && FIELD == 0 && prm.mode == LRVOL_STEP_HEURISTIC) || grid.x * grid.y <= kPairCtas)
+    if (take_pairs<P, FIELD, STORE, FIXED>(prm, (int64_t)grid.x * grid.y, sms))
       return launch_render_f<P, FIELD, STORE, FIXED, TREES, true, TRACE>(prm, s);
   }
   return launch_render_f<P, FIELD, STORE, FIXED, TREES, false, TRACE>(prm, s);
