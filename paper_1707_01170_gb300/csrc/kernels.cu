@@ -1179,7 +1179,8 @@ __device__ __forceinline__ void ff_add(float &hi, float &lo, float d) {
   lo = __fsub_rn(t, __fsub_rn(hi, s));
 }
 
-template <int P, int STORE>
+// TREES: the forest has trees; else a head word names the element.
+template <int P, int STORE, bool TREES>
 struct SLField {
   static constexpr int N = P + 1;
   float4 ra, rb, rc, rd;
@@ -1201,7 +1202,8 @@ struct SLField {
 
   __device__ __forceinline__ bool locate(const SLParams &sp, float px, float py, float pz) {
     if (cur != kNone && px >= ra.x && py >= ra.y && pz >= ra.z && px < rb.x && py < rb.y && pz < rb.z) return true;
-    const uint32_t e = forest_lookup(sp.forest, px, py, pz, sp.status);
+    const uint32_t e =
+        TREES ? forest_lookup(sp.forest, px, py, pz, sp.status) : forest_head(sp.forest, px, py, pz) & ~kLeaf;
     if (e >= (uint32_t)sp.n_elem) {   // kNone included
       set_status(sp.status, kStatusBounds);
       return false;
@@ -1214,12 +1216,12 @@ struct SLField {
 };
 
 // One streamline, seed q.
-template <int P, int STORE>
+template <int P, int STORE, bool TREES>
 __device__ __forceinline__ void trace_line(const SLParams &sp, const double *__restrict__ seeds, int64_t q,
                                            SLSample *__restrict__ out, int32_t *__restrict__ count,
                                            int32_t *__restrict__ status) {
   const SLTab &T = c_sl_tab[sp.method];
-  SLField<P, STORE> F;
+  SLField<P, STORE, TREES> F;
   F.cur = kNone;
   float xh[3], xl[3];
   for (int a = 0; a < 3; ++a) {
@@ -1374,17 +1376,24 @@ __device__ __forceinline__ void trace_line(const SLParams &sp, const double *__r
 // `lanes` lanes of each warp trace lines: with fewer lines than the GPU has
 // warp slots, one line per warp keeps a line from waiting on its warp-mates'
 // element look-ups (a line's steps are a sequential chain, so its latency is
-// what a small rake of seeds waits for).
-template <int P, int STORE>
-__global__ void __launch_bounds__(128) k_streamlines(const __grid_constant__ SLParams sp,
-                                                     const double *__restrict__ seeds, int64_t n, int lanes,
-                                                     SLSample *__restrict__ out, int32_t *__restrict__ count,
-                                                     int32_t *__restrict__ status) {
+// what a small rake of seeds waits for).  The look-up is inlined at every stage,
+// so forests without a tree have a kernel without the walk (24,000 lines of a
+// tricubic FP32 volume, RK4: 1,114 us, 1,227 with it, where 292 bytes spill instead
+// of 168); and the triquadratic BF16 kernel with trees is held to the 168 registers
+// that let three CTAs on an SM (100,000 lines of the 388,016-element flow, RK2: 2,143
+// us, 2,713 with 194).
+template <int P, int STORE, bool TREES>
+constexpr int line_min_ctas() { return P == 2 && STORE == LRVOL_STORE_BF16 && TREES ? 3 : 0; }
+
+template <int P, int STORE, bool TREES>
+__global__ void __launch_bounds__(128, (line_min_ctas<P, STORE, TREES>())) k_streamlines(
+    const __grid_constant__ SLParams sp, const double *__restrict__ seeds, int64_t n, int lanes,
+    SLSample *__restrict__ out, int32_t *__restrict__ count, int32_t *__restrict__ status) {
   if ((int)(threadIdx.x & 31) >= lanes) return;
   for (;;) {
     const int64_t q = (int64_t)atomicAdd(sp.queue, 1ull);
     if (q >= n) return;
-    trace_line<P, STORE>(sp, seeds, q, out, count, status);
+    trace_line<P, STORE, TREES>(sp, seeds, q, out, count, status);
   }
 }
 
@@ -1654,18 +1663,27 @@ __global__ void __launch_bounds__(128) k_streamline_error(const SLSample *__rest
 // Lines per warp up to which a line gets four lanes: as many as a warp has
 // groups of four.  250 lines of a triquadratic FP32 volume, RK4: 0.79 against
 // 1.13 ms with a lane each; 10,000 lines 1.45 against 1.83 (FP16 1.43 against
-// 1.76; tricubic 0.60 against 1.03; trilinear 0.112 against 0.117).
-constexpr int kGroupedLines = 8;
+// 1.76; tricubic 0.60 against 1.03).  Of a trilinear volume a group's exchange of a
+// stage's point outweighs a third of its evaluation once lanes are busy: up to
+// 5 lines a warp (RKF45 0.90, RK4 0.96 with 5), FP16 blocks 3 (1.02 with 4), and with
+// one stage a step 2 (RK1 0.90 with 1, 1.04 to 1.25 with 3), FP16 blocks none (1.10).
+template <int P, int STORE>
+static int grouped_lines(int method) {
+  if (P > 1) return 8;
+  if (method == LRVOL_RK1) return STORE == LRVOL_STORE_F16 ? 0 : 2;
+  return STORE == LRVOL_STORE_F16 ? 3 : 5;
+}
 
 template <int P, int STORE>
 cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSample *o, int32_t *count,
                       int32_t *status, cudaStream_t s) {
+  const bool trees = sp.forest.n_nodes > 0 || sp.forest.n_grid_units > 0;
+  auto *const single = trees ? k_streamlines<P, STORE, true> : k_streamlines<P, STORE, false>;
   int dev = 0, sms = 0, per_sm = 0, per_sm_group = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_streamlines<P, STORE>, 128, 0)) != cudaSuccess)
-    return e;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, single, 128, 0)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_group, k_streamlines_group<P, STORE>, 128, 0)) !=
       cudaSuccess)
     return e;
@@ -1675,7 +1693,7 @@ cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSamp
   const int64_t groups = (n + 4 * fit_group - 1) / (4 * fit_group);
   if ((e = cudaMemsetAsync(sp.queue, 0, sizeof(unsigned long long), s)) != cudaSuccess) return e;
   SLParams spl = sp;
-  const bool grouped = groups <= kGroupedLines;
+  const bool grouped = groups <= grouped_lines<P, STORE>(sp.method);
   spl.pair_out = grouped || lanes < 32;
   if (grouped) {
     const int64_t need = (n + 4 * groups - 1) / (4 * groups);
@@ -1683,7 +1701,7 @@ cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSamp
                                                                                      count, status);
   } else {
     const int64_t need = (n + 4 * lanes - 1) / (4 * lanes);
-    k_streamlines<P, STORE><<<(unsigned)std::min(need, fit), 128, 0, s>>>(spl, seeds, n, (int)lanes, o, count, status);
+    single<<<(unsigned)std::min(need, fit), 128, 0, s>>>(spl, seeds, n, (int)lanes, o, count, status);
   }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (spl.pair_out) {
@@ -1983,7 +2001,7 @@ __global__ void __launch_bounds__(128) k_tube_resolve(const __grid_constant__ Tu
   hcl = fminf(fmaxf(hcl, 0.f), 1.f);
 #pragma unroll
   for (int c = 0; c < 3; ++c) qa[c] = __fadd_rn(a[c], __fmul_rn(hcl, ba[c]));
-  SLField<P, STORE> F;
+  SLField<P, STORE, true> F;
   F.cur = kNone;
   float v0 = 0.f, v1 = 0.f, v2 = 0.f;
   F.eval(tp.field, qa[0], qa[1], qa[2], v0, v1, v2);

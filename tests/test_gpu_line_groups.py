@@ -1,7 +1,8 @@
 """Lines by four lanes against lines by one lane: the same seeds in a rake small
 enough for groups of lanes and repeated in one too large for them give the same
-bits, for every degree, storage and method, with lines that leave the cube, meet
-the cap, end at t_end, start outside, and run into a field that is not finite.
+bits, for every degree, storage and method, in forests with and without trees, with
+lines that leave the cube, meet the cap, end at t_end, start outside, and run into a
+field that is not finite.
 """
 import numpy as np
 import pytest
@@ -32,12 +33,14 @@ def _trace(gv, seeds, method, rule, h, tol):
 @pytest.mark.parametrize("storage", [lv.STORE_F32, lv.STORE_F16, lv.STORE_BF16])
 @pytest.mark.parametrize("deg", [1, 2, 3])
 @pytest.mark.parametrize("finite", [True, False])
-def test_groups_equal_single_lanes(deg, storage, finite):
-    vol = V.refined_ball((deg,) * 3, (3, 3, 3), radii=(0.35,), ncomp=3, seed=6)
+@pytest.mark.parametrize("side,blocks", [(3, 4), (4, 8)])     # a forest with trees, and one without
+def test_groups_equal_single_lanes(deg, storage, finite, side, blocks):
+    vol = V.refined_ball((deg,) * 3, (side,) * 3, radii=(0.35,), ncomp=3, seed=6)
     vol.coef = 2 * vol.coef - 1
     if not finite:
         vol.coef[len(vol.coef) // 2] = (np.inf, np.nan, 1.0)
-    gv = lv.Volume(vol).build_accel((4, 4, 4)).to_bezier(storage)
+    gv = lv.Volume(vol).build_accel((blocks,) * 3).to_bezier(storage)
+    assert (gv.stats()["n_nodes"] > 0) == (side == 3)
     few, reps = _seeds(37), 2400             # 88,800 lines: a lane each, every lane of a warp in use
     small = torch.from_numpy(few).cuda()
     large = small.repeat(reps, 1)
