@@ -1871,7 +1871,7 @@ __global__ void __launch_bounds__(32 * kTubeWarps) k_tube_raster(const __grid_co
                                                                  int split) {
   __shared__ TubeSlot slots[kTubeWarps][32];
   const int lane = threadIdx.x & 31;
-  const int64_t wid = (int64_t)blockIdx.x * kTubeWarps + (threadIdx.x >> 5);
+  const int64_t wid = ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * kTubeWarps + (threadIdx.x >> 5);
   const int64_t at = wid / split, line = at / strides;
   const int part = (int)(wid - at * split);
   if (line >= tp.n_lines) return;                      // whole warp
@@ -2045,8 +2045,10 @@ cudaError_t launch_tubes(TubeParams tp, int degree, int storage, cudaStream_t s)
     split = std::min<int64_t>(std::max<int64_t>(split, 1), 256);
     const int64_t strides = std::min<int64_t>(std::max<int64_t>(64 * (int64_t)sms / lines, 1), std::min<int64_t>(groups, 256));
     split = (split + strides - 1) / strides;
-    const int64_t warps = lines * strides * split;
-    k_tube_raster<<<(unsigned)((warps + kTubeWarps - 1) / kTubeWarps), 32 * kTubeWarps, 0, s>>>(tp, (int)strides, (int)split);
+    // up to 2^32 lines: in rows of CTAs past what one row holds
+    const int64_t ctas = (lines * strides * split + kTubeWarps - 1) / kTubeWarps, row = std::min(ctas, (int64_t)1 << 30);
+    const dim3 grid((unsigned)row, (unsigned)((ctas + row - 1) / row));
+    k_tube_raster<<<grid, 32 * kTubeWarps, 0, s>>>(tp, (int)strides, (int)split);
   }
   const unsigned blocks = (unsigned)((npix + 127) / 128);
 #define LRVOL_TUBE_CASE(P_, S_) k_tube_resolve<P_, S_><<<blocks, 128, 0, s>>>(tp)

@@ -78,3 +78,23 @@ def test_tubes_few_large_segments_split_over_warps():
     assert np.array_equal(img[..., 3] > 0, ref[..., 3] > 0)
     assert (ref[..., 3] > 0).mean() > 0.05
     assert np.abs(img - ref).max() <= 1e-4
+
+
+def test_tubes_of_more_lines_than_a_grid_row():
+    """2^31 + 3 lines of two samples (137 GB of them), all but three empty: the image of the three alone."""
+    n = 2 ** 31 + 3
+    if torch.cuda.mem_get_info()[0] < n * 68 + (1 << 33):
+        pytest.skip("needs 155 GB of device memory")
+    gv = lv.Volume(TU._field_z()).build_accel((8, 8, 8)).to_bezier()
+    s, c = TU._lines([[0.2, 0.3, 0.3], [0.5, 0.35, 0.4]], [[0.3, 0.8, 0.6], [0.45, 0.5, 0.5]], [[0.5, 0.2, 0.8], [0.55, 0.6, 0.2]])
+    s, c = torch.from_numpy(s).cuda(), torch.from_numpy(c.astype(np.int32)).cuda()
+    cam = V.orbit_camera(V.Stream(31), 96, 64)
+    want = lv.tubes(gv, cam, s, c, 0.06, TU._cmap())
+    at = torch.tensor([0, 2 ** 31 - 1, n - 1], device="cuda")
+    many, count = torch.empty((n, 2, 4), dtype=torch.float64, device="cuda"), torch.zeros(n, dtype=torch.int32, device="cuda")
+    many[at], count[at] = s, c
+    got = lv.tubes(gv, cam, many, count, 0.06, TU._cmap())
+    del many, count
+    torch.cuda.empty_cache()
+    gv.close()
+    assert (want[..., 3] > 0).float().mean() > 0.05 and torch.equal(got, want)
