@@ -120,26 +120,6 @@ __device__ __forceinline__ void dmonomials(float u, float *d) {
   }
 }
 
-// sum_{k,j,i} c[k][j][i] bx[i] by[j] bz[k], x fastest
-template <int P>
-__device__ __forceinline__ float contract(const float *c, const float *bx, const float *by, const float *bz) {
-  constexpr int N = P + 1;
-  float f = 0.f;
-#pragma unroll
-  for (int k = 0; k < N; ++k) {
-    float t = 0.f;
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      float s = 0.f;
-#pragma unroll
-      for (int i = 0; i < N; ++i) s = fmaf(c[(k * N + j) * N + i], bx[i], s);
-      t = fmaf(s, by[j], t);
-    }
-    f = fmaf(t, bz[k], f);
-  }
-  return f;
-}
-
 // u = (p - lo) / (hi - lo) as (p - lo_RU) * iw + (lo_RU - lo) * iw: one fused rounding after
 // the subtraction, which is exact when p is near lo_RU (the offset term is tiny).
 __device__ __forceinline__ float local_u(float p, float lo_ru, float off, float iw) {

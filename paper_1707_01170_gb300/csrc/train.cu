@@ -163,10 +163,12 @@ __device__ __forceinline__ void store_input_grad(float *h, const f2 (&acc)[R / 3
 // between barriers, not by the FMA rate (8,192 rows: 456 MFLOP, 6 us at the
 // FP32 peak): 29 us a step through the binding, against 3,558 us for a launch
 // per layer and direction whose weight-gradient threads walked all rows alone.
+// (One CTA an SM is stated: left open, the registers are cut to 80 and 100 of 169
+// and 145, and a step takes 2 us more.)
 template <int R>
-__global__ void __launch_bounds__(kTrainThreads, R == 32 ? 2 : 1) k_mlp_tiles(const float *__restrict__ x, const float *__restrict__ tgt,
-                                                            int64_t n, const float *__restrict__ p,
-                                                            float *__restrict__ part, float *__restrict__ loss_part) {
+__global__ void __launch_bounds__(kTrainThreads, 1) k_mlp_tiles(const float *__restrict__ x, const float *__restrict__ tgt,
+                                                                int64_t n, const float *__restrict__ p,
+                                                                float *__restrict__ part, float *__restrict__ loss_part) {
   extern __shared__ __align__(16) unsigned char train_smem[];
   TrainSmem<R> &S = *reinterpret_cast<TrainSmem<R> *>(train_smem);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
