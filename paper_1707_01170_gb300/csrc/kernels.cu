@@ -8,7 +8,7 @@
 //   k_streamlines, k_streamline_error, k_tube_*
 //                  Sec. 5 streamlines (Eq. 4 steps), the Eq. 7 error, tubes.
 //   k_trim_raster  Sec. 4.1 trimming: per-pixel interval of a boundary mesh.
-//   (k_render, the per-pixel ray casting of Sec. 4, is in render.cu, a volume's
+//   (k_render, the per-pixel ray casting of Sec. 4, is in render_kernel.cuh, a volume's
 //   change of basis in setup.cu, look-up and evaluation at points in points.cu;
 //   the device helpers these files share are in device_common.cuh.)
 #include <algorithm>

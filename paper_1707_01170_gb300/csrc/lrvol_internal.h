@@ -68,7 +68,7 @@ struct ForestView {
   const float4 *grids;           // GridUnit
   uint32_t n_grid_units;
   uint32_t head_sy, head_sz;     // strides of y and z
-  uint32_t head_bias;            // 0x4b000000 (1 + head_sy + head_sz) mod 2^32, see forest_lookup
+  uint32_t head_bias;            // 0x4b000000 (1 + head_sy + head_sz) mod 2^32, see forest_head
   float fbx, fby, fbz;           // block counts (powers of two)
 };
 

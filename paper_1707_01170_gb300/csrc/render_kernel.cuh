@@ -49,7 +49,9 @@ namespace {
 // code compiles out) runs the same march for a list of pixels, one thread per
 // listed pixel, and also writes each sample's (t, element id, field value,
 // segment length), the composited sample count and the pixel's RGBA.  It is
-// the parity hook that compares this kernel's own samples with the oracle.
+// the parity hook that compares a kernel's own samples with the oracle.  It takes
+// one sample a pass: the kernels that take two are held to its pixels and counts,
+// bit for bit, and to those of the untraced kernels that take one.
 //
 // FIELD 3 renders a scalar volume with gradient shading (Sec. 4.1): each
 // sample also evaluates the block's gradient, and C_src is scaled by
@@ -58,8 +60,8 @@ namespace {
 // 64 registers a lane (4 CTAs of 128 threads), 16-bit pairs of an FP16 block
 // 32 (5 CTAs); the triquadratic 3-vector FP16 block (42 registers instead of
 // 83) also fits 5.  The shaded tricubic kernel keeps the gradient's partial
-// sums too: at 4 CTAs it spills 88 bytes and still beats 3 CTAs without
-// spills by 5 % (measured); forcing 5 CTAs on the FP32 kernels spills
+// sums too: at 4 CTAs it spills (16 bytes without trees, up to 40 with them)
+// and still beats 3 CTAs without spills by 5 % (measured); forcing 5 CTAs on the FP32 kernels spills
 // inside the sample loop and costs 37-51 %.
 template <int P, int FIELD, int STORE>
 constexpr int render_min_ctas() {

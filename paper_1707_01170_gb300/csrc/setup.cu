@@ -818,7 +818,10 @@ cudaError_t launch_to_bezier(const lrvol_s *v, int32_t *todo, uint32_t *n_todo, 
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (v->n_basis <= 32) return e;   // no list that the kernel leaves over
-    blocks = std::min<int64_t>(blocks, 1216);   // usually nothing is left: a grid that strides over the list
+    int dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+    blocks = std::min<int64_t>(blocks, 8 * sms);   // usually nothing is left: a grid that strides over the list
   }
   k_to_bezier<<<(unsigned)blocks, 32 * kBezWarps, 0, s>>>(v->d_box, v->d_knots, v->d_coef, v->d_weight, v->d_inc_ptr,
                                                          v->d_inc_idx, v->p[0], v->p[1], v->p[2], v->nc, v->kw,
