@@ -13,6 +13,7 @@
 //   the device helpers these files share are in device_common.cuh.)
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "device_common.cuh"
 
@@ -560,7 +561,11 @@ __global__ void __launch_bounds__(128) k_labels_lane(const __grid_constant__ Ren
 // rays: 12.0 ms for a 320x180 camera of a 174,000-element tricubic volume with
 // seven candidates, 2.8 ms here.  Held to 128 registers for four CTAs an SM: with the 146 it
 // would take, three fit and it is a fifth slower, and five CTAs spill.
-template <int P>
+// EARLY: longer candidates than one that failed get no end.  The votes and registers
+// for it cost up to 3 % of a march, so it is taken where the longest candidate reaches
+// past 2.5 chunks (seven candidates, 320x180, h_fine 1/2048: trilinear volume 1.47 ->
+// 0.76 ms, tricubic 1.60 -> 1.46; candidates up to 64 steps 4.84 -> 1.96).
+template <int P, bool EARLY>
 __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ RenderParams prm, float h_fine, float tau,
                                                 const float *__restrict__ cand, int n_cand,
                                                 int32_t *__restrict__ label) {
@@ -655,11 +660,7 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
     // fine composites over [t, te)
     float F0 = 0.f, F1 = 0.f, F2 = 0.f, FT = 1.f;
     bool need = lane < n_cand && t < te;
-    auto last_end = [&]() { return __uint_as_float(__reduce_max_sync(kAll, need ? __float_as_uint(te) : 0u)); };   // te >= 0
-    auto error = [&]() {
-      return Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
-    };
-    float te_max = last_end();
+    const float te_max = __uint_as_float(__reduce_max_sync(kAll, need ? __float_as_uint(te) : 0u));   // te >= 0
     // fine samples before te: a quotient, corrected with the samples' own places
     int nf = 0;
     if (need) {
@@ -668,8 +669,8 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
       while (nf < kMaxSamplesPerRay && __fmaf_rn((float)nf, h_fine, t) < te) ++nf;
     }
     float cT = 1.f, cC0 = 0.f, cC1 = 0.f, cC2 = 0.f;   // composite of the earlier chunks
-    unsigned open_ends = __ballot_sync(kAll, need);
-    for (int kb = 0; kb < kMaxSamplesPerRay && open_ends; kb += 32) {
+    unsigned open_ends = EARLY ? __ballot_sync(kAll, need) : 0u;
+    for (int kb = 0; kb < kMaxSamplesPerRay && (EARLY ? open_ends != 0u : __any_sync(kAll, need)); kb += 32) {
       const float ts = __fmaf_rn((float)(kb + lane), h_fine, t), tn = __fmaf_rn((float)(kb + lane + 1), h_fine, t);
       const bool act = ts < te_max;
       float4 src = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -709,20 +710,21 @@ __global__ void __launch_bounds__(128, 4) k_labels(const __grid_constant__ Rende
       cC0 += __shfl_sync(kAll, s0, 31);
       cC1 += __shfl_sync(kAll, s1, 31);
       cC2 += __shfl_sync(kAll, s2, 31);
-      const unsigned before_chunk = open_ends;
-      open_ends = __ballot_sync(kAll, need);
-      // candidates ended while others are open: the label is the one before the first
-      // that fails, so those behind a failed one need no end
-      if ((before_chunk & ~open_ends) > 1u && open_ends > 1u) {
-        const unsigned failed = __ballot_sync(kAll, is_cand && fin && !(error() <= tau));
-        if (failed) {
-          need &= lane < __ffs(failed);
-          te_max = last_end();
-          open_ends = __ballot_sync(kAll, need);
+      if constexpr (EARLY) {
+        // the label is the candidate before the first that fails: those behind one that failed need no end
+        open_ends = __ballot_sync(kAll, need);
+        if (open_ends > 1u) {
+          const float err = Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
+          const unsigned failed = __ballot_sync(kAll, is_cand && fin && !(err <= tau));
+          if (failed) {
+            need &= lane < __ffs(failed);
+            open_ends &= failed ^ (failed - 1u);   // up to the first that failed
+          }
         }
       }
     }
-    const unsigned bad = __ballot_sync(kAll, is_cand && !(error() <= tau));
+    const float err = Tfront * fmaxf(fmaxf(fabsf(A0 - F0), fabsf(A1 - F1)), fmaxf(fabsf(A2 - F2), fabsf(AT - FT)));
+    const unsigned bad = __ballot_sync(kAll, is_cand && !(err <= tau));
     if (lane == 0) atomicMin(label + e, bad ? __ffs(bad) - 2 : n_cand - 1);
     Tfront *= __shfl_sync(kAll, FT, 0);
     t = tb;
@@ -773,6 +775,11 @@ cudaError_t launch_mlp_infer(const float *x, int64_t n, const uint16_t *packed, 
   return cudaGetLastError();
 }
 
+struct LabelRoute {
+  bool by_lane;   // k_labels_lane; else k_labels ...
+  bool early;     // ... with EARLY
+};
+
 // Whether a lane a ray is faster than a warp a ray.  A warp wastes lanes on a visit
 // of few samples, lanes need many rays to fill the GPU and march again for every
 // candidate.  Per ray and visit the lane's work is its samples (1 + 0.091 each), the
@@ -785,8 +792,8 @@ cudaError_t launch_mlp_infer(const float *x, int64_t n, const uint16_t *packed, 
 // in which the choice is within 5 % of the faster kernel for 97 % and 0.5 % on average.
 // 174,000 tricubic elements, lane / warp: 640x360 rays, one candidate, h_fine 1/256 0.49 /
 // 4.9 ms; 320x180, seven candidates, h_fine 1/2048 12.0 / 2.8 ms.
-static bool labels_by_lane(const LabelCost &cost, int64_t rays, int sms, double h_fine, double tau, const float *cand,
-                           int n_cand) {
+static LabelRoute label_route(const LabelCost &cost, int64_t rays, int sms, double h_fine, double tau, const float *cand,
+                              int n_cand) {
   const double pass = 1 / (1 + std::exp(-2.23 - 0.66 * std::log10(tau / 4e-4)));
   double samples = cost.chord / h_fine, farthest = cost.chord, steps = 0, reached = 1;
   for (int c = 1; c < n_cand; ++c) {
@@ -797,8 +804,10 @@ static bool labels_by_lane(const LabelCost &cost, int64_t rays, int sms, double 
     steps = std::max(steps, length / sc);
   }
   const double per_sm = (double)rays / sms;
-  return 1.29 * (1 + 0.091 * samples) * (1 + per_sm / 2540) <
-         1.05 * (1 + 0.257 * farthest / (32 * h_fine) + 0.0256 * steps) * (1 + per_sm / 85);
+  const double chunks = farthest / (32 * h_fine);
+  return {1.29 * (1 + 0.091 * samples) * (1 + per_sm / 2540) <
+              1.05 * (1 + 0.257 * chunks + 0.0256 * steps) * (1 + per_sm / 85),
+          n_cand > 1 && chunks > 2.5};
 }
 
 cudaError_t launch_labels(const RenderParams &prm, int degree, const LabelCost &cost, float h_fine, float tau,
@@ -808,22 +817,23 @@ cudaError_t launch_labels(const RenderParams &prm, int degree, const LabelCost &
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const int w = prm.width, h = prm.row_end - prm.row_begin;
-  if (labels_by_lane(cost, (int64_t)w * h, sms, h_fine, tau, cand_host, n_cand)) {
-    const dim3 grid((unsigned)((w + 15) / 16), (unsigned)((h + 7) / 8));
-    switch (degree) {
-      case 1: k_labels_lane<1><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-      case 2: k_labels_lane<2><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-      case 3: k_labels_lane<3><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-      default: return cudaErrorInvalidValue;
-    }
-  } else {
-    const dim3 grid((unsigned)((w + 1) / 2), (unsigned)((h + 1) / 2));   // four rays a CTA, a 2x2 patch
-    switch (degree) {
-      case 1: k_labels<1><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-      case 2: k_labels<2><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-      case 3: k_labels<3><<<grid, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label); break;
-      default: return cudaErrorInvalidValue;
-    }
+  const LabelRoute route = label_route(cost, (int64_t)w * h, sms, h_fine, tau, cand_host, n_cand);
+  auto launch = [&](auto degree_c) {
+    constexpr int P = decltype(degree_c)::value;
+    const dim3 patches((unsigned)((w + 1) / 2), (unsigned)((h + 1) / 2));   // four rays a CTA, a 2x2 patch
+    if (route.by_lane)
+      k_labels_lane<P><<<dim3((unsigned)((w + 15) / 16), (unsigned)((h + 7) / 8)), 128, 0, s>>>(prm, h_fine, tau, cand,
+                                                                                             n_cand, label);
+    else if (route.early)
+      k_labels<P, true><<<patches, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label);
+    else
+      k_labels<P, false><<<patches, 128, 0, s>>>(prm, h_fine, tau, cand, n_cand, label);
+  };
+  switch (degree) {
+    case 1: launch(std::integral_constant<int, 1>()); break;
+    case 2: launch(std::integral_constant<int, 2>()); break;
+    case 3: launch(std::integral_constant<int, 3>()); break;
+    default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();
 }
