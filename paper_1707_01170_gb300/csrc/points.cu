@@ -36,8 +36,9 @@ __device__ __forceinline__ uint32_t find_element(const ForestView &f, int64_t n_
 
 // One point a thread, with the renderer's block code (256-bit loads, packed
 // FP32 contraction): a dependent head load, then the record and the block.
-// Scattered points are bound by the L2: 1,000,003 gradients of a tricubic FP32
-// volume read 336 bytes each and take 52 us, 6.5 TB/s (350 us when the block
+// Scattered points are bound by L1's data path, 86 % busy (a scattered 256-bit
+// load is eight wavefronts), with the L2 at 58 % of its rate: 1,000,003 gradients of
+// a tricubic FP32 volume read 336 bytes each and take 52 us (350 us when the block
 // went through a local array, a scalar load a coefficient, under loops over
 // any degree); points in grid order share blocks and take 29 us (190).
 // Gathering a warp's blocks to shared memory with neighbouring lanes on one
