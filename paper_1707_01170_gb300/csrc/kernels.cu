@@ -790,7 +790,7 @@ struct LabelRoute {
 // larger tau is.  The constants are a fit to 5,271 timings (seven volumes of degree 1 to
 // 3, 64x36 to 1280x720 rays, 1 to 16 candidates, h_fine 1/64 to 1/8192, tau 1e-5 to 1e-2),
 // in which the choice is within 5 % of the faster kernel for 97 % and 0.5 % on average.
-// 174,000 tricubic elements, lane / warp: 640x360 rays, one candidate, h_fine 1/256 0.49 /
+// 174,000 tricubic elements, lane / warp: 640x360 rays, one candidate, h_fine 1/256 0.51 /
 // 4.9 ms; 320x180, seven candidates, h_fine 1/2048 12.0 / 2.8 ms.
 static LabelRoute label_route(const LabelCost &cost, int64_t rays, int sms, double h_fine, double tau, const float *cand,
                               int n_cand) {
