@@ -1389,14 +1389,9 @@ __device__ __forceinline__ void trace_line(const SLParams &sp, const double *__r
 // what a small rake of seeds waits for).  The look-up is inlined at every stage,
 // so forests without a tree have a kernel without the walk (24,000 lines of a
 // tricubic FP32 volume, RK4: 1,114 us, 1,227 with it, where 292 bytes spill instead
-// of 168); and the triquadratic BF16 kernel with trees is held to the 168 registers
-// that let three CTAs on an SM (100,000 lines of the 388,016-element flow, RK2: 2,143
-// us, 2,713 with 194).
-template <int P, int STORE, bool TREES>
-constexpr int line_min_ctas() { return P == 2 && STORE == LRVOL_STORE_BF16 && TREES ? 3 : 0; }
-
-template <int P, int STORE, bool TREES>
-__global__ void __launch_bounds__(128, (line_min_ctas<P, STORE, TREES>())) k_streamlines(
+// of 168).  MIN: CTAs on an SM that the registers have to allow, 0 for any (launch_sl).
+template <int P, int STORE, bool TREES, int MIN>
+__global__ void __launch_bounds__(128, MIN) k_streamlines(
     const __grid_constant__ SLParams sp, const double *__restrict__ seeds, int64_t n, int lanes,
     SLSample *__restrict__ out, int32_t *__restrict__ count, int32_t *__restrict__ status) {
   if ((int)(threadIdx.x & 31) >= lanes) return;
@@ -1688,7 +1683,7 @@ template <int P, int STORE>
 cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSample *o, int32_t *count,
                       int32_t *status, cudaStream_t s) {
   const bool trees = sp.forest.n_nodes > 0 || sp.forest.n_grid_units > 0;
-  auto *const single = trees ? k_streamlines<P, STORE, true> : k_streamlines<P, STORE, false>;
+  auto *single = trees ? k_streamlines<P, STORE, true, 0> : k_streamlines<P, STORE, false, 0>;
   int dev = 0, sms = 0, per_sm = 0, per_sm_group = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1697,6 +1692,16 @@ cudaError_t launch_sl(const SLParams &sp, const double *seeds, int64_t n, SLSamp
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm_group, k_streamlines_group<P, STORE>, 128, 0)) !=
       cudaSuccess)
     return e;
+  // The triquadratic BF16 kernel with trees takes 194 registers, two CTAs an SM; held to
+  // the 168 that allow three it spills, and is faster once lines are 1.5 times the two CTAs'
+  // lanes (the 388,016-element flow, RK2 / RK4, 100,000 lines: 2,143 / 2,561 us, 2,713 /
+  // 3,111 with two; 40,000 lines 1,419 / 1,756, 1,389 / 1,647 with two).
+  if constexpr (P == 2 && STORE == LRVOL_STORE_BF16) {
+    if (trees && per_sm < 3 && 2 * n > 3 * 128 * (int64_t)sms * std::max(per_sm, 1)) {
+      single = k_streamlines<P, STORE, true, 3>;
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, single, 128, 0)) != cudaSuccess) return e;
+    }
+  }
   const int64_t fit = (int64_t)sms * std::max(per_sm, 1);               // resident CTAs of 4 warps
   const int64_t fit_group = (int64_t)sms * std::max(per_sm_group, 1);
   int64_t lanes = std::min<int64_t>(std::max<int64_t>((n + 4 * fit - 1) / (4 * fit), 1), 32);   // lines per warp
